@@ -1,8 +1,11 @@
-"""ctypes binding of libquantpipe.so: argument marshalling only.
+"""Binding of libquantpipe.so: argument marshalling only.
 
 Every step of the path runs in the CUDA library; this module turns torch tensors into
-pointers and sizes, passes the current CUDA stream, and raises on error codes.  There is no
-CPU fallback: if the library has not been built, loading fails with an error.
+pointers and sizes, passes the current CUDA stream, and raises on error codes.  ctypes loads
+the library and calls its host functions; the calls that enqueue work on the GPU go through
+the small extension module _qpcall (csrc/qp_call.c), because at the sizes of one image the
+marshalling is what such a call costs.  There is no CPU fallback: if the library has not been
+built, loading fails with an error.
 """
 from __future__ import annotations
 
@@ -84,6 +87,8 @@ class QuantPipeError(RuntimeError):
 
 
 _lib = None
+_call = _call64 = _tensor_in = None                 # of _qpcall, once load() has run
+_addr: dict = {}                                    # addresses of the entry points called through it
 
 
 def load() -> C.CDLL:
@@ -164,8 +169,22 @@ def load() -> C.CDLL:
         if name not in ("qp_last_error", "qp_status_string", "qp_packed_bytes", "qp_aciq_F", "qp_launch_count",
                         "qp_controller_payload_bytes", "qp_graph_replays"):
             fn.restype = i32
+    _load_call_path(L)
     _lib = L
     return L
+
+
+def _load_call_path(L: C.CDLL) -> None:
+    global _call, _call64, _tensor_in
+    try:
+        from . import _qpcall
+    except ImportError as e:
+        raise RuntimeError("_qpcall is missing: build it with `python -m paper_2211_04515_b200.build` "
+                           "(there is no CPU fallback)") from e
+    _qpcall.setup(torch.float32, torch.bfloat16)
+    _call, _call64, _tensor_in = _qpcall.call, _qpcall.call64, _qpcall.tensor_in
+    for name in EXPORTS:
+        _addr[name] = C.cast(getattr(L, name), C.c_void_p).value
 
 
 # ------------------------------------------------------------- host, pure
@@ -284,6 +303,17 @@ def _stream(device) -> int:
     return torch.cuda.current_stream(device).cuda_stream
 
 
+_raw_stream = torch._C._cuda_getCurrentRawStream    # device index -> current stream, without the Stream object
+
+
+def _input(x: torch.Tensor):
+    """(numel, dtype code) of a contiguous CUDA tensor of a dtype that the library takes."""
+    n, code = _tensor_in(x)
+    if code < 0:
+        raise QuantPipeError(QP_ERR_UNSUPPORTED_DTYPE, f"unsupported dtype {x.dtype}")
+    return n, code
+
+
 def _as_struct(t: torch.Tensor, cls):
     """Copies a device byte buffer holding one struct to the host (synchronises)."""
     raw = t.detach().cpu().contiguous().numpy().tobytes()
@@ -299,16 +329,18 @@ class Context:
             raise QuantPipeError(QP_ERR_INVALID_ARG, "a CUDA device is required")
         self.device = torch.device("cuda", dev.index if dev.index is not None else torch.cuda.current_device())
         self._lib = load()
+        self._index = self.device.index
         handle = C.c_void_p()
         rc = self._lib.qp_create(self.device.index, C.byref(handle))
         if rc != QP_OK:
             raise QuantPipeError(rc, "qp_create failed: " + qp_status_string(rc))
         self._h = handle
+        self._hv = handle.value                     # the same as a plain integer, for _call
 
     def close(self):
         if getattr(self, "_h", None):
             self._lib.qp_destroy(self._h)
-            self._h = None
+            self._h = self._hv = None
 
     def __del__(self):
         try:
@@ -322,25 +354,33 @@ class Context:
             raise QuantPipeError(rc, self._lib.qp_last_error(self._h).decode())
         return int(rc)
 
+    def _run(self, name: str, *args) -> None:
+        """One call on this context and torch's current stream (the last parameter of every device call)."""
+        rc = _call(_addr[name], self._hv, *args, _raw_stream(self._index))
+        if rc < 0:
+            self._check(rc)
+
     def _bytes(self, nbytes: int) -> torch.Tensor:
         return torch.empty(nbytes, dtype=torch.uint8, device=self.device)
 
+    def _packed(self, n: int, bits: int) -> torch.Tensor:
+        return self._bytes(_call64(_addr["qp_packed_bytes"], n, bits))
+
     def _qp_arg(self, qp):
-        """(pointer, on_device, keepalive) for a host QParams struct or a device byte tensor."""
+        """(pointer, on_device) for a host QParams struct or a device byte tensor; `qp` outlives the call."""
         if isinstance(qp, QParams):
-            return C.cast(C.pointer(qp), C.c_void_p), 0, qp
+            return C.addressof(qp), 0
         if isinstance(qp, torch.Tensor) and qp.is_cuda:
-            return C.c_void_p(qp.data_ptr()), 1, qp
+            return qp, 1
         raise QuantPipeError(QP_ERR_INVALID_ARG, "qp must be a QParams struct or a device tensor")
 
     # -- a1
     def qp_stats(self, x: torch.Tensor, out: torch.Tensor | None = None, hist_bins: int = 0) -> torch.Tensor:
         """Statistics of x into an 80-byte device buffer (returned); hist_bins > 0 also asks
         for the peak of the search's histogram."""
-        assert x.is_cuda and x.is_contiguous()
+        n, code = _input(x)
         out = self._bytes(C.sizeof(Stats)) if out is None else out
-        self._check(self._lib.qp_stats(self._h, x.data_ptr(), _dtype_code(x), x.numel(), hist_bins, out.data_ptr(),
-                                       _stream(self.device)))
+        self._run("qp_stats", x, code, n, hist_bins, out)
         return out
 
     # -- a3
@@ -348,15 +388,13 @@ class Context:
                                dist: int = QP_DIST_LAPLACE, bmode: int = QP_B_MAD,
                                out: torch.Tensor | None = None) -> torch.Tensor:
         out = self._bytes(C.sizeof(QParams)) if out is None else out
-        self._check(self._lib.qp_clip_qparams_device(self._h, d_stats.data_ptr(), bits, method, dist, bmode,
-                                                     out.data_ptr(), _stream(self.device)))
+        self._run("qp_clip_qparams_device", d_stats, bits, method, dist, bmode, out)
         return out
 
     def qp_aciq_qparams_device(self, d_stats: torch.Tensor, bits: int, dist: int = QP_DIST_LAPLACE,
                                bmode: int = QP_B_MAD, out: torch.Tensor | None = None) -> torch.Tensor:
         out = self._bytes(C.sizeof(QParams)) if out is None else out
-        self._check(self._lib.qp_aciq_qparams_device(self._h, d_stats.data_ptr(), bits, dist, bmode, out.data_ptr(),
-                                                     _stream(self.device)))
+        self._run("qp_aciq_qparams_device", d_stats, bits, dist, bmode, out)
         return out
 
     # -- a2 + a4
@@ -364,12 +402,10 @@ class Context:
                          steps: int = QP_DEFAULT_STEPS, hist_bins: int = QP_DEFAULT_HIST_BINS,
                          out_result: torch.Tensor | None = None, out_qp: torch.Tensor | None = None):
         """Directed search; returns (device DSResult bytes, device QParams bytes)."""
-        assert x.is_cuda and x.is_contiguous()
+        n, code = _input(x)
         out_result = self._bytes(C.sizeof(DSResult)) if out_result is None else out_result
         out_qp = self._bytes(C.sizeof(QParams)) if out_qp is None else out_qp
-        self._check(self._lib.qp_dsaciq_search(self._h, x.data_ptr(), _dtype_code(x), x.numel(), d_stats.data_ptr(),
-                                               bits, bmode, steps, hist_bins, out_result.data_ptr(), out_qp.data_ptr(),
-                                               _stream(self.device)))
+        self._run("qp_dsaciq_search", x, code, n, d_stats, bits, bmode, steps, hist_bins, out_result, out_qp)
         return out_result, out_qp
 
     def qp_set_search_path(self, path: int):
@@ -411,14 +447,11 @@ class Context:
 
     # -- a5
     def qp_quantize_pack(self, x: torch.Tensor, bits: int, qp, out: torch.Tensor | None = None) -> torch.Tensor:
-        assert x.is_cuda and x.is_contiguous()
-        need = qp_packed_bytes(x.numel(), bits)
+        n, code = _input(x)
         if out is None:
-            out = self._bytes(need)
-        ptr, on_dev, _keep = self._qp_arg(qp)
-        self._check(self._lib.qp_quantize_pack(self._h, x.data_ptr(), _dtype_code(x), x.numel(), bits, ptr, on_dev,
-                                               out.data_ptr(), out.numel() * out.element_size(),
-                                               _stream(self.device)))
+            out = self._packed(n, bits)
+        ptr, on_dev = self._qp_arg(qp)
+        self._run("qp_quantize_pack", x, code, n, bits, ptr, on_dev, out, out.nbytes)
         return out
 
     # -- a6
@@ -427,13 +460,12 @@ class Context:
         assert packed.is_cuda and packed.is_contiguous()
         if out is None:
             out = torch.empty(n, dtype=out_dtype, device=self.device)
-        assert out.numel() >= n and out.is_contiguous()
-        need = qp_packed_bytes(n, bits)
-        if packed.numel() * packed.element_size() < need:
+        room, code = _input(out)
+        assert room >= n
+        if packed.nbytes < _call64(_addr["qp_packed_bytes"], n, bits):
             raise QuantPipeError(QP_ERR_BUFFER_TOO_SMALL, "packed buffer shorter than qp_packed_bytes(n, bits)")
-        ptr, on_dev, _keep = self._qp_arg(qp)
-        self._check(self._lib.qp_unpack_dequantize(self._h, packed.data_ptr(), n, bits, ptr, on_dev, out.data_ptr(),
-                                                   _dtype_code(out), _stream(self.device)))
+        ptr, on_dev = self._qp_arg(qp)
+        self._run("qp_unpack_dequantize", packed, n, bits, ptr, on_dev, out, code)
         return out
 
     # -- whole sender on device buffers
@@ -442,22 +474,19 @@ class Context:
                          bmode: int = QP_B_MAD, steps: int = QP_DEFAULT_STEPS, hist_bins: int = QP_DEFAULT_HIST_BINS):
         """stats -> clip -> quantize+pack in one call; returns (packed, device QParams bytes).
         use_ds: False/True (ACIQ / directed search) or a QP_CLIP_* method."""
-        assert x.is_cuda and x.is_contiguous()
-        out_packed = self._bytes(qp_packed_bytes(x.numel(), bits)) if out_packed is None else out_packed
+        n, code = _input(x)
+        out_packed = self._packed(n, bits) if out_packed is None else out_packed
         out_qp = self._bytes(C.sizeof(QParams)) if out_qp is None else out_qp
-        self._check(self._lib.qp_sender_device(self._h, x.data_ptr(), _dtype_code(x), x.numel(), bits,
-                                               int(use_ds), bmode, steps, hist_bins, out_packed.data_ptr(),
-                                               out_packed.numel() * out_packed.element_size(), out_qp.data_ptr(),
-                                               out_stats.data_ptr() if out_stats is not None else None,
-                                               _stream(self.device)))
+        self._run("qp_sender_device", x, code, n, bits, int(use_ds), bmode, steps, hist_bins, out_packed, out_packed.nbytes,
+                  out_qp, out_stats)
         return out_packed, out_qp
 
     # -- channel-wise variant: x is [rows, channels], the last dimension contiguous
     def qp_stats_channels(self, x: torch.Tensor, channels: int, out: torch.Tensor | None = None) -> torch.Tensor:
-        assert x.is_cuda and x.is_contiguous() and x.numel() % channels == 0
+        n, code = _input(x)
+        assert n % channels == 0
         out = self._bytes(C.sizeof(Stats) * channels) if out is None else out
-        self._check(self._lib.qp_stats_channels(self._h, x.data_ptr(), _dtype_code(x), x.numel() // channels, channels,
-                                                out.data_ptr(), _stream(self.device)))
+        self._run("qp_stats_channels", x, code, n // channels, channels, out)
         return out
 
     def qp_dsaciq_search_channels(self, x: torch.Tensor, channels: int, d_stats: torch.Tensor, bits: int,
@@ -465,12 +494,12 @@ class Context:
                                   hist_bins: int = QP_DEFAULT_HIST_BINS, out_result: torch.Tensor | None = None,
                                   out_qp: torch.Tensor | None = None):
         """Directed search per channel; returns (device DSResult[channels] bytes, device QParams[channels] bytes)."""
-        assert x.is_cuda and x.is_contiguous() and x.numel() % channels == 0
+        n, code = _input(x)
+        assert n % channels == 0
         out_result = self._bytes(C.sizeof(DSResult) * channels) if out_result is None else out_result
         out_qp = self._bytes(C.sizeof(QParams) * channels) if out_qp is None else out_qp
-        self._check(self._lib.qp_dsaciq_search_channels(self._h, x.data_ptr(), _dtype_code(x), x.numel() // channels,
-                                                        channels, d_stats.data_ptr(), bits, bmode, steps, hist_bins,
-                                                        out_result.data_ptr(), out_qp.data_ptr(), _stream(self.device)))
+        self._run("qp_dsaciq_search_channels", x, code, n // channels, channels, d_stats, bits, bmode, steps, hist_bins,
+                  out_result, out_qp)
         return out_result, out_qp
 
     def qp_dsaciq_curve_channels(self, channel: int, steps: int):
@@ -482,86 +511,77 @@ class Context:
                                         dist: int = QP_DIST_LAPLACE, bmode: int = QP_B_MAD,
                                         out: torch.Tensor | None = None) -> torch.Tensor:
         out = self._bytes(C.sizeof(QParams) * channels) if out is None else out
-        self._check(self._lib.qp_clip_qparams_channels_device(self._h, d_stats.data_ptr(), channels, bits, method, dist,
-                                                              bmode, out.data_ptr(), _stream(self.device)))
+        self._run("qp_clip_qparams_channels_device", d_stats, channels, bits, method, dist, bmode, out)
         return out
 
     def qp_quantize_pack_channels(self, x: torch.Tensor, channels: int, bits: int, d_qp: torch.Tensor,
                                   out: torch.Tensor | None = None) -> torch.Tensor:
-        assert x.is_cuda and x.is_contiguous() and x.numel() % channels == 0
-        out = self._bytes(qp_packed_bytes(x.numel(), bits)) if out is None else out
-        self._check(self._lib.qp_quantize_pack_channels(self._h, x.data_ptr(), _dtype_code(x), x.numel() // channels,
-                                                        channels, bits, d_qp.data_ptr(), out.data_ptr(),
-                                                        out.numel() * out.element_size(), _stream(self.device)))
+        n, code = _input(x)
+        assert n % channels == 0
+        out = self._packed(n, bits) if out is None else out
+        self._run("qp_quantize_pack_channels", x, code, n // channels, channels, bits, d_qp, out, out.nbytes)
         return out
 
     def qp_unpack_dequantize_channels(self, packed: torch.Tensor, rows: int, channels: int, bits: int, d_qp: torch.Tensor,
                                       out: torch.Tensor | None = None, out_dtype=torch.float32) -> torch.Tensor:
         out = torch.empty(rows * channels, dtype=out_dtype, device=packed.device) if out is None else out
-        self._check(self._lib.qp_unpack_dequantize_channels(self._h, packed.data_ptr(), rows, channels, bits,
-                                                            d_qp.data_ptr(), out.data_ptr(), _dtype_code(out),
-                                                            _stream(self.device)))
+        self._run("qp_unpack_dequantize_channels", packed, rows, channels, bits, d_qp, out, _dtype_code(out))
         return out
 
     def qp_sender_channels_device(self, x: torch.Tensor, channels: int, bits: int, method: int = QP_CLIP_ACIQ,
                                   bmode: int = QP_B_MAD, out_packed: torch.Tensor | None = None,
                                   out_qp: torch.Tensor | None = None, out_stats: torch.Tensor | None = None):
         """Channel-wise statistics -> clip -> quantize+pack in one call; returns (packed, device QParams[channels])."""
-        assert x.is_cuda and x.is_contiguous() and x.numel() % channels == 0
-        out_packed = self._bytes(qp_packed_bytes(x.numel(), bits)) if out_packed is None else out_packed
+        n, code = _input(x)
+        assert n % channels == 0
+        out_packed = self._packed(n, bits) if out_packed is None else out_packed
         out_qp = self._bytes(C.sizeof(QParams) * channels) if out_qp is None else out_qp
-        self._check(self._lib.qp_sender_channels_device(
-            self._h, x.data_ptr(), _dtype_code(x), x.numel() // channels, channels, bits, method, bmode,
-            out_packed.data_ptr(), out_packed.numel() * out_packed.element_size(), out_qp.data_ptr(),
-            out_stats.data_ptr() if out_stats is not None else None, _stream(self.device)))
+        self._run("qp_sender_channels_device", x, code, n // channels, channels, bits, method, bmode, out_packed,
+                  out_packed.nbytes, out_qp, out_stats)
         return out_packed, out_qp
 
     # -- token-wise variant: x is [tokens, channels], a token = a row of `channels` contiguous elements
     def qp_stats_tokens(self, x: torch.Tensor, channels: int, out: torch.Tensor | None = None) -> torch.Tensor:
-        assert x.is_cuda and x.is_contiguous() and x.numel() % channels == 0
-        tokens = x.numel() // channels
+        n, code = _input(x)
+        assert n % channels == 0
+        tokens = n // channels
         out = self._bytes(C.sizeof(Stats) * tokens) if out is None else out
-        self._check(self._lib.qp_stats_tokens(self._h, x.data_ptr(), _dtype_code(x), tokens, channels, out.data_ptr(),
-                                              _stream(self.device)))
+        self._run("qp_stats_tokens", x, code, tokens, channels, out)
         return out
 
     def qp_clip_qparams_tokens_device(self, d_stats: torch.Tensor, tokens: int, bits: int, method: int = QP_CLIP_ACIQ,
                                       dist: int = QP_DIST_LAPLACE, bmode: int = QP_B_MAD,
                                       out: torch.Tensor | None = None) -> torch.Tensor:
         out = self._bytes(C.sizeof(QParams) * tokens) if out is None else out
-        self._check(self._lib.qp_clip_qparams_tokens_device(self._h, d_stats.data_ptr(), tokens, bits, method, dist, bmode,
-                                                            out.data_ptr(), _stream(self.device)))
+        self._run("qp_clip_qparams_tokens_device", d_stats, tokens, bits, method, dist, bmode, out)
         return out
 
     def qp_quantize_pack_tokens(self, x: torch.Tensor, channels: int, bits: int, d_qp: torch.Tensor,
                                 out: torch.Tensor | None = None) -> torch.Tensor:
-        assert x.is_cuda and x.is_contiguous() and x.numel() % channels == 0
-        out = self._bytes(qp_packed_bytes(x.numel(), bits)) if out is None else out
-        self._check(self._lib.qp_quantize_pack_tokens(self._h, x.data_ptr(), _dtype_code(x), x.numel() // channels, channels,
-                                                      bits, d_qp.data_ptr(), out.data_ptr(),
-                                                      out.numel() * out.element_size(), _stream(self.device)))
+        n, code = _input(x)
+        assert n % channels == 0
+        out = self._packed(n, bits) if out is None else out
+        self._run("qp_quantize_pack_tokens", x, code, n // channels, channels, bits, d_qp, out, out.nbytes)
         return out
 
     def qp_unpack_dequantize_tokens(self, packed: torch.Tensor, tokens: int, channels: int, bits: int, d_qp: torch.Tensor,
                                     out: torch.Tensor | None = None, out_dtype=torch.float32) -> torch.Tensor:
         out = torch.empty(tokens * channels, dtype=out_dtype, device=packed.device) if out is None else out
-        self._check(self._lib.qp_unpack_dequantize_tokens(self._h, packed.data_ptr(), tokens, channels, bits,
-                                                          d_qp.data_ptr(), out.data_ptr(), _dtype_code(out),
-                                                          _stream(self.device)))
+        self._run("qp_unpack_dequantize_tokens", packed, tokens, channels, bits, d_qp, out, _dtype_code(out))
         return out
 
     def qp_sender_tokens_device(self, x: torch.Tensor, channels: int, bits: int, method: int = QP_CLIP_ACIQ,
                                 bmode: int = QP_B_MAD, out_packed: torch.Tensor | None = None,
                                 out_qp: torch.Tensor | None = None, stats_work: torch.Tensor | None = None):
         """Token-wise statistics -> clip -> quantize+pack in one call; returns (packed, device QParams[tokens])."""
-        assert x.is_cuda and x.is_contiguous() and x.numel() % channels == 0
-        tokens = x.numel() // channels
-        out_packed = self._bytes(qp_packed_bytes(x.numel(), bits)) if out_packed is None else out_packed
+        n, code = _input(x)
+        assert n % channels == 0
+        tokens = n // channels
+        out_packed = self._packed(n, bits) if out_packed is None else out_packed
         out_qp = self._bytes(C.sizeof(QParams) * tokens) if out_qp is None else out_qp
         stats_work = self._bytes(C.sizeof(Stats) * tokens) if stats_work is None else stats_work
-        self._check(self._lib.qp_sender_tokens_device(
-            self._h, x.data_ptr(), _dtype_code(x), tokens, channels, bits, method, bmode, out_packed.data_ptr(),
-            out_packed.numel() * out_packed.element_size(), out_qp.data_ptr(), stats_work.data_ptr(), _stream(self.device)))
+        self._run("qp_sender_tokens_device", x, code, tokens, channels, bits, method, bmode, out_packed, out_packed.nbytes,
+                  out_qp, stats_work)
         return out_packed, out_qp
 
     # -- host-buffer sender / receiver
@@ -570,18 +590,13 @@ class Context:
                        bmode: int = QP_B_MAD, steps: int = QP_DEFAULT_STEPS, hist_bins: int = QP_DEFAULT_HIST_BINS):
         """Host tensor in, packed host bytes + quantizer out (valid after a stream synchronise)."""
         assert not h_x.is_cuda and h_x.is_contiguous() and not h_packed.is_cuda
-        self._check(self._lib.qp_sender_host(self._h, h_x.data_ptr(), _dtype_code(h_x), h_x.numel(), bits,
-                                             int(use_ds), bmode, steps, hist_bins, d_x_work.data_ptr(),
-                                             d_packed_work.data_ptr(), h_packed.data_ptr(),
-                                             h_packed.numel() * h_packed.element_size(), C.byref(h_qp_out),
-                                             _stream(self.device)))
+        self._run("qp_sender_host", h_x, _dtype_code(h_x), h_x.numel(), bits, int(use_ds), bmode, steps, hist_bins, d_x_work,
+                  d_packed_work, h_packed, h_packed.nbytes, C.addressof(h_qp_out))
 
     def qp_receiver_host(self, h_packed: torch.Tensor, n: int, bits: int, h_qp: QParams, d_packed_work: torch.Tensor,
                          d_y_work: torch.Tensor, h_y: torch.Tensor):
         assert not h_packed.is_cuda and not h_y.is_cuda and h_y.is_contiguous() and h_y.numel() >= n
-        self._check(self._lib.qp_receiver_host(self._h, h_packed.data_ptr(), n, bits, C.byref(h_qp),
-                                               d_packed_work.data_ptr(), d_y_work.data_ptr(), h_y.data_ptr(),
-                                               _dtype_code(h_y), _stream(self.device)))
+        self._run("qp_receiver_host", h_packed, n, bits, C.addressof(h_qp), d_packed_work, d_y_work, h_y, _dtype_code(h_y))
 
     def qp_launch_count(self) -> int:
         return int(self._lib.qp_launch_count(self._h))

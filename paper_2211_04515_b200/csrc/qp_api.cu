@@ -277,12 +277,22 @@ static double gauss_F(int bits)
     return a;
 }
 
+// The multipliers are constants of (bits, dist): solved once, not on every sender call.
 double qp_host_aciq_F(int bits, int dist)
 {
+    struct Table {
+        double laplace[17], gauss[17];
+        Table()
+        {
+            for (int b = 0; b <= 16; ++b) {
+                laplace[b] = qp_bits_ok(b) ? lambert_w0(3.0 * pow(4.0, (double)b)) : 0.0;
+                gauss[b] = qp_bits_ok(b) ? gauss_F(b) : 0.0;
+            }
+        }
+    };
+    static const Table table;
     if (!qp_bits_ok(bits)) return 0.0;
-    if (dist == QP_DIST_LAPLACE) return lambert_w0(3.0 * pow(4.0, (double)bits));
-    if (dist == QP_DIST_GAUSS) return gauss_F(bits);
-    return 0.0;
+    return dist == QP_DIST_LAPLACE ? table.laplace[bits] : dist == QP_DIST_GAUSS ? table.gauss[bits] : 0.0;
 }
 
 extern "C" double qp_aciq_F(int bits, int dist) { return qp_host_aciq_F(bits, dist); }

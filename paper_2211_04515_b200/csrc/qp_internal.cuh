@@ -121,12 +121,15 @@ int32_t qp_fail(qp_ctx* ctx, int32_t status, const char* what);
 int32_t qp_check_launch(qp_ctx* ctx, const char* what);
 
 struct qp_device_guard {                 // makes ctx->device current for the scope
-    int prev;
+    int prev;                            // the device to go back to; -1: it was current already
     bool ok;
     explicit qp_device_guard(int dev) : prev(-1), ok(true)
     {
-        if (cudaGetDevice(&prev) != cudaSuccess) { ok = false; return; }
-        if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
+        int now = -1;
+        if (cudaGetDevice(&now) != cudaSuccess) { ok = false; return; }
+        if (now == dev) return;
+        prev = now;
+        if (cudaSetDevice(dev) != cudaSuccess) ok = false;
     }
     ~qp_device_guard() { if (prev >= 0) cudaSetDevice(prev); }
 };
