@@ -134,6 +134,19 @@ struct qp_device_guard {                 // makes ctx->device current for the sc
     ~qp_device_guard() { if (prev >= 0) cudaSetDevice(prev); }
 };
 
+// Launch shape of the warp-tile kernels (a warp per tile of 1024 elements, `max_warps` warps per block at
+// most).  A tensor of fewer tiles than the GPU has SMs x max_warps is spread over all SMs with fewer warps
+// per block instead of filling a few SMs; up to 64 blocks per SM, beyond that the grid walks.
+struct qp_grid_shape { unsigned blocks, threads; };
+static inline qp_grid_shape qp_tile_grid(const qp_ctx* ctx, uint64_t ntiles, int max_warps)
+{
+    const uint64_t sms = (uint64_t)ctx->sm_count;
+    int warps = max_warps;
+    while (warps > 1 && (ntiles + warps - 1) / warps < sms) warps >>= 1;
+    const uint64_t want = (ntiles + warps - 1) / warps, cap = sms * 64;
+    return {(unsigned)(want > cap ? cap : want), (unsigned)warps * 32u};
+}
+
 // Shared host arithmetic (one definition each, in qp_api.cu).
 double qp_host_aciq_F(int bits, int dist);
 static inline bool qp_bits_ok(int bits) { return (bits >= 1 && bits <= 8) || bits == 16; }

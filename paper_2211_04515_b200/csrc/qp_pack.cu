@@ -14,7 +14,8 @@
 // stores are 128-byte coalesced.
 //
 // bits = 16: one uint16 per element, plain vectorised map.
-// Ragged tails (n mod 1024), pad bytes and misaligned inputs go through a scalar kernel.
+// The last, partial tile and the pad words are guarded iterations of the same loop, and an input that
+// is not 16-byte aligned takes the same kernel with element loads: one launch for every shape.
 #include "qp_internal.cuh"
 
 namespace {
@@ -50,11 +51,14 @@ __device__ __forceinline__ unsigned quad_of(const float* e, const QP4& q)
     return r;
 }
 
-template <int BITS, typename T>
-__global__ void __launch_bounds__(QP_THREADS) pack_kernel(const T* __restrict__ x, uint64_t ntiles,
+// ntiles counts the last, partial tile too: its missing elements are NaN (code 0) and its words are
+// written up to nwords, pad words included.  VEC: x is 16-byte aligned.  Otherwise every lane loads the
+// elements of its vectors one by one (the four loads of a vector touch the same lines, so they hit L1).
+template <int BITS, typename T, bool VEC>
+__global__ void __launch_bounds__(QP_THREADS) pack_kernel(const T* __restrict__ x, uint64_t n, uint64_t ntiles,
                                                           const qp_qparams_t* __restrict__ d_qp, qp_qparams_t h_qp,
-                                                          uint32_t* __restrict__ out, unsigned* __restrict__ status,
-                                                          int reverse)
+                                                          uint32_t* __restrict__ out, uint64_t nwords,
+                                                          unsigned* __restrict__ status, int reverse)
 {
     constexpr int EPV = qp_span<T>::EPV;          // 4 (f32) or 8 (bf16) elements per 16-byte vector
     constexpr int NLOAD = TILE / (32 * EPV);      // 8 or 4 vector loads per lane
@@ -62,16 +66,36 @@ __global__ void __launch_bounds__(QP_THREADS) pack_kernel(const T* __restrict__ 
     const QP4 q = load_qp(d_qp, h_qp, BITS, status);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t* sw = stage[warp];
-    const uint64_t wstride = (uint64_t)gridDim.x * WARPS;
+    const unsigned warps = blockDim.x >> 5;
+    const uint64_t wstride = (uint64_t)gridDim.x * warps;
 
     // `reverse`: the grid walks the tensor from its end (the tiles are the same), for a call that
     // follows a pass which ended there and left that part of x in L2
-    for (uint64_t it = (uint64_t)blockIdx.x * WARPS + warp; it < ntiles; it += wstride) {
+    for (uint64_t it = (uint64_t)blockIdx.x * warps + warp; it < ntiles; it += wstride) {
         const uint64_t tile = reverse ? ntiles - 1 - it : it;
         const T* xt = x + tile * TILE;
+        const bool full = (tile + 1) * TILE <= n;                 // warp-uniform
         float e[NLOAD][EPV];
+        if (full) {
 #pragma unroll
-        for (int j = 0; j < NLOAD; ++j) qp_load_vec(xt + (j * 32 + lane) * EPV, e[j]);
+            for (int j = 0; j < NLOAD; ++j) {
+                if constexpr (VEC) {
+                    qp_load_vec(xt + (j * 32 + lane) * EPV, e[j]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < EPV; ++i) e[j][i] = qp_load_one(xt + (j * 32 + lane) * EPV + i);
+                }
+            }
+        } else {
+            const int have = (int)(n - tile * TILE);
+#pragma unroll
+            for (int j = 0; j < NLOAD; ++j)
+#pragma unroll
+                for (int i = 0; i < EPV; ++i) {
+                    const int k = (j * 32 + lane) * EPV + i;
+                    e[j][i] = k < have ? qp_load_one(xt + k) : __int_as_float(0x7FC00000);
+                }
+        }
 #pragma unroll
         for (int j = 0; j < NLOAD; ++j) {
             if constexpr (EPV == 4) {
@@ -98,52 +122,26 @@ __global__ void __launch_bounds__(QP_THREADS) pack_kernel(const T* __restrict__ 
             if (sh + QB > 32) w[(word + 1) % BITS] |= qd[k] >> (32 - sh);
         }
         uint32_t* ot = out + tile * (32 * BITS);
-        if constexpr (BITS == 8) {
+        if (full && BITS == 8) {
             uint4* o = reinterpret_cast<uint4*>(ot + lane * 8);
-            o[0] = make_uint4(w[0], w[1], w[2], w[3]);
-            o[1] = make_uint4(w[4], w[5], w[6], w[7]);
-        } else if constexpr (BITS == 4) {
-            *reinterpret_cast<uint4*>(ot + lane * 4) = make_uint4(w[0], w[1], w[2], w[3]);
-        } else if constexpr (BITS == 2) {
-            *reinterpret_cast<uint2*>(ot + lane * 2) = make_uint2(w[0], w[1]);
-        } else if constexpr (BITS == 1) {
-            ot[lane] = w[0];
+            o[0] = make_uint4(w[0], w[1 % BITS], w[2 % BITS], w[3 % BITS]);
+            o[1] = make_uint4(w[4 % BITS], w[5 % BITS], w[6 % BITS], w[7 % BITS]);
+        } else if (full && BITS == 4) {
+            *reinterpret_cast<uint4*>(ot + lane * 4) = make_uint4(w[0], w[1 % BITS], w[2 % BITS], w[3 % BITS]);
+        } else if (full && BITS == 2) {
+            *reinterpret_cast<uint2*>(ot + lane * 2) = make_uint2(w[0], w[1 % BITS]);
         } else {
             __syncwarp();
 #pragma unroll
             for (int m = 0; m < BITS; ++m) sw[lane * BITS + m] = w[m];
             __syncwarp();
+            const int room = (int)min((uint64_t)(32 * BITS), nwords - tile * (32 * BITS));
 #pragma unroll
-            for (int m = 0; m < BITS; ++m) ot[m * 32 + lane] = sw[m * 32 + lane];
+            for (int m = 0; m < BITS; ++m)
+                if (m * 32 + lane < room) ot[m * 32 + lane] = sw[m * 32 + lane];
         }
         __syncwarp();
     }
-}
-
-// Scalar path: thread t packs elements [first + 32t, first + 32t + 32) that exist (missing
-// ones count as code 0) into `bits` words, and writes those below nwords.
-template <typename T>
-__global__ void __launch_bounds__(QP_THREADS) pack_tail_kernel(const T* __restrict__ x, uint64_t first, uint64_t n,
-                                                               int bits, const qp_qparams_t* __restrict__ d_qp,
-                                                               qp_qparams_t h_qp, uint32_t* __restrict__ out,
-                                                               uint64_t nwords, unsigned* __restrict__ status)
-{
-    const QP4 q = load_qp(d_qp, h_qp, bits, status);
-    const uint64_t t = (uint64_t)blockIdx.x * QP_THREADS + threadIdx.x;
-    const uint64_t w0 = t * (uint64_t)bits;
-    if (w0 >= nwords) return;
-    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    const uint64_t e0 = first + t * 32;
-    for (int i = 0; i < 32; ++i) {
-        const uint64_t idx = e0 + i;
-        if (idx >= n) break;
-        const unsigned c = qp_code(qp_load_one(x + idx), q.lo, q.hi, q.inv, q.mask);
-        const int bit = i * bits, word = bit >> 5, sh = bit & 31;
-        w[word] |= c << sh;
-        if (sh + bits > 32) w[word + 1] |= c >> (32 - sh);
-    }
-    for (int m = 0; m < bits; ++m)
-        if (w0 + m < nwords) out[w0 + m] = w[m];
 }
 
 // bits = 16: thread t converts the 8 elements [8t, 8t+8) to one 16-byte vector of uint16 codes.
@@ -196,34 +194,25 @@ int32_t pack_typed(qp_ctx* ctx, const T* x, uint64_t n, int bits, const qp_qpara
             pack16_kernel<T, false><<<blocks, QP_THREADS, 0, s>>>(x, n, d_qp, h_qp, static_cast<uint4*>(d_packed), nvec_out, ctx->d_status);
         return qp_check_launch(ctx, "qp_quantize_pack");
     }
-    const uint64_t ntiles = aligned ? n / TILE : 0;
+    const uint64_t nwords = qp_packed_bytes(n, bits) / 4;
+    const uint64_t ntiles = (n + TILE - 1) / TILE;
     uint32_t* out = static_cast<uint32_t*>(d_packed);
     // a hint, not a dependency: start where the last pass over this tensor stopped
     const int reverse = (ctx->last_x == static_cast<const void*>(x) && ctx->last_x_end) ? 1 : 0;
     ctx->last_x = x;
     ctx->last_x_end = reverse ? 0 : 1;
-    if (ntiles) {
-        uint64_t want = (ntiles + WARPS - 1) / WARPS;
-        const uint64_t cap = (uint64_t)ctx->sm_count * 64;
-        const int blocks = (int)(want > cap ? cap : want);
-        ctx->launches += 1;
-#define QP_PACK_CASE(B) case B: pack_kernel<B, T><<<blocks, QP_THREADS, 0, s>>>(x, ntiles, d_qp, h_qp, out, ctx->d_status, reverse); break;
-        switch (bits) {
-            QP_PACK_CASE(1) QP_PACK_CASE(2) QP_PACK_CASE(3) QP_PACK_CASE(4)
-            QP_PACK_CASE(5) QP_PACK_CASE(6) QP_PACK_CASE(7) QP_PACK_CASE(8)
-        }
+    const qp_grid_shape g = qp_tile_grid(ctx, ntiles, WARPS);
+    ctx->launches += 1;
+#define QP_PACK_CASE(B)                                                                                                        \
+    case B:                                                                                                                    \
+        if (aligned) pack_kernel<B, T, true><<<g.blocks, g.threads, 0, s>>>(x, n, ntiles, d_qp, h_qp, out, nwords, ctx->d_status, reverse); \
+        else pack_kernel<B, T, false><<<g.blocks, g.threads, 0, s>>>(x, n, ntiles, d_qp, h_qp, out, nwords, ctx->d_status, reverse);        \
+        break;
+    switch (bits) {
+        QP_PACK_CASE(1) QP_PACK_CASE(2) QP_PACK_CASE(3) QP_PACK_CASE(4)
+        QP_PACK_CASE(5) QP_PACK_CASE(6) QP_PACK_CASE(7) QP_PACK_CASE(8)
+    }
 #undef QP_PACK_CASE
-    }
-    const uint64_t done_words = ntiles * 32 * (uint64_t)bits;
-    const uint64_t total_words = qp_packed_bytes(n, bits) / 4;
-    if (total_words > done_words) {
-        const uint64_t nwords = total_words - done_words;
-        const uint64_t threads = (nwords + bits - 1) / bits;
-        const uint64_t blocks = (threads + QP_THREADS - 1) / QP_THREADS;
-        ctx->launches += 1;
-        pack_tail_kernel<T><<<(unsigned)blocks, QP_THREADS, 0, s>>>(x, ntiles * TILE, n, bits, d_qp, h_qp,
-                                                                     out + done_words, nwords, ctx->d_status);
-    }
     return qp_check_launch(ctx, "qp_quantize_pack");
 }
 

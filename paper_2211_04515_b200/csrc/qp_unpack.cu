@@ -7,7 +7,8 @@
 // bits 1,2,4,8; 128-byte coalesced through shared memory otherwise), cuts them into the 8
 // "quads" (4 codes each) of its 32 consecutive elements, and the quads cross the warp
 // through a chunk-swizzled 1 KB staging buffer so that lane l then expands quad j*32+l and
-// stores 16-byte vectors that are fully coalesced across the warp.
+// stores 16-byte vectors that are fully coalesced across the warp.  The last, partial tile is a guarded
+// iteration of the same loop, and an output that is not aligned takes element stores: one launch.
 #include "qp_internal.cuh"
 
 namespace {
@@ -51,38 +52,43 @@ __device__ __forceinline__ void store_out(unsigned short* y, uint64_t i4, const 
 __device__ __forceinline__ void store_one(float* y, uint64_t i, float v) { y[i] = v; }
 __device__ __forceinline__ void store_one(unsigned short* y, uint64_t i, float v) { y[i] = qp_f32_to_bf16(v); }
 
-template <int BITS, typename TO>
-__global__ void __launch_bounds__(QP_THREADS) unpack_kernel(const uint32_t* __restrict__ in, uint64_t ntiles,
-                                                            const qp_qparams_t* __restrict__ d_qp, qp_qparams_t h_qp,
-                                                            TO* __restrict__ y, unsigned* __restrict__ status)
+// ntiles counts the last, partial tile too: its words are read up to nwords and its elements written up
+// to n.  VEC: y is aligned for 4-element stores; otherwise the elements are stored one by one.
+template <int BITS, typename TO, bool VEC>
+__global__ void __launch_bounds__(QP_THREADS) unpack_kernel(const uint32_t* __restrict__ in, uint64_t n, uint64_t nwords,
+                                                            uint64_t ntiles, const qp_qparams_t* __restrict__ d_qp,
+                                                            qp_qparams_t h_qp, TO* __restrict__ y,
+                                                            unsigned* __restrict__ status)
 {
     __shared__ __align__(16) uint32_t stage[WARPS][256];
     const DQ q = load_dq(d_qp, h_qp, BITS, status);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t* sw = stage[warp];
-    const uint64_t wstride = (uint64_t)gridDim.x * WARPS;
+    const unsigned warps = blockDim.x >> 5;
+    const uint64_t wstride = (uint64_t)gridDim.x * warps;
     constexpr unsigned MASK = (1u << BITS) - 1u;
     constexpr int QB = 4 * BITS;
     constexpr unsigned QMASK = QB >= 32 ? 0xFFFFFFFFu : ((1u << (QB & 31)) - 1u);
 
-    for (uint64_t tile = (uint64_t)blockIdx.x * WARPS + warp; tile < ntiles; tile += wstride) {
+    for (uint64_t tile = (uint64_t)blockIdx.x * warps + warp; tile < ntiles; tile += wstride) {
         const uint32_t* it = in + tile * (32 * BITS);
+        const bool full = (tile + 1) * TILE <= n;                 // warp-uniform
         uint32_t w[BITS];
-        if constexpr (BITS == 8) {
+        if (full && BITS == 8) {
             const uint4 a = __ldg(reinterpret_cast<const uint4*>(it + lane * 8));
             const uint4 b = __ldg(reinterpret_cast<const uint4*>(it + lane * 8) + 1);
-            w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
-        } else if constexpr (BITS == 4) {
+            w[0] = a.x; w[1 % BITS] = a.y; w[2 % BITS] = a.z; w[3 % BITS] = a.w;
+            w[4 % BITS] = b.x; w[5 % BITS] = b.y; w[6 % BITS] = b.z; w[7 % BITS] = b.w;
+        } else if (full && BITS == 4) {
             const uint4 a = __ldg(reinterpret_cast<const uint4*>(it + lane * 4));
-            w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
-        } else if constexpr (BITS == 2) {
+            w[0] = a.x; w[1 % BITS] = a.y; w[2 % BITS] = a.z; w[3 % BITS] = a.w;
+        } else if (full && BITS == 2) {
             const uint2 a = __ldg(reinterpret_cast<const uint2*>(it + lane * 2));
-            w[0] = a.x; w[1] = a.y;
-        } else if constexpr (BITS == 1) {
-            w[0] = __ldg(it + lane);
+            w[0] = a.x; w[1 % BITS] = a.y;
         } else {
+            const int room = (int)min((uint64_t)(32 * BITS), nwords - tile * (32 * BITS));
 #pragma unroll
-            for (int m = 0; m < BITS; ++m) sw[m * 32 + lane] = __ldg(it + m * 32 + lane);
+            for (int m = 0; m < BITS; ++m) sw[m * 32 + lane] = m * 32 + lane < room ? __ldg(it + m * 32 + lane) : 0u;
             __syncwarp();
 #pragma unroll
             for (int m = 0; m < BITS; ++m) w[m] = sw[lane * BITS + m];
@@ -102,39 +108,22 @@ __global__ void __launch_bounds__(QP_THREADS) unpack_kernel(const uint32_t* __re
         uint32_t mine[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) mine[j] = sw[swz(j * 32 + lane)];
+        const int have = full ? TILE : (int)(n - tile * TILE);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             float v[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) v[i] = dequant((mine[j] >> (BITS * i)) & MASK, q);
-            store_out(y, tile * (TILE / 4) + j * 32 + lane, v);
+            const int k = (j * 32 + lane) * 4;
+            if (VEC && (full || k + 4 <= have)) {
+                store_out(y, tile * (TILE / 4) + j * 32 + lane, v);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (k + i < have) store_one(y, tile * TILE + k + i, v[i]);
+            }
         }
         __syncwarp();
-    }
-}
-
-// Scalar path: thread t expands elements [first + 32t, first + 32t + 32) that exist.
-template <typename TO>
-__global__ void __launch_bounds__(QP_THREADS) unpack_tail_kernel(const uint32_t* __restrict__ in, uint64_t first,
-                                                                 uint64_t n, int bits,
-                                                                 const qp_qparams_t* __restrict__ d_qp, qp_qparams_t h_qp,
-                                                                 TO* __restrict__ y, unsigned* __restrict__ status)
-{
-    const DQ q = load_dq(d_qp, h_qp, bits, status);
-    const uint64_t t = (uint64_t)blockIdx.x * QP_THREADS + threadIdx.x;
-    const uint64_t e0 = first + t * 32;
-    if (e0 >= n) return;
-    const uint32_t* wp = in + t * (uint64_t)bits;          // `in` already points at the word of element `first`
-    const unsigned mask = (1u << bits) - 1u;
-    const int cnt = (int)((n - e0) < 32 ? (n - e0) : 32);
-    const int nw = (cnt * bits + 31) >> 5;                  // words that hold existing elements
-    uint32_t w[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int m = 0; m < nw; ++m) w[m] = __ldg(wp + m);
-    for (int i = 0; i < cnt; ++i) {
-        const int bit = i * bits, word = bit >> 5, sh = bit & 31;
-        uint32_t c = w[word] >> sh;
-        if (sh + bits > 32) c |= w[word + 1] << (32 - sh);
-        store_one(y, e0 + i, dequant(c & mask, q));
     }
 }
 
@@ -185,27 +174,19 @@ int32_t unpack_typed(qp_ctx* ctx, const void* d_packed, uint64_t n, int bits, co
         return qp_check_launch(ctx, "qp_unpack_dequantize");
     }
     const uint32_t* in = static_cast<const uint32_t*>(d_packed);
-    const uint64_t ntiles = aligned ? n / TILE : 0;
-    if (ntiles) {
-        uint64_t want = (ntiles + WARPS - 1) / WARPS;
-        const uint64_t cap = (uint64_t)ctx->sm_count * 64;
-        const int blocks = (int)(want > cap ? cap : want);
-        ctx->launches += 1;
-#define QP_UNPACK_CASE(B) case B: unpack_kernel<B, TO><<<blocks, QP_THREADS, 0, s>>>(in, ntiles, d_qp, h_qp, y, ctx->d_status); break;
-        switch (bits) {
-            QP_UNPACK_CASE(1) QP_UNPACK_CASE(2) QP_UNPACK_CASE(3) QP_UNPACK_CASE(4)
-            QP_UNPACK_CASE(5) QP_UNPACK_CASE(6) QP_UNPACK_CASE(7) QP_UNPACK_CASE(8)
-        }
+    const uint64_t nwords = qp_packed_bytes(n, bits) / 4, ntiles = (n + TILE - 1) / TILE;
+    const qp_grid_shape g = qp_tile_grid(ctx, ntiles, WARPS);
+    ctx->launches += 1;
+#define QP_UNPACK_CASE(B)                                                                                                    \
+    case B:                                                                                                                  \
+        if (aligned) unpack_kernel<B, TO, true><<<g.blocks, g.threads, 0, s>>>(in, n, nwords, ntiles, d_qp, h_qp, y, ctx->d_status); \
+        else unpack_kernel<B, TO, false><<<g.blocks, g.threads, 0, s>>>(in, n, nwords, ntiles, d_qp, h_qp, y, ctx->d_status);        \
+        break;
+    switch (bits) {
+        QP_UNPACK_CASE(1) QP_UNPACK_CASE(2) QP_UNPACK_CASE(3) QP_UNPACK_CASE(4)
+        QP_UNPACK_CASE(5) QP_UNPACK_CASE(6) QP_UNPACK_CASE(7) QP_UNPACK_CASE(8)
+    }
 #undef QP_UNPACK_CASE
-    }
-    const uint64_t first = ntiles * TILE;
-    if (n > first) {
-        const uint64_t threads = (n - first + 31) / 32;
-        const uint64_t blocks = (threads + QP_THREADS - 1) / QP_THREADS;
-        ctx->launches += 1;
-        unpack_tail_kernel<TO><<<(unsigned)blocks, QP_THREADS, 0, s>>>(in + ntiles * 32 * (uint64_t)bits, first, n, bits,
-                                                                       d_qp, h_qp, y, ctx->d_status);
-    }
     return qp_check_launch(ctx, "qp_unpack_dequantize");
 }
 
