@@ -229,6 +229,74 @@ __device__ __forceinline__ unsigned qp_code(float x, float lo, float hi, float i
     return __float_as_uint(__fadd_rn(qp_grid_pos(x, lo, hi, inv_scale), QP_MAGIC)) & mask;
 }
 
+// Two fp32 values in a register pair: Blackwell adds, multiplies and fuses both with one instruction
+// (each rounded on its own, as the scalar forms), which halves the issue slots of such chains.
+typedef unsigned long long qp_f2;
+__device__ __forceinline__ qp_f2 qp_pack2(float a, float b)
+{
+    qp_f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void qp_unpack2(qp_f2 v, float& a, float& b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ qp_f2 qp_add2(qp_f2 a, qp_f2 b)
+{
+    qp_f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// (through scalar products: a packed multiply whose result goes into a packed add came out contracted to one
+// rounding, which moved codes next to a rounding boundary)
+__device__ __forceinline__ qp_f2 qp_mul2(qp_f2 a, qp_f2 b)
+{
+    float a0, a1, b0, b1;
+    qp_unpack2(a, a0, a1);
+    qp_unpack2(b, b0, b1);
+    return qp_pack2(__fmul_rn(a0, b0), __fmul_rn(a1, b1));
+}
+__device__ __forceinline__ qp_f2 qp_fma2(qp_f2 a, qp_f2 b, qp_f2 c)
+{
+    qp_f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// smallest / largest of three (one instruction)
+__device__ __forceinline__ float qp_min3(float a, float b, float c)
+{
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float qp_max3(float a, float b, float c)
+{
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// The codes of 4 consecutive elements as one word of 4 * BITS bits: qp_code on pairs, and the fields put
+// together by adding the shifted words and taking the magic constant's bits off once (codes have no bits
+// above BITS, so nothing carries).
+template <int BITS>
+__device__ __forceinline__ unsigned qp_quad(const float* e, float lo, float hi, float inv)
+{
+    const qp_f2 nlo = qp_pack2(-lo, -lo), inv2 = qp_pack2(inv, inv), magic = qp_pack2(QP_MAGIC, QP_MAGIC);
+    constexpr unsigned MB = QP_MAGIC_BITS;
+    constexpr unsigned offs = MB + (MB << BITS) + (BITS < 16 ? MB << ((2 * BITS) & 31) : 0u) + (3 * BITS < 32 ? MB << ((3 * BITS) & 31) : 0u);
+    unsigned r = 0u - offs;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float a = fminf(fmaxf(e[2 * h], lo), hi), b = fminf(fmaxf(e[2 * h + 1], lo), hi);
+        float pa, pb;
+        qp_unpack2(qp_add2(qp_mul2(qp_add2(qp_pack2(a, b), nlo), inv2), magic), pa, pb);
+        r += (__float_as_uint(pa) << (2 * h * BITS)) + (__float_as_uint(pb) << ((2 * h + 1) * BITS));
+    }
+    return r;
+}
+
 // monotone map float -> uint32 (finite values; -0 sorts directly below +0), and back
 __device__ __forceinline__ unsigned qp_key_of(float x)
 {

@@ -4,7 +4,7 @@
 // quantizer that the per-tensor functions give for its row alone.  Bit-width and packed layout
 // are shared, so the receiver needs the `tokens` quantizers (24 bytes each) with the stream.
 //
-//   tok_stats_kernel    a warp per token: the row is read once from HBM (sums, min, max), the mean
+//   tok_stats_kernel    (rows that do not suit tok_rows_kernel) a warp per token: the row is read once from HBM (sums, min, max), the mean
 //                       comes out of a warp reduction, and the second pass over the row (deviations)
 //                       finds it in L1; fp32 partials per lane folded into fp64, fixed shuffle order
 //   tok_pack_kernel     the per-tensor packer's warp tile (1024 elements = 32 * bits words, coalesced
@@ -14,6 +14,8 @@
 //                       are 128 elements apart, so the token index moves on by a compare instead of
 //                       a division
 //   tok_unpack_kernel   the mirror image
+//   tok_rows_kernel     the same statistics from rows in shared memory and, in the sender, clip, quantize and
+//                       pack of the row as well
 //   tok_*_scalar        any shape and alignment: a thread per 32 elements, token by division
 #include "qp_internal.cuh"
 
@@ -163,7 +165,6 @@ __global__ void __launch_bounds__(QP_THREADS) tok_pack_kernel(const T* __restric
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t* sw = stage[warp];
     const uint64_t wstride = (uint64_t)gridDim.x * WARPS;
-    constexpr unsigned mask = (1u << BITS) - 1u;
     bool mismatch = false;
     for (uint64_t tile = (uint64_t)blockIdx.x * WARPS + warp; tile < ntiles; tile += wstride) {
         const T* xt = x + tile * TILE;
@@ -179,10 +180,7 @@ __global__ void __launch_bounds__(QP_THREADS) tok_pack_kernel(const T* __restric
             unsigned quads[EPV / 4];
 #pragma unroll
             for (int h = 0; h < EPV / 4; ++h) {
-                unsigned r = 0;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) r |= qp_code(e[j][4 * h + i], lo, hi, inv, mask) << (BITS * i);
-                quads[h] = r;
+                quads[h] = qp_quad<BITS>(e[j] + 4 * h, lo, hi, inv);
             }
             if constexpr (EPV == 4) sw[swz(j * 32 + lane)] = quads[0];
             else *reinterpret_cast<uint2*>(&sw[swz(2 * (j * 32 + lane))]) = make_uint2(quads[0], quads[1]);
@@ -350,6 +348,349 @@ __global__ void __launch_bounds__(QP_THREADS) tok_unpack_scalar(const uint32_t* 
     if (mismatch) atomicOr(status, QP_DEV_BITS_MISMATCH);
 }
 
+// ---------------------------------------------------------------------------- rows in shared memory
+//
+// A warp takes a token, copies its row into its own piece of shared memory (asynchronous 16-byte copies)
+// and does everything to it from there: statistics and, in the sender, clip, quantize and pack as well.
+// The row is read from HBM once and the packed words written once: the sender is bound by those bytes (161 MB
+// for the ViT-Huge tensor at 8 bits, 24.7 us at the copy peak), where the three kernels read the tensor twice
+// and took 76 us (statistics 49, clip 2.5, pack 24.5).  The row is not kept in registers: with 128 of
+// them only 16 warps fit an SM and the chains of one token do not overlap enough with the others'
+// (53 us).  What a token costs beside its elements is kept small by giving the lanes different work: the two
+// sums of a pass reduce together (half a warp each), and the quotients of the statistics and of the
+// quantizer are one division with another numerator in every lane.
+
+// s0 and s1 summed over the warp, both results in every lane; fixed order
+__device__ __forceinline__ void tok_reduce2(double& s0, double& s1, int lane)
+{
+    const bool upper = (lane & 16) != 0;
+    double v = upper ? s1 : s0;
+    v += __shfl_xor_sync(0xFFFFFFFFu, upper ? s0 : s1, 16);
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    s0 = __shfl_sync(0xFFFFFFFFu, v, 0);
+    s1 = __shfl_sync(0xFFFFFFFFu, v, 16);
+}
+
+// 8 consecutive-vector elements of the row as four pairs: vectors v and v + 32 of fp32, vector v of bf16
+template <typename T>
+__device__ __forceinline__ void tok_lds8(const T* row, int v, qp_f2 (&p)[4])
+{
+    if constexpr (sizeof(T) == 4) {
+        const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(row + v * 4);
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(row + (v + 32) * 4);
+        p[0] = a.x; p[1] = a.y; p[2] = b.x; p[3] = b.y;
+    } else {
+        const uint4 r = *reinterpret_cast<const uint4*>(row + v * 8);
+        const unsigned w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) p[i] = qp_pack2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u));
+    }
+}
+
+// a 16-byte vector of the row as floats
+template <typename T>
+__device__ __forceinline__ void tok_lds(const T* p, float (&e)[qp_span<T>::EPV])
+{
+    const uint4 r = *reinterpret_cast<const uint4*>(p);
+    const unsigned w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if constexpr (sizeof(T) == 4) {
+            e[i] = __uint_as_float(w[i]);
+        } else {
+            e[2 * i] = __uint_as_float(w[i] << 16);
+            e[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+        }
+    }
+}
+
+// sum of 8 magnitudes as a tree, and of 8 values: no longer chain of roundings than a run of four
+__device__ __forceinline__ float tok_abs8(const qp_f2 (&p)[4])
+{
+    float a[4], b[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) qp_unpack2(p[i], a[i], b[i]);
+    return ((fabsf(a[0]) + fabsf(a[1])) + (fabsf(a[2]) + fabsf(a[3]))) + ((fabsf(b[0]) + fabsf(b[1])) + (fabsf(b[2]) + fabsf(b[3])));
+}
+__device__ __forceinline__ float tok_sum8(const qp_f2 (&p)[4])
+{
+    float a, b;
+    qp_unpack2(qp_add2(qp_add2(p[0], p[1]), qp_add2(p[2], p[3])), a, b);
+    return a + b;
+}
+
+// statistics of the row in shared memory (nvec whole vectors), the same in every lane; true if it holds
+// non-finite values.  The loops over whole groups of 32 lanes x 8 elements are uniform; what is left of the
+// row (less than one such group) is padded: with copies of nothing (zero) for the sums, and skipped in the
+// deviations by an infinite value.
+template <typename T>
+__device__ __forceinline__ bool tok_row_stats(const T* row, int nvec, uint32_t C, int lane, qp_stats_t& st)
+{
+    constexpr int EPV = qp_span<T>::EPV;
+    constexpr int STEP = 8 / EPV * 32;                        // vectors of one round: 64 (fp32), 32 (bf16)
+    const float inf = __int_as_float(0x7F800000);
+    // first moments: fp32 over 8 elements, then fp64
+    double s = 0.0, sa = 0.0;
+    float mn = inf, mx = -inf;
+    unsigned bad = 0u;
+    bool odd = false;                                         // a NaN or Inf (or an fp32 overflow) in this lane
+    auto tail8 = [&](int v0, float missing, qp_f2 (&p)[4]) {  // the last, partial round
+        float e[8];
+#pragma unroll
+        for (int h = 0; h < 8 / EPV; ++h) {
+            const int v = v0 + h * 32 + lane;
+            float a[EPV];
+            if (v < nvec) tok_lds<T>(row + v * EPV, a);
+#pragma unroll
+            for (int i = 0; i < EPV; ++i) e[h * EPV + i] = v < nvec ? a[i] : missing;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) p[i] = qp_pack2(e[2 * i], e[2 * i + 1]);
+    };
+    auto moments = [&](const qp_f2 (&p)[4]) {
+        const float psa = tok_abs8(p);
+        s += (double)tok_sum8(p);
+        sa += (double)psa;
+        odd |= !(psa < inf);
+    };
+    const int whole = nvec / STEP * STEP;
+#pragma unroll 2
+    for (int v0 = 0; v0 < whole; v0 += STEP) {
+        qp_f2 p[4];
+        tok_lds8<T>(row, v0 + lane, p);
+        moments(p);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float a, b;
+            qp_unpack2(p[i], a, b);
+            mn = qp_min3(mn, a, b);
+            mx = qp_max3(mx, a, b);
+        }
+    }
+    if (whole < nvec) {
+        qp_f2 p[4];
+        tail8(whole, 0.f, p);
+        moments(p);
+#pragma unroll
+        for (int h = 0; h < 8 / EPV; ++h)
+            if (whole + h * 32 + lane < nvec) {
+                float a[EPV];
+                tok_lds<T>(row + (whole + h * 32 + lane) * EPV, a);
+#pragma unroll
+                for (int i = 0; i < EPV; i += 2) { mn = qp_min3(mn, a[i], a[i + 1]); mx = qp_max3(mx, a[i], a[i + 1]); }
+            }
+    }
+    const bool guard = __any_sync(0xFFFFFFFFu, odd);
+    if (guard) {                                              // rare: the row again, element by element
+        s = 0.0; sa = 0.0; mn = inf; mx = -inf;
+        for (int v = lane; v < nvec; v += 32) {
+            float e[EPV];
+            tok_lds<T>(row + v * EPV, e);
+#pragma unroll
+            for (int i = 0; i < EPV; ++i) {
+                if (qp_is_finite(e[i])) {
+                    s += (double)e[i];
+                    sa += (double)fabsf(e[i]);
+                    mn = fminf(mn, e[i]);
+                    mx = fmaxf(mx, e[i]);
+                } else {
+                    ++bad;
+                }
+            }
+        }
+        bad = __reduce_add_sync(0xFFFFFFFFu, bad);
+    }
+    tok_reduce2(s, sa, lane);
+    {
+        const bool upper = (lane & 16) != 0;                  // min of x in one half, min of -x in the other
+        float v = upper ? -mx : mn;
+        v = fminf(v, __shfl_xor_sync(0xFFFFFFFFu, upper ? mn : -mx, 16));
+        for (int o = 8; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+        mn = __shfl_sync(0xFFFFFFFFu, v, 0);
+        mx = -__shfl_sync(0xFFFFFFFFu, v, 16);
+    }
+    const unsigned nf = C - bad;
+    const double mean = nf ? s / (double)nf : 0.0;
+    const float m_hi = (float)mean, m_lo = (float)(mean - (double)m_hi);   // the mean as an unevaluated fp32 pair
+
+    // deviations
+    double sd = 0.0, sv = 0.0;
+    const qp_f2 nhi = qp_pack2(-m_hi, -m_hi), nlo = qp_pack2(-m_lo, -m_lo);
+    auto deviations = [&](const qp_f2 (&p)[4], bool check) {
+        qp_f2 d[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) d[i] = qp_add2(qp_add2(p[i], nhi), nlo);
+        if (check) {                                          // uniform: non-finite values, or elements that do not exist
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float a, b, da, db;
+                qp_unpack2(p[i], a, b);
+                qp_unpack2(d[i], da, db);
+                d[i] = qp_pack2(qp_is_finite(a) ? da : 0.f, qp_is_finite(b) ? db : 0.f);
+            }
+        }
+        sd += (double)tok_abs8(d);
+        qp_f2 q2 = qp_fma2(d[0], d[0], 0ull);
+#pragma unroll
+        for (int i = 1; i < 4; ++i) q2 = qp_fma2(d[i], d[i], q2);
+        float qa, qb;
+        qp_unpack2(q2, qa, qb);
+        sv += (double)(qa + qb);
+    };
+#pragma unroll 2
+    for (int v0 = 0; v0 < whole; v0 += STEP) {
+        qp_f2 p[4];
+        tok_lds8<T>(row, v0 + lane, p);
+        deviations(p, guard);
+    }
+    if (whole < nvec) {
+        qp_f2 p[4];
+        tail8(whole, inf, p);
+        deviations(p, true);
+    }
+    tok_reduce2(sd, sv, lane);
+
+    const double q = (lane == 0 ? sa : lane == 1 ? sd : sv) / (double)(nf ? nf : 1u);   // the three means in three lanes
+    st.n = C;
+    st.nonfinite = bad;
+    st.mean = mean;
+    st.mean_abs = nf ? __shfl_sync(0xFFFFFFFFu, q, 0) : 0.0;
+    st.mad = nf ? __shfl_sync(0xFFFFFFFFu, q, 1) : 0.0;
+    st.var = nf ? __shfl_sync(0xFFFFFFFFu, q, 2) : 0.0;
+    st.min = nf ? (double)mn : 0.0;
+    st.max = nf ? (double)mx : 0.0;
+    st.hist_peak = 0;
+    st.hist_bins = 0;
+    st.reserved = 0;
+    return bad != 0u;
+}
+
+constexpr int TR_WARPS = 8;                                   // warps per block
+
+// bytes of shared memory a warp needs for a row (a multiple of 16): the row, and in the sender its quads
+__host__ __device__ constexpr size_t tok_row_bytes(uint32_t C, size_t esz, bool sender)
+{
+    return (size_t)C * esz + (sender ? (size_t)C : 0);
+}
+
+// BITS = 0: statistics only (any row of whole vectors).  BITS = 1..8: the whole sender, rows of whole
+// 32-element groups (a row is then whole words).
+template <int BITS, typename T>
+__global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __restrict__ x, uint64_t tokens, uint32_t C, int method,
+                                                                 int bmode, double F, uint32_t* __restrict__ out,
+                                                                 uint64_t nwords, qp_qparams_t* __restrict__ qp_out,
+                                                                 qp_stats_t* __restrict__ st_out, unsigned* __restrict__ status)
+{
+    extern __shared__ __align__(16) unsigned char raw[];
+    constexpr int EPV = qp_span<T>::EPV;
+    const int lane = threadIdx.x & 31;
+    T* row = reinterpret_cast<T*>(raw + (threadIdx.x >> 5) * tok_row_bytes(C, sizeof(T), BITS > 0));
+    const int nvec = (int)(C / EPV);
+    unsigned raise = 0u;
+    const uint64_t wstride = (uint64_t)gridDim.x * TR_WARPS;
+    for (uint64_t t = (uint64_t)blockIdx.x * TR_WARPS + (threadIdx.x >> 5); t < tokens; t += wstride) {
+        const T* src = x + t * C;
+        auto fetch = [&](int v) {
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(row + v * EPV)),
+                         "l"(src + (size_t)v * EPV)
+                         : "memory");
+        };
+#pragma unroll 4
+        for (int v0 = 0; v0 < (nvec & ~31); v0 += 32) fetch(v0 + lane);
+        if ((nvec & ~31) + lane < nvec) fetch((nvec & ~31) + lane);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncwarp();
+
+        qp_stats_t st;
+        if (tok_row_stats<T>(row, nvec, C, lane, st)) raise |= QP_DEV_NONFINITE;
+        if (lane == 0) st_out[t] = st;
+        if constexpr (BITS > 0) {
+            constexpr unsigned mask = (1u << BITS) - 1u;
+            uint32_t* sw = reinterpret_cast<uint32_t*>(row + C);
+            const int groups = (int)(C / 32);
+            double lo_d, hi_d;
+            qp_clip_ends(st, method, QP_DIST_LAPLACE, bmode, BITS, F, lo_d, hi_d);
+            qp_qparams_t q;
+            q.lo = (float)lo_d;
+            q.hi = (float)hi_d;
+            q.bits = BITS;
+            q.flags = (!(q.hi > q.lo) || !(q.lo - q.lo == 0.f) || !(q.hi - q.hi == 0.f)) ? 1 : 0;
+            q.scale = q.inv_scale = 0.f;
+            if (q.flags) {
+                raise |= QP_DEV_DEGENERATE;
+            } else {                                         // scale and its reciprocal in two lanes
+                const double range = (double)q.hi - (double)q.lo, levels_m1 = (double)mask;
+                const double num = lane == 0 ? range : levels_m1, den = lane == 0 ? levels_m1 : range;
+                const float v = (float)(num / den);
+                q.scale = __shfl_sync(0xFFFFFFFFu, v, 0);
+                q.inv_scale = __shfl_sync(0xFFFFFFFFu, v, 1);
+            }
+            if (lane == 0) qp_out[t] = q;
+            uint32_t* orow = out + t * (uint64_t)(groups * BITS);
+            auto quantize = [&](int v) {                     // vector v: its quads to the output (8 bits: a quad is a word) or to `sw`
+                float e[EPV];
+                tok_lds<T>(row + v * EPV, e);
+                if constexpr (EPV == 4) {
+                    const unsigned qd = qp_quad<BITS>(e, q.lo, q.hi, q.inv_scale);
+                    if constexpr (BITS == 8) orow[v] = qd;
+                    else sw[swz(v)] = qd;
+                } else {
+                    const uint2 qd = make_uint2(qp_quad<BITS>(e, q.lo, q.hi, q.inv_scale),
+                                                qp_quad<BITS>(e + 4, q.lo, q.hi, q.inv_scale));
+                    if constexpr (BITS == 8) reinterpret_cast<uint2*>(orow)[v] = qd;
+                    else if constexpr (BITS == 4) orow[v] = qd.x | (qd.y << 16);
+                    else *reinterpret_cast<uint2*>(&sw[swz(2 * v)]) = qd;
+                }
+            };
+            const int whole = nvec & ~31;
+#pragma unroll 4
+            for (int v0 = 0; v0 < whole; v0 += 32) quantize(v0 + lane);
+            if (whole + lane < nvec) quantize(whole + lane);
+            if constexpr (BITS != 8 && !(BITS == 4 && EPV == 8)) {
+                // quads across the warp: 32 elements = BITS words per lane
+                __syncwarp();
+                uint32_t* words = reinterpret_cast<uint32_t*>(row);   // the row is no longer needed: room for its words
+                for (int g = lane; g < groups; g += 32) {
+                    const uint4 a = *reinterpret_cast<const uint4*>(&sw[swz(8 * g)]);
+                    const uint4 b = *reinterpret_cast<const uint4*>(&sw[swz(8 * g + 4)]);
+                    const uint32_t qd[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+                    uint32_t w[BITS];
+#pragma unroll
+                    for (int m = 0; m < BITS; ++m) w[m] = 0u;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        constexpr int QB = 4 * BITS;
+                        const int bit = QB * i, word = bit >> 5, sh = bit & 31;
+                        w[word] |= qd[i] << sh;
+                        if (sh + QB > 32) w[(word + 1) % BITS] |= qd[i] >> (32 - sh);
+                    }
+                    if constexpr (BITS == 4) {               // 4, 2, 1: a lane's words are one aligned vector
+                        *reinterpret_cast<uint4*>(orow + g * 4) = make_uint4(w[0], w[1], w[2], w[3]);
+                    } else if constexpr (BITS == 2) {
+                        *reinterpret_cast<uint2*>(orow + g * 2) = make_uint2(w[0], w[1]);
+                    } else if constexpr (BITS == 1) {
+                        orow[g] = w[0];
+                    } else {
+#pragma unroll
+                        for (int m = 0; m < BITS; ++m) words[g * BITS + m] = w[m];
+                    }
+                }
+                if constexpr (BITS != 4 && BITS != 2 && BITS != 1) {
+                    __syncwarp();
+                    for (int i = lane; i < groups * BITS; i += 32) orow[i] = words[i];
+                }
+            }
+            if (t == tokens - 1) {                           // pad words
+                const uint64_t end = tokens * (uint64_t)(groups * BITS);
+                if (lane < (int)(nwords - end)) out[end + lane] = 0u;
+            }
+        }
+        __syncwarp();                                        // the row may be overwritten
+    }
+    if (raise && lane == 0) atomicOr(status, raise);
+}
+
 // ---------------------------------------------------------------------------- host side
 
 int32_t tok_check(qp_ctx* ctx, uint64_t tokens, uint32_t channels)
@@ -424,6 +765,50 @@ int32_t unpack_tokens_typed(qp_ctx* ctx, const void* d_packed, uint64_t n, uint3
     return qp_check_launch(ctx, "qp_unpack_dequantize_tokens");
 }
 
+// Rows go through shared memory where a row fits: TR_WARPS of them in the 48 KB every block may have would
+// stop at 1536 fp32 channels; blocks ask for more, up to what leaves two blocks (16 warps) per SM.
+constexpr size_t TR_SMEM_MAX = 112 * 1024;
+bool tok_rows_apply(const void* x, int dtype, uint32_t C, bool sender)
+{
+    if (!x || (dtype != QP_F32 && dtype != QP_BF16)) return false;
+    const size_t esz = dtype == QP_F32 ? 4 : 2;
+    return C >= 32 && C % (sender ? 32 : 16 / esz) == 0 && ((uintptr_t)x & 15u) == 0 &&
+           tok_row_bytes(C, esz, sender) * TR_WARPS <= TR_SMEM_MAX;
+}
+
+template <int BITS, typename T>
+int32_t launch_rows(qp_ctx* ctx, const T* x, uint64_t tokens, uint32_t C, int method, int bmode, uint32_t* out,
+                    qp_qparams_t* d_qp, qp_stats_t* d_stats, cudaStream_t s)
+{
+    const size_t smem = tok_row_bytes(C, sizeof(T), BITS > 0) * TR_WARPS;
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(tok_rows_kernel<BITS, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)TR_SMEM_MAX) != cudaSuccess)
+        return qp_check_launch(ctx, "token rows (shared memory)");
+    const uint64_t want = (tokens + TR_WARPS - 1) / TR_WARPS, cap = (uint64_t)ctx->sm_count * 64;
+    tok_rows_kernel<BITS, T><<<(unsigned)(want < cap ? want : cap), TR_WARPS * 32, smem, s>>>(
+        x, tokens, C, method, bmode, BITS > 0 ? qp_host_aciq_F(BITS, QP_DIST_LAPLACE) : 0.0, out,
+        BITS > 0 ? qp_packed_bytes(tokens * C, BITS) / 4 : 0, d_qp, d_stats, ctx->d_status);
+    ctx->launches += 1;
+    return qp_check_launch(ctx, "token rows");
+}
+
+template <typename T>
+int32_t sender_tokens_typed(qp_ctx* ctx, const T* x, uint64_t tokens, uint32_t C, int bits, int method, int bmode, void* d_packed,
+                            qp_qparams_t* d_qp, qp_stats_t* d_stats, cudaStream_t s)
+{
+    uint32_t* out = static_cast<uint32_t*>(d_packed);
+    switch (bits) {
+        case 1: return launch_rows<1>(ctx, x, tokens, C, method, bmode, out, d_qp, d_stats, s);
+        case 2: return launch_rows<2>(ctx, x, tokens, C, method, bmode, out, d_qp, d_stats, s);
+        case 3: return launch_rows<3>(ctx, x, tokens, C, method, bmode, out, d_qp, d_stats, s);
+        case 4: return launch_rows<4>(ctx, x, tokens, C, method, bmode, out, d_qp, d_stats, s);
+        case 5: return launch_rows<5>(ctx, x, tokens, C, method, bmode, out, d_qp, d_stats, s);
+        case 6: return launch_rows<6>(ctx, x, tokens, C, method, bmode, out, d_qp, d_stats, s);
+        case 7: return launch_rows<7>(ctx, x, tokens, C, method, bmode, out, d_qp, d_stats, s);
+        default: return launch_rows<8>(ctx, x, tokens, C, method, bmode, out, d_qp, d_stats, s);
+    }
+}
+
 }  // namespace
 
 extern "C" int32_t qp_stats_tokens(qp_ctx* ctx, const void* d_x, int dtype, uint64_t tokens, uint32_t channels,
@@ -440,6 +825,11 @@ extern "C" int32_t qp_stats_tokens(qp_ctx* ctx, const void* d_x, int dtype, uint
     qp_device_guard guard(ctx->device);
     if (!guard.ok) return qp_fail(ctx, QP_ERR_CUDA, "cannot select device");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (tok_rows_apply(d_x, dtype, channels, false)) {
+        if (dtype == QP_F32)
+            return launch_rows<0>(ctx, static_cast<const float*>(d_x), tokens, channels, 0, 0, nullptr, nullptr, d_out, s);
+        return launch_rows<0>(ctx, static_cast<const unsigned short*>(d_x), tokens, channels, 0, 0, nullptr, nullptr, d_out, s);
+    }
     const unsigned blocks = tok_grid(ctx, tokens);
     const bool aligned = ((uintptr_t)d_x & 15u) == 0;
     if (dtype == QP_F32) {
@@ -525,7 +915,27 @@ extern "C" int32_t qp_sender_tokens_device(qp_ctx* ctx, const void* d_x, int dty
 {
     if (!ctx) return QP_ERR_INVALID_ARG;
     if (tokens > 0 && (!d_qp_out || !d_stats_work)) return qp_fail(ctx, QP_ERR_INVALID_ARG, "null d_qp_out / d_stats_work");
-    int32_t rc = qp_stats_tokens(ctx, d_x, dtype, tokens, channels, d_stats_work, stream);
+    int32_t rc;
+    if (tokens > 0 && bits >= 1 && bits <= 8 && qp_clip_method_closed_form(method) &&
+        (bmode == QP_B_MAD || bmode == QP_B_MEAN_ABS) && tok_rows_apply(d_x, dtype, channels, true)) {
+        // the checks of the three calls that this one launch does not get to otherwise
+        rc = tok_check(ctx, tokens, channels);
+        if (rc) return rc;
+        if (packed_capacity < qp_packed_bytes(tokens * channels, bits))
+            return qp_fail(ctx, QP_ERR_BUFFER_TOO_SMALL, "packed_capacity < qp_packed_bytes(n, bits)");
+        if (!d_packed) return qp_fail(ctx, QP_ERR_INVALID_ARG, "null pointer");
+        if (((uintptr_t)d_packed & 15u) || ((uintptr_t)d_qp_out & 3u) || ((uintptr_t)d_stats_work & 7u))
+            return qp_fail(ctx, QP_ERR_ALIGNMENT, "d_packed (16 bytes), d_qp_out or d_stats_work not aligned");
+        qp_device_guard guard(ctx->device);
+        if (!guard.ok) return qp_fail(ctx, QP_ERR_CUDA, "cannot select device");
+        cudaStream_t s = static_cast<cudaStream_t>(stream);
+        if (dtype == QP_F32)
+            return sender_tokens_typed<float>(ctx, static_cast<const float*>(d_x), tokens, channels, bits, method, bmode, d_packed,
+                                              d_qp_out, d_stats_work, s);
+        return sender_tokens_typed<unsigned short>(ctx, static_cast<const unsigned short*>(d_x), tokens, channels, bits, method,
+                                                   bmode, d_packed, d_qp_out, d_stats_work, s);
+    }
+    rc = qp_stats_tokens(ctx, d_x, dtype, tokens, channels, d_stats_work, stream);
     if (rc < 0) return rc;
     rc = qp_clip_qparams_tokens_device(ctx, d_stats_work, tokens, bits, method, QP_DIST_LAPLACE, bmode, d_qp_out, stream);
     if (rc < 0) return rc;

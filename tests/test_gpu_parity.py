@@ -1358,6 +1358,19 @@ def test_tokens_shapes_ragged_and_methods(ctx, channels, tokens):
     ctx.qp_get_status()                                         # one-channel tokens have no spread: degenerate
 
 
+# rows in shared memory: less than a round of lanes, whole and partial rounds, the longest rows and one beyond
+@pytest.mark.parametrize("channels,bits", [(32, 3), (96, 8), (160, 4), (256, 2), (1056, 8), (1312, 7), (2848, 6), (2880, 6)])
+def test_tokens_rows_edges(ctx, channels, bits):
+    x = si.vit_activation((1, 37, channels), 500 + channels).reshape(-1)
+    check_tokens(ctx, x, dev(x), channels, bits)
+    x[[5, channels, 36 * channels + 7]] = [np.nan, np.inf, -np.inf]       # rows that are gone through element by element
+    x[3 * channels:4 * channels] = np.float32(-0.75)                     # a constant row
+    h = si.to_bf16_bits(x)
+    d = torch.from_numpy(h.view(np.int16)).cuda().view(torch.bfloat16)
+    check_tokens(ctx, oracle.widen_bf16(h), d, channels, bits)
+    assert ctx.qp_get_status() == qp.QP_DEV_NONFINITE | qp.QP_DEV_DEGENERATE
+
+
 def test_tokens_misaligned_nonfinite_bf16_and_errors(ctx):
     x = si.vit_activation((1, 301, 96), 167, outlier_frac=0.03).reshape(-1).astype(np.float32)
     big = dev(np.concatenate([np.zeros(1, np.float32), x]))
