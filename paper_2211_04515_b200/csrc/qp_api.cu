@@ -758,6 +758,10 @@ extern "C" int32_t qp_unpack_dequantize(qp_ctx* ctx, const void* d_packed, uint6
 
 // ------------------------------------------- whole sender on device buffers
 
+// Above this many elements statistics, search and packing are one launch of the streaming kernel; the small-tensor launch
+// ends there at the latest (closed-form clips), and the separate calls' launches serve what is between the two.
+constexpr uint64_t QP_ONE_LAUNCH_MIN_N = 1ull << 21;
+
 // statistics -> clip -> quantize+pack on device buffers: one cooperative launch where that
 // applies (small tensors), the kernel chain of the separate calls otherwise
 static int32_t sender_on_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int bits, int method, int bmode,
@@ -784,6 +788,22 @@ static int32_t sender_on_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_
                                     static_cast<cudaStream_t>(stream));
         if (rc == QP_OK && use_ds) { ctx->last_steps = steps; ctx->last_bits = bits; }
         if (rc != QP_WARN_INFEASIBLE) return rc;               // else: this device cannot hold the grid
+    }
+    if (use_ds && ctx->sender_path == QP_SENDER_AUTO && ctx->stats_path == QP_STATS_AUTO && ctx->search_path == QP_SEARCH_AUTO &&
+        n > QP_ONE_LAUNCH_MIN_N && check_x(ctx, d_x, dtype, n) == QP_OK && steps >= 1 && d_packed && !((uintptr_t)d_packed & 15u) &&
+        !((uintptr_t)st & 7u) && !((uintptr_t)d_qp_out & 3u) && (bmode == QP_B_MAD || bmode == QP_B_MEAN_ABS) &&
+        qp_stats_search_applies(ctx, d_x, dtype, n, hist_bins, bits, steps)) {
+        qp_device_guard guard(ctx->device);
+        if (!guard.ok) return qp_fail(ctx, QP_ERR_CUDA, "cannot select device");
+        rc = qp_launch_stats_search(ctx, d_x, dtype, n, nullptr, st, hist_bins, bits, search_mode, steps,
+                                    qp_host_aciq_F(bits, QP_DIST_LAPLACE), nullptr, d_qp_out, d_packed,
+                                    static_cast<cudaStream_t>(stream));
+        if (rc < 0) return rc;
+        ctx->last_steps = steps;
+        ctx->last_bits = bits;
+        ctx->last_x = d_x;
+        ctx->last_x_end = 0;
+        return rc;
     }
     rc = qp_stats(ctx, d_x, dtype, n, use_ds ? hist_bins : 0, st, stream);
     if (rc < 0) return rc;

@@ -48,4 +48,24 @@ __device__ __forceinline__ bool barrier(unsigned* bar, unsigned target, unsigned
     return *s_ok != 0;
 }
 
+// The wait alone, for a block that has arrived before (arrive_release by one thread behind a block barrier).
+__device__ __forceinline__ bool wait(const unsigned* bar, unsigned target, unsigned spin_limit, unsigned* status, int* s_ok)
+{
+    if (threadIdx.x == 0) {
+        int ok = 1;
+        unsigned spins = 0;
+        while (ld_acquire(bar) < target) {
+            if (++spins > spin_limit) {
+                ok = 0;
+                atomicOr(status, QP_DEV_STREAM_TIMEOUT);
+                break;
+            }
+            if (spins > 64) __nanosleep(64);
+        }
+        *s_ok = ok;
+    }
+    __syncthreads();
+    return *s_ok != 0;
+}
+
 }  // namespace qp_grid

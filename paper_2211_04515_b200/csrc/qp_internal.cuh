@@ -79,6 +79,7 @@ struct qp_ctx {
     int stats_path;                      // 0 auto, 1 two kernels, 2 one cooperative launch where it applies
     int fused_checked, fused_ok;         // whether this device can hold the cooperative sender's grid
     int stats_fused_checked, stats_fused_ok;   // the same for the one-launch statistics
+    int ss_checked, ss_ok;               // the same for statistics and search in one launch
     long long wait_cycles;               // limit of a wait for a tile copy (clock cycles)
     unsigned spin_limit;                 // limit of a grid-barrier wait (polls)
     int bar_extra;                       // test only: arrivals a grid barrier waits for beyond the grid size
@@ -110,9 +111,12 @@ struct qp_ctx {
     char err[256];
 };
 
-// Scratch of the cooperative kernels (d_fused): 256 bytes of barrier counters and the whole-sender
-// kernel's histogram (4096 x 8 bytes).
-constexpr size_t QP_FUSED_BYTES = 256 + sizeof(unsigned long long) * 4096;
+// Scratch of the cooperative kernels (d_fused): 256 bytes of barrier counters and the histogram (4096 x 8 bytes), both
+// zero between launches, and the interval totals of the search (count and sum, 8 bytes each).
+constexpr int QP_SS_MAX_CAND = 256;              // candidates of the search in one launch with the statistics
+constexpr int QP_SS_TOTALS = 4096;
+constexpr size_t QP_FUSED_TOTALS_AT = 256 + sizeof(unsigned long long) * 4096;
+constexpr size_t QP_FUSED_BYTES = QP_FUSED_TOTALS_AT + 16 * (size_t)QP_SS_TOTALS;
 
 constexpr long long QP_WAIT_CYCLES_DEFAULT = 4000000000ll;   // about two seconds
 constexpr unsigned QP_SPIN_LIMIT_DEFAULT = 1u << 22;          // x 64 ns sleeps: a quarter of a second at least
@@ -540,6 +544,10 @@ int32_t qp_launch_channel_interval_sums(qp_ctx* ctx, const void* d_x, int dtype,
 int32_t qp_launch_interval_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, const qp_stats_t* d_stats,
                                   int bits, int bmode, int steps, int hist_bins, double F, qp_ds_result_t* d_out,
                                   qp_qparams_t* d_qp_out, cudaStream_t s);
+bool qp_stats_search_applies(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int hist_bins, int bits, int steps);
+int32_t qp_launch_stats_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, const qp_stats_t* st_in, qp_stats_t* st_out,
+                               int hist_bins, int bits, int bmode, int steps, double F, qp_ds_result_t* d_out,
+                               qp_qparams_t* d_qp_out, void* d_packed, cudaStream_t s);
 bool qp_sender_fused_applies(uint64_t n, int use_ds, int steps, int hist_bins, bool forced);
 int32_t qp_launch_sender_fused(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int bits, int method, int bmode,
                                int steps, int hist_bins, double F, void* d_packed, qp_qparams_t* d_qp_out,

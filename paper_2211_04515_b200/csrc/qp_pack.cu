@@ -16,11 +16,11 @@
 // bits = 16: one uint16 per element, plain vectorised map.
 // The last, partial tile and the pad words are guarded iterations of the same loop, and an input that
 // is not 16-byte aligned takes the same kernel with element loads: one launch for every shape.
-#include "qp_internal.cuh"
+#include "qp_packtile.cuh"
 
 namespace {
 
-constexpr int TILE = 1024;                 // elements per warp tile
+constexpr int TILE = QP_TILE;
 constexpr int WARPS = QP_THREADS / 32;
 
 struct QP4 { float lo, hi, inv; unsigned mask; };
@@ -39,109 +39,22 @@ __device__ __forceinline__ QP4 load_qp(const qp_qparams_t* __restrict__ d_qp, co
     return q;
 }
 
-// physical word of quad p in a warp's 256-word staging buffer: 16-byte chunk index XOR bit 3
-__device__ __forceinline__ int swz(int p) { return ((((p >> 2) ^ ((p >> 5) & 1)) << 2) | (p & 3)); }
-
-template <int BITS>
-__device__ __forceinline__ unsigned quad_of(const float* e, const QP4& q)
-{
-    unsigned r = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) r |= qp_code(e[i], q.lo, q.hi, q.inv, q.mask) << (BITS * i);
-    return r;
-}
-
-// ntiles counts the last, partial tile too: its missing elements are NaN (code 0) and its words are
-// written up to nwords, pad words included.  VEC: x is 16-byte aligned.  Otherwise every lane loads the
-// elements of its vectors one by one (the four loads of a vector touch the same lines, so they hit L1).
+// ntiles counts the last, partial tile too.
 template <int BITS, typename T, bool VEC>
 __global__ void __launch_bounds__(QP_THREADS) pack_kernel(const T* __restrict__ x, uint64_t n, uint64_t ntiles,
                                                           const qp_qparams_t* __restrict__ d_qp, qp_qparams_t h_qp,
                                                           uint32_t* __restrict__ out, uint64_t nwords,
                                                           unsigned* __restrict__ status, int reverse)
 {
-    constexpr int EPV = qp_span<T>::EPV;          // 4 (f32) or 8 (bf16) elements per 16-byte vector
-    constexpr int NLOAD = TILE / (32 * EPV);      // 8 or 4 vector loads per lane
     __shared__ __align__(16) uint32_t stage[WARPS][256];
     const QP4 q = load_qp(d_qp, h_qp, BITS, status);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t* sw = stage[warp];
     const unsigned warps = blockDim.x >> 5;
     const uint64_t wstride = (uint64_t)gridDim.x * warps;
-
     // `reverse`: the grid walks the tensor from its end (the tiles are the same), for a call that
     // follows a pass which ended there and left that part of x in L2
-    for (uint64_t it = (uint64_t)blockIdx.x * warps + warp; it < ntiles; it += wstride) {
-        const uint64_t tile = reverse ? ntiles - 1 - it : it;
-        const T* xt = x + tile * TILE;
-        const bool full = (tile + 1) * TILE <= n;                 // warp-uniform
-        float e[NLOAD][EPV];
-        if (full) {
-#pragma unroll
-            for (int j = 0; j < NLOAD; ++j) {
-                if constexpr (VEC) {
-                    qp_load_vec(xt + (j * 32 + lane) * EPV, e[j]);
-                } else {
-#pragma unroll
-                    for (int i = 0; i < EPV; ++i) e[j][i] = qp_load_one(xt + (j * 32 + lane) * EPV + i);
-                }
-            }
-        } else {
-            const int have = (int)(n - tile * TILE);
-#pragma unroll
-            for (int j = 0; j < NLOAD; ++j)
-#pragma unroll
-                for (int i = 0; i < EPV; ++i) {
-                    const int k = (j * 32 + lane) * EPV + i;
-                    e[j][i] = k < have ? qp_load_one(xt + k) : __int_as_float(0x7FC00000);
-                }
-        }
-#pragma unroll
-        for (int j = 0; j < NLOAD; ++j) {
-            if constexpr (EPV == 4) {
-                sw[swz(j * 32 + lane)] = quad_of<BITS>(e[j], q);
-            } else {
-                uint2 two;
-                two.x = quad_of<BITS>(e[j], q);
-                two.y = quad_of<BITS>(e[j] + 4, q);
-                *reinterpret_cast<uint2*>(&sw[swz(2 * (j * 32 + lane))]) = two;
-            }
-        }
-        __syncwarp();
-        const uint4 a = *reinterpret_cast<const uint4*>(&sw[swz(8 * lane)]);
-        const uint4 b = *reinterpret_cast<const uint4*>(&sw[swz(8 * lane + 4)]);
-        const uint32_t qd[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        uint32_t w[BITS];
-#pragma unroll
-        for (int m = 0; m < BITS; ++m) w[m] = 0u;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            constexpr int QB = 4 * BITS;
-            const int bit = QB * k, word = bit >> 5, sh = bit & 31;
-            w[word] |= qd[k] << sh;
-            if (sh + QB > 32) w[(word + 1) % BITS] |= qd[k] >> (32 - sh);
-        }
-        uint32_t* ot = out + tile * (32 * BITS);
-        if (full && BITS == 8) {
-            uint4* o = reinterpret_cast<uint4*>(ot + lane * 8);
-            o[0] = make_uint4(w[0], w[1 % BITS], w[2 % BITS], w[3 % BITS]);
-            o[1] = make_uint4(w[4 % BITS], w[5 % BITS], w[6 % BITS], w[7 % BITS]);
-        } else if (full && BITS == 4) {
-            *reinterpret_cast<uint4*>(ot + lane * 4) = make_uint4(w[0], w[1 % BITS], w[2 % BITS], w[3 % BITS]);
-        } else if (full && BITS == 2) {
-            *reinterpret_cast<uint2*>(ot + lane * 2) = make_uint2(w[0], w[1 % BITS]);
-        } else {
-            __syncwarp();
-#pragma unroll
-            for (int m = 0; m < BITS; ++m) sw[lane * BITS + m] = w[m];
-            __syncwarp();
-            const int room = (int)min((uint64_t)(32 * BITS), nwords - tile * (32 * BITS));
-#pragma unroll
-            for (int m = 0; m < BITS; ++m)
-                if (m * 32 + lane < room) ot[m * 32 + lane] = sw[m * 32 + lane];
-        }
-        __syncwarp();
-    }
+    for (uint64_t it = (uint64_t)blockIdx.x * warps + warp; it < ntiles; it += wstride)
+        qp_pack_tile<BITS, T, VEC>(x, n, reverse ? ntiles - 1 - it : it, lane, q.lo, q.hi, q.inv, out, nwords, stage[warp]);
 }
 
 // bits = 16: thread t converts the 8 elements [8t, 8t+8) to one 16-byte vector of uint16 codes.

@@ -919,6 +919,9 @@ int32_t qp_launch_stats(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int
     // histogram rides along (66.3 us against 72.5; equal without it, 59 us): QP_STATS_AUTO takes the one launch
     // without the histogram and the two kernels with it; QP_STATS_FUSED and QP_STATS_TWO_KERNELS force either.
     const bool with_hist = hist_bins >= 1 && hist_bins <= ST_FUSED_HIST_MAX;
+    if (ctx->stats_path == QP_STATS_AUTO && with_hist && ntiles >= 8 &&
+        qp_stats_search_applies(ctx, d_x, dtype, n, hist_bins, 0, 0))
+        return qp_launch_stats_search(ctx, d_x, dtype, n, nullptr, d_out, hist_bins, 0, 0, 0, 0.0, nullptr, nullptr, nullptr, s);
     const bool one_launch = ctx->stats_path == QP_STATS_FUSED || (ctx->stats_path == QP_STATS_AUTO && !with_hist);
     if (ntiles >= 8 && one_launch && stats_fused_usable(ctx)) {
         if (dtype == QP_F32) return launch_fused<float>(ctx, static_cast<const float*>(d_x), n, hist_bins, d_out, s);

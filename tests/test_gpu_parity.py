@@ -948,6 +948,77 @@ def test_search_forms_agree_beyond_two_waves(ctx, n):
     assert ctx.qp_get_status() == 0
 
 
+# statistics and search in one launch (the default from 2^20 elements on, the sender above 2^21): every width it takes, tile
+# remainders, the largest and smallest number of steps, tables with few replicas, and the exact-threshold form
+SS_CASES = [(1, 0, 100, 100, (1 << 21) + 1, "vit"), (2, 0, 100, 100, (1 << 21) + 1023, "outliers"), (3, 0, 100, 100, (1 << 21) + 1024, "vit"),
+            (4, 0, 100, 100, (1 << 21) + 5, "outliers"), (4, qp.QP_B_MIDRISE, 255, 4096, (1 << 21) + 77, "vit"),
+            (2, qp.QP_B_GAUSS, 1, 1, (1 << 21) + 512, "vit"), (3, qp.QP_B_MEAN_ABS, 37, 1000, (1 << 21) + 31, "nonfinite"),
+            (4, 0, 100, 100, (1 << 21) + 9, "offset"), (2, 0, 100, 100, (1 << 21) + 9, "offset"),
+            (4, 0, 255, 100, (1 << 21) + 9, "constant"), (2, 0, 100, 100, (1 << 21) + 2048, "two_levels"),
+            (3, 0, 100, 100, (1 << 21) + 3, "tiny")]
+
+
+@pytest.mark.parametrize("bits,bmode,steps,nb,n,data", SS_CASES)
+@pytest.mark.parametrize("bf16", [False, True])
+def test_stats_and_search_in_one_launch(ctx, bits, bmode, steps, nb, n, data, bf16):
+    x = si.vit_activation((1, n // 256 + 1, 256), 700 + bits, outlier_frac=0.02 if data == "outliers" else 0.0).reshape(-1)[:n].copy()
+    if data == "nonfinite":
+        x[[0, 1023, n // 2, n - 1]] = [np.nan, np.inf, -np.inf, np.nan]
+    elif data == "offset":                               # clip ends coarse against the step: exact thresholds
+        x = (np.float32(4096.0) + x).astype(np.float32)
+        x[::5000] += np.float32(300.0)
+    elif data == "constant":
+        x[:] = np.float32(-2.5)
+    elif data == "two_levels":
+        x = np.where(np.arange(n) % 3 == 0, np.float32(-1.0), np.float32(2.0)).astype(np.float32)
+    elif data == "tiny":
+        x *= np.float32(1e-20)
+    d = dev(x)
+    if bf16:
+        h = si.to_bf16_bits(x)
+        d, x = torch.from_numpy(h.view(np.int16)).cuda().view(torch.bfloat16), oracle.widen_bf16(h)
+    st_o = oracle.stats(x)
+    st = ctx.read_stats(ctx.qp_stats(d, hist_bins=nb))
+    if data != "constant":
+        check_stats(st, st_o)
+        assert st.hist_peak == int(oracle.hist_peak(x, st_o.min, st_o.max, nb)[1].max())
+    assert st.hist_bins == nb
+    result = oracle.ds_search(x, st_o, bits, bmode, steps, nb)
+    if data == "constant":
+        d_res, d_qp = ctx.qp_dsaciq_search(d, ctx.qp_stats(d), bits, bmode, steps, nb)       # counts for itself
+        res, q = ctx.read_ds_result(d_res), ctx.read_qparams(d_qp)
+        assert res.k_star == 0 and res.mse_star == 0.0 and q.flags == 1 and (q.lo, q.hi) == (-2.5, -2.5)
+    else:
+        before = ctx.qp_launch_count()
+        # (two atoms feel an ulp of a clip end: every step on the library's own quantizers there)
+        check_search(ctx, x, d, bits, bmode, steps, nb, exact_steps=None if data == "two_levels" else [0, steps // 2, steps],
+                     oracle_result=result)
+        assert ctx.qp_launch_count() - before == 2       # the statistics and the search
+        first = ctx.qp_dsaciq_curve(steps)
+        d_plain = ctx.qp_stats(d)                        # no histogram in them: the search counts for itself
+        ctx.qp_dsaciq_search(d, d_plain, bits, bmode, steps, nb)
+        second = np.array(ctx.qp_dsaciq_curve(steps))
+        assert data == "two_levels" or np.all(np.abs(second - first) <= 2e-6 * np.abs(first) + 1e-300)
+    if bmode & qp.QP_B_GAUSS == 0:                       # the sender: the same launch packs as well
+        method = qp.QP_CLIP_DSACIQ | (qp.QP_CLIP_MIDRISE if bmode & qp.QP_B_MIDRISE else 0)
+        whole, packed = guarded(qp.qp_packed_bytes(n, bits))
+        before = ctx.qp_launch_count()
+        _, d_qp = ctx.qp_sender_device(d, bits, method, out_packed=packed, bmode=bmode & 0xF, steps=steps, hist_bins=nb)
+        assert ctx.qp_launch_count() - before == 1
+        again, d_qp2 = ctx.qp_sender_device(d, bits, method, bmode=bmode & 0xF, steps=steps, hist_bins=nb)
+        assert torch.equal(packed, again) and torch.equal(d_qp, d_qp2)                # bit-reproducible
+        assert canaries_intact(whole, packed.numel())
+        q = ctx.read_qparams(d_qp)
+        if data != "constant":
+            cand = ctx.qp_dsaciq_candidates(steps)
+            k = [i for i in range(steps + 1) if (cand[i].lo, cand[i].hi) == (q.lo, q.hi)][0]
+            curve = np.array(ctx.qp_dsaciq_curve(steps))
+            assert curve[k] == curve.min()
+        o = oracle.QParams(q.lo, q.hi, q.scale, q.inv_scale, q.bits, q.flags)
+        assert np.array_equal(packed.cpu().numpy(), oracle.quantize_pack(x, o))
+    assert ctx.qp_get_status() & ~(qp.QP_DEV_NONFINITE | qp.QP_DEV_DEGENERATE) == 0
+
+
 # ------------------------------------------------------------------ graph replay (execution option)
 
 @pytest.mark.parametrize("n_images,path", [(6, qp.QP_SEARCH_CANDIDATES), (40, qp.QP_SEARCH_AUTO)])
