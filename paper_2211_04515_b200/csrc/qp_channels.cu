@@ -733,6 +733,9 @@ extern "C" int32_t qp_stats_channels(qp_ctx* ctx, const void* d_x, int dtype, ui
             return qp_check_launch(ctx, "qp_stats_channels");
         return QP_OK;
     }
+    if (qp_channel_strips_apply(ctx, rows, channels, 0))
+        return qp_launch_channel_strips(ctx, d_x, dtype, rows, channels, nullptr, d_out, 0, 0, QP_DEFAULT_STEPS, 0, 0, 0.0, nullptr,
+                                        nullptr, nullptr, nullptr, nullptr, s);
     if (dtype == QP_F32) return stats_channels_typed<float>(ctx, static_cast<const float*>(d_x), rows, channels, d_out, s);
     return stats_channels_typed<unsigned short>(ctx, static_cast<const unsigned short*>(d_x), rows, channels, d_out, s);
 }
@@ -980,6 +983,17 @@ extern "C" int32_t qp_sender_channels_device(qp_ctx* ctx, const void* d_x, int d
             ctx->ch_stats_bytes = need;
         }
         st = static_cast<qp_stats_t*>(ctx->d_ch_stats);
+    }
+    if (use_ds && rows > 0 && d_x && (dtype == QP_F32 || dtype == QP_BF16) && !((uintptr_t)d_x & (dtype == QP_F32 ? 3u : 1u)) &&
+        !((uintptr_t)st & 7u) && !((uintptr_t)d_qp_out & 3u) && ((bmode & ~(QP_B_MIDRISE | QP_B_GAUSS)) == QP_B_MAD ||
+        (bmode & ~QP_B_MIDRISE) == QP_B_MEAN_ABS)) {
+        qp_device_guard guard(ctx->device);
+        if (!guard.ok) return qp_fail(ctx, QP_ERR_CUDA, "cannot select device");
+        rc = qp_stats_search_channels(ctx, d_x, dtype, rows, channels, st, bits, bmode | ((method & QP_CLIP_MIDRISE) ? QP_B_MIDRISE : 0),
+                                      QP_DEFAULT_STEPS, QP_DEFAULT_HIST_BINS, d_qp_out, static_cast<cudaStream_t>(stream));
+        if (rc < 0) return rc;
+        if (rc == QP_OK)
+            return qp_quantize_pack_channels(ctx, d_x, dtype, rows, channels, bits, d_qp_out, d_packed, packed_capacity, stream);
     }
     rc = qp_stats_channels(ctx, d_x, dtype, rows, channels, st, stream);
     if (rc < 0) return rc;

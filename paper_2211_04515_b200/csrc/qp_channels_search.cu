@@ -213,8 +213,8 @@ __global__ void __launch_bounds__(128) ch_pick_kernel(const double* __restrict__
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
 template <typename T>
-int32_t search_channels_typed(qp_ctx* ctx, const T* x, uint64_t rows, uint32_t C, const qp_stats_t* d_stats, int bits,
-                              int bmode, int steps, int nb, double F, qp_ds_result_t* d_out, qp_qparams_t* d_qp_out,
+int32_t search_channels_typed(qp_ctx* ctx, const T* x, uint64_t rows, uint32_t C, const qp_stats_t* d_stats, qp_stats_t* st_out,
+                              int bits, int bmode, int steps, int nb, double F, qp_ds_result_t* d_out, qp_qparams_t* d_qp_out,
                               cudaStream_t s)
 {
     const int ncp = (steps + 1 + CK - 1) / CK * CK;          // candidates padded to whole groups
@@ -227,8 +227,10 @@ int32_t search_channels_typed(qp_ctx* ctx, const T* x, uint64_t rows, uint32_t C
     if (row_blocks > (rows + min_rows - 1) / min_rows) row_blocks = (rows + min_rows - 1) / min_rows;
     if (row_blocks < 1) row_blocks = 1;
     // interval moments where they apply (qp_set_search_path(QP_SEARCH_CANDIDATES) keeps the scoring of every candidate)
-    const bool intervals = ctx->search_path != QP_SEARCH_CANDIDATES && qp_channel_interval_applies(rows, bits, steps);
-    if (intervals) row_blocks = 1;
+    // (up to 4 bits in the strips kernel)
+    const bool strips = ctx->search_path != QP_SEARCH_CANDIDATES && qp_channel_strips_apply(ctx, rows, C, bits);
+    const bool intervals = !strips && ctx->search_path != QP_SEARCH_CANDIDATES && qp_channel_interval_applies(rows, bits, steps);
+    if (intervals || strips) row_blocks = 1;
     const uint64_t rows_per_block = (rows + row_blocks - 1) / row_blocks;
 
     size_t off = 0;
@@ -258,6 +260,15 @@ int32_t search_channels_typed(qp_ctx* ctx, const T* x, uint64_t rows, uint32_t C
     double* curve = reinterpret_cast<double*>(b + o_curve);
     double* part = reinterpret_cast<double*>(b + o_part);
 
+    ctx->ch_last_steps = steps;
+    ctx->ch_last_ncp = ncp;
+    ctx->ch_last_channels = C;
+    ctx->ch_curve_offset = o_curve;
+    ctx->ch_cand_offset = o_cand;
+    ctx->ch_last_bits = bits;
+    if (strips)
+        return qp_launch_channel_strips(ctx, x, sizeof(T) == 4 ? QP_F32 : QP_BF16, rows, C, d_stats, st_out, bits, bmode, steps, ncp,
+                                        nb, F, cand, valid, curve, d_out, d_qp_out, s);
     if (cudaMemsetAsync(hist, 0, sizeof(unsigned) * (size_t)C * nb, s) != cudaSuccess)
         return qp_check_launch(ctx, "qp_dsaciq_search_channels (histogram reset)");
     const size_t hist_smem = sizeof(unsigned) * CS_HIST_CH * (size_t)nb;
@@ -282,16 +293,24 @@ int32_t search_channels_typed(qp_ctx* ctx, const T* x, uint64_t rows, uint32_t C
     ch_pick_kernel<<<C, 128, 0, s>>>(part, (int)row_blocks, C, steps, ncp, nb, bits, valid, cand, setup, curve, d_out,
                                      d_qp_out, ctx->d_status);
     ctx->launches += 1;
-    ctx->ch_last_steps = steps;
-    ctx->ch_last_ncp = ncp;
-    ctx->ch_last_channels = C;
-    ctx->ch_curve_offset = o_curve;
-    ctx->ch_cand_offset = o_cand;
-    ctx->ch_last_bits = bits;
     return qp_check_launch(ctx, "qp_dsaciq_search_channels");
 }
 
 }  // namespace
+
+// Statistics and search in one call (the channel-wise sender; arguments checked there): QP_WARN_INFEASIBLE where the strips
+// kernel does not apply.
+int32_t qp_stats_search_channels(qp_ctx* ctx, const void* d_x, int dtype, uint64_t rows, uint32_t channels, qp_stats_t* st_out,
+                                 int bits, int bmode, int steps, int hist_bins, qp_qparams_t* d_qp_out, cudaStream_t s)
+{
+    if (ctx->search_path == QP_SEARCH_CANDIDATES || !qp_channel_strips_apply(ctx, rows, channels, bits)) return QP_WARN_INFEASIBLE;
+    const double F = qp_host_aciq_F(bits, (bmode & QP_B_GAUSS) ? QP_DIST_GAUSS : QP_DIST_LAPLACE);
+    if (dtype == QP_F32)
+        return search_channels_typed<float>(ctx, static_cast<const float*>(d_x), rows, channels, nullptr, st_out, bits, bmode, steps,
+                                            hist_bins, F, nullptr, d_qp_out, s);
+    return search_channels_typed<unsigned short>(ctx, static_cast<const unsigned short*>(d_x), rows, channels, nullptr, st_out, bits,
+                                                 bmode, steps, hist_bins, F, nullptr, d_qp_out, s);
+}
 
 extern "C" int32_t qp_dsaciq_search_channels(qp_ctx* ctx, const void* d_x, int dtype, uint64_t rows, uint32_t channels,
                                              const qp_stats_t* d_stats, int bits, int bmode, int steps, int hist_bins,
@@ -319,9 +338,9 @@ extern "C" int32_t qp_dsaciq_search_channels(qp_ctx* ctx, const void* d_x, int d
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const double F = qp_host_aciq_F(bits, (bmode & QP_B_GAUSS) ? QP_DIST_GAUSS : QP_DIST_LAPLACE);
     if (dtype == QP_F32)
-        return search_channels_typed<float>(ctx, static_cast<const float*>(d_x), rows, channels, d_stats, bits, bmode, steps,
+        return search_channels_typed<float>(ctx, static_cast<const float*>(d_x), rows, channels, d_stats, nullptr, bits, bmode, steps,
                                             hist_bins, F, d_out, d_qp_out, s);
-    return search_channels_typed<unsigned short>(ctx, static_cast<const unsigned short*>(d_x), rows, channels, d_stats, bits,
+    return search_channels_typed<unsigned short>(ctx, static_cast<const unsigned short*>(d_x), rows, channels, d_stats, nullptr, bits,
                                                  bmode, steps, hist_bins, F, d_out, d_qp_out, s);
 }
 

@@ -1,0 +1,694 @@
+// Channel-wise statistics and directed search (paper Sec. 3, Eq. 1, run per column of a [rows, channels] tensor) in one
+// launch: a cluster of S blocks owns a strip of w neighbouring channels, each block a part of the rows, so nothing is
+// merged across the grid.
+//
+//   phase A   sum x, sum |x|, min, max, non-finite count per channel
+//   phase B   sum |x - mean|, sum (x - mean)^2, histogram over the channel's [min, max]
+//   phase C   per channel, the count and the sum of the elements of every interval between the candidates' thresholds
+//             (qp_affine.cuh), in shared memory
+//   finish    two warps per channel (a side each): prefix sums over the intervals, the error of every candidate from 2^bits
+//             differences, first minimum, quantizer
+// Between the phases the blocks of a cluster add up their parts through distributed shared memory.  A thread stays with one
+// channel and walks its rows, sixteen loads ahead; the first pass takes the strip from DRAM, the others from L2.
+//
+// What bounds it: the instructions (A 4, B 11, C 14 + 2 per code boundary and element) and, as a strip's row is 4 w bytes,
+// the L1 look-ups, one or two per row and pass.  12608 x 1024 fp32 at 4 bits (52 MB): see the table of measurements in the
+// kernel list; the ten kernels before (four for the statistics, histogram, set-up, thresholds sorted per channel, a
+// pass with binary searches, error curves, pick) took 255 us.
+#include <cooperative_groups.h>
+
+#include <type_traits>
+
+#include "qp_affine.cuh"
+
+namespace cg = cooperative_groups;
+
+QP_CK_UNIT
+
+namespace {
+
+constexpr int CT_THREADS = 512;
+constexpr int CT_WARPS = CT_THREADS / 32;
+constexpr int CT_MAX_W = 16;                       // channels of a strip
+constexpr int CT_MAX_S = 8;                        // blocks of a cluster
+constexpr int CT_AHEAD = 16;                       // loads in flight per thread
+constexpr float CT_INF = __builtin_huge_valf();
+constexpr int CT_MAX_CAND = QP_CH_MAX_STEPS + 1;
+constexpr size_t CT_TABLE_BYTES = 2 * SS_SUMS_AT;  // interval tables (counts, then sums) of the strip
+constexpr size_t CT_DYN_BYTES = CT_TABLE_BYTES + (size_t)CT_MAX_W * (QP_CH_MAX_HIST_BINS + 1) * sizeof(unsigned);
+
+struct CtArgs {
+    const void* x;
+    uint64_t rows;
+    uint32_t C;
+    int w;                                         // channels per strip
+    uint64_t rows_pb;                              // rows per block of a cluster
+    int nb, steps, bmode, ncp, ub;
+    double F;
+    const qp_stats_t* st_in;                       // search only: the caller's statistics
+    qp_stats_t* st_out;
+    float4* cand;                                  // [C][ncp]
+    int* valid;                                    // [C][ncp]
+    double* curve;                                 // [C][ncp]
+    qp_ds_result_t* ds_out;
+    qp_qparams_t* qp_out;
+    unsigned* status;
+};
+
+// The m rows p, p + st, p + 2 st, ... of a column, CT_AHEAD loads ahead of their use: f.one(value) for each, f.fold() after
+// every CT_AHEAD of them and at the end.
+template <typename T, typename F>
+__device__ __forceinline__ void ct_column(const T* p, uint32_t st, int m, F& f)
+{
+    if (m <= 0) return;
+    using Raw = typename std::conditional<sizeof(T) == 4, float, unsigned short>::type;
+    auto load = [](const T* q) { return __ldg(reinterpret_cast<const Raw*>(q)); };
+    auto value = [](Raw r) {
+        if constexpr (sizeof(T) == 4) return (float)r;
+        else return qp_bf16_to_f32(r);
+    };
+    Raw v[CT_AHEAD];
+    const int full = m / CT_AHEAD, rest = m - full * CT_AHEAD;
+    if (full) {
+#pragma unroll
+        for (int j = 0; j < CT_AHEAD; ++j) v[j] = load(p + j * st);
+        for (int b = 1; b <= full; ++b) {
+            if (b < full) p += (uint64_t)CT_AHEAD * st;
+#pragma unroll
+            for (int j = 0; j < CT_AHEAD; ++j) {
+                const Raw r = v[j];
+                if (b < full) v[j] = load(p + j * st);
+                f.one(value(r));
+            }
+            f.fold();
+        }
+        p += (uint64_t)CT_AHEAD * st;
+    }
+    if (rest) {
+#pragma unroll
+        for (int j = 0; j < CT_AHEAD; ++j)
+            if (j < rest) v[j] = load(p + j * st);
+#pragma unroll
+        for (int j = 0; j < CT_AHEAD; ++j)
+            if (j < rest) f.one(value(v[j]));
+        f.fold();
+    }
+}
+
+struct CtMoments {
+    double s = 0.0, sa = 0.0;
+    float mn = CT_INF, mx = -CT_INF, ps = 0.f, psa = 0.f;
+    __device__ __forceinline__ void one(float v)
+    {
+        ps += v;
+        psa += fabsf(v);
+        mn = fminf(mn, v);
+        mx = fmaxf(mx, v);
+    }
+    __device__ __forceinline__ void fold()
+    {
+        s += (double)ps;
+        sa += (double)psa;
+        ps = psa = 0.f;
+    }
+};
+struct CtMomentsGuarded {                          // a column with non-finite values (or an fp32 overflow)
+    double s = 0.0, sa = 0.0, bad = 0.0;
+    float mn = CT_INF, mx = -CT_INF;
+    __device__ __forceinline__ void one(float v)
+    {
+        if (qp_is_finite(v)) {
+            s += (double)v;
+            sa += (double)fabsf(v);
+            mn = fminf(mn, v);
+            mx = fmaxf(mx, v);
+        } else {
+            bad += 1.0;
+        }
+    }
+    __device__ __forceinline__ void fold() {}
+};
+
+// Deviations about the fp32 mean, summed in fp64 (as the per-tensor kernel), and the histogram.
+template <bool SUMS, bool HIST, bool GUARD>
+struct CtDeviations {
+    float m, mn, inv_w;
+    unsigned base, nb;                             // byte address of the channel's first bin, less what the float's bits bring
+    double sd = 0.0, sv = 0.0;
+    unsigned below = 0u;
+    __device__ __forceinline__ void one(float v)
+    {
+        if (GUARD && !qp_is_finite(v)) return;
+        if (SUMS) {
+            const float y = __fsub_rn(v, m);
+            const double d = (double)y;
+            sv = fma(d, d, sv);
+            sd += fabs(d);
+            below += __float_as_uint(y) >> 31;
+        }
+        if (HIST) {                                // bin = floor((x - min) * inv_w), each operation rounded; x = max may give nb
+            const float pos = __fmul_rn(__fsub_rn(v, mn), inv_w);
+            const unsigned b = QP_CK(__float_as_uint(__fadd_rd(pos, SS_MAGIC)) - SS_ONE, nb + 1) + SS_ONE;
+            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(b * 4u + base) : "memory");
+        }
+    }
+    __device__ __forceinline__ void fold() {}
+};
+
+template <int HH, bool GUARD>
+struct CtCounter {
+    const SsPlan<HH>& p;
+    const SsTable& tb;
+    __device__ __forceinline__ void one(float v)
+    {
+        if (!GUARD || qp_is_finite(v)) ss_count<HH>(p, tb, v);
+    }
+    __device__ __forceinline__ void fold() {}
+};
+
+// N quantities of every thread added up (OPS: 0 sum, 1 min, 2 max) over the row lanes of its channel: a fixed tree; the
+// result is in the threads of row lane 0.  red: N * CT_THREADS doubles.
+template <int... OPS>
+__device__ __forceinline__ void ct_reduce(double (&v)[sizeof...(OPS)], double* red, int rl, int nl, int w)
+{
+    constexpr int N = sizeof...(OPS);
+    constexpr int ops[N] = {OPS...};
+#pragma unroll
+    for (int j = 0; j < N; ++j) red[j * CT_THREADS + threadIdx.x] = v[j];
+    __syncthreads();
+    int off = 1;
+    while (off < nl) off <<= 1;
+    for (off >>= 1; off > 0; off >>= 1) {
+        if (rl < off && rl + off < nl) {
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                const double t = red[j * CT_THREADS + threadIdx.x + off * w];
+                v[j] = ops[j] == 0 ? v[j] + t : (ops[j] == 1 ? fmin(v[j], t) : fmax(v[j], t));
+                red[j * CT_THREADS + threadIdx.x] = v[j];
+            }
+        }
+        __syncthreads();
+    }
+}
+
+__device__ __forceinline__ void ct_team_sync(int team) { asm volatile("barrier.sync %0, 64;" ::"r"(team + 1) : "memory"); }
+
+// STATS: phases A and B (otherwise the statistics come with st_in and B only counts the histogram).  HH: code boundaries above
+// the centre, 2^bits / 2 - 1; -1: statistics only.
+template <typename T, bool STATS, int HH>
+__global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
+{
+    constexpr bool SEARCH = HH >= 0;
+    constexpr int H = SEARCH ? HH : 0;
+    constexpr int BITS = H == 0 ? 1 : H == 1 ? 2 : H == 3 ? 3 : 4;
+    extern __shared__ __align__(16) unsigned char raw[];
+    __shared__ double s_a[CT_MAX_W][5], s_b[CT_MAX_W][3];     // this block's parts, read by the whole cluster
+    __shared__ qp_stats_t s_st[CT_MAX_W];
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int w = a.w, lane = threadIdx.x & 31;
+    const uint32_t c0 = blockIdx.x / (unsigned)S * (uint32_t)w;
+    const int nch = (int)min((uint32_t)w, a.C - c0);
+    const int slot = threadIdx.x % w, rl = threadIdx.x / w, nl = CT_THREADS / w;
+    const uint64_t r0 = min((uint64_t)rank * a.rows_pb, a.rows), r1 = min(r0 + a.rows_pb, a.rows);
+    const bool active = rl < nl && slot < nch && r0 + rl < r1;
+    const int m = active ? (int)((r1 - r0 - rl + nl - 1) / nl) : 0;                // rows of this thread
+    const uint32_t st = (uint32_t)nl * a.C;
+    const T* px = static_cast<const T*>(a.x) + (active ? (r0 + rl) * a.C + c0 + slot : 0);
+    const double inf = __longlong_as_double(0x7FF0000000000000ll);
+    double* red = reinterpret_cast<double*>(raw);
+    unsigned* bins = reinterpret_cast<unsigned*>(raw + CT_TABLE_BYTES);            // [w][nb + 1]
+
+    if constexpr (SEARCH)
+        for (int i = threadIdx.x; i < w * (a.nb + 1); i += CT_THREADS) bins[i] = 0u;
+
+    // ---- phase A
+    if constexpr (STATS) {
+        double v5[5] = {0.0, 0.0, inf, -inf, 0.0};
+        {
+            CtMoments acc;
+            ct_column<T>(px, st, m, acc);
+            if (acc.sa < inf) {
+                v5[0] = acc.s; v5[1] = acc.sa; v5[2] = (double)acc.mn; v5[3] = (double)acc.mx;
+            } else {                                          // rare: the column again, element by element
+                CtMomentsGuarded g;
+                ct_column<T>(px, st, m, g);
+                v5[0] = g.s; v5[1] = g.sa; v5[2] = (double)g.mn; v5[3] = (double)g.mx; v5[4] = g.bad;
+            }
+        }
+        ct_reduce<0, 0, 1, 2, 0>(v5, red, rl, nl, w);
+        if (rl == 0)
+#pragma unroll
+            for (int j = 0; j < 5; ++j) s_a[slot][j] = v5[j];
+        cluster.sync();
+        if ((int)threadIdx.x < nch) {                         // every block the same sums, in rank order
+            double t[5] = {0.0, 0.0, inf, -inf, 0.0};
+            for (int r = 0; r < S; ++r) {
+                const double* q = cluster.map_shared_rank(&s_a[threadIdx.x][0], r);
+                t[0] += q[0];
+                t[1] += q[1];
+                t[2] = fmin(t[2], q[2]);
+                t[3] = fmax(t[3], q[3]);
+                t[4] += q[4];
+            }
+            const unsigned long long bad = (unsigned long long)t[4], nf = a.rows - bad;
+            qp_stats_t& o = s_st[threadIdx.x];
+            o.n = a.rows;
+            o.nonfinite = bad;
+            o.mean = nf ? t[0] / (double)nf : 0.0;
+            o.mean_abs = nf ? t[1] / (double)nf : 0.0;
+            o.min = nf ? t[2] : 0.0;
+            o.max = nf ? t[3] : 0.0;
+            o.mad = o.var = 0.0;
+            o.hist_peak = 0;
+            o.hist_bins = 0;
+            o.reserved = 0;
+        }
+    } else {
+        if ((int)threadIdx.x < nch) s_st[threadIdx.x] = a.st_in[c0 + threadIdx.x];
+    }
+    __syncthreads();
+    bool odd = false;                                         // a channel with non-finite values: uniform over the cluster
+    for (int i = 0; i < nch; ++i) odd |= s_st[i].nonfinite != 0;
+
+    // ---- phase B
+    {
+        const qp_stats_t& my = s_st[slot < nch ? slot : 0];
+        double v3[3];
+        auto pass = [&](auto guard_tag) {
+            CtDeviations<STATS, SEARCH, decltype(guard_tag)::value> d;
+            d.m = (float)my.mean;
+            d.mn = (float)my.min;
+            d.inv_w = SEARCH && my.max > my.min ? (float)((double)a.nb / (my.max - my.min)) : 0.f;
+            d.nb = (unsigned)a.nb;
+            d.base = (unsigned)__cvta_generic_to_shared(bins + slot * (a.nb + 1)) - SS_ONE * 4u;
+            ct_column<T>(px, st, m, d);
+            v3[0] = d.sd; v3[1] = d.sv; v3[2] = (double)d.below;
+        };
+        if (odd) pass(std::true_type{}); else pass(std::false_type{});
+        if constexpr (STATS) {
+            ct_reduce<0, 0, 0>(v3, red, rl, nl, w);
+            if (rl == 0)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) s_b[slot][j] = v3[j];
+        }
+        cluster.sync();                                       // (orders the histogram counters of the cluster, too)
+        if (STATS && (int)threadIdx.x < nch) {
+            double t[3] = {0.0, 0.0, 0.0};
+            for (int r = 0; r < S; ++r) {
+                const double* q = cluster.map_shared_rank(&s_b[threadIdx.x][0], r);
+#pragma unroll
+                for (int j = 0; j < 3; ++j) t[j] += q[j];
+            }
+            qp_stats_t& o = s_st[threadIdx.x];
+            const double nf = (double)(o.n - o.nonfinite), dm = o.mean - (double)(float)o.mean;
+            o.mad = nf > 0.0 ? fmax(0.0, t[0] - dm * (nf - 2.0 * t[2])) / nf : 0.0;
+            o.var = nf > 0.0 ? fmax(0.0, t[1] / nf - dm * dm) : 0.0;
+            if (rank == 0) {
+                if (a.st_out) a.st_out[c0 + threadIdx.x] = o;
+                if (o.nonfinite) atomicOr(a.status, QP_DEV_NONFINITE);
+            }
+        }
+    }
+
+    // ---- phase C
+    if constexpr (SEARCH) {
+        __shared__ unsigned s_top[CT_MAX_W];
+        __shared__ SsPlan<H> s_plan[CT_MAX_W];
+        __shared__ qp_ds_setup s_setup[CT_MAX_W];
+        // (in the histogram's room, which is free by then)
+        double (*s_v)[CT_MAX_CAND] = reinterpret_cast<double (*)[CT_MAX_CAND]>(raw + CT_TABLE_BYTES);
+        int (*s_edge)[SS_GRID + 1] = reinterpret_cast<int (*)[SS_GRID + 1]>(raw + CT_TABLE_BYTES + sizeof(double) * (CT_WARPS / 2) * CT_MAX_CAND);
+        static_assert((CT_WARPS / 2) * (CT_MAX_CAND * sizeof(double) + (SS_GRID + 1) * sizeof(int)) <= CT_DYN_BYTES - CT_TABLE_BYTES, "room");
+        __shared__ unsigned s_n[CT_WARPS / 2][2];
+        const int ncand = a.steps + 1, ni = SS_GRID + 1 + H * ncand;
+        if (threadIdx.x < CT_MAX_W) s_top[threadIdx.x] = 0u;
+        for (int i = threadIdx.x; i < w * ni; i += CT_THREADS)                     // w * 2 ni words of counts and of sums
+            reinterpret_cast<uint2*>(raw)[i] = reinterpret_cast<uint2*>(raw + SS_SUMS_AT)[i] = make_uint2(0u, 0u);
+        __syncthreads();
+        for (int i = threadIdx.x; i < nch * a.nb; i += CT_THREADS) {               // peak of the histogram
+            const int sl = i / a.nb, b = i - sl * a.nb;
+            unsigned c = 0u;
+            for (int r = 0; r < S; ++r) {
+                const unsigned* q = cluster.map_shared_rank(bins, r) + sl * (a.nb + 1) + b;
+                c += q[0];
+                if (b == a.nb - 1) c += q[1];
+            }
+            atomicMax(&s_top[sl], c);
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < nch * 8) {                     // eight threads per channel: the common part, and a boundary each
+            const int sl = threadIdx.x >> 3, part = (threadIdx.x & 7) - 1;
+            qp_ds_setup su;
+            qp_ds_make_setup(&s_st[sl], s_st[sl].max > s_st[sl].min ? s_top[sl] : 0u, a.nb, a.bmode, a.F, su);
+            su.g_lo = su.g_hi = su.inv_gw = su.inv_u = su.gw = su.pad2 = 0.f;
+            su.u = 0.0;
+            if (part < 0) s_setup[sl] = su;
+            const double k = su.F * ((a.bmode & QP_B_MIDRISE) ? 1.0 - 1.0 / (double)(1 << BITS) : 1.0);
+            ss_make_plan<H>(s_plan[sl], part, s_st[sl].mean, k * su.b_e, k * (su.degenerate ? su.b_e : su.b_r),
+                            su.degenerate ? 1 : ncand, BITS, a.ub);
+        }
+        __syncthreads();
+        {
+            const SsPlan<H> p = s_plan[slot < nch ? slot : 0];
+            SsTable tb;
+            tb.mul = 4u;
+            tb.base = (unsigned)__cvta_generic_to_shared(raw) + (unsigned)(slot * 2 * ni) * 4u - SS_ONE * 4u;
+            tb.half = (unsigned)ni * 4u;
+            tb.ni = (unsigned)ni;
+            tb.ub = (unsigned)a.ub;
+            tb.scale = (float)(SS_GRID << a.ub);
+            const int mine = p.hard ? 0 : m;                  // (a hard channel is scored candidate by candidate below)
+            if (odd) {
+                CtCounter<H, true> f = {p, tb};
+                ct_column<T>(px, st, mine, f);
+            } else {
+                CtCounter<H, false> f = {p, tb};
+                ct_column<T>(px, st, mine, f);
+            }
+        }
+        cluster.sync();
+
+        // ---- finish: channel slots rank, rank + S, ... of the strip are this block's; a team of two warps takes one, a side each
+        const int team = threadIdx.x >> 6, side = (threadIdx.x >> 5) & 1;
+        for (int sl = rank + team * S; sl < nch; sl += (CT_WARPS / 2) * S) {
+            const SsPlan<H>& p = s_plan[sl];
+            if (p.hard) continue;                             // uniform over the team
+            const uint32_t c = c0 + sl;
+            for (int g = threadIdx.x & 63; g <= SS_GRID; g += 64) s_edge[team][g] = ss_cell_start(p, g);
+            ct_team_sync(team);
+            unsigned* cnt = reinterpret_cast<unsigned*>(raw) + (2 * sl + side) * ni;
+            unsigned* sum = reinterpret_cast<unsigned*>(raw + SS_SUMS_AT) + (2 * sl + side) * ni;
+            // totals over the cluster, in place: count | high bits of the sum << 24 (rows <= 65535, at most 8 sums of 32 bits)
+            const int per = (ni + 31) / 32, i0 = min(lane * per, ni), i1 = min(i0 + per, ni);
+            int cell = 0;
+            {
+                int hi = SS_GRID;                             // grid cell of interval i0
+                while (cell < hi) { const int mid = (cell + hi + 1) >> 1; if (s_edge[team][mid] <= i0) cell = mid; else hi = mid - 1; }
+            }
+            const int cell0 = cell;
+            unsigned n_all = 0u;
+            unsigned long long s_all = 0ull;
+            for (int i = i0; i < i1; ++i) {
+                while (cell < SS_GRID && s_edge[team][cell + 1] <= i) ++cell;
+                unsigned n = 0u;
+                unsigned long long s = 0ull;
+                for (int r = 0; r < S; ++r) {
+                    n += *cluster.map_shared_rank(cnt + i, r);
+                    s += *cluster.map_shared_rank(sum + i, r);
+                }
+                cnt[i] = n | (unsigned)(s >> 32) << 24;
+                sum[i] = (unsigned)s;
+                n_all += n;
+                s_all += s + ((unsigned long long)n * (unsigned)cell << a.ub);
+            }
+            // exclusive prefix sums, in place: count in 17 bits | high bits of the sum << 17, low word of the sum
+            unsigned np = n_all;
+            unsigned long long sp = s_all;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned tn = __shfl_up_sync(0xFFFFFFFFu, np, o);
+                const unsigned long long ts = __shfl_up_sync(0xFFFFFFFFu, sp, o);
+                if (lane >= o) { np += tn; sp += ts; }
+            }
+            const unsigned n_side = __shfl_sync(0xFFFFFFFFu, np, 31);
+            np -= n_all;
+            sp -= s_all;
+            cell = cell0;
+            for (int i = i0; i < i1; ++i) {
+                while (cell < SS_GRID && s_edge[team][cell + 1] <= i) ++cell;
+                const unsigned n = cnt[i] & 0xFFFFFFu;
+                const unsigned long long s = (unsigned long long)(cnt[i] >> 24) << 32 | sum[i];
+                cnt[i] = np | (unsigned)(sp >> 32) << 17;
+                sum[i] = (unsigned)sp;
+                np += n;
+                sp += s + ((unsigned long long)n * (unsigned)cell << a.ub);
+            }
+            if (lane == 0) s_n[team][side] = n_side;
+            ct_team_sync(team);
+
+            const qp_stats_t& q = s_st[sl];
+            const qp_ds_setup su = s_setup[sl];
+            const double nf = (double)(q.n - q.nonfinite), dm = q.mean - (double)p.m;
+            const double s_abs = nf * q.mad + dm * ((double)s_n[team][0] - (double)s_n[team][1]);
+            const double s_side = 0.5 * (side ? s_abs - nf * dm : s_abs + nf * dm);    // sum |y| of this side
+            const bool flat = !(p.inv_e > 0.f);
+            double v[CT_MAX_CAND / 32];
+#pragma unroll
+            for (int j = 0; j < CT_MAX_CAND / 32; ++j) {
+                const int k = lane + 32 * j;
+                v[j] = 0.0;
+                if (k >= ncand) continue;
+                float4 cd;
+                int ok;
+                qp_ds_candidate(su, k, a.steps, BITS, a.bmode & QP_B_MIDRISE, cd, ok);
+                if (side) {
+                    a.cand[(size_t)c * a.ncp + k] = cd;
+                    a.valid[(size_t)c * a.ncp + k] = ok;
+                }
+                double N0 = 0.0, S0 = 0.0;
+                for (int i = 0; ok && i <= H; ++i) {          // code i of this side, outwards
+                    const int p1 = i == H || flat ? ni : QP_CK(ss_place(p, k, i + 1), ni);
+                    double N1 = (double)n_side, S1 = s_side;
+                    if (p1 < ni) {
+                        const unsigned w0 = cnt[p1];
+                        N1 = (double)(w0 & 0x1FFFFu);
+                        S1 = p.u * (double)((unsigned long long)(w0 >> 17) << 32 | sum[p1]);
+                    }
+                    double lv = ss_level(cd, side ? H - i : H + 1 + i, p.m);
+                    if (side) lv = -lv;                       // distance from the centre, as |y|
+                    v[j] += (N1 - N0) * lv * lv - 2.0 * lv * (S1 - S0);
+                    N0 = N1;
+                    S0 = S1;
+                }
+                if (!ok) v[j] = inf;
+                if (side) s_v[team][k] = v[j];
+            }
+            ct_team_sync(team);
+            if (side == 0) {                                  // both sides, then the first minimum
+                double bv = inf;
+                int bk = 1 << 30;
+#pragma unroll
+                for (int j = 0; j < CT_MAX_CAND / 32; ++j) {
+                    const int k = lane + 32 * j;
+                    if (k >= ncand) continue;
+                    const double other = s_v[team][k];
+                    const double mse = other < inf ? (nf > 0.0 ? (nf * (q.var + dm * dm) + (v[j] + other)) / nf : 0.0) : inf;
+                    a.curve[(size_t)c * a.ncp + k] = mse;
+                    s_v[team][k] = mse;
+                    if (mse < bv) { bv = mse; bk = k; }
+                }
+                for (int o = 16; o > 0; o >>= 1) {
+                    const double ov = __shfl_down_sync(0xFFFFFFFFu, bv, o);
+                    const int ok = __shfl_down_sync(0xFFFFFFFFu, bk, o);
+                    if (ov < bv || (ov == bv && ok < bk)) { bv = ov; bk = ok; }
+                }
+                if (lane == 0) {
+                    const int best = bk < ncand ? bk : 0;     // (every error infinite or NaN: keep b_E)
+                    float4 cd;
+                    int ok;
+                    qp_ds_candidate(su, best, a.steps, BITS, a.bmode & QP_B_MIDRISE, cd, ok);
+                    qp_ds_write_result(best, s_v[team], su, a.steps, a.nb, BITS, cd, a.ds_out ? a.ds_out + c : nullptr,
+                                       a.qp_out + c, a.status);
+                }
+            }
+            ct_team_sync(team);                               // s_v, s_edge and s_n are free again
+        }
+
+        // ---- hard channels (clip ends coarse against the step): every candidate scored on every element
+        bool any_hard = false;
+        for (int i = 0; i < nch; ++i) any_hard |= s_plan[i].hard != 0;
+        cluster.sync();                                       // nobody reads this block's tables any more
+        if (!any_hard) return;                                // uniform over the cluster
+        constexpr int K = QP_EVAL_K;
+        const int groups = (ncand + K - 1) / K, lanes = CT_THREADS / groups;
+        const int g = threadIdx.x % groups, sub = threadIdx.x / groups;
+        for (int sl = 0; sl < nch; ++sl) {
+            if (!s_plan[sl].hard) continue;
+            const uint32_t c = c0 + sl;
+            const qp_ds_setup su = s_setup[sl];
+            float4 q[K];
+            int ok[K];
+            double acc[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                qp_ds_candidate(su, min(g * K + k, ncand - 1), a.steps, BITS, a.bmode & QP_B_MIDRISE, q[k], ok[k]);
+                acc[k] = 0.0;
+            }
+            if (sub < lanes)
+                for (uint64_t r = r0 + sub; r < r1; r += lanes) {
+                    const float v = qp_load_one(static_cast<const T*>(a.x) + r * a.C + c);
+                    if (!qp_is_finite(v)) continue;
+#pragma unroll
+                    for (int k = 0; k < K; ++k) {
+                        const float pos = qp_grid_pos(v, q[k].x, q[k].y, q[k].w);
+                        const float lev = __fsub_rn(__fadd_rn(pos, QP_MAGIC), QP_MAGIC);
+                        const float d = __fsub_rn(fmaf(lev, q[k].z, q[k].x), v);
+                        acc[k] += (double)(d * d);
+                    }
+                }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < K; ++k) red[threadIdx.x * K + k] = acc[k];
+            __syncthreads();
+            for (int k = threadIdx.x; k < ncand; k += CT_THREADS) {
+                double t = 0.0;
+                for (int l = 0; l < lanes; ++l) t += red[(l * groups + k / K) * K + k % K];
+                s_v[0][k] = t;
+            }
+            cluster.sync();
+            if (sl % S == rank) {
+                const double nf = (double)(s_st[sl].n - s_st[sl].nonfinite);
+                for (int k = threadIdx.x; k < ncand; k += CT_THREADS) {
+                    double t = 0.0;
+                    for (int r = 0; r < S; ++r) t += *cluster.map_shared_rank(&s_v[0][k], r);
+                    float4 cd;
+                    int valid;
+                    qp_ds_candidate(su, k, a.steps, BITS, a.bmode & QP_B_MIDRISE, cd, valid);
+                    a.cand[(size_t)c * a.ncp + k] = cd;
+                    a.valid[(size_t)c * a.ncp + k] = valid;
+                    const double mse = !valid ? inf : nf > 0.0 ? t / nf : 0.0;
+                    a.curve[(size_t)c * a.ncp + k] = mse;
+                    s_v[1][k] = mse;
+                }
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    int best = 0;
+                    for (int k = 1; k < ncand; ++k)
+                        if (s_v[1][k] < s_v[1][best]) best = k;
+                    float4 cd;
+                    int valid;
+                    qp_ds_candidate(su, best, a.steps, BITS, a.bmode & QP_B_MIDRISE, cd, valid);
+                    qp_ds_write_result(best, s_v[1], su, a.steps, a.nb, BITS, cd, a.ds_out ? a.ds_out + c : nullptr, a.qp_out + c,
+                                       a.status);
+                }
+            }
+            cluster.sync();
+        }
+    } else {
+        cluster.sync();                                       // nobody leaves while its parts may still be read
+    }
+}
+
+template <typename T>
+void* ct_kernel(bool stats, int bits)                         // bits 0: statistics only
+{
+    if (bits == 0) return (void*)ch_strip_kernel<T, true, -1>;
+    if (stats) return bits == 1 ? (void*)ch_strip_kernel<T, true, 0> : bits == 2 ? (void*)ch_strip_kernel<T, true, 1>
+                    : bits == 3 ? (void*)ch_strip_kernel<T, true, 3> : (void*)ch_strip_kernel<T, true, 7>;
+    return bits == 1 ? (void*)ch_strip_kernel<T, false, 0> : bits == 2 ? (void*)ch_strip_kernel<T, false, 1>
+         : bits == 3 ? (void*)ch_strip_kernel<T, false, 3> : (void*)ch_strip_kernel<T, false, 7>;
+}
+
+cudaLaunchConfig_t ct_config(cudaLaunchAttribute* at, unsigned blocks, int S, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(CT_THREADS);
+    cfg.dynamicSmemBytes = CT_DYN_BYTES;
+    cfg.stream = s;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)S;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// Once per context: whether the device holds the kernels, and how many clusters of each size at a time.
+bool ct_usable(qp_ctx* ctx)
+{
+    if (!ctx->ct_checked) {
+        ctx->ct_checked = 1;
+        int optin = 0;
+        bool ok = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device) == cudaSuccess;
+        for (int bits = 0; ok && bits <= 4; ++bits)
+            for (int v = 0; ok && v < (bits ? 4 : 2); ++v) {
+                void* k = (v & 1) ? ct_kernel<unsigned short>(v < 2, bits) : ct_kernel<float>(v < 2, bits);
+                cudaFuncAttributes fa;
+                ok = cudaFuncGetAttributes(&fa, k) == cudaSuccess && (size_t)optin >= fa.sharedSizeBytes + CT_DYN_BYTES &&
+                     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CT_DYN_BYTES) == cudaSuccess;
+            }
+        for (int S = 1; ok && S <= CT_MAX_S; ++S) {
+            cudaLaunchAttribute at;
+            const cudaLaunchConfig_t cfg = ct_config(&at, (unsigned)(S * ctx->sm_count), S, nullptr);
+            if (cudaOccupancyMaxActiveClusters(&ctx->ct_clusters[S], ct_kernel<float>(true, 4), &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                ctx->ct_clusters[S] = 0;
+            }
+        }
+        ok = ok && ctx->ct_clusters[1] > 0;
+        if (!ok) cudaGetLastError();
+        ctx->ct_ok = ok ? 1 : 0;
+    }
+    return ctx->ct_ok != 0;
+}
+
+// Strip width w and cluster size S: the fewest row-elements on the busiest SM, counting 2 more elements per row of a strip
+// (its cache lines are looked up one by one) and 6000 per wave (prologue, plan and finish, ~20 us).  A block's part stays
+// below 8192 rows where clusters allow it, so that offsets keep 19 bits.
+void ct_choose(const qp_ctx* ctx, uint64_t rows, uint32_t C, int max_w, int& w, int& S)
+{
+    double best = 1e300;
+    w = S = 1;
+    for (int s = 1; s <= CT_MAX_S; ++s) {
+        if (ctx->ct_clusters[s] < 1 || (s > 1 && (uint64_t)s > rows)) continue;
+        for (int v = 1; v <= max_w && (uint32_t)v <= C; ++v) {
+            const uint64_t strips = (C + v - 1) / v, waves = (strips + ctx->ct_clusters[s] - 1) / ctx->ct_clusters[s];
+            const uint64_t rows_pb = (rows + s - 1) / s;
+            double cost = (double)waves * ((double)rows_pb * (v + 2) + 6000.0);
+            if (rows_pb > 8191) cost *= 4.0;
+            if (cost < best) { best = cost; w = v; S = s; }
+        }
+    }
+}
+
+}  // namespace
+
+// Statistics per channel (bits = 0), the search on the caller's statistics (st_in), or both.  Rows up to 65535: the packed
+// prefix sums hold 17 bits of count.
+bool qp_channel_strips_apply(qp_ctx* ctx, uint64_t rows, uint32_t C, int bits)
+{
+    return rows >= 1 && rows <= 65535 && bits <= 4 && (uint64_t)C * rows < (1ull << 40) && ct_usable(ctx);
+}
+
+int32_t qp_launch_channel_strips(qp_ctx* ctx, const void* d_x, int dtype, uint64_t rows, uint32_t C, const qp_stats_t* st_in,
+                                 qp_stats_t* st_out, int bits, int bmode, int steps, int ncp, int nb, double F, float4* cand,
+                                 int* valid, double* curve, qp_ds_result_t* d_out, qp_qparams_t* d_qp_out, cudaStream_t s)
+{
+    // (statistics always with the strips of the default search, so that they come out the same with and without it)
+    const int hh = bits ? (1 << bits) / 2 - 1 : 0;
+    const int ni = SS_GRID + 1 + hh * (steps + 1);
+    int max_w = CT_MAX_W;
+    while (max_w > 1 && (size_t)max_w * 2 * ni * sizeof(unsigned) > (size_t)SS_SUMS_AT) --max_w;
+    int w, S;
+    ct_choose(ctx, rows, C, max_w, w, S);
+    CtArgs a;
+    a.x = d_x;
+    a.rows = rows;
+    a.C = C;
+    a.w = w;
+    a.rows_pb = (rows + S - 1) / S;
+    a.nb = nb;
+    a.steps = steps;
+    a.bmode = bmode;
+    a.ncp = ncp;
+    // offsets are at most 2^ub and a block's sums of them stay below 2^32; 22 bits keep the grid's integers below 2^28
+    a.ub = 22;
+    while (a.ub > 0 && (a.rows_pb << a.ub) >= (1ull << 32)) --a.ub;
+    a.F = F;
+    a.st_in = st_in;
+    a.st_out = st_out;
+    a.cand = cand;
+    a.valid = valid;
+    a.curve = curve;
+    a.ds_out = d_out;
+    a.qp_out = d_qp_out;
+    a.status = ctx->d_status;
+    void* k = dtype == QP_F32 ? ct_kernel<float>(st_in == nullptr, bits) : ct_kernel<unsigned short>(st_in == nullptr, bits);
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = ct_config(&at, (unsigned)((C + w - 1) / w * S), S, s);
+    void* params[] = {&a};
+    if (cudaLaunchKernelExC(&cfg, k, params) != cudaSuccess) return qp_check_launch(ctx, "channel strips");
+    ctx->launches += 1;
+    return qp_check_launch(ctx, "channel strips");
+}

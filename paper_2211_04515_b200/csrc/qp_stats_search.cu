@@ -11,23 +11,10 @@
 //   exit      block 0 turns the interval sums into the error of every candidate, picks the first minimum and writes
 //             the quantizer; in the sender the other blocks wait for it and all pack
 //
-// Phase C needs no table of thresholds.  The candidates' clip half-widths are a_k = a_0 + k d, so the
-// thresholds of one code boundary i above the centre are the equally spaced points c_i a_k, and the number
-// of them at or below |x - mean| is a clamped affine function of it: floor(K sat(A_i |y| + B_i)), two
-// instructions.  The sum over the boundaries of one side, plus the cell of a uniform grid of 64 cells,
-// numbers the intervals of the merged partition of that side.  Where a threshold really lies differs from
-// that formula by the rounding of the clip ends, s ~ 1e-7 of the clip: an element between the two is exchanged between
-// two codes whose reconstruction errors differ by less than 2 s, so a candidate's error moves by 12 (s / step)^2
-// relative (below 1e-8).  Where the clip ends are coarse against the step (|mean| beyond 250 steps), the "hard" form
-// below takes the exact thresholds instead.
-//
-// Per element: 1 is added to the interval's count and d to its sum by two 32-bit shared-memory atomics, d = the
-// offset from the grid cell's left edge.  The grid spans a power of two E above the widest clip, a cell is E / 2^6 and
-// d counts units of E / 2^25, so d is exact for |y| >= E / 4 and rounded to half a unit below (which counts 2 level
-// times in an element's squared error; the roundings of different elements are independent).  The tables hold a
-// replica per lane (per two lanes at 4 bits), so a warp's atomics meet neither the same counter nor the same bank.
-// They are emptied into 64-bit sums before they can wrap.  Integer sums: the
-// result does not depend on the order.
+// Phase C needs no table of thresholds (qp_affine.cuh).  Its tables hold a replica per lane (per two lanes at 4 bits), so a
+// warp's atomics meet neither the same counter nor the same bank.  They are emptied into 64-bit sums before they can
+// wrap.  Integer sums: the result does not depend on the order.  Tensors whose clip ends are coarse against the quantization
+// step take the "hard" form below, with the exact thresholds.
 //
 // What bounds it, on 129 MB (fp32, 2 bits): phase A the read from DRAM (24 us); B and C the read, most of which L2
 // still holds, together with 9 and 12 instructions and one and two shared atomics per element (18 and 21 us); the packing
@@ -36,6 +23,7 @@
 // the statistics, five for the search and one for the packing took 171 and 107.
 #include <type_traits>
 
+#include "qp_affine.cuh"
 #include "qp_gridbar.cuh"
 #include "qp_packtile.cuh"
 
@@ -46,13 +34,9 @@ namespace {
 constexpr int SS_THREADS = 512;                   // 128 registers a thread; 768 and 1024 threads spill and were slower
 constexpr int SS_WARPS = SS_THREADS / 32;
 constexpr int SS_TILE = 1024;                     // phases A and B: 32 elements per lane
-constexpr int SS_GRID = 64;                       // uniform cells per side
 constexpr unsigned SS_UNIT_BITS = 19;             // offsets are counted in cell / 2^19
-constexpr unsigned SS_ONE = 0x4B000000u;          // bits of 2^23: the offset sits in the low mantissa bits
-constexpr float SS_MAGIC = 8388608.0f;
 constexpr int SS_MAX_HIST = 4096;
-constexpr size_t SS_TABLE_BYTES = 200 * 1024;     // dynamic shared memory: interval tables, the exit's arrays
-constexpr int SS_SUMS_AT = (int)(SS_TABLE_BYTES / 2);   // the sums' half of the interval tables
+constexpr size_t SS_TABLE_BYTES = 2 * SS_SUMS_AT; // dynamic shared memory: interval tables (counts, then sums), the exit's arrays
 constexpr size_t SS_HIST_BYTES = 16512;           // and the histogram behind them (room for 4096 bins and one more)
 constexpr size_t SS_DYN_BYTES = SS_TABLE_BYTES + SS_HIST_BYTES;
 constexpr int SS_MERGE = 5;                       // block partials per lane that are in flight in a merge
@@ -280,72 +264,6 @@ struct SsDeviationsOf {                                       // the stream's vi
     __device__ __forceinline__ void end() { d.end(); }
 };
 
-// ---- the candidates' partition
-template <int HH>
-struct SsPlan {
-    float m;                                                  // fp32 mean; y = x - m
-    float inv_e, cell;                                        // 1 / E; width of a grid cell E / 64: powers of two
-    float kf;                                                 // number of candidates
-    float span[HH ? HH : 1];                                  // 1 / A
-    float A[HH ? HH : 1], B[HH ? HH : 1];                     // boundary i: thresholds passed / K = sat(A_i |y| + B_i)
-    double u, w;
-    int ncand, down, hard;                                    // down: the half-widths fall with k
-};
-
-// Threads 0..31 (one warp).  mean, a0, a1: centre and half-widths of the first and the last valid candidate.
-template <int HH>
-__device__ inline void ss_make_plan(SsPlan<HH>& p, double mean, double a0, double a1, int ncand, int bits)
-{
-    const double a_min = fmin(a0, a1), R = fmax(a0, a1), L1 = (double)((1 << bits) - 1);
-    const bool any = R > 1e-30 && R < 1e30;
-    const int i = threadIdx.x - 1;                            // thread 0: the common part; thread 1 + i: boundary i
-    if (i < 0) {
-        int e = 0;
-        if (any) frexp(R, &e);                                // R < 2^e
-        p.m = (float)mean;
-        p.ncand = ncand;
-        p.kf = (float)ncand;
-        p.down = a1 < a0;
-        p.inv_e = any ? (float)ldexp(1.0, -e) : 0.f;
-        p.w = any ? ldexp(1.0, e - 6) : 0.0;
-        p.cell = (float)p.w;
-        p.u = any ? ldexp(1.0, e - 6 - (int)SS_UNIT_BITS) : 1.0;
-        // clip ends that are coarse against the smallest step (an ulp of the mean beyond 2^-15 of it, where a candidate's
-        // error would move by 1e-8), or clips beyond what the formula's fp32 constants hold: the exact thresholds
-        p.hard = HH > 0 && R > 0.0 && (!any || fabs(mean) * 1.1920928955078125e-7 > 3.0517578125e-5 * (2.0 * a_min / L1));
-    } else if (i < HH) {
-        const double c = 2.0 * (i + 1) / L1, t0 = c * a_min;
-        const double gap = ncand > 1 ? c * (R - a_min) / (double)(ncand - 1) : 0.0;
-        // thresholds t0 + q gap, q = 0 .. K - 1.  (Candidates closer together than 1e-6 of the clip are spread
-        // that far: it moves a threshold by less than its element's share of the error can show.)
-        const double span = fmax((double)ncand * gap, 1e-6 * c * R);
-        p.A[i] = any ? (float)(1.0 / span) : 0.f;
-        p.B[i] = any ? (float)(1.0 / (double)ncand - t0 / span) : 0.f;
-        p.span[i] = (float)span;
-    }
-}
-
-// Phase C.  |y| is clamped to E by the saturating product t = |y| / E, exact because E is a power of two; d = t as an integer in
-// units of 2^-25 (the conversion pipe is idle otherwise), less the grid cell's.  What lies beyond E counts in the last interval
-// of its side, whose sum is not used: the sum over a whole side is known from the statistics.
-// base of the table: byte address of this lane's replica of interval 0 of the upper side; the lower side
-// follows `half` bytes later; the sums are SS_SUMS_AT bytes behind the counts.
-struct SsTable { unsigned mul, base, half, ni; };
-template <int HH>
-__device__ __forceinline__ void ss_count(const SsPlan<HH>& p, const SsTable& tb, float x)
-{
-    const float y = __fsub_rn(x, p.m), a = fabsf(y);
-    const float t = __saturatef(__fmul_rn(a, p.inv_e));
-    const float g = __fmaf_rd(t, (float)SS_GRID, SS_MAGIC);   // grid cell, then interval number, in the low bits
-    float r = g;
-#pragma unroll
-    for (int i = 0; i < HH; ++i) r = __fmaf_rd(__saturatef(fmaf(a, p.A[i], p.B[i])), p.kf, r);
-    const unsigned d = __float2uint_rn(__fmul_rn(t, (float)(SS_GRID << SS_UNIT_BITS))) - (__float_as_uint(g) << SS_UNIT_BITS);
-    unsigned addr = (QP_CK(__float_as_uint(r) - SS_ONE, tb.ni) + SS_ONE) * tb.mul + tb.base;
-    addr += (__float_as_uint(y) >> 31) * tb.half;
-    asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory");
-    asm volatile("red.shared.add.u32 [%0+%2], %1;" ::"r"(addr), "r"(d), "n"(SS_SUMS_AT) : "memory");
-}
 template <int HH, bool GUARD>
 struct SsCounter {
     const SsPlan<HH>& p;
@@ -472,11 +390,6 @@ __device__ inline void ss_pick(const SsArgs& a, int ncand, const double* s_curve
     }
 }
 
-__device__ __forceinline__ double ss_level(const float4& q, int j, float m)   // reconstruction of code j, relative to m
-{
-    return (double)fmaf((float)j, q.z, q.x) - (double)m;
-}
-
 // Block 0, after its arrival: where the boundaries of every candidate lie among the intervals (in shared memory), while
 // the other blocks are still on their way.  s_cell[i]: grid cell of interval i; pos[k][i]: first interval of
 // code i of a side, i = 0..HH; pos[k][HH + 1] = ni.
@@ -484,29 +397,11 @@ template <int HH>
 __device__ inline void ss_places(const SsPlan<HH>& p, int ncand, int ni, int* s_edge, unsigned char* s_cell, int* pos)
 {
     constexpr int C = HH + 1;
-    auto passed = [&](int i, float x) { return (int)(__float_as_uint(__fmaf_rd(__saturatef(fmaf(x, p.A[i], p.B[i])), p.kf, SS_MAGIC)) - SS_ONE); };
-    for (int g = threadIdx.x; g <= SS_GRID; g += SS_THREADS) {
-        int e = g;
-#pragma unroll
-        for (int i = 0; i < HH; ++i) e += passed(i, (float)g * p.cell);
-        s_edge[g] = g ? e : 0;
-    }
+    for (int g = threadIdx.x; g <= SS_GRID; g += SS_THREADS) s_edge[g] = ss_cell_start(p, g);
     const bool flat = !(p.inv_e > 0.f);                       // no width at all: everything has the first code of its side
-    const float inv_k = 1.0f / p.kf;
     for (int w = threadIdx.x; w < ncand * (C + 1); w += SS_THREADS) {
         const int k = w / (C + 1), b = w - k * (C + 1);       // boundary b = 1..HH of candidate k
-        int r = b == 0 ? 0 : ni;
-        if (b >= 1 && b <= HH && !flat) {
-            const int q = p.down ? p.ncand - 1 - k : k;
-            float T = 0.f;
-#pragma unroll
-            for (int o = 0; o < HH; ++o)
-                if (o == b - 1) T = ((float)(q + 1) * inv_k - p.B[o]) * p.span[o];
-            r = q + 1 + (int)(__float_as_uint(__fmaf_rd(__saturatef(__fmul_rn(T, p.inv_e)), (float)SS_GRID, SS_MAGIC)) - SS_ONE);
-#pragma unroll
-            for (int o = 0; o < HH; ++o) r += o == b - 1 ? 0 : passed(o, T);
-        }
-        pos[w] = QP_CK(r, ni + 1);
+        pos[w] = QP_CK(b == 0 ? 0 : (b > HH || flat) ? ni : ss_place(p, k, b), ni + 1);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < ni; i += SS_THREADS) {      // cell of an interval: the last one that starts at or before it
@@ -909,7 +804,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArg
             if (threadIdx.x < 32) {
                 if (lane == 0) s_setup = su;
                 const double k = su.F * ((a.bmode & QP_B_MIDRISE) ? 1.0 - 1.0 / (double)(1 << BITS) : 1.0);
-                ss_make_plan<H>(s_plan, s_st.mean, k * su.b_e, k * (su.degenerate ? su.b_e : su.b_r), su.degenerate ? 1 : ncand, BITS);
+                ss_make_plan<H>(s_plan, (int)threadIdx.x - 1, s_st.mean, k * su.b_e, k * (su.degenerate ? su.b_e : su.b_r), su.degenerate ? 1 : ncand, BITS, SS_UNIT_BITS);
             } else {
                 for (int k = threadIdx.x - 32; k < ncand; k += SS_THREADS - 32) {
                     float4 c;
@@ -932,6 +827,8 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArg
             tb.base = (unsigned)__cvta_generic_to_shared(raw) + 4u * (lane & ((1 << a.rep_shift) - 1)) - SS_ONE * tb.mul;
             tb.half = (unsigned)ni * tb.mul;
             tb.ni = (unsigned)ni;
+            tb.ub = SS_UNIT_BITS;
+            tb.scale = (float)(SS_GRID << SS_UNIT_BITS);
             ulonglong2* row = a.rows + (size_t)blockIdx.x * (2 * ni);
             const uint64_t per = (uint64_t)a.flush_tiles * step;      // tiles of all warps between two flushes
             const uint64_t ntiles = a.ntiles * (SS_TILE / CT);
