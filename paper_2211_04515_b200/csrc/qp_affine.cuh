@@ -88,34 +88,31 @@ __device__ __forceinline__ void ss_count(const SsPlan<HH>& p, const SsTable& tb,
     asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory");
     asm volatile("red.shared.add.u32 [%0+%2], %1;" ::"r"(addr), "r"(d), "n"(SS_SUMS_AT) : "memory");
 }
-// thresholds of boundary i (0-based) at or below x on its side
+// interval that x on a side belongs to, as ss_count numbers it
 template <int HH>
-__device__ __forceinline__ int ss_passed(const SsPlan<HH>& p, int i, float x)
+__device__ __forceinline__ int ss_interval(const SsPlan<HH>& p, float x)
 {
-    return (int)(__float_as_uint(__fmaf_rd(__saturatef(fmaf(x, p.A[i], p.B[i])), p.kf, SS_MAGIC)) - SS_ONE);
+    float r = __fmaf_rd(__saturatef(__fmul_rn(x, p.inv_e)), (float)SS_GRID, SS_MAGIC);
+#pragma unroll
+    for (int i = 0; i < HH; ++i) r = __fmaf_rd(__saturatef(fmaf(x, p.A[i], p.B[i])), p.kf, r);
+    return (int)(__float_as_uint(r) - SS_ONE);
 }
-// first interval of code b (1..HH) of candidate k on a side
+// first interval of code b (1..HH) of candidate k on a side: the interval of its threshold, in which the thresholds of
+// its own boundary, counted exactly, take the place of the formula's (which may be one off at the threshold itself)
 template <int HH>
 __device__ __forceinline__ int ss_place(const SsPlan<HH>& p, int k, int b)
 {
     const int q = p.down ? p.ncand - 1 - k : k;
-    float T = 0.f;
-#pragma unroll
-    for (int o = 0; o < HH; ++o)
-        if (o == b - 1) T = ((float)(q + 1) * (1.0f / p.kf) - p.B[o]) * p.span[o];
-    int r = q + 1 + (int)(__float_as_uint(__fmaf_rd(__saturatef(__fmul_rn(T, p.inv_e)), (float)SS_GRID, SS_MAGIC)) - SS_ONE);
-#pragma unroll
-    for (int o = 0; o < HH; ++o) r += o == b - 1 ? 0 : ss_passed(p, o, T);
-    return r;
+    const float A = p.A[b - 1], B = p.B[b - 1];
+    const float T = ((float)(q + 1) * (1.0f / p.kf) - B) * p.span[b - 1];
+    const int own = (int)(__float_as_uint(__fmaf_rd(__saturatef(fmaf(T, A, B)), p.kf, SS_MAGIC)) - SS_ONE);
+    return ss_interval(p, T) - own + q + 1;
 }
 // interval that grid cell g starts with
 template <int HH>
 __device__ __forceinline__ int ss_cell_start(const SsPlan<HH>& p, int g)
 {
-    int e = g;
-#pragma unroll
-    for (int i = 0; i < HH; ++i) e += ss_passed(p, i, (float)g * p.cell);
-    return g ? e : 0;
+    return g ? g + ss_interval(p, (float)g * p.cell) - (int)(__float_as_uint(__fmaf_rd(__saturatef(__fmul_rn((float)g * p.cell, p.inv_e)), (float)SS_GRID, SS_MAGIC)) - SS_ONE) : 0;
 }
 __device__ __forceinline__ double ss_level(const float4& q, int j, float m)   // reconstruction of code j, relative to m
 {

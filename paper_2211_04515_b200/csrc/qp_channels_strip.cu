@@ -27,11 +27,13 @@ QP_CK_UNIT
 
 namespace {
 
-constexpr int CT_THREADS = 512;
-constexpr int CT_WARPS = CT_THREADS / 32;
+constexpr int CT_THREADS = 1024;
+constexpr int CT_TEAMS = 8;                        // teams of the finish: a channel each
+constexpr int CT_TEAM = CT_THREADS / CT_TEAMS;     // threads of a team (two warps at least: a side each)
 constexpr int CT_MAX_W = 16;                       // channels of a strip
 constexpr int CT_MAX_S = 8;                        // blocks of a cluster
-constexpr int CT_AHEAD = 16;                       // loads in flight per thread
+constexpr int CT_AHEAD = 8;                        // loads in flight per thread: a batch
+constexpr int CT_PREFETCH = 4;                     // batches that the first pass is prefetched ahead of its loads
 constexpr float CT_INF = __builtin_huge_valf();
 constexpr int CT_MAX_CAND = QP_CH_MAX_STEPS + 1;
 constexpr size_t CT_TABLE_BYTES = 2 * SS_SUMS_AT;  // interval tables (counts, then sums) of the strip
@@ -55,14 +57,20 @@ struct CtArgs {
     unsigned* status;
 };
 
-// The m rows p, p + st, p + 2 st, ... of a column, CT_AHEAD loads ahead of their use: f.one(value) for each, f.fold() after
-// every CT_AHEAD of them and at the end.
-template <typename T, typename F>
-__device__ __forceinline__ void ct_column(const T* p, uint32_t st, int m, F& f)
+// A thread's rows of a column: at byte offsets at, at + st, ... from the block's rows (32 bits: one instruction per address).
+struct CtRows { const unsigned char* base; unsigned at, st; };
+
+// CT_AHEAD loads ahead of their use: f.one(value) for each row, f.fold() after every CT_AHEAD of them and at the end.
+// ahead(b) is called before batch b's loads are issued, b = 1, 2, ...
+struct CtNothing { __device__ __forceinline__ void operator()(int) const {} };
+template <typename T, typename F, typename A = CtNothing>
+__device__ __forceinline__ void ct_column(const CtRows& rows, int m, F& f, const A& ahead = A())
 {
     if (m <= 0) return;
     using Raw = typename std::conditional<sizeof(T) == 4, float, unsigned short>::type;
-    auto load = [](const T* q) { return __ldg(reinterpret_cast<const Raw*>(q)); };
+    unsigned at = rows.at;
+    const unsigned st = rows.st;
+    auto load = [&](int j) { return __ldg(reinterpret_cast<const Raw*>(rows.base + (at + (unsigned)j * st))); };
     auto value = [](Raw r) {
         if constexpr (sizeof(T) == 4) return (float)r;
         else return qp_bf16_to_f32(r);
@@ -71,23 +79,27 @@ __device__ __forceinline__ void ct_column(const T* p, uint32_t st, int m, F& f)
     const int full = m / CT_AHEAD, rest = m - full * CT_AHEAD;
     if (full) {
 #pragma unroll
-        for (int j = 0; j < CT_AHEAD; ++j) v[j] = load(p + j * st);
-        for (int b = 1; b <= full; ++b) {
-            if (b < full) p += (uint64_t)CT_AHEAD * st;
+        for (int j = 0; j < CT_AHEAD; ++j) v[j] = load(j);
+        for (int b = 1; b < full; ++b) {
+            at += CT_AHEAD * st;
+            ahead(b);
 #pragma unroll
             for (int j = 0; j < CT_AHEAD; ++j) {
                 const Raw r = v[j];
-                if (b < full) v[j] = load(p + j * st);
+                v[j] = load(j);
                 f.one(value(r));
             }
             f.fold();
         }
-        p += (uint64_t)CT_AHEAD * st;
+        at += CT_AHEAD * st;
+#pragma unroll
+        for (int j = 0; j < CT_AHEAD; ++j) f.one(value(v[j]));
+        f.fold();
     }
     if (rest) {
 #pragma unroll
         for (int j = 0; j < CT_AHEAD; ++j)
-            if (j < rest) v[j] = load(p + j * st);
+            if (j < rest) v[j] = load(j);
 #pragma unroll
         for (int j = 0; j < CT_AHEAD; ++j)
             if (j < rest) f.one(value(v[j]));
@@ -191,7 +203,7 @@ __device__ __forceinline__ void ct_reduce(double (&v)[sizeof...(OPS)], double* r
     }
 }
 
-__device__ __forceinline__ void ct_team_sync(int team) { asm volatile("barrier.sync %0, 64;" ::"r"(team + 1) : "memory"); }
+__device__ __forceinline__ void ct_team_sync(int team) { asm volatile("barrier.sync %0, %1;" ::"r"(team + 1), "n"(CT_TEAM) : "memory"); }
 
 // STATS: phases A and B (otherwise the statistics come with st_in and B only counts the histogram).  HH: code boundaries above
 // the centre, 2^bits / 2 - 1; -1: statistics only.
@@ -213,8 +225,9 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
     const uint64_t r0 = min((uint64_t)rank * a.rows_pb, a.rows), r1 = min(r0 + a.rows_pb, a.rows);
     const bool active = rl < nl && slot < nch && r0 + rl < r1;
     const int m = active ? (int)((r1 - r0 - rl + nl - 1) / nl) : 0;                // rows of this thread
-    const uint32_t st = (uint32_t)nl * a.C;
-    const T* px = static_cast<const T*>(a.x) + (active ? (r0 + rl) * a.C + c0 + slot : 0);
+    const CtRows mine = {static_cast<const unsigned char*>(a.x) + r0 * a.C * sizeof(T),
+                         active ? ((unsigned)rl * a.C + c0 + (unsigned)slot) * (unsigned)sizeof(T) : 0u,
+                         (unsigned)nl * a.C * (unsigned)sizeof(T)};
     const double inf = __longlong_as_double(0x7FF0000000000000ll);
     double* red = reinterpret_cast<double*>(raw);
     unsigned* bins = reinterpret_cast<unsigned*>(raw + CT_TABLE_BYTES);            // [w][nb + 1]
@@ -226,13 +239,30 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
     if constexpr (STATS) {
         double v5[5] = {0.0, 0.0, inf, -inf, 0.0};
         {
+            // The strips of a rank walk the same rows side by side.  Left to their own loads they ask DRAM for 4 w bytes at a
+            // time and wait for it (52 MB: 25 us); so each brings its share of the rows that all of them need four batches
+            // later into L2, in one contiguous piece.
+            const uint64_t strips = (a.C + w - 1) / w, row_bytes = (uint64_t)a.C * sizeof(T), batch_rows = (uint64_t)nl * CT_AHEAD;
+            const unsigned char* base = reinterpret_cast<const unsigned char*>(((uintptr_t)a.x + 15u) & ~(uintptr_t)15u);
+            const uint64_t skip = (uint64_t)(base - static_cast<const unsigned char*>(a.x));
+            auto prefetch = [&](uint64_t batch) {             // this strip's share of a batch of its rank's rows
+                const uint64_t b0 = min((r0 + batch * batch_rows), r1) * row_bytes, b1 = min((r0 + (batch + 1) * batch_rows), r1) * row_bytes;
+                const uint64_t share = ((b1 - b0) / strips + 16) & ~(uint64_t)15u, at = blockIdx.x / (unsigned)S * share;
+                const uint64_t f0 = (b0 + at) & ~(uint64_t)15u, f1 = min(b0 + at + share, b1) & ~(uint64_t)15u;
+                if (f1 > f0 && f1 + skip <= a.rows * row_bytes)
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(base + f0), "r"((unsigned)(f1 - f0)) : "memory");
+            };
+            if (threadIdx.x == 0)
+                for (uint64_t b = 0; b < CT_PREFETCH; ++b) prefetch(b);
             CtMoments acc;
-            ct_column<T>(px, st, m, acc);
+            ct_column<T>(mine, m, acc, [&](int b) {
+                if (threadIdx.x == 0) prefetch((uint64_t)b - 1 + CT_PREFETCH);
+            });
             if (acc.sa < inf) {
                 v5[0] = acc.s; v5[1] = acc.sa; v5[2] = (double)acc.mn; v5[3] = (double)acc.mx;
             } else {                                          // rare: the column again, element by element
                 CtMomentsGuarded g;
-                ct_column<T>(px, st, m, g);
+                ct_column<T>(mine, m, g);
                 v5[0] = g.s; v5[1] = g.sa; v5[2] = (double)g.mn; v5[3] = (double)g.mx; v5[4] = g.bad;
             }
         }
@@ -282,7 +312,7 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
             d.inv_w = SEARCH && my.max > my.min ? (float)((double)a.nb / (my.max - my.min)) : 0.f;
             d.nb = (unsigned)a.nb;
             d.base = (unsigned)__cvta_generic_to_shared(bins + slot * (a.nb + 1)) - SS_ONE * 4u;
-            ct_column<T>(px, st, m, d);
+            ct_column<T>(mine, m, d);
             v3[0] = d.sd; v3[1] = d.sv; v3[2] = (double)d.below;
         };
         if (odd) pass(std::true_type{}); else pass(std::false_type{});
@@ -318,9 +348,9 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
         __shared__ qp_ds_setup s_setup[CT_MAX_W];
         // (in the histogram's room, which is free by then)
         double (*s_v)[CT_MAX_CAND] = reinterpret_cast<double (*)[CT_MAX_CAND]>(raw + CT_TABLE_BYTES);
-        int (*s_edge)[SS_GRID + 1] = reinterpret_cast<int (*)[SS_GRID + 1]>(raw + CT_TABLE_BYTES + sizeof(double) * (CT_WARPS / 2) * CT_MAX_CAND);
-        static_assert((CT_WARPS / 2) * (CT_MAX_CAND * sizeof(double) + (SS_GRID + 1) * sizeof(int)) <= CT_DYN_BYTES - CT_TABLE_BYTES, "room");
-        __shared__ unsigned s_n[CT_WARPS / 2][2];
+        int (*s_edge)[SS_GRID + 1] = reinterpret_cast<int (*)[SS_GRID + 1]>(raw + CT_TABLE_BYTES + sizeof(double) * (CT_TEAMS) * CT_MAX_CAND);
+        static_assert((CT_TEAMS) * (CT_MAX_CAND * sizeof(double) + (SS_GRID + 1) * sizeof(int)) <= CT_DYN_BYTES - CT_TABLE_BYTES, "room");
+        __shared__ unsigned s_n[CT_TEAMS][2];
         const int ncand = a.steps + 1, ni = SS_GRID + 1 + H * ncand;
         if (threadIdx.x < CT_MAX_W) s_top[threadIdx.x] = 0u;
         for (int i = threadIdx.x; i < w * ni; i += CT_THREADS)                     // w * 2 ni words of counts and of sums
@@ -358,125 +388,142 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
             tb.ni = (unsigned)ni;
             tb.ub = (unsigned)a.ub;
             tb.scale = (float)(SS_GRID << a.ub);
-            const int mine = p.hard ? 0 : m;                  // (a hard channel is scored candidate by candidate below)
+            const int rows = p.hard ? 0 : m;                  // (a hard channel is scored candidate by candidate below)
             if (odd) {
                 CtCounter<H, true> f = {p, tb};
-                ct_column<T>(px, st, mine, f);
+                ct_column<T>(mine, rows, f);
             } else {
                 CtCounter<H, false> f = {p, tb};
-                ct_column<T>(px, st, mine, f);
+                ct_column<T>(mine, rows, f);
             }
         }
         cluster.sync();
 
-        // ---- finish: channel slots rank, rank + S, ... of the strip are this block's; a team of two warps takes one, a side each
-        const int team = threadIdx.x >> 6, side = (threadIdx.x >> 5) & 1;
-        for (int sl = rank + team * S; sl < nch; sl += (CT_WARPS / 2) * S) {
+        // ---- finish: channel slots rank, rank + S, ... of the strip are this block's.  Their totals over the cluster, in place:
+        // count | high bits of the sum << 24 (rows <= 65535, at most 8 sums of 32 bits); eight entries' loads in flight.
+        if (S > 1) {
+            const int own = (nch - rank + S - 1) / S, len = 2 * ni;
+            unsigned* cnt = reinterpret_cast<unsigned*>(raw);
+            unsigned* sum = reinterpret_cast<unsigned*>(raw + SS_SUMS_AT);
+            for (int e0 = threadIdx.x; e0 < own * len; e0 += 8 * CT_THREADS) {
+                unsigned n[8];
+                unsigned long long t[8];
+                int at[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int e = e0 + j * CT_THREADS, sl = e / len;
+                    at[j] = e < own * len ? (rank + sl * S) * len + (e - sl * len) : 0;
+                    n[j] = 0u;
+                    t[j] = 0ull;
+                }
+                for (int r = 0; r < S; ++r) {
+                    const unsigned* rc = cluster.map_shared_rank(cnt, r);
+                    const unsigned* rs = cluster.map_shared_rank(sum, r);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        n[j] += rc[at[j]];
+                        t[j] += rs[at[j]];
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (e0 + j * CT_THREADS < own * len) {
+                        cnt[at[j]] = n[j] | (unsigned)(t[j] >> 32) << 24;
+                        sum[at[j]] = (unsigned)t[j];
+                    }
+            }
+            __syncthreads();
+        }
+        // a team takes a channel: its first two warps a side each for the prefix sums, then all of it the candidates
+        const int team = threadIdx.x / CT_TEAM, tt = threadIdx.x % CT_TEAM, side = tt >> 5;
+        for (int sl = rank + team * S; sl < nch; sl += (CT_TEAMS) * S) {
             const SsPlan<H>& p = s_plan[sl];
             if (p.hard) continue;                             // uniform over the team
             const uint32_t c = c0 + sl;
-            for (int g = threadIdx.x & 63; g <= SS_GRID; g += 64) s_edge[team][g] = ss_cell_start(p, g);
+            for (int g = tt; g <= SS_GRID; g += CT_TEAM) s_edge[team][g] = ss_cell_start(p, g);
             ct_team_sync(team);
-            unsigned* cnt = reinterpret_cast<unsigned*>(raw) + (2 * sl + side) * ni;
-            unsigned* sum = reinterpret_cast<unsigned*>(raw + SS_SUMS_AT) + (2 * sl + side) * ni;
-            // totals over the cluster, in place: count | high bits of the sum << 24 (rows <= 65535, at most 8 sums of 32 bits)
-            const int per = (ni + 31) / 32, i0 = min(lane * per, ni), i1 = min(i0 + per, ni);
-            int cell = 0;
-            {
-                int hi = SS_GRID;                             // grid cell of interval i0
-                while (cell < hi) { const int mid = (cell + hi + 1) >> 1; if (s_edge[team][mid] <= i0) cell = mid; else hi = mid - 1; }
-            }
-            const int cell0 = cell;
-            unsigned n_all = 0u;
-            unsigned long long s_all = 0ull;
-            for (int i = i0; i < i1; ++i) {
-                while (cell < SS_GRID && s_edge[team][cell + 1] <= i) ++cell;
-                unsigned n = 0u;
-                unsigned long long s = 0ull;
-                for (int r = 0; r < S; ++r) {
-                    n += *cluster.map_shared_rank(cnt + i, r);
-                    s += *cluster.map_shared_rank(sum + i, r);
+            if (side < 2) {
+                unsigned* cnt = reinterpret_cast<unsigned*>(raw) + (2 * sl + side) * ni;
+                unsigned* sum = reinterpret_cast<unsigned*>(raw + SS_SUMS_AT) + (2 * sl + side) * ni;
+                const int per = (ni + 31) / 32, i0 = min(lane * per, ni), i1 = min(i0 + per, ni);
+                int cell = 0;
+                {
+                    int hi = SS_GRID;                             // grid cell of interval i0
+                    while (cell < hi) { const int mid = (cell + hi + 1) >> 1; if (s_edge[team][mid] <= i0) cell = mid; else hi = mid - 1; }
                 }
-                cnt[i] = n | (unsigned)(s >> 32) << 24;
-                sum[i] = (unsigned)s;
-                n_all += n;
-                s_all += s + ((unsigned long long)n * (unsigned)cell << a.ub);
+                const int cell0 = cell;
+                unsigned n_all = 0u;
+                unsigned long long s_all = 0ull;
+                for (int i = i0; i < i1; ++i) {
+                    while (cell < SS_GRID && s_edge[team][cell + 1] <= i) ++cell;
+                    const unsigned n = cnt[i] & 0xFFFFFFu;
+                    n_all += n;
+                    s_all += ((unsigned long long)(cnt[i] >> 24) << 32 | sum[i]) + ((unsigned long long)n * (unsigned)cell << a.ub);
+                }
+                // exclusive prefix sums, in place: count in 17 bits | high bits of the sum << 17, low word of the sum
+                unsigned np = n_all;
+                unsigned long long sp = s_all;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned tn = __shfl_up_sync(0xFFFFFFFFu, np, o);
+                    const unsigned long long ts = __shfl_up_sync(0xFFFFFFFFu, sp, o);
+                    if (lane >= o) { np += tn; sp += ts; }
+                }
+                const unsigned n_side = __shfl_sync(0xFFFFFFFFu, np, 31);
+                np -= n_all;
+                sp -= s_all;
+                cell = cell0;
+                for (int i = i0; i < i1; ++i) {
+                    while (cell < SS_GRID && s_edge[team][cell + 1] <= i) ++cell;
+                    const unsigned n = cnt[i] & 0xFFFFFFu;
+                    const unsigned long long s = (unsigned long long)(cnt[i] >> 24) << 32 | sum[i];
+                    cnt[i] = np | (unsigned)(sp >> 32) << 17;
+                    sum[i] = (unsigned)sp;
+                    np += n;
+                    sp += s + ((unsigned long long)n * (unsigned)cell << a.ub);
+                }
+                if (lane == 0) s_n[team][side] = n_side;
             }
-            // exclusive prefix sums, in place: count in 17 bits | high bits of the sum << 17, low word of the sum
-            unsigned np = n_all;
-            unsigned long long sp = s_all;
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned tn = __shfl_up_sync(0xFFFFFFFFu, np, o);
-                const unsigned long long ts = __shfl_up_sync(0xFFFFFFFFu, sp, o);
-                if (lane >= o) { np += tn; sp += ts; }
-            }
-            const unsigned n_side = __shfl_sync(0xFFFFFFFFu, np, 31);
-            np -= n_all;
-            sp -= s_all;
-            cell = cell0;
-            for (int i = i0; i < i1; ++i) {
-                while (cell < SS_GRID && s_edge[team][cell + 1] <= i) ++cell;
-                const unsigned n = cnt[i] & 0xFFFFFFu;
-                const unsigned long long s = (unsigned long long)(cnt[i] >> 24) << 32 | sum[i];
-                cnt[i] = np | (unsigned)(sp >> 32) << 17;
-                sum[i] = (unsigned)sp;
-                np += n;
-                sp += s + ((unsigned long long)n * (unsigned)cell << a.ub);
-            }
-            if (lane == 0) s_n[team][side] = n_side;
             ct_team_sync(team);
 
             const qp_stats_t& q = s_st[sl];
             const qp_ds_setup su = s_setup[sl];
             const double nf = (double)(q.n - q.nonfinite), dm = q.mean - (double)p.m;
             const double s_abs = nf * q.mad + dm * ((double)s_n[team][0] - (double)s_n[team][1]);
-            const double s_side = 0.5 * (side ? s_abs - nf * dm : s_abs + nf * dm);    // sum |y| of this side
+            const double s_up = 0.5 * (s_abs + nf * dm), s_down = 0.5 * (s_abs - nf * dm);     // sum |y| of each side
             const bool flat = !(p.inv_e > 0.f);
-            double v[CT_MAX_CAND / 32];
-#pragma unroll
-            for (int j = 0; j < CT_MAX_CAND / 32; ++j) {
-                const int k = lane + 32 * j;
-                v[j] = 0.0;
-                if (k >= ncand) continue;
+            const unsigned* c_up = reinterpret_cast<unsigned*>(raw) + 2 * sl * ni;
+            const unsigned* t_up = reinterpret_cast<unsigned*>(raw + SS_SUMS_AT) + 2 * sl * ni;
+            for (int k = tt; k < ncand; k += CT_TEAM) {
                 float4 cd;
                 int ok;
                 qp_ds_candidate(su, k, a.steps, BITS, a.bmode & QP_B_MIDRISE, cd, ok);
-                if (side) {
-                    a.cand[(size_t)c * a.ncp + k] = cd;
-                    a.valid[(size_t)c * a.ncp + k] = ok;
-                }
-                double N0 = 0.0, S0 = 0.0;
-                for (int i = 0; ok && i <= H; ++i) {          // code i of this side, outwards
+                a.cand[(size_t)c * a.ncp + k] = cd;
+                a.valid[(size_t)c * a.ncp + k] = ok;
+                double v = 0.0, n_up = 0.0, n_down = 0.0, x_up = 0.0, x_down = 0.0;
+                for (int i = 0; ok && i <= H; ++i) {          // code i of both sides, outwards
                     const int p1 = i == H || flat ? ni : QP_CK(ss_place(p, k, i + 1), ni);
-                    double N1 = (double)n_side, S1 = s_side;
+                    double n1 = (double)s_n[team][0], n2 = (double)s_n[team][1], x1 = s_up, x2 = s_down;
                     if (p1 < ni) {
-                        const unsigned w0 = cnt[p1];
-                        N1 = (double)(w0 & 0x1FFFFu);
-                        S1 = p.u * (double)((unsigned long long)(w0 >> 17) << 32 | sum[p1]);
+                        const unsigned w1 = c_up[p1], w2 = c_up[ni + p1];
+                        n1 = (double)(w1 & 0x1FFFFu);
+                        n2 = (double)(w2 & 0x1FFFFu);
+                        x1 = p.u * (double)((unsigned long long)(w1 >> 17) << 32 | t_up[p1]);
+                        x2 = p.u * (double)((unsigned long long)(w2 >> 17) << 32 | t_up[ni + p1]);
                     }
-                    double lv = ss_level(cd, side ? H - i : H + 1 + i, p.m);
-                    if (side) lv = -lv;                       // distance from the centre, as |y|
-                    v[j] += (N1 - N0) * lv * lv - 2.0 * lv * (S1 - S0);
-                    N0 = N1;
-                    S0 = S1;
+                    const double l1 = ss_level(cd, H + 1 + i, p.m), l2 = -ss_level(cd, H - i, p.m);   // distances from the centre
+                    v += ((n1 - n_up) * l1 * l1 - 2.0 * l1 * (x1 - x_up)) + ((n2 - n_down) * l2 * l2 - 2.0 * l2 * (x2 - x_down));
+                    n_up = n1; n_down = n2; x_up = x1; x_down = x2;
                 }
-                if (!ok) v[j] = inf;
-                if (side) s_v[team][k] = v[j];
+                const double mse = !ok ? inf : nf > 0.0 ? (nf * (q.var + dm * dm) + v) / nf : 0.0;
+                a.curve[(size_t)c * a.ncp + k] = mse;
+                s_v[team][k] = mse;
             }
             ct_team_sync(team);
-            if (side == 0) {                                  // both sides, then the first minimum
+            if (side == 0) {                                  // the first minimum
                 double bv = inf;
                 int bk = 1 << 30;
-#pragma unroll
-                for (int j = 0; j < CT_MAX_CAND / 32; ++j) {
-                    const int k = lane + 32 * j;
-                    if (k >= ncand) continue;
-                    const double other = s_v[team][k];
-                    const double mse = other < inf ? (nf > 0.0 ? (nf * (q.var + dm * dm) + (v[j] + other)) / nf : 0.0) : inf;
-                    a.curve[(size_t)c * a.ncp + k] = mse;
-                    s_v[team][k] = mse;
-                    if (mse < bv) { bv = mse; bk = k; }
-                }
+                for (int k = lane; k < ncand; k += 32)
+                    if (s_v[team][k] < bv) { bv = s_v[team][k]; bk = k; }
                 for (int o = 16; o > 0; o >>= 1) {
                     const double ov = __shfl_down_sync(0xFFFFFFFFu, bv, o);
                     const int ok = __shfl_down_sync(0xFFFFFFFFu, bk, o);
@@ -645,10 +692,10 @@ void ct_choose(const qp_ctx* ctx, uint64_t rows, uint32_t C, int max_w, int& w, 
 }  // namespace
 
 // Statistics per channel (bits = 0), the search on the caller's statistics (st_in), or both.  Rows up to 65535: the packed
-// prefix sums hold 17 bits of count.
+// prefix sums hold 17 bits of count (and a block's byte offsets, below 65536 * 4096 * 4, 32 bits).
 bool qp_channel_strips_apply(qp_ctx* ctx, uint64_t rows, uint32_t C, int bits)
 {
-    return rows >= 1 && rows <= 65535 && bits <= 4 && (uint64_t)C * rows < (1ull << 40) && ct_usable(ctx);
+    return rows >= 1 && rows <= 65535 && bits <= 4 && C <= QP_MAX_CHANNELS && ct_usable(ctx);
 }
 
 int32_t qp_launch_channel_strips(qp_ctx* ctx, const void* d_x, int dtype, uint64_t rows, uint32_t C, const qp_stats_t* st_in,

@@ -1353,6 +1353,27 @@ def test_search_channels_full_size_sampled(ctx, name, bits):
     assert ctx.qp_get_status() & ~qp.QP_DEV_DEGENERATE == 0
 
 
+# strips of channels: clusters of every size (rows), the last strip's remainder, one row, and channels whose clip ends are
+# coarse against the step (every candidate scored) beside ordinary ones
+@pytest.mark.parametrize("channels,rows,bits", [(17, 8191, 4), (16, 8193, 3), (33, 20000, 4), (2, 57345, 1), (100, 1, 2), (197, 130, 4)])
+def test_search_channels_strips(ctx, channels, rows, bits):
+    x = si.vit_activation((1, rows, channels), 170 + channels % 5, outlier_frac=0.1).reshape(rows, channels).copy()
+    if rows > 1:
+        x[:, 1] += np.float32(5000.0)
+        x[:, channels - 1] = np.round(x[:, channels - 1])
+    x = x.reshape(-1)
+    check_search_channels(ctx, x, dev(x), channels, bits, steps=100 if rows < 50000 else 20)
+    d_stats = ctx.qp_stats_channels(dev(x), channels)
+    want_st = torch.empty_like(d_stats)
+    packed, d_qp = ctx.qp_sender_channels_device(dev(x), channels, bits, qp.QP_CLIP_DSACIQ, out_stats=want_st)
+    _, d_qp2 = ctx.qp_dsaciq_search_channels(dev(x), channels, d_stats, bits)
+    assert torch.equal(d_qp, d_qp2)                      # the same bits with the statistics in the launch and before it
+    assert torch.equal(packed, ctx.qp_quantize_pack_channels(dev(x), channels, bits, d_qp))
+    a, b = _read_array(want_st, qp.Stats, channels), _read_array(d_stats, qp.Stats, channels)
+    assert all((u.mean, u.mad, u.var, u.min, u.max) == (v.mean, v.mad, v.var, v.min, v.max) for u, v in zip(a, b))
+    ctx.qp_get_status()
+
+
 @pytest.mark.parametrize("rows", [65535, 65536])
 def test_search_channels_at_the_row_limit_of_the_interval_form(ctx, rows):
     """65535 rows is the most the interval form's 16-bit counts hold; one more row and the call scores every
