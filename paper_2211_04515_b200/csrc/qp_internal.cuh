@@ -80,6 +80,7 @@ struct qp_ctx {
     int fused_checked, fused_ok;         // whether this device can hold the cooperative sender's grid
     int stats_fused_checked, stats_fused_ok;   // the same for the one-launch statistics
     int ss_checked, ss_ok;               // the same for statistics and search in one launch
+    int op_checked, op_ok;               // the same for the one-pass statistics
     int ct_checked, ct_ok;               // the same for the channel strips, and
     int ct_clusters[9];                  // how many clusters of 1..8 blocks run at a time
     long long wait_cycles;               // limit of a wait for a tile copy (clock cycles)
@@ -548,6 +549,9 @@ int32_t qp_launch_interval_search(qp_ctx* ctx, const void* d_x, int dtype, uint6
                                   qp_qparams_t* d_qp_out, cudaStream_t s);
 int32_t qp_stats_search_channels(qp_ctx* ctx, const void* d_x, int dtype, uint64_t rows, uint32_t channels, qp_stats_t* st_out,
                                  int bits, int bmode, int steps, int hist_bins, qp_qparams_t* d_qp_out, cudaStream_t s);
+bool qp_stats_onepass_applies(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n);
+int32_t qp_launch_stats_onepass(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, qp_stats_t* st_out, int bits, int method,
+                                int bmode, double F, qp_qparams_t* d_qp_out, void* d_packed, cudaStream_t s);
 bool qp_channel_strips_apply(qp_ctx* ctx, uint64_t rows, uint32_t C, int bits);
 int32_t qp_launch_channel_strips(qp_ctx* ctx, const void* d_x, int dtype, uint64_t rows, uint32_t C, const qp_stats_t* st_in,
                                  qp_stats_t* st_out, int bits, int bmode, int steps, int ncp, int nb, double F, float4* cand,

@@ -1,0 +1,554 @@
+// Statistics (paper Sec. 3), and in the sender with a closed-form clip the clip and the packing as well: one cooperative
+// launch, one block of 16 independent warps per SM.  Two forms, chosen by the tensor's size.
+//
+// Two passes, while L2 still holds the tensor when the second one comes (which walks it backwards): sum x, sum |x|, min and
+// max; a grid barrier; sum |x - mean| and sum (x - mean)^2; a second barrier, and every block knows the clip and packs.
+// What bounds it: two barriers and merges of 2.5 us each, then L2 and the instructions.  Against one launch of 32 KB
+// tiles copied by TMA: 12.5 against 14.5 us at 2^20 elements, 20.4 / 21.7 at 2^23, 26.7 / 28.6 at 2^24 fp32.
+//
+// One pass above that.  sum |x - mean| needs the mean first, so the deviations are taken about a pilot centre c, y = x - c,
+// and the split point is moved to the mean afterwards: with D = mean - c > 0
+//     sum |x - mean| = sum |y| + D (N(y < 0) - N(y >= 0)) + 2 sum over 0 <= y < D of (D - y),
+// mirrored for D < 0.  The last sum is over the few elements between c and the mean: the elements within delta of c (six
+// standard errors of the pilot, under half a per cent of a bell-shaped tensor) are counted and added up in cells of 1/64
+// octave of |y|, so that every cell but the mean's own lies on a known side.  That one is taken as evenly filled, which is
+// accepted where even the worst filling could not change the result by 1e-8; otherwise (and where the mean lies further
+// than delta from c, or a cell's counter might have wrapped) the second pass runs after all.
+// What bounds it: the read, 171 us for 1 GiB of fp32 (6.3 TB/s) of 193 in all, where two passes took 319; the rest is the
+// pilot (3 us for its loads: 64 bytes per sample, one DRAM burst; 16-byte samples took 16 us on 1 GiB), three
+// barriers, and blocks that end up to 8 us apart.  fp32 of 134, 268 and 537 MB: 41, 62 and 102 us against 45, 82 and 157.
+// The window must cost next to nothing: one test per four elements, and behind it one predicated look-up for the lane's hit
+// (all elements through the look-up took 275 us on 1 GiB, four look-ups behind the test 221).
+//
+// Packing here rather than in a launch of its own: 5 to 10 us less (no clip launch, no gaps, and what L2 still holds is not
+// read again), 1 GiB at 8 bits 383 against 394 us, 2^24 fp32 at 2 bits 35 against 44.
+#include "qp_gridbar.cuh"
+#include "qp_packtile.cuh"
+#include "qp_tiles.cuh"
+
+QP_CK_UNIT
+
+namespace {
+
+constexpr int OP_SAMPLE = 4;                       // most pilot vectors per thread
+constexpr int OP_OCTAVES = 8;                      // octaves of |y| below delta that have cells of their own
+constexpr int OP_CELLS = 64 * OP_OCTAVES + 1;      // per side; cell 0: what is below them
+constexpr int OP_REPS = 3;                         // log2 of the lane replicas of a cell
+constexpr unsigned OP_FULL = 65000u;               // most elements of a cell's replica: offsets of 16 bits add up to a word
+constexpr uint64_t OP_ONE_MIN_BYTES = 96ull << 20; // tensors from which one pass is the faster form
+constexpr float OP_MAGIC = 8388608.0f;
+constexpr unsigned OP_ONE = 0x4B000000u;
+constexpr size_t OP_DYN_BYTES = (size_t)(2 * OP_CELLS * 2 << OP_REPS) * sizeof(unsigned);   // >= 16 KB: the packer's staging
+constexpr int OP_SUMS_AT = (int)(OP_DYN_BYTES / 2);
+
+struct OpArgs {
+    const void* x;
+    uint64_t n, ntiles;                            // ntiles: whole tiles
+    qp_stats_t* st_out;
+    qp_qparams_t* qp_out;                          // sender: the quantizer, and
+    uint32_t* packed;                              // the packed stream
+    uint64_t nwords;
+    int method, bmode;
+    double F;
+    int one;                                       // one pass, or two
+    int sample;                                    // pilot vectors per thread
+    double* part;                                  // [4][grid][8]
+    unsigned* bar;                                 // [0] arrivals, [1] blocks that have left; zero at entry and at exit
+    unsigned* status;
+    unsigned spin_limit, bar_extra;
+};
+
+__device__ __forceinline__ unsigned op_hash(unsigned v)
+{
+    v ^= v >> 16; v *= 0x7FEB352Du;
+    v ^= v >> 15; v *= 0x846CA68Bu;
+    return v ^ (v >> 16);
+}
+
+// ONE: the pass about the pilot centre; otherwise the first of two passes (c = 0, no deviations and no window)
+template <bool ONE>
+struct OpPass {
+    float c, delta, inv_u;                         // inv_u: 2^16 / delta
+    int cell_off;                                  // |y|'s top bits less this: cell - 1
+    unsigned mul, base, half;                      // window table of this lane, as byte addresses
+    double sy, sa, sv, sx;                         // sum y, |y|, y^2, |x|
+    float mn, mx;
+    unsigned below, odd;
+    qp_f2 nc, y2[2], v2[2];
+    float a2[2], x2[2], lo, hi, w0, w1;
+    __device__ __forceinline__ void begin()
+    {
+        y2[0] = y2[1] = v2[0] = v2[1] = 0ull;
+        a2[0] = a2[1] = x2[0] = x2[1] = 0.f;
+        lo = mn;
+        hi = mx;
+    }
+    __device__ __forceinline__ void window(float y) const
+    {
+        const float a = fabsf(y);
+        const int cell = min(max((int)(__float_as_uint(a) >> 17) - cell_off, 0), OP_CELLS - 1);
+        const unsigned addr = (unsigned)cell * mul + base + (__float_as_uint(y) >> 31) * half;
+        const unsigned d = __float_as_uint(fmaf(a, inv_u, OP_MAGIC)) - OP_ONE;
+        asm volatile("{ .reg .pred p; setp.lt.f32 p, %3, %4; @p red.shared.add.u32 [%0], 1; @p red.shared.add.u32 [%0+%2], %1; }"
+                     ::"r"(addr), "r"(d), "n"(OP_SUMS_AT), "f"(a), "f"(delta) : "memory");
+    }
+    __device__ __forceinline__ void pair(float a, float b, int i)
+    {
+        if constexpr (!ONE) {
+            y2[i & 1] = qp_add2(y2[i & 1], qp_pack2(a, b));
+            x2[0] += fabsf(a);
+            x2[1] += fabsf(b);
+            lo = qp_min3(lo, a, b);
+            hi = qp_max3(hi, a, b);
+            return;
+        }
+        const qp_f2 y = qp_add2(qp_pack2(a, b), nc);
+        float ya, yb;
+        qp_unpack2(y, ya, yb);
+        y2[i & 1] = qp_add2(y2[i & 1], y);
+        v2[i & 1] = qp_fma2(y, y, v2[i & 1]);
+        a2[0] += fabsf(ya);
+        a2[1] += fabsf(yb);
+        x2[0] += fabsf(a);
+        x2[1] += fabsf(b);
+        lo = qp_min3(lo, a, b);
+        hi = qp_max3(hi, a, b);
+        below += __float_as_uint(ya) >> 31;
+        below += __float_as_uint(yb) >> 31;
+        // four elements per test: outside the branch the window costs an instruction and a half per element
+        if (i & 1) {
+            if (fminf(qp_min3(fabsf(w0), fabsf(w1), fabsf(ya)), fabsf(yb)) < delta) {
+                const bool h0 = fabsf(w0) < delta, h1 = fabsf(w1) < delta, h2 = fabsf(ya) < delta, h3 = fabsf(yb) < delta;
+                window(h0 ? w0 : h1 ? w1 : h2 ? ya : yb);
+                if ((h0 & h1) | ((h0 | h1) & h2) | ((h0 | h1 | h2) & h3)) {
+                    if (h0 && h1) window(w1);
+                    if ((h0 || h1) && h2) window(ya);
+                    if ((h0 || h1 || h2) && h3) window(yb);
+                }
+            }
+        } else {
+            w0 = ya;
+            w1 = yb;
+        }
+    }
+    __device__ __forceinline__ void end()
+    {
+        const float psa = a2[0] + a2[1], psx = x2[0] + x2[1];
+        if ((ONE ? psa : 0.f) + psx < __int_as_float(0x7F800000)) {        // every element finite (and no fp32 overflow)
+            float u, v;
+            qp_unpack2(qp_add2(y2[0], y2[1]), u, v);
+            sy += (double)(u + v);
+            if constexpr (ONE) {
+                qp_unpack2(qp_add2(v2[0], v2[1]), u, v);
+                sv += (double)(u + v);
+                sa += (double)psa;
+            }
+            sx += (double)psx;
+            mn = lo;
+            mx = hi;
+        } else {
+            ++odd;
+        }
+    }
+};
+// element by element: a lane's share with non-finite values, and what is behind the last tile
+struct OpOnes {
+    double sy = 0.0, sa = 0.0, sv = 0.0, sx = 0.0, below = 0.0, bad = 0.0;
+    float mn, mx;
+    __device__ __forceinline__ void one(float v, float c)
+    {
+        if (!qp_is_finite(v)) { bad += 1.0; return; }
+        const double y = (double)__fsub_rn(v, c);
+        sy += y;
+        sa += fabs(y);
+        sv += y * y;
+        sx += (double)fabsf(v);
+        below += y < 0.0 ? 1.0 : 0.0;
+        mn = fminf(mn, v);
+        mx = fmaxf(mx, v);
+    }
+};
+// the second pass, where it has to run: deviations about the mean itself
+template <bool GUARD>
+struct OpDeviations {
+    qp_f2 nhi, nlo;
+    double sd, sv;
+    float a2[2];
+    qp_f2 v2;
+    __device__ __forceinline__ void begin()
+    {
+        a2[0] = a2[1] = 0.f;
+        v2 = 0ull;
+    }
+    __device__ __forceinline__ void pair(float a, float b, int)
+    {
+        qp_f2 d = qp_add2(qp_add2(qp_pack2(a, b), nhi), nlo);
+        float da, db;
+        qp_unpack2(d, da, db);
+        if (GUARD) {
+            da = qp_is_finite(a) ? da : 0.f;
+            db = qp_is_finite(b) ? db : 0.f;
+            d = qp_pack2(da, db);
+        }
+        v2 = qp_fma2(d, d, v2);
+        a2[0] += fabsf(da);
+        a2[1] += fabsf(db);
+    }
+    __device__ __forceinline__ void end()
+    {
+        float u, v;
+        qp_unpack2(v2, u, v);
+        sd += (double)(a2[0] + a2[1]);
+        sv += (double)(u + v);
+    }
+};
+
+// N partials of every block, in order, by one warp with all loads in flight; the result in s (shared), for everybody
+// behind the block barrier at the end.  OPS: 0 sum, 1 min, 2 max.
+template <int... OPS>
+__device__ __forceinline__ void op_merge(const double* part, unsigned G, double* s)
+{
+    constexpr int N = sizeof...(OPS);
+    constexpr int ops[N] = {OPS...};
+    const double inf = __longlong_as_double(0x7FF0000000000000ll);
+    if (threadIdx.x < 32) {
+        double m[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) m[j] = ops[j] == 0 ? 0.0 : ops[j] == 1 ? inf : -inf;
+        for (unsigned b0 = threadIdx.x; b0 < G; b0 += 32 * SS_MERGE) {
+            double p[SS_MERGE][N];
+#pragma unroll
+            for (int u = 0; u < SS_MERGE; ++u)
+#pragma unroll
+                for (int j = 0; j < N; ++j)
+                    p[u][j] = b0 + 32 * u < G ? __ldcg(part + (size_t)(b0 + 32 * u) * 8 + j) : (ops[j] == 0 ? 0.0 : ops[j] == 1 ? inf : -inf);
+#pragma unroll
+            for (int u = 0; u < SS_MERGE; ++u)
+#pragma unroll
+                for (int j = 0; j < N; ++j)
+                    m[j] = ops[j] == 0 ? m[j] + p[u][j] : (ops[j] == 1 ? fmin(m[j], p[u][j]) : fmax(m[j], p[u][j]));
+        }
+        ss_warp_reduce<OPS...>(m);
+        if (threadIdx.x == 0)
+#pragma unroll
+            for (int j = 0; j < N; ++j) s[j] = m[j];
+    }
+    __syncthreads();
+}
+
+// BITS = 0: statistics only; 1..8: the sender.
+template <typename T, int BITS>
+__global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpArgs a)
+{
+    extern __shared__ __align__(16) unsigned char raw[];
+    using Tiles = SsTiles<T, SS_TILE>;
+    constexpr int EPV = Tiles::EPV;
+    __shared__ double s_red[SS_WARPS * 8];
+    __shared__ double s_sum[8];
+    __shared__ int s_ok, s_full;
+    __shared__ qp_qparams_t s_qp;
+    const T* x = static_cast<const T*>(a.x);
+    const int lane = threadIdx.x & 31;
+    const unsigned G = gridDim.x;
+    const uint64_t first = (uint64_t)blockIdx.x * SS_WARPS + (threadIdx.x >> 5), step = (uint64_t)G * SS_WARPS;
+    const uint64_t tail0 = a.ntiles * SS_TILE;
+    const double inf = __longlong_as_double(0x7FF0000000000000ll);
+    unsigned* table = reinterpret_cast<unsigned*>(raw);
+    unsigned waits = 0;
+    auto meet = [&]() {
+        ++waits;
+        return qp_grid::barrier(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
+    };
+    for (int i = threadIdx.x; i < (int)(OP_DYN_BYTES / 16); i += SS_THREADS) reinterpret_cast<uint4*>(raw)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (threadIdx.x == 0) s_full = 0;
+
+    // ---- pilot: sample i, four neighbouring vectors (the bytes of one DRAM burst) by four lanes, lies at a random place of
+    // the i-th of equal parts of the tensor
+    float c = 0.f, delta = 1.f;
+    if (a.one) {
+        const uint64_t nv4 = a.n / (4 * EPV);
+        const unsigned total = (unsigned)a.sample * G * (SS_THREADS / 4);
+        const uint64_t part = nv4 / total;                    // >= 1
+        float e[OP_SAMPLE][EPV];
+#pragma unroll
+        for (int j = 0; j < OP_SAMPLE; ++j) {
+            const unsigned i = ((unsigned)j * G + blockIdx.x) * (SS_THREADS / 4) + threadIdx.x / 4;
+            const uint64_t v = (i * part + ((uint64_t)op_hash(i) * part >> 32)) * 4 + (lane & 3);
+            if (j < a.sample) qp_load_vec(x + v * EPV, e[j]);
+        }
+        float x0 = qp_load_one(x);                            // (any value near the tensor's: the sums are taken about it)
+        if (!qp_is_finite(x0)) x0 = 0.f;
+        float p1 = 0.f, p2 = 0.f, pn = 0.f;
+#pragma unroll
+        for (int j = 0; j < OP_SAMPLE; ++j) {
+            if (j >= a.sample) break;
+            float m = 0.f;
+#pragma unroll
+            for (int k = 0; k < EPV; ++k) m += e[j][k] - x0;
+            m *= 0.25f / EPV;
+            m += __shfl_xor_sync(0xFFFFFFFFu, m, 1);
+            m += __shfl_xor_sync(0xFFFFFFFFu, m, 2);
+            if (m * m < __int_as_float(0x7F800000)) { p1 += m; p2 = fmaf(m, m, p2); pn += 1.f; }
+        }
+        double v3[3] = {(double)p1, (double)p2, (double)pn};
+        ss_reduce<0, 0, 0>(v3, s_red);
+        if (threadIdx.x == 0)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) a.part[(size_t)(2 * G + blockIdx.x) * 8 + j] = v3[j];
+        if (!meet()) return;
+        op_merge<0, 0, 0>(a.part + (size_t)2 * G * 8, G, s_sum);
+        // (every sample was counted by its four lanes)
+        const double k = s_sum[2] > 0.0 ? s_sum[2] : 1.0, m = s_sum[0] / k, var = s_sum[1] / k - m * m;
+        c = (float)((double)x0 + m);
+        if (!qp_is_finite(c)) c = 0.f;
+        const double want = fmax(fmax(12.0 * sqrt(fmax(var, 0.0) / k), fabs((double)c) * 3.814697265625e-6), 1e-30);
+        delta = (float)fmin(want, 1e30);
+    }
+
+    // ---- the pass
+    double v8[8];
+    const int cell_off = (int)(__float_as_uint(delta) >> 17) - (OP_CELLS - 1);   // delta's own cell is the last
+    auto pass = [&](auto& f) {
+        f.c = c;
+        f.delta = delta;
+        f.inv_u = 65536.0f / delta;
+        f.cell_off = cell_off;
+        f.mul = 4u << OP_REPS;
+        f.base = (unsigned)__cvta_generic_to_shared(table + (lane & ((1 << OP_REPS) - 1)));
+        f.half = (unsigned)OP_CELLS * f.mul;
+        f.sy = f.sa = f.sv = f.sx = 0.0;
+        f.mn = __int_as_float(0x7F800000);
+        f.mx = -f.mn;
+        f.below = f.odd = 0u;
+        f.nc = qp_pack2(-c, -c);
+        Tiles::template run<false>(x, a.ntiles, first, step, lane, f);
+        OpOnes o;
+        o.mn = f.mn;
+        o.mx = f.mx;
+        if (f.odd) {                                          // rare: this lane's share again (its window counts stand)
+            o.mn = __int_as_float(0x7F800000);
+            o.mx = -o.mn;
+            for (uint64_t t = first; t < a.ntiles; t += step)
+                for (int j = 0; j < SS_TILE / 32 / EPV; ++j)
+                    for (int i = 0; i < EPV; ++i) o.one(qp_load_one(x + t * SS_TILE + (j * 32 + lane) * EPV + i), c);
+        } else {
+            o.sy = f.sy; o.sa = f.sa; o.sv = f.sv; o.sx = f.sx;
+            o.below = (double)f.below;
+        }
+        if (blockIdx.x == G - 1)
+            for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) {
+                const float v = qp_load_one(x + i);
+                o.one(v, c);
+                if (a.one && qp_is_finite(v)) f.window(__fsub_rn(v, c));
+            }
+        v8[0] = o.sy; v8[1] = o.sa; v8[2] = o.sv; v8[3] = o.sx; v8[4] = (double)o.mn; v8[5] = (double)o.mx; v8[6] = o.below; v8[7] = o.bad;
+    };
+    if (a.one) {
+        OpPass<true> f;
+        pass(f);
+    } else {
+        OpPass<false> f;
+        pass(f);
+    }
+    ss_reduce<0, 0, 0, 0, 1, 2, 0, 0>(v8, s_red);             // (its barriers also order the window's counters)
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) a.part[(size_t)blockIdx.x * 8 + j] = v8[j];
+    if (!meet()) return;
+    op_merge<0, 0, 0, 0, 1, 2, 0, 0>(a.part, G, s_sum);
+    qp_stats_t st;
+    const double sum_abs = s_sum[1], sum_sq = s_sum[2], below = s_sum[6];
+    double D, nf;
+    {
+        const unsigned long long bad = (unsigned long long)s_sum[7];
+        nf = (double)(a.n - bad);
+        D = nf > 0.0 ? s_sum[0] / nf : 0.0;
+        st.n = a.n;
+        st.nonfinite = bad;
+        st.mean = nf > 0.0 ? (double)c + D : 0.0;
+        st.mean_abs = nf > 0.0 ? s_sum[3] / nf : 0.0;
+        st.min = nf > 0.0 ? s_sum[4] : 0.0;
+        st.max = nf > 0.0 ? s_sum[5] : 0.0;
+        st.hist_peak = 0;
+        st.hist_bins = 0;
+        st.reserved = 0;
+        st.var = nf > 0.0 ? fmax(0.0, sum_sq / nf - D * D) : 0.0;
+        st.mad = 0.0;
+    }
+    bool again = !a.one || !(fabs(D) < (double)delta) || !(sum_sq < inf);
+    // ---- this block's share of the elements between c and the mean
+    if (!again) {                                             // uniform over the grid
+        const int side = D < 0.0;
+        const float aD = (float)fabs(D);
+        const int own = max((int)(__float_as_uint(aD) >> 17) - cell_off, 0);
+        double v4[4] = {0.0, 0.0, 0.0, 0.0};                  // count and sum below the mean's cell, count in it, overflow
+        for (int i = threadIdx.x; i < OP_CELLS; i += SS_THREADS) {
+            const unsigned* cnt = table + ((size_t)(side * OP_CELLS + i) << OP_REPS);
+            const unsigned* sum = reinterpret_cast<const unsigned*>(raw + OP_SUMS_AT) + ((size_t)(side * OP_CELLS + i) << OP_REPS);
+            unsigned long long cn = 0ull, cs = 0ull;
+            for (int r = 0; r < (1 << OP_REPS); ++r) {
+                const int rr = (r + threadIdx.x) & ((1 << OP_REPS) - 1);
+                cn += cnt[rr];
+                cs += sum[rr];
+                if (cnt[rr] > OP_FULL) s_full = 1;            // benign race: every writer writes 1
+            }
+            if (i < own) { v4[0] += (double)cn; v4[1] += (double)cs; }
+            if (i == own) v4[2] += (double)cn;
+        }
+        ss_reduce<0, 0, 0, 0>(v4, s_red);
+        if (threadIdx.x == 0) {
+            double* p = a.part + (size_t)(G + blockIdx.x) * 8;
+            p[0] = v4[0]; p[1] = v4[1]; p[2] = v4[2]; p[3] = s_full ? 1.0 : 0.0;
+        }
+        if (!meet()) return;
+        op_merge<0, 0, 0, 0>(a.part + (size_t)G * 8, G, s_sum);
+        const double d = fabs(D), u = (double)delta / 65536.0;
+        const double lo = own ? (double)__uint_as_float((unsigned)(own + cell_off) << 17) : 0.0;
+        const double hi = (double)__uint_as_float((unsigned)(own + 1 + cell_off) << 17), w = hi - lo;
+        const double own_part = s_sum[2] * (d - lo) * (d - lo) / (2.0 * w);       // evenly filled
+        const double between = d * s_sum[0] - u * s_sum[1] + own_part;
+        const double neg = side ? nf - below : below;         // elements on the other side of c
+        const double sd = sum_abs + d * (neg - (nf - neg)) + 2.0 * between;
+        st.mad = nf > 0.0 ? fmax(0.0, sd) / nf : 0.0;
+        again = s_sum[3] > 0.0 || !(s_sum[2] * w * 0.5 <= 1e-8 * sum_abs);
+        if (sum_abs == 0.0) again = false;                    // (every element is c)
+    }
+    if (again) {                                              // uniform over the grid
+        __syncthreads();
+        const float m_hi = (float)st.mean, m_lo = (float)(st.mean - (double)m_hi);    // the mean as an unevaluated fp32 pair
+        const qp_f2 nhi = qp_pack2(-m_hi, -m_hi), nlo = qp_pack2(-m_lo, -m_lo);
+        double v2[2];
+        if (st.nonfinite) {
+            OpDeviations<true> f = {nhi, nlo, 0.0, 0.0};
+            Tiles::template run<true>(x, a.ntiles, first, step, lane, f);
+            v2[0] = f.sd; v2[1] = f.sv;
+        } else {
+            OpDeviations<false> f = {nhi, nlo, 0.0, 0.0};
+            Tiles::template run<true>(x, a.ntiles, first, step, lane, f);
+            v2[0] = f.sd; v2[1] = f.sv;
+        }
+        if (blockIdx.x == G - 1)
+            for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) {
+                const float v = qp_load_one(x + i);
+                if (!qp_is_finite(v)) continue;
+                const float dd = __fsub_rn(__fsub_rn(v, m_hi), m_lo);
+                v2[0] += (double)fabsf(dd);
+                v2[1] += (double)(dd * dd);
+            }
+        ss_reduce<0, 0>(v2, s_red);
+        if (threadIdx.x == 0) {                               // (rows of their own: a slow block may still read the others)
+            a.part[(size_t)(3 * G + blockIdx.x) * 8] = v2[0];
+            a.part[(size_t)(3 * G + blockIdx.x) * 8 + 1] = v2[1];
+        }
+        if (!meet()) return;
+        op_merge<0, 0>(a.part + (size_t)3 * G * 8, G, s_sum);
+        st.mad = nf > 0.0 ? s_sum[0] / nf : 0.0;
+        st.var = nf > 0.0 ? s_sum[1] / nf : 0.0;
+    }
+    if (threadIdx.x == 0) {
+        if (blockIdx.x == 0) {
+            *a.st_out = st;
+            if (st.nonfinite) atomicOr(a.status, QP_DEV_NONFINITE);
+        }
+        if constexpr (BITS > 0) {
+            double lo, hi;
+            qp_clip_ends(st, a.method, QP_DIST_LAPLACE, a.bmode, BITS, a.F, lo, hi);
+            const int rc = qp_fill_qparams(lo, hi, BITS, &s_qp);
+            if (blockIdx.x == 0) {
+                *a.qp_out = s_qp;
+                if (rc == QP_WARN_DEGENERATE) atomicOr(a.status, QP_DEV_DEGENERATE);
+            }
+        }
+    }
+    __syncthreads();
+    if constexpr (BITS > 0) {                                 // from the tensor's end, which L2 holds
+        uint32_t* sw = reinterpret_cast<uint32_t*>(raw) + (threadIdx.x >> 5) * 256;
+        const float lo = s_qp.lo, hi = s_qp.hi, inv = s_qp.inv_scale;
+        const uint64_t tiles = (a.n + QP_TILE - 1) / QP_TILE;
+        for (uint64_t it = first; it < tiles; it += step)
+            qp_pack_tile<BITS, T, true>(x, a.n, tiles - 1 - it, lane, lo, hi, inv, a.packed, a.nwords, sw);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0 && atomicInc(a.bar + 1, G - 1) == G - 1) atomicExch(a.bar, 0u);       // the last block out
+}
+
+template <typename T>
+void* op_kernel(int bits)
+{
+    switch (bits) {
+        case 0: return (void*)stats_onepass_kernel<T, 0>;
+        case 1: return (void*)stats_onepass_kernel<T, 1>;
+        case 2: return (void*)stats_onepass_kernel<T, 2>;
+        case 3: return (void*)stats_onepass_kernel<T, 3>;
+        case 4: return (void*)stats_onepass_kernel<T, 4>;
+        case 5: return (void*)stats_onepass_kernel<T, 5>;
+        case 6: return (void*)stats_onepass_kernel<T, 6>;
+        case 7: return (void*)stats_onepass_kernel<T, 7>;
+        default: return (void*)stats_onepass_kernel<T, 8>;
+    }
+}
+
+bool op_usable(qp_ctx* ctx)
+{
+    if (!ctx->op_checked) {
+        ctx->op_checked = 1;
+        int coop = 0;
+        bool ok = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device) == cudaSuccess && coop &&
+                  (size_t)ctx->sm_count * 32 * sizeof(double) <= sizeof(qp_stats_partial) * QP_MAX_BLOCKS;
+        for (int bits = 0; ok && bits <= 8; ++bits)
+            for (int v = 0; ok && v < 2; ++v) {
+                void* k = v ? op_kernel<unsigned short>(bits) : op_kernel<float>(bits);
+                int per_sm = 0;
+                ok = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OP_DYN_BYTES) == cudaSuccess &&
+                     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, SS_THREADS, OP_DYN_BYTES) == cudaSuccess && per_sm >= 1;
+            }
+        if (!ok) cudaGetLastError();
+        ctx->op_ok = ok ? 1 : 0;
+    }
+    return ctx->op_ok != 0;
+}
+
+}  // namespace
+
+bool qp_stats_onepass_applies(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n)
+{
+    (void)dtype;
+    return !((uintptr_t)d_x & 15u) && n >= 8 * SS_TILE && op_usable(ctx);
+}
+
+// Statistics (bits = 0), or with bits 1..8 the sender with a closed-form clip.
+int32_t qp_launch_stats_onepass(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, qp_stats_t* st_out, int bits, int method,
+                                int bmode, double F, qp_qparams_t* d_qp_out, void* d_packed, cudaStream_t s)
+{
+    static_assert(OP_DYN_BYTES >= SS_WARPS * 1024, "the packer's staging");
+    OpArgs a;
+    a.x = d_x;
+    a.n = n;
+    a.ntiles = n / SS_TILE;
+    a.st_out = st_out;
+    a.qp_out = d_qp_out;
+    a.packed = static_cast<uint32_t*>(d_packed);
+    a.nwords = bits ? qp_packed_bytes(n, bits) / 4 : 0;
+    a.method = method;
+    a.bmode = bmode;
+    a.F = F;
+    a.part = reinterpret_cast<double*>(ctx->d_part);
+    a.bar = reinterpret_cast<unsigned*>(ctx->d_fused) + 24;   // words 24, 25 of the barrier scratch
+    a.status = ctx->d_status;
+    a.spin_limit = ctx->spin_limit;
+    a.bar_extra = (unsigned)ctx->bar_extra;
+    const uint64_t want = (a.ntiles + SS_WARPS - 1) / SS_WARPS;
+    const unsigned G = (unsigned)(want < (uint64_t)ctx->sm_count ? want : (uint64_t)ctx->sm_count);
+    const uint64_t share = n / (dtype == QP_F32 ? 4 : 8) / ((uint64_t)G * SS_THREADS * 16);   // a sixteenth of the tensor
+    // Two passes while the second one finds the tensor in L2, where it costs less than the pilot and the window; fp32 of 67, 134
+    // and 268 MB: 30.6, 41 and 62 us in one pass, 28.6, 45 and 82 us in two; bf16 of 34, 67 and 134 MB: 28.8, 38.9 and 57,
+    // and 26.7, 39.0 and 63.
+    a.one = n * (dtype == QP_F32 ? 4 : 2) >= OP_ONE_MIN_BYTES;
+    a.sample = share < 1 ? 1 : share < OP_SAMPLE ? (int)share : OP_SAMPLE;
+    void* k = dtype == QP_F32 ? op_kernel<float>(bits) : op_kernel<unsigned short>(bits);
+    void* params[] = {&a};
+    if (cudaLaunchCooperativeKernel(k, dim3(G), dim3(SS_THREADS), params, OP_DYN_BYTES, s) != cudaSuccess)
+        return qp_check_launch(ctx, "one-pass statistics (cooperative launch)");
+    ctx->launches += 1;
+    return qp_check_launch(ctx, "one-pass statistics");
+}

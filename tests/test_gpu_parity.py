@@ -948,6 +948,52 @@ def test_search_forms_agree_beyond_two_waves(ctx, n):
     assert ctx.qp_get_status() == 0
 
 
+# statistics about a pilot centre (96 MB and more: 25165824 fp32 elements) and in two streaming passes (below), tiles of 1024
+# elements, 16 warps a block; with the closed-form sender from 2^21 + 2^19 elements.  Data that the one pass cannot
+# finish ("mass", "two_levels") or finishes at once, and elements that its sums must leave out.
+@pytest.mark.parametrize("n,data,bf16", [(8 * 1024, "plain", False), (8 * 1024 + 1, "nonfinite", True), (16 * 1024 + 1023, "plain", False),
+                                         (148 * 16 * 1024 + 7, "nonfinite", False), ((5 << 19) + 1, "offset", False),
+                                         ((5 << 19) + 1031, "plain", True), ((96 << 18) - 1, "plain", False),
+                                         (96 << 18, "plain", False), ((96 << 18) + 1025, "nonfinite", False),
+                                         (96 << 18, "mass", False), (96 << 18, "two_levels", False), (96 << 18, "constant", False),
+                                         (96 << 18, "outliers", False), (96 << 18, "offset", False), ((96 << 19) + 9, "plain", True)])
+def test_stats_streaming(ctx, n, data, bf16):
+    x = np.tile(si.flat_iid(min(n, 1 << 20), 31, "laplace"), -(-n // (1 << 20)))[:n] * np.float32(0.7) + np.float32(0.1)
+    if data == "nonfinite":
+        x[[0, 1023, n // 2, n - 1]] = [np.nan, np.inf, -np.inf, np.nan]
+    elif data == "offset":
+        x += np.float32(500.0)
+    elif data == "mass":                                 # half of the elements at the mean
+        x = np.where(np.arange(n) % 2 == 0, np.float32(0.0), x - x.mean(dtype=np.float64).astype(np.float32))
+    elif data == "two_levels":
+        x = np.where(np.arange(n) % 3 == 0, np.float32(-1.0), np.float32(2.0))
+    elif data == "constant":
+        x[:] = np.float32(-2.5)
+    elif data == "outliers":
+        x[::9973] *= np.float32(1e4)
+    x = x.astype(np.float32)
+    d = dev(x)
+    if bf16:
+        h = si.to_bf16_bits(x)
+        d, x = torch.from_numpy(h.view(np.int16)).cuda().view(torch.bfloat16), oracle.widen_bf16(h)
+    st_o = oracle.stats(x)
+    out = ctx.qp_stats(d)
+    st = ctx.read_stats(out)
+    check_stats(st, st_o)
+    assert abs(st.mad - st_o.mad) <= 3e-7 * st_o.mad
+    assert bytes(st) == bytes(ctx.read_stats(ctx.qp_stats(d)))
+    if n > (5 << 19):
+        before = ctx.qp_launch_count()
+        st_s = torch.zeros(80, dtype=torch.uint8, device="cuda")
+        packed, q = ctx.qp_sender_device(d, 6, False, out_stats=st_s)
+        assert ctx.qp_launch_count() - before == 1
+        assert bytes(ctx.read_stats(st_s)) == bytes(st)
+        want = ctx.qp_clip_qparams_device(out, 6, qp.QP_CLIP_ACIQ)
+        assert torch.equal(q.view(torch.uint8).reshape(-1), want.view(torch.uint8).reshape(-1))
+        assert torch.equal(packed, ctx.qp_quantize_pack(d, 6, want))
+    ctx.qp_get_status()
+
+
 # statistics and search in one launch (the default from 2^20 elements on, the sender above 2^21): every width it takes, tile
 # remainders, the largest and smallest number of steps, tables with few replicas, and the exact-threshold form
 SS_CASES = [(1, 0, 100, 100, (1 << 21) + 1, "vit"), (2, 0, 100, 100, (1 << 21) + 1023, "outliers"), (3, 0, 100, 100, (1 << 21) + 1024, "vit"),
