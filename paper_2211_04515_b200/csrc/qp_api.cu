@@ -763,6 +763,16 @@ extern "C" int32_t qp_unpack_dequantize(qp_ctx* ctx, const void* d_packed, uint6
 // launches serve what is between the two.
 constexpr uint64_t QP_ONE_LAUNCH_MIN_N = 1ull << 21;
 
+// Where the directed search with statistics and packing in front of and behind it is one launch of the streaming kernel: that
+// spends about 20 us whatever the size (barriers, and block 0's scoring, which grows with the levels), the
+// small-tensor launch scores every element against the candidates.  At 2^16, 151296, 2^18, 2^19 and 2^20 elements: 24.8,
+// 28.9, 32.9, 43 and 64 us in the small-tensor launch; streaming 27 to 29 us at 2 bits and 37 to 35 at 4.
+static bool streaming_search(uint64_t n, int bits)
+{
+    const uint64_t from = bits <= 2 ? 1ull << 17 : bits == 3 ? 3ull << 16 : 3ull << 17;
+    return n > QP_ONE_LAUNCH_MIN_N || (n >= from && n <= 15ull << 17);
+}
+
 // statistics -> clip -> quantize+pack on device buffers: one cooperative launch where that
 // applies (small tensors), the kernel chain of the separate calls otherwise
 static int32_t sender_on_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int bits, int method, int bmode,
@@ -772,6 +782,22 @@ static int32_t sender_on_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_
     int32_t rc;
     const int use_ds = (method & 0xF) == QP_CLIP_DSACIQ;
     const int search_mode = bmode | ((method & QP_CLIP_MIDRISE) ? QP_B_MIDRISE : 0);
+    if (use_ds && ctx->sender_path == QP_SENDER_AUTO && ctx->stats_path == QP_STATS_AUTO && ctx->search_path == QP_SEARCH_AUTO &&
+        streaming_search(n, bits) && check_x(ctx, d_x, dtype, n) == QP_OK && steps >= 1 && d_packed && !((uintptr_t)d_packed & 15u) &&
+        !((uintptr_t)st & 7u) && !((uintptr_t)d_qp_out & 3u) && (bmode == QP_B_MAD || bmode == QP_B_MEAN_ABS) &&
+        qp_stats_search_applies(ctx, d_x, dtype, n, hist_bins, bits, steps)) {
+        qp_device_guard guard(ctx->device);
+        if (!guard.ok) return qp_fail(ctx, QP_ERR_CUDA, "cannot select device");
+        rc = qp_launch_stats_search(ctx, d_x, dtype, n, nullptr, st, hist_bins, bits, search_mode, steps,
+                                    qp_host_aciq_F(bits, QP_DIST_LAPLACE), nullptr, d_qp_out, d_packed,
+                                    static_cast<cudaStream_t>(stream));
+        if (rc < 0) return rc;
+        ctx->last_steps = steps;
+        ctx->last_bits = bits;
+        ctx->last_x = d_x;
+        ctx->last_x_end = 0;
+        return rc;
+    }
     if (ctx->sender_path != QP_SENDER_CHAIN &&
         qp_sender_fused_applies(n, use_ds, steps, hist_bins, ctx->sender_path == QP_SENDER_FUSED)) {
         // the checks of the separate calls
@@ -789,22 +815,6 @@ static int32_t sender_on_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_
                                     static_cast<cudaStream_t>(stream));
         if (rc == QP_OK && use_ds) { ctx->last_steps = steps; ctx->last_bits = bits; }
         if (rc != QP_WARN_INFEASIBLE) return rc;               // else: this device cannot hold the grid
-    }
-    if (use_ds && ctx->sender_path == QP_SENDER_AUTO && ctx->stats_path == QP_STATS_AUTO && ctx->search_path == QP_SEARCH_AUTO &&
-        n > QP_ONE_LAUNCH_MIN_N && check_x(ctx, d_x, dtype, n) == QP_OK && steps >= 1 && d_packed && !((uintptr_t)d_packed & 15u) &&
-        !((uintptr_t)st & 7u) && !((uintptr_t)d_qp_out & 3u) && (bmode == QP_B_MAD || bmode == QP_B_MEAN_ABS) &&
-        qp_stats_search_applies(ctx, d_x, dtype, n, hist_bins, bits, steps)) {
-        qp_device_guard guard(ctx->device);
-        if (!guard.ok) return qp_fail(ctx, QP_ERR_CUDA, "cannot select device");
-        rc = qp_launch_stats_search(ctx, d_x, dtype, n, nullptr, st, hist_bins, bits, search_mode, steps,
-                                    qp_host_aciq_F(bits, QP_DIST_LAPLACE), nullptr, d_qp_out, d_packed,
-                                    static_cast<cudaStream_t>(stream));
-        if (rc < 0) return rc;
-        ctx->last_steps = steps;
-        ctx->last_bits = bits;
-        ctx->last_x = d_x;
-        ctx->last_x_end = 0;
-        return rc;
     }
     // the closed-form clip in one launch, except that the packer's own launch reads a large bf16 tensor faster: 2^26, 2^27 and
     // 2^28 elements at 8 bits take 89, 158 and 292 us in one launch, 94, 155 and 279 in three
