@@ -764,13 +764,21 @@ extern "C" int32_t qp_unpack_dequantize(qp_ctx* ctx, const void* d_packed, uint6
 constexpr uint64_t QP_ONE_LAUNCH_MIN_N = 1ull << 21;
 
 // Where the directed search with statistics and packing in front of and behind it is one launch of the streaming kernel: that
-// spends about 20 us whatever the size (barriers, and block 0's scoring, which grows with the levels), the
-// small-tensor launch scores every element against the candidates.  At 2^16, 151296, 2^18, 2^19 and 2^20 elements: 24.8,
-// 28.9, 32.9, 43 and 64 us in the small-tensor launch; streaming 27 to 29 us at 2 bits and 37 to 35 at 4.
+// spends 15 to 25 us whatever the size (barriers, and one block's scoring, which grows with the levels), the
+// small-tensor launch scores every element against every candidate.  At 2^15, 2^16, 2^17, 2^18, 2^19 and 2^20 elements: 23.5,
+// 24.7, 26.8, 32.9, 43 and 64 us in the small-tensor launch; streaming 22.7, 23.5, 23, 24.7, 28.8, 28.8 at 2 bits, 26.7, 28.7,
+// 26.8, 28.8, 32, 33 at 3 and 31 to 33 up to 2^18, 35 to 37 from there on at 4.
 static bool streaming_search(uint64_t n, int bits)
 {
-    const uint64_t from = bits <= 2 ? 1ull << 17 : bits == 3 ? 3ull << 16 : 3ull << 17;
+    const uint64_t from = bits <= 2 ? 1ull << 15 : bits == 3 ? 3ull << 16 : 3ull << 17;
     return n > QP_ONE_LAUNCH_MIN_N || (n >= from && n <= 15ull << 17);
+}
+
+// And the closed-form clip: as one cluster (12.4 us up to 2^18 elements, against 14.4 in the small-tensor launch, which is
+// as fast from there on), and above what the small-tensor launch holds.
+static bool streaming_closed_form(uint64_t n)
+{
+    return n > QP_ONE_LAUNCH_MIN_N + (1u << 19) || n <= 1u << 18;
 }
 
 // statistics -> clip -> quantize+pack on device buffers: one cooperative launch where that
@@ -798,6 +806,17 @@ static int32_t sender_on_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_
         ctx->last_x_end = 0;
         return rc;
     }
+    // the closed-form clip in one launch, except that the packer's own launch reads a large bf16 tensor faster: 2^26, 2^27 and
+    // 2^28 elements at 8 bits take 89, 158 and 292 us in one launch, 94, 155 and 279 in three
+    if (!use_ds && (dtype == QP_F32 || n <= (1ull << 26)) && ctx->sender_path == QP_SENDER_AUTO &&
+        ctx->stats_path == QP_STATS_AUTO && streaming_closed_form(n) && bits <= 8 &&
+        check_x(ctx, d_x, dtype, n) == QP_OK && d_packed && !((uintptr_t)d_packed & 15u) && !((uintptr_t)st & 7u) &&
+        !((uintptr_t)d_qp_out & 3u) && (bmode == QP_B_MAD || bmode == QP_B_MEAN_ABS) && qp_stats_onepass_applies(ctx, d_x, dtype, n)) {
+        qp_device_guard guard(ctx->device);
+        if (!guard.ok) return qp_fail(ctx, QP_ERR_CUDA, "cannot select device");
+        return qp_launch_stats_onepass(ctx, d_x, dtype, n, st, bits, method, bmode, qp_host_aciq_F(bits, QP_DIST_LAPLACE), d_qp_out,
+                                       d_packed, static_cast<cudaStream_t>(stream));
+    }
     if (ctx->sender_path != QP_SENDER_CHAIN &&
         qp_sender_fused_applies(n, use_ds, steps, hist_bins, ctx->sender_path == QP_SENDER_FUSED)) {
         // the checks of the separate calls
@@ -815,17 +834,6 @@ static int32_t sender_on_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_
                                     static_cast<cudaStream_t>(stream));
         if (rc == QP_OK && use_ds) { ctx->last_steps = steps; ctx->last_bits = bits; }
         if (rc != QP_WARN_INFEASIBLE) return rc;               // else: this device cannot hold the grid
-    }
-    // the closed-form clip in one launch, except that the packer's own launch reads a large bf16 tensor faster: 2^26, 2^27 and
-    // 2^28 elements at 8 bits take 89, 158 and 292 us in one launch, 94, 155 and 279 in three
-    if (!use_ds && (dtype == QP_F32 || n <= (1ull << 26)) && ctx->sender_path == QP_SENDER_AUTO &&
-        ctx->stats_path == QP_STATS_AUTO && n > QP_ONE_LAUNCH_MIN_N + (1u << 19) && bits <= 8 &&
-        check_x(ctx, d_x, dtype, n) == QP_OK && d_packed && !((uintptr_t)d_packed & 15u) && !((uintptr_t)st & 7u) &&
-        !((uintptr_t)d_qp_out & 3u) && (bmode == QP_B_MAD || bmode == QP_B_MEAN_ABS) && qp_stats_onepass_applies(ctx, d_x, dtype, n)) {
-        qp_device_guard guard(ctx->device);
-        if (!guard.ok) return qp_fail(ctx, QP_ERR_CUDA, "cannot select device");
-        return qp_launch_stats_onepass(ctx, d_x, dtype, n, st, bits, method, bmode, qp_host_aciq_F(bits, QP_DIST_LAPLACE), d_qp_out,
-                                       d_packed, static_cast<cudaStream_t>(stream));
     }
     rc = qp_stats(ctx, d_x, dtype, n, use_ds ? hist_bins : 0, st, stream);
     if (rc < 0) return rc;

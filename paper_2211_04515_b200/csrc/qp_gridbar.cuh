@@ -68,4 +68,9 @@ __device__ __forceinline__ bool wait(const unsigned* bar, unsigned target, unsig
     return *s_ok != 0;
 }
 
+// A grid that is one thread-block cluster has the hardware's barrier instead (about 0.4 us against 1.2): all threads
+// arrive, then all wait; it orders global memory like the counter does, and its blocks are resident together by definition.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
 }  // namespace qp_grid

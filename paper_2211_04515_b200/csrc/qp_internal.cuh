@@ -80,6 +80,7 @@ struct qp_ctx {
     int fused_checked, fused_ok;         // whether this device can hold the cooperative sender's grid
     int stats_fused_checked, stats_fused_ok;   // the same for the one-launch statistics
     int ss_checked, ss_ok;               // the same for statistics and search in one launch
+    int ss_cluster, op_cluster;          // whether these two also run as one cluster of up to QP_CLUSTER_BLOCKS blocks
     int op_checked, op_ok;               // the same for the one-pass statistics
     int ct_checked, ct_ok;               // the same for the channel strips, and
     int ct_clusters[9];                  // how many clusters of 1..8 blocks run at a time

@@ -56,6 +56,7 @@ struct OpArgs {
     unsigned* bar;                                 // [0] arrivals, [1] blocks that have left; zero at entry and at exit
     unsigned* status;
     unsigned spin_limit, bar_extra;
+    int cluster;                                   // the grid is one thread-block cluster
 };
 
 __device__ __forceinline__ unsigned op_hash(unsigned v)
@@ -256,6 +257,11 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
     unsigned* table = reinterpret_cast<unsigned*>(raw);
     unsigned waits = 0;
     auto meet = [&]() {
+        if (a.cluster) {
+            qp_grid::cluster_arrive();
+            qp_grid::cluster_wait();
+            return true;
+        }
         ++waits;
         return qp_grid::barrier(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
     };
@@ -467,8 +473,9 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
         const uint64_t tiles = (a.n + QP_TILE - 1) / QP_TILE;
         for (uint64_t it = first; it < tiles; it += step)
             qp_pack_tile<BITS, T, true>(x, a.n, tiles - 1 - it, lane, lo, hi, inv, a.packed, a.nwords, sw);
-        __syncthreads();
     }
+    if (a.cluster) return;
+    __syncthreads();
     if (threadIdx.x == 0 && atomicInc(a.bar + 1, G - 1) == G - 1) atomicExch(a.bar, 0u);       // the last block out
 }
 
@@ -502,6 +509,10 @@ bool op_usable(qp_ctx* ctx)
                 ok = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OP_DYN_BYTES) == cudaSuccess &&
                      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, SS_THREADS, OP_DYN_BYTES) == cudaSuccess && per_sm >= 1;
             }
+        ctx->op_cluster = ok;
+        for (int bits = 0; ok && bits <= 8; ++bits)
+            for (int v = 0; v < 2; ++v)
+                ctx->op_cluster &= qp_cluster_fits(v ? op_kernel<unsigned short>(bits) : op_kernel<float>(bits), SS_THREADS, OP_DYN_BYTES);
         if (!ok) cudaGetLastError();
         ctx->op_ok = ok ? 1 : 0;
     }
@@ -538,7 +549,9 @@ int32_t qp_launch_stats_onepass(qp_ctx* ctx, const void* d_x, int dtype, uint64_
     a.spin_limit = ctx->spin_limit;
     a.bar_extra = (unsigned)ctx->bar_extra;
     const uint64_t want = (a.ntiles + SS_WARPS - 1) / SS_WARPS;
-    const unsigned G = (unsigned)(want < (uint64_t)ctx->sm_count ? want : (uint64_t)ctx->sm_count);
+    a.cluster = qp_cluster_wanted(ctx, ctx->op_cluster, n);
+    const unsigned most = a.cluster ? QP_CLUSTER_BLOCKS : (unsigned)ctx->sm_count;
+    const unsigned G = (unsigned)(want < most ? want : most);
     const uint64_t share = n / (dtype == QP_F32 ? 4 : 8) / ((uint64_t)G * SS_THREADS * 16);   // a sixteenth of the tensor
     // Two passes while the second one finds the tensor in L2, where it costs less than the pilot and the window; fp32 of 67, 134
     // and 268 MB: 30.6, 41 and 62 us in one pass, 28.6, 45 and 82 us in two; bf16 of 34, 67 and 134 MB: 28.8, 38.9 and 57,
@@ -547,7 +560,7 @@ int32_t qp_launch_stats_onepass(qp_ctx* ctx, const void* d_x, int dtype, uint64_
     a.sample = share < 1 ? 1 : share < OP_SAMPLE ? (int)share : OP_SAMPLE;
     void* k = dtype == QP_F32 ? op_kernel<float>(bits) : op_kernel<unsigned short>(bits);
     void* params[] = {&a};
-    if (cudaLaunchCooperativeKernel(k, dim3(G), dim3(SS_THREADS), params, OP_DYN_BYTES, s) != cudaSuccess)
+    if (qp_launch_together(k, G, SS_THREADS, params, OP_DYN_BYTES, a.cluster, s) != cudaSuccess)
         return qp_check_launch(ctx, "one-pass statistics (cooperative launch)");
     ctx->launches += 1;
     return qp_check_launch(ctx, "one-pass statistics");

@@ -58,6 +58,7 @@ struct SsArgs {
     unsigned* bar;                                // [0] arrivals, [1] blocks that have left; zero at entry and at exit
     unsigned* status;
     unsigned spin_limit, bar_extra;
+    int cluster;                                   // the grid is one thread-block cluster
     int hist_shift;                               // log2 of the lane replicas of a histogram bin
     int rep_shift;                                // log2 of the lane replicas of an interval
     int flush_tiles;                              // tiles per warp after which the interval tables are emptied
@@ -250,6 +251,24 @@ __device__ __forceinline__ void ss_slices(const SsArgs& a, int count, unsigned c
         }
         __syncthreads();
     }
+}
+
+// The same for all intervals by one block, for the few rows of a cluster; the block barrier at the end makes them the
+// block's to read.
+__device__ __forceinline__ void ss_all_slices(const SsArgs& a, int count)
+{
+    const int G = (int)gridDim.x;
+    for (int i = threadIdx.x; i < count; i += SS_THREADS) {
+        unsigned long long n = 0, s = 0;
+#pragma unroll 8
+        for (int b = 0; b < G; ++b) {
+            const ulonglong2 v = __ldcg(a.rows + (size_t)b * count + i);
+            n += v.x;
+            s += v.y;
+        }
+        a.tot[i] = make_ulonglong2(n, s);
+    }
+    __syncthreads();
 }
 
 // Exclusive prefix sums of n[0..len), s[0..len) (n[len], s[len]: the totals), by `threads` threads (a multiple of
@@ -528,13 +547,30 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArg
     const double inf = __longlong_as_double(0x7FF0000000000000ll);
     unsigned* bins = reinterpret_cast<unsigned*>(raw + SS_TABLE_BYTES);
     unsigned waits = 0;
+    const bool cluster = a.cluster;
     auto meet = [&]() {
+        if (cluster) {
+            qp_grid::cluster_arrive();
+            qp_grid::cluster_wait();
+            return true;
+        }
         ++waits;
         return qp_grid::barrier(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
     };
     auto arrive = [&]() {
         __syncthreads();
+        if (cluster) {
+            qp_grid::cluster_arrive();
+            return;
+        }
         if (threadIdx.x == 0) qp_grid::arrive_release(a.bar);
+    };
+    auto wait = [&](unsigned target) {                        // behind arrive
+        if (cluster) {
+            qp_grid::cluster_wait();
+            return true;
+        }
+        return qp_grid::wait(a.bar, target + a.bar_extra, a.spin_limit, a.status, &s_ok);
     };
     auto scratch_clean = [&]() {                              // one block, when nobody needs the scratch any more
         for (int b = threadIdx.x; b < a.nb; b += SS_THREADS) a.hist[b] = 0ull;
@@ -797,13 +833,17 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArg
             }
             ss_hard_flush(h, row, fresh);
         }
-        if (!meet()) return;
-        ss_slices(a, hard ? h.M + 1 : 2 * ni, raw + SS_TABLE_BYTES);
+        const int count = hard ? h.M + 1 : 2 * ni;
+        if (!cluster) {
+            if (!meet()) return;
+            ss_slices(a, count, raw + SS_TABLE_BYTES);
+        }
         arrive();
         if (blockIdx.x == 0) {
             int* pos = reinterpret_cast<int*>(raw + SS_TABLE_BYTES);          // [ncand][H + 2] in the histogram's room (the slices are stored)
             if (!hard) ss_places<H>(s_plan, ncand, ni, s_edge, s_cell, pos);
-            if (!qp_grid::wait(a.bar, (waits + 1) * G + a.bar_extra, a.spin_limit, a.status, &s_ok)) return;
+            if (!wait((waits + 1) * G)) return;
+            if (cluster) ss_all_slices(a, count);
             if (!hard) {
                 ss_finish<H>(a, s_plan, s_st, ncand, ni, s_cell, pos, s_cand, s_valid, s_curve, s_red, reinterpret_cast<double*>(raw));
             } else {
@@ -821,16 +861,21 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArg
                 return;
             }
             arrive();
-        } else if (!a.packed) {
-            return;
+        } else {
+            if (cluster) {
+                wait(0);
+                if (a.packed) arrive();
+            }
+            if (!a.packed) return;
         }
         if constexpr (STATS) {                                // the sender: everybody packs, from the tensor's end
-            if (!qp_grid::wait(a.bar, (waits + 1) * G + 1 + a.bar_extra, a.spin_limit, a.status, &s_ok)) return;
+            if (!wait((waits + 1) * G + 1)) return;
             const float lo = __ldcg(&a.qp_out->lo), hi = __ldcg(&a.qp_out->hi), inv = __ldcg(&a.qp_out->inv_scale);
             uint32_t* sw = reinterpret_cast<uint32_t*>(raw) + (threadIdx.x >> 5) * 256;
             const uint64_t tiles = (a.n + QP_TILE - 1) / QP_TILE;
             for (uint64_t it = first; it < tiles; it += step)
                 qp_pack_tile<BITS, T, true>(x, a.n, tiles - 1 - it, lane, lo, hi, inv, a.packed, a.nwords, sw);
+            if (cluster) return;
             __syncthreads();
             if (threadIdx.x == 0 && atomicInc(a.bar + 1, G - 1) == G - 1) atomicExch(a.bar, 0u);   // the last block out
         }
@@ -867,6 +912,11 @@ bool ss_usable(qp_ctx* ctx)
                      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SS_DYN_BYTES) == cudaSuccess &&
                      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, SS_THREADS, SS_DYN_BYTES) == cudaSuccess && per_sm >= 1;
             }
+        ctx->ss_cluster = ok;
+        for (int bits = 0; ok && bits <= 4; ++bits)
+            for (int v = 0; v < (bits ? 4 : 2); ++v)
+                ctx->ss_cluster &= qp_cluster_fits((v & 1) ? ss_kernel<unsigned short>(v < 2, bits) : ss_kernel<float>(v < 2, bits),
+                                                   SS_THREADS, SS_DYN_BYTES);
         if (!ok) cudaGetLastError();
         ctx->ss_ok = ok ? 1 : 0;
     }
@@ -934,10 +984,12 @@ int32_t qp_launch_stats_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t
     a.flush_tiles = ((8191 - 64) << a.rep_shift) / (SS_WARPS * ss_ctile(hh));
     if (a.flush_tiles < 1) return qp_fail(ctx, QP_ERR_INVALID_ARG, "statistics and search: tables too small");
     const uint64_t want = (a.ntiles + SS_WARPS - 1) / SS_WARPS;
-    const unsigned G = (unsigned)(want < (uint64_t)ctx->sm_count ? want : (uint64_t)ctx->sm_count);
+    a.cluster = qp_cluster_wanted(ctx, ctx->ss_cluster, n);
+    const unsigned most = a.cluster ? QP_CLUSTER_BLOCKS : (unsigned)ctx->sm_count;
+    const unsigned G = (unsigned)(want < most ? want : most);
     void* k = dtype == QP_F32 ? ss_kernel<float>(st_in == nullptr, bits) : ss_kernel<unsigned short>(st_in == nullptr, bits);
     void* params[] = {&a};
-    if (cudaLaunchCooperativeKernel(k, dim3(G), dim3(SS_THREADS), params, SS_DYN_BYTES, s) != cudaSuccess)
+    if (qp_launch_together(k, G, SS_THREADS, params, SS_DYN_BYTES, a.cluster, s) != cudaSuccess)
         return qp_check_launch(ctx, "statistics and search (cooperative launch)");
     ctx->launches += 1;
     return qp_check_launch(ctx, "statistics and search");

@@ -90,3 +90,51 @@ struct SsStream {
 };
 template <typename T, int ELEMS> using SsTiles = SsStream<T, ELEMS / 32 / qp_span<T>::EPV>;
 
+
+// ---- launches whose blocks wait for one another: a cooperative grid, or one thread-block cluster
+constexpr unsigned QP_CLUSTER_BLOCKS = 16;        // the largest cluster (above 8: by attribute, where the device has the SMs)
+
+// One cluster while every warp of it has at most one tile; the search with 2 bits at 2^17, 2^18 and 3 * 2^17 elements takes 23,
+// 24.7 and 28.8 us in a cluster, 26.7, 28.1 and 28.8 in a grid, at 2^20 35 and 28.8.
+constexpr uint64_t QP_CLUSTER_MAX_N = (uint64_t)QP_CLUSTER_BLOCKS * SS_WARPS * SS_TILE;
+
+inline cudaLaunchConfig_t qp_cluster_config(cudaLaunchAttribute* at, unsigned G, unsigned threads, size_t bytes, cudaStream_t s)
+{
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = G;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(G);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// whether the device can hold `kernel` as a cluster of every size up to QP_CLUSTER_BLOCKS (the largest one tells)
+inline int qp_cluster_fits(const void* kernel, unsigned threads, size_t bytes)
+{
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = qp_cluster_config(&at, QP_CLUSTER_BLOCKS, threads, bytes, nullptr);
+    int clusters = 0;
+    const bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters >= 1;
+    if (!ok) cudaGetLastError();
+    return ok ? 1 : 0;
+}
+
+// (the tests that make a barrier's wait run out have the counting barrier)
+inline int qp_cluster_wanted(const qp_ctx* ctx, int fits, uint64_t n)
+{
+    return fits && n <= QP_CLUSTER_MAX_N && ctx->bar_extra == 0;
+}
+
+inline cudaError_t qp_launch_together(void* kernel, unsigned G, unsigned threads, void** params, size_t bytes, int cluster, cudaStream_t s)
+{
+    if (!cluster) return cudaLaunchCooperativeKernel(kernel, dim3(G), dim3(threads), params, bytes, s);
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = qp_cluster_config(&at, G, threads, bytes, s);
+    return cudaLaunchKernelExC(&cfg, kernel, params);
+}

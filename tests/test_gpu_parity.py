@@ -948,10 +948,44 @@ def test_search_forms_agree_beyond_two_waves(ctx, n):
     assert ctx.qp_get_status() == 0
 
 
+# the sender's search in the streaming launch: as one cluster of blocks (up to 2^18 elements: 1, 3, 15 and 16 blocks of 16 tiles)
+# and as a grid, at the ends of the ranges that it serves; the winner is a candidate of the separate search's
+@pytest.mark.parametrize("bits,n,bf16", [(1, 1 << 15, False), (2, 1 << 16, True), (2, 33 * 1024 + 5, False), (2, 240 * 1024 + 1023, False),
+                                         (3, 3 << 16, False), (1, 1 << 18, True), (3, (1 << 18) + 1, False), (4, 3 << 17, True),
+                                         (4, 1 << 20, False), (2, 15 << 17, False)])
+@pytest.mark.parametrize("data", ["plain", "offset"])
+def test_sender_search_streaming(ctx, bits, n, bf16, data):
+    from types import SimpleNamespace
+    x = si.vit_activation((1, n, 1), 40 + bits, outlier_frac=0.001).reshape(-1)
+    if data == "offset":                                 # clip ends coarse against the step: exact thresholds
+        x = (np.float32(4096.0) + x).astype(np.float32)
+    d = dev(x)
+    if bf16:
+        h = si.to_bf16_bits(x)
+        d, x = torch.from_numpy(h.view(np.int16)).cuda().view(torch.bfloat16), oracle.widen_bf16(h)
+    st = torch.zeros(80, dtype=torch.uint8, device="cuda")
+    before = ctx.qp_launch_count()
+    packed, q = ctx.qp_sender_device(d, bits, True, out_stats=st)
+    assert ctx.qp_launch_count() - before == 1
+    curve = np.array(ctx.qp_dsaciq_curve(100))
+    st_o = oracle.stats(x)
+    check_stats(ctx.read_stats(st), st_o)
+    _, res_o, _, curve_o = oracle.ds_search(x, st_o, bits, 0, 100, 100)
+    got = ctx.read_qparams(q)
+    cand = ctx.qp_dsaciq_candidates(100)
+    hits = [k for k in range(101) if np.isfinite(curve[k]) and (cand[k].lo, cand[k].hi) == (got.lo, got.hi)]
+    assert hits
+    res = SimpleNamespace(k_star=hits[0], alpha_star=oracle_candidate_ends(st_o, res_o, bits, 0, 100, hits[0])[2])  # (its ends are)
+    check_candidates_and_pick(x, st_o, res_o, curve_o, res, curve, cand, bits, 0, 100, exact_steps=None if data == "offset" else (0, 37, 100))
+    assert torch.equal(packed, ctx.qp_quantize_pack(d, bits, q))
+    ctx.qp_get_status()
+
+
 # statistics about a pilot centre (96 MB and more: 25165824 fp32 elements) and in two streaming passes (below), tiles of 1024
 # elements, 16 warps a block; with the closed-form sender from 2^21 + 2^19 elements.  Data that the one pass cannot
 # finish ("mass", "two_levels") or finishes at once, and elements that its sums must leave out.
-@pytest.mark.parametrize("n,data,bf16", [(8 * 1024, "plain", False), (8 * 1024 + 1, "nonfinite", True), (16 * 1024 + 1023, "plain", False),
+@pytest.mark.parametrize("n,data,bf16", [(8 * 1024, "plain", False), ((1 << 15) + 1, "plain", True), (1 << 18, "outliers", False),
+                                         ((1 << 18) - 1025, "nonfinite", False), (8 * 1024 + 1, "nonfinite", True), (16 * 1024 + 1023, "plain", False),
                                          (148 * 16 * 1024 + 7, "nonfinite", False), ((5 << 19) + 1, "offset", False),
                                          ((5 << 19) + 1031, "plain", True), ((96 << 18) - 1, "plain", False),
                                          (96 << 18, "plain", False), ((96 << 18) + 1025, "nonfinite", False),
@@ -982,7 +1016,7 @@ def test_stats_streaming(ctx, n, data, bf16):
     check_stats(st, st_o)
     assert abs(st.mad - st_o.mad) <= 3e-7 * st_o.mad
     assert bytes(st) == bytes(ctx.read_stats(ctx.qp_stats(d)))
-    if n > (5 << 19):
+    if n > (5 << 19) or n <= (1 << 18):
         before = ctx.qp_launch_count()
         st_s = torch.zeros(80, dtype=torch.uint8, device="cuda")
         packed, q = ctx.qp_sender_device(d, 6, False, out_stats=st_s)
