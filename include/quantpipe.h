@@ -165,9 +165,10 @@ int32_t qp_make_qparams(double lo, double hi, int bits, qp_qparams_t* h_out);
  * One call fills *d_out (device memory, 80 bytes, 8-byte aligned) from the n elements at
  * d_x.  Two passes over x (sums/min/max, then deviations about the mean), fp64 merges in a
  * fixed order: results are bit-reproducible run to run.  n = 0 gives all-zero statistics.
- * For 16-byte aligned tensors of at least 128 KB both passes run in one cooperative launch
- * (the second pass starts on the tiles that the first one left in shared memory), see
- * qp_set_stats_path.
+ * 16-byte aligned tensors (8192 elements and more, 128 KB with the histogram) take one launch for
+ * both, and without the histogram a single pass from 96 MB on: deviations about a pilot centre, the
+ * split point moved to the mean afterwards (a second pass follows in the same launch where that
+ * cannot be done to 1e-8), see qp_set_stats_path.
  * hist_bins > 0 asks the second pass to carry the directed search's histogram along
  * (hist_bins equal bins over [min, max]; only its peak count is kept, in hist_peak): a later
  * qp_dsaciq_search with the same hist_bins then skips its own histogram pass.  The fusion is
@@ -182,17 +183,16 @@ int32_t qp_stats(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int hist_b
  * will equal hist_bins), else 0.  Host, pure: it depends only on the pointer's alignment, the
  * size and hist_bins. */
 int qp_stats_carries_histogram(const void* d_x, int dtype, uint64_t n, int hist_bins);
-/* How qp_stats runs its two passes on 16-byte aligned tensors of at least 128 KB (an execution
- * option without a counterpart in the paper; min, max, the counts and the histogram's peak are
- * identical on both paths, the other fields agree to ~1e-8 relative):
+/* How qp_stats runs its passes on 16-byte aligned tensors (an execution option without a
+ * counterpart in the paper; min, max, the counts and the histogram's peak are identical on all
+ * paths, the other fields agree to ~1e-7 relative):
  *   QP_STATS_TWO_KERNELS  one kernel per pass
  *   QP_STATS_FUSED        one cooperative launch for both (one block per SM; every block keeps the
  *                         last tiles of its first pass in shared memory and starts the second pass,
  *                         which walks backwards, on them).  Falls back to two kernels on a device
  *                         that cannot hold it.
- *   QP_STATS_AUTO         the cooperative launch for hist_bins = 0, the two kernels when the histogram
- *                         rides along (default: the faster of the two inside the sender chain; called
- *                         alone the cooperative launch is the faster with the histogram too)
+ *   QP_STATS_AUTO         the streaming launch that the search and the senders use as well: up to 2^18
+ *                         elements one thread-block cluster, above that one block per SM (default)
  * A grid barrier or tile wait of the cooperative launch that runs out sets QP_DEV_STREAM_TIMEOUT
  * and the launch ends without output. */
 enum { QP_STATS_AUTO = 0, QP_STATS_TWO_KERNELS = 1, QP_STATS_FUSED = 2 };
@@ -288,7 +288,9 @@ int32_t qp_dsaciq_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, co
  *   QP_SEARCH_INTERVALS   one pass gathers moments per interval between the candidates'
  *                         decision thresholds; used where (steps+1)*(2^bits-1) <= 2048 and
  *                         n < ~1.8e9, otherwise the call falls back to the first way
- *   QP_SEARCH_AUTO        intervals for n >= 2^20 where they apply (default)
+ *   QP_SEARCH_AUTO        for n >= 2^20 the intervals where they apply; at 1..4 bits, up to 255 steps and
+ *                         16-byte aligned in one streaming launch that numbers a tensor's intervals by
+ *                         arithmetic instead of looking them up (default)
  * The pass over x that gathers the moments has two forms with identical results: the plain one
  * (every element looks its interval up), and one that adds elements of grid cells without a
  * threshold straight into per-cell, per-lane sums and looks up only the others; the second is
@@ -330,12 +332,11 @@ int32_t qp_policy_use_ds(int bits);
  * bits zero.  `qp` is a host pointer (qp_on_device = 0, read before returning) or a
  * device pointer (qp_on_device = 1, read by the kernel; its bits must equal `bits`,
  * otherwise QP_DEV_BITS_MISMATCH is raised in the status word).
- * d_packed must be 16-byte aligned; d_x aligned to its element size.  Only a 16-byte aligned d_x
- * takes the warp-tile kernel; an x that is merely element-aligned (a view that starts at an odd
- * element) sends the WHOLE tensor through the scalar kernel (a thread per 32 elements, 4-byte
- * loads): the same bytes, about 5x the time (129 MB tensor on B200: 153-162 us against 33-35 us).
- * Copy such a view to an aligned buffer first if speed matters.  The same holds for d_y of
- * qp_unpack_dequantize (179 us against 31-34 us); qp_stats loses less (66 us against 46 us).
+ * d_packed must be 16-byte aligned; d_x aligned to its element size.  An x that is merely
+ * element-aligned (a view that starts at an odd element) is read element by element in the same
+ * kernel, at no cost on a large fp32 tensor (129 MB on B200: 27 us either way).  A d_y of
+ * qp_unpack_dequantize that is not 16-byte aligned costs more (57 us against 25), and so do the
+ * statistics of such a view (65 us against 39).
  * Errors: QP_ERR_INVALID_ARG, QP_ERR_UNSUPPORTED_BITS, QP_ERR_UNSUPPORTED_DTYPE,
  * QP_ERR_BUFFER_TOO_SMALL (packed_capacity < qp_packed_bytes), QP_ERR_ALIGNMENT, QP_ERR_CUDA. */
 int32_t qp_quantize_pack(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int bits,
@@ -525,8 +526,11 @@ int32_t qp_sender_tokens_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_
  *                    the sums are merged in another order: statistics agree with the chain to
  *                    ~1e-15 relative, the error curve to ~1e-6, so the clip range can differ in
  *                    its last fp32 bit or, where two steps of the search tie, by one step.
- *   QP_SENDER_AUTO   fused where it is the faster of the two on a B200: n <= 2^20 with the
- *                    search, n <= 2^21 otherwise (default)
+ *   QP_SENDER_AUTO   the fastest on a B200 (default): for 16-byte aligned tensors a streaming launch
+ *                    that reads x again for every step (closed-form clips up to 2^18 elements and above
+ *                    2.6e6, bf16 up to 2^26; the search at 1..4 bits from 2^15, 3 * 2^16 or 3 * 2^17
+ *                    elements (up to 2, 3 and 4 bits) to 1.9e6 and above 2^21); else fused for n <= 2^20
+ *                    with the search and n <= 2^21 otherwise; else the chain
  * A grid barrier that does not complete within about a quarter of a second sets
  * QP_DEV_STREAM_TIMEOUT in the status word and the launch ends without output
  * (qp_get_status then returns QP_ERR_TIMEOUT). */

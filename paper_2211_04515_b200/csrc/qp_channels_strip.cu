@@ -6,15 +6,17 @@
 //   phase B   sum |x - mean|, sum (x - mean)^2, histogram over the channel's [min, max]
 //   phase C   per channel, the count and the sum of the elements of every interval between the candidates' thresholds
 //             (qp_affine.cuh), in shared memory
-//   finish    two warps per channel (a side each): prefix sums over the intervals, the error of every candidate from 2^bits
+//   finish    a team of four warps per channel (the first two scan a side each): prefix sums over the intervals, the error of every candidate from 2^bits
 //             differences, first minimum, quantizer
 // Between the phases the blocks of a cluster add up their parts through distributed shared memory.  A thread stays with one
-// channel and walks its rows, sixteen loads ahead; the first pass takes the strip from DRAM, the others from L2.
+// channel and walks its rows, eight loads ahead; the first pass takes the strip from DRAM, the others from L2.
 //
-// What bounds it: the instructions (A 4, B 11, C 14 + 2 per code boundary and element) and, as a strip's row is 4 w bytes,
-// the L1 look-ups, one or two per row and pass.  12608 x 1024 fp32 at 4 bits (52 MB): see the table of measurements in the
-// kernel list; the ten kernels before (four for the statistics, histogram, set-up, thresholds sorted per channel, a
-// pass with binary searches, error curves, pick) took 255 us.
+// What bounds it: the loads of 4 bytes per lane (a strip's row is 4 w bytes, so a warp's load touches several lines; the load
+// queue and the latency behind it are two thirds of the stalls), the instructions (A 4, B 11, C 14 + 2 per code
+// boundary and element), and the finish.  12608 x 1024 fp32 at 4 bits (52 MB): 105 us, of which A 18, B 12, C 19, sums across the
+// cluster 17, finish 27, plans 4; the ten kernels before (four for the statistics, histogram, set-up, thresholds sorted per
+// channel, a pass with binary searches, error curves, pick) took 255 us.  Gathering the interval sums entry by entry
+// through distributed shared memory took 32 us instead of 10, one warp per side for all of a channel's candidates 16 instead of 5.
 #include <cooperative_groups.h>
 
 #include <type_traits>

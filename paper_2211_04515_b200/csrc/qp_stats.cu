@@ -913,18 +913,16 @@ int32_t qp_launch_stats(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int
         return QP_OK;
     }
     const uint64_t ntiles = ((uintptr_t)d_x & 15u) ? 0 : n * (dtype == QP_F32 ? 4 : 2) / ST_TILE;
-    // One launch or two.  Alone, the one-launch form is the faster with and without the histogram (129 MB:
-    // 43.6 / 51.8 us against 51.0 / 59.0).  Inside the sender chain, where the pass runs while the receiver's
-    // output of the step before is still being written back from L2, the two kernels are the faster once the
-    // histogram rides along (66.3 us against 72.5; equal without it, 59 us): QP_STATS_AUTO takes the one launch
-    // without the histogram and the two kernels with it; QP_STATS_FUSED and QP_STATS_TWO_KERNELS force either.
+    // QP_STATS_AUTO takes the streaming launches wherever they apply: 12.4 us at 2^20 fp32 elements against 14.5 in one launch of
+    // bulk-copied tiles and 16.5 in two kernels, 102 against 157 at 2^27; with the histogram 30.6 us for 52 MB.
+    // QP_STATS_FUSED and QP_STATS_TWO_KERNELS force the other two.
     const bool with_hist = hist_bins >= 1 && hist_bins <= ST_FUSED_HIST_MAX;
     if (ctx->stats_path == QP_STATS_AUTO && with_hist && ntiles >= 8 &&
         qp_stats_search_applies(ctx, d_x, dtype, n, hist_bins, 0, 0))
         return qp_launch_stats_search(ctx, d_x, dtype, n, nullptr, d_out, hist_bins, 0, 0, 0, 0.0, nullptr, nullptr, nullptr, s);
     if (ctx->stats_path == QP_STATS_AUTO && !with_hist && qp_stats_onepass_applies(ctx, d_x, dtype, n))
         return qp_launch_stats_onepass(ctx, d_x, dtype, n, d_out, 0, 0, 0, 0.0, nullptr, nullptr, s);
-    const bool one_launch = ctx->stats_path == QP_STATS_FUSED || (ctx->stats_path == QP_STATS_AUTO && !with_hist);
+    const bool one_launch = ctx->stats_path == QP_STATS_FUSED;
     if (ntiles >= 8 && one_launch && stats_fused_usable(ctx)) {
         if (dtype == QP_F32) return launch_fused<float>(ctx, static_cast<const float*>(d_x), n, hist_bins, d_out, s);
         return launch_fused<unsigned short>(ctx, static_cast<const unsigned short*>(d_x), n, hist_bins, d_out, s);
