@@ -926,6 +926,8 @@ extern "C" int32_t qp_receiver_host(qp_ctx* ctx, const void* h_packed, uint64_t 
     {
         qp_device_guard guard(ctx->device);
         if (!guard.ok) return qp_fail(ctx, QP_ERR_CUDA, "cannot select device");
+        const int32_t one = qp_launch_unpack_host(ctx, h_packed, n, bits, *h_qp, d_packed_work, d_y_work, h_y, out_dtype, s);
+        if (one != QP_WARN_INFEASIBLE) return one;
         if (need && cudaMemcpyAsync(d_packed_work, h_packed, need, cudaMemcpyHostToDevice, s) != cudaSuccess)
             return qp_check_launch(ctx, "qp_receiver_host (copy in)");
     }

@@ -569,5 +569,7 @@ int32_t qp_launch_aciq_device(qp_ctx* ctx, const qp_stats_t* d_stats, int bits, 
                               qp_qparams_t* d_qp_out, cudaStream_t s);
 int32_t qp_launch_pack(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int bits, const qp_qparams_t* d_qp,
                        qp_qparams_t h_qp, void* d_packed, cudaStream_t s);
+int32_t qp_launch_unpack_host(qp_ctx* ctx, const void* h_packed, uint64_t n, int bits, const qp_qparams_t& h_qp, void* d_packed,
+                              void* d_y, void* h_y, int out_dtype, cudaStream_t s);
 int32_t qp_launch_unpack(qp_ctx* ctx, const void* d_packed, uint64_t n, int bits, const qp_qparams_t* d_qp,
                          qp_qparams_t h_qp, void* d_y, int out_dtype, cudaStream_t s);

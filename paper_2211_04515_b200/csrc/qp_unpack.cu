@@ -9,6 +9,11 @@
 // through a chunk-swizzled 1 KB staging buffer so that lane l then expands quad j*32+l and
 // stores 16-byte vectors that are fully coalesced across the warp.  The last, partial tile is a guarded
 // iteration of the same loop, and an output that is not aligned takes element stores: one launch.
+//
+// HOST: the receiver on host buffers.  The kernel reads the packed words from page-locked memory and writes the elements to
+// the work buffer and to page-locked memory, so both directions of the link are busy at once and the two copies around the
+// kernel, 4 us each and in series with it, are gone.  What bounds it: the link, 49 GB/s of stores (a copy engine's 55).  One image
+// at 8 bits: 19 us against 35 (bf16 14.5 / 26), 1.2 M elements 111 / 126 (bf16 65 / 84), 4.2 M 389 / 391 (230 / 246).
 #include "qp_internal.cuh"
 
 namespace {
@@ -54,11 +59,12 @@ __device__ __forceinline__ void store_one(unsigned short* y, uint64_t i, float v
 
 // ntiles counts the last, partial tile too: its words are read up to nwords and its elements written up
 // to n.  VEC: y is aligned for 4-element stores; otherwise the elements are stored one by one.
-template <int BITS, typename TO, bool VEC>
+template <int BITS, typename TO, bool VEC, bool HOST = false>
 __global__ void __launch_bounds__(QP_THREADS) unpack_kernel(const uint32_t* __restrict__ in, uint64_t n, uint64_t nwords,
                                                             uint64_t ntiles, const qp_qparams_t* __restrict__ d_qp,
                                                             qp_qparams_t h_qp, TO* __restrict__ y,
-                                                            unsigned* __restrict__ status)
+                                                            unsigned* __restrict__ status, uint32_t* __restrict__ work = nullptr,
+                                                            TO* __restrict__ y_host = nullptr)
 {
     __shared__ __align__(16) uint32_t stage[WARPS][256];
     const DQ q = load_dq(d_qp, h_qp, BITS, status);
@@ -72,6 +78,7 @@ __global__ void __launch_bounds__(QP_THREADS) unpack_kernel(const uint32_t* __re
 
     for (uint64_t tile = (uint64_t)blockIdx.x * warps + warp; tile < ntiles; tile += wstride) {
         const uint32_t* it = in + tile * (32 * BITS);
+        uint32_t* wk = HOST ? work + tile * (32 * BITS) : nullptr;
         const bool full = (tile + 1) * TILE <= n;                 // warp-uniform
         uint32_t w[BITS];
         if (full && BITS == 8) {
@@ -79,16 +86,26 @@ __global__ void __launch_bounds__(QP_THREADS) unpack_kernel(const uint32_t* __re
             const uint4 b = __ldg(reinterpret_cast<const uint4*>(it + lane * 8) + 1);
             w[0] = a.x; w[1 % BITS] = a.y; w[2 % BITS] = a.z; w[3 % BITS] = a.w;
             w[4 % BITS] = b.x; w[5 % BITS] = b.y; w[6 % BITS] = b.z; w[7 % BITS] = b.w;
+            if constexpr (HOST) {
+                *reinterpret_cast<uint4*>(wk + lane * 8) = a;
+                *(reinterpret_cast<uint4*>(wk + lane * 8) + 1) = b;
+            }
         } else if (full && BITS == 4) {
             const uint4 a = __ldg(reinterpret_cast<const uint4*>(it + lane * 4));
             w[0] = a.x; w[1 % BITS] = a.y; w[2 % BITS] = a.z; w[3 % BITS] = a.w;
+            if constexpr (HOST) *reinterpret_cast<uint4*>(wk + lane * 4) = a;
         } else if (full && BITS == 2) {
             const uint2 a = __ldg(reinterpret_cast<const uint2*>(it + lane * 2));
             w[0] = a.x; w[1 % BITS] = a.y;
+            if constexpr (HOST) *reinterpret_cast<uint2*>(wk + lane * 2) = a;
         } else {
             const int room = (int)min((uint64_t)(32 * BITS), nwords - tile * (32 * BITS));
 #pragma unroll
-            for (int m = 0; m < BITS; ++m) sw[m * 32 + lane] = m * 32 + lane < room ? __ldg(it + m * 32 + lane) : 0u;
+            for (int m = 0; m < BITS; ++m) {
+                const uint32_t v = m * 32 + lane < room ? __ldg(it + m * 32 + lane) : 0u;
+                sw[m * 32 + lane] = v;
+                if (HOST && m * 32 + lane < room) wk[m * 32 + lane] = v;
+            }
             __syncwarp();
 #pragma unroll
             for (int m = 0; m < BITS; ++m) w[m] = sw[lane * BITS + m];
@@ -117,10 +134,14 @@ __global__ void __launch_bounds__(QP_THREADS) unpack_kernel(const uint32_t* __re
             const int k = (j * 32 + lane) * 4;
             if (VEC && (full || k + 4 <= have)) {
                 store_out(y, tile * (TILE / 4) + j * 32 + lane, v);
+                if constexpr (HOST) store_out(y_host, tile * (TILE / 4) + j * 32 + lane, v);
             } else {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if (k + i < have) store_one(y, tile * TILE + k + i, v[i]);
+                    if (k + i < have) {
+                        store_one(y, tile * TILE + k + i, v[i]);
+                        if constexpr (HOST) store_one(y_host, tile * TILE + k + i, v[i]);
+                    }
             }
         }
         __syncwarp();
@@ -190,7 +211,56 @@ int32_t unpack_typed(qp_ctx* ctx, const void* d_packed, uint64_t n, int bits, co
     return qp_check_launch(ctx, "qp_unpack_dequantize");
 }
 
+template <typename TO>
+int32_t unpack_host_typed(qp_ctx* ctx, const uint32_t* in, uint64_t n, int bits, const qp_qparams_t& h_qp, uint32_t* work, TO* y,
+                          TO* y_host, cudaStream_t s)
+{
+    const uint64_t nwords = qp_packed_bytes(n, bits) / 4, ntiles = (n + TILE - 1) / TILE;
+    const qp_grid_shape g = qp_tile_grid(ctx, ntiles, WARPS);
+    ctx->launches += 1;
+#define QP_UNPACK_CASE(B)                                                                                                              case B:                                                                                                                                unpack_kernel<B, TO, true, true><<<g.blocks, g.threads, 0, s>>>(in, n, nwords, ntiles, nullptr, h_qp, y, ctx->d_status, work,                                                                         y_host);                                                           break;
+    switch (bits) {
+        QP_UNPACK_CASE(1) QP_UNPACK_CASE(2) QP_UNPACK_CASE(3) QP_UNPACK_CASE(4)
+        QP_UNPACK_CASE(5) QP_UNPACK_CASE(6) QP_UNPACK_CASE(7) QP_UNPACK_CASE(8)
+    }
+#undef QP_UNPACK_CASE
+    return qp_check_launch(ctx, "qp_receiver_host");
+}
+
+// the device's address of [p, p + bytes) in page-locked host memory, or NULL
+void* mapped(const void* p, uint64_t bytes)
+{
+    cudaPointerAttributes a, b;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
+        cudaPointerGetAttributes(&b, static_cast<const char*>(p) + bytes - 1) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    const bool ok = a.type == cudaMemoryTypeHost && b.type == cudaMemoryTypeHost && a.devicePointer && b.devicePointer &&
+                    static_cast<char*>(b.devicePointer) - static_cast<char*>(a.devicePointer) == (ptrdiff_t)(bytes - 1);
+    return ok ? a.devicePointer : nullptr;
+}
+
 }  // namespace
+
+// The receiver on page-locked, 16-byte aligned buffers in one launch; QP_WARN_INFEASIBLE where it does not apply: copy engines
+// move more than 16 MB of elements as fast or faster (their rate is the better one, and the copies' latencies no longer show).
+int32_t qp_launch_unpack_host(qp_ctx* ctx, const void* h_packed, uint64_t n, int bits, const qp_qparams_t& h_qp, void* d_packed,
+                              void* d_y, void* h_y, int out_dtype, cudaStream_t s)
+{
+    const uint64_t esz = out_dtype == QP_F32 ? 4 : 2;
+    if (n == 0 || bits > 8 || h_qp.bits != bits || n * esz > 16ull << 20 ||
+        (((uintptr_t)h_packed | (uintptr_t)d_packed | (uintptr_t)d_y | (uintptr_t)h_y) & 15u))
+        return QP_WARN_INFEASIBLE;
+    const void* in = mapped(h_packed, qp_packed_bytes(n, bits));
+    void* out = in ? mapped(h_y, n * esz) : nullptr;
+    if (!out) return QP_WARN_INFEASIBLE;
+    if (out_dtype == QP_F32)
+        return unpack_host_typed<float>(ctx, static_cast<const uint32_t*>(in), n, bits, h_qp, static_cast<uint32_t*>(d_packed),
+                                        static_cast<float*>(d_y), static_cast<float*>(out), s);
+    return unpack_host_typed<unsigned short>(ctx, static_cast<const uint32_t*>(in), n, bits, h_qp, static_cast<uint32_t*>(d_packed),
+                                             static_cast<unsigned short*>(d_y), static_cast<unsigned short*>(out), s);
+}
 
 int32_t qp_launch_unpack(qp_ctx* ctx, const void* d_packed, uint64_t n, int bits, const qp_qparams_t* d_qp,
                          qp_qparams_t h_qp, void* d_y, int out_dtype, cudaStream_t s)

@@ -828,6 +828,27 @@ def test_sender_and_receiver_host_buffers(ctx):
         assert np.max(np.abs(h_y.numpy().astype(np.float64) - y_o.astype(np.float64))) <= 1e-6
 
 
+# page-locked buffers: one kernel that reads and writes host memory, partial and whole tiles of 1024; pageable or unaligned ones,
+# 16 bits and more than 16 MB of elements: copies around the ordinary kernel
+@pytest.mark.parametrize("n", [1, 31, 1023, 1024, 4101, 8 * 1024 * 148 * 2 + 77, (4 << 20) + 1])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_receiver_host_buffers_edges(ctx, n, dtype):
+    x = torch.from_numpy(si.vit_activation((1, n, 1), 5).reshape(-1)).cuda()
+    for bits in (1, 2, 3, 4, 5, 6, 7, 8, 16) if n < 10000 else (3, 8):
+        packed, q = ctx.qp_sender_device(x, bits, False)
+        packed = packed.view(torch.uint8).reshape(-1)
+        h_qp = ctx.read_qparams(q)
+        want = ctx.qp_unpack_dequantize(packed, n, bits, h_qp, out_dtype=dtype)
+        for off, pinned in ((0, True), (1, True), (0, False)):
+            h_p = torch.empty(packed.numel(), dtype=torch.uint8, pin_memory=pinned).copy_(packed)
+            h_y = torch.full((n + 9,), 7.0, dtype=dtype, pin_memory=pinned)
+            d_p, d_y = torch.full_like(packed, 0xA5), torch.full_like(want, -1.0)
+            ctx.qp_receiver_host(h_p, n, bits, h_qp, d_p, d_y, h_y[off:off + n])
+            torch.cuda.synchronize()
+            assert torch.equal(d_p, packed) and torch.equal(d_y, want) and torch.equal(h_y[off:off + n], want.cpu())
+            assert (h_y[:off] == 7.0).all() and (h_y[off + n:] == 7.0).all()
+
+
 # ----------------------------------------------------- full-size configurations
 
 def full_pack_unpack(ctx, x, d, qp_o, bits, label=""):
