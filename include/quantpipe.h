@@ -288,9 +288,9 @@ int32_t qp_dsaciq_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, co
  *   QP_SEARCH_INTERVALS   one pass gathers moments per interval between the candidates'
  *                         decision thresholds; used where (steps+1)*(2^bits-1) <= 2048 and
  *                         n < ~1.8e9, otherwise the call falls back to the first way
- *   QP_SEARCH_AUTO        for n >= 2^20 the intervals where they apply; at 1..4 bits, up to 255 steps and
- *                         16-byte aligned in one streaming launch that numbers a tensor's intervals by
- *                         arithmetic instead of looking them up (default)
+ *   QP_SEARCH_AUTO        at 1..4 bits, up to 255 steps, 16-byte aligned and n >= 8192 (4 bits: 32768) the
+ *                         intervals in one streaming launch that numbers them by arithmetic instead of
+ *                         looking them up; otherwise for n >= 2^20 the intervals where they apply (default)
  * The pass over x that gathers the moments has two forms with identical results: the plain one
  * (every element looks its interval up), and one that adds elements of grid cells without a
  * threshold straight into per-cell, per-lane sums and looks up only the others; the second is

@@ -308,8 +308,7 @@ int32_t qp_launch_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, co
                          int bmode, int steps, int hist_bins, double F, qp_ds_result_t* d_out, qp_qparams_t* d_qp_out,
                          cudaStream_t s)
 {
-    if (ctx->search_path == QP_SEARCH_AUTO && n >= (1ull << 20) &&
-        qp_stats_search_applies(ctx, d_x, dtype, n, hist_bins, bits, steps))
+    if (ctx->search_path == QP_SEARCH_AUTO && qp_stats_search_applies(ctx, d_x, dtype, n, hist_bins, bits, steps))
         return qp_launch_stats_search(ctx, d_x, dtype, n, d_stats, nullptr, hist_bins, bits, bmode, steps, F, d_out, d_qp_out,
                                       nullptr, s);
     if (dtype == QP_F32)

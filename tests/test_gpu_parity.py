@@ -1002,6 +1002,21 @@ def test_sender_search_streaming(ctx, bits, n, bf16, data):
     ctx.qp_get_status()
 
 
+# the separate search in that launch, from its smallest tensor (8 tiles) to the last cluster and the first grid
+@pytest.mark.parametrize("bits", [1, 2, 3, 4])
+@pytest.mark.parametrize("n", [8 * 1024, 16 * 1024 + 1, (1 << 18) - 3, 1 << 18, (1 << 18) + 1])
+def test_search_streaming_small(ctx, bits, n):
+    x = si.vit_activation((1, n, 1), 60 + bits, outlier_frac=0.001).reshape(-1)
+    before = ctx.qp_launch_count()
+    d = dev(x)
+    d_stats = ctx.qp_stats(d, hist_bins=100)
+    at = ctx.qp_launch_count()
+    ctx.qp_dsaciq_search(d, d_stats, bits, 0, 100, 100)
+    assert at > before
+    assert bits == 4 and n < 32768 or ctx.qp_launch_count() - at <= 2  # the histogram where the statistics do not carry it
+    check_search(ctx, x, d, bits, exact_steps=None if n < 1 << 17 else (0, 50, 100))
+
+
 # statistics about a pilot centre (96 MB and more: 25165824 fp32 elements) and in two streaming passes (below), tiles of 1024
 # elements, 16 warps a block; with the closed-form sender from 2^21 + 2^19 elements.  Data that the one pass cannot
 # finish ("mass", "two_levels") or finishes at once, and elements that its sums must leave out.
