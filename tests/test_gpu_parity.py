@@ -847,6 +847,7 @@ def test_receiver_host_buffers_edges(ctx, n, dtype):
             torch.cuda.synchronize()
             assert torch.equal(d_p, packed) and torch.equal(d_y, want) and torch.equal(h_y[off:off + n], want.cpu())
             assert (h_y[:off] == 7.0).all() and (h_y[off + n:] == 7.0).all()
+    ctx.qp_get_status()                                  # (one element: degenerate)
 
 
 # ----------------------------------------------------- full-size configurations
