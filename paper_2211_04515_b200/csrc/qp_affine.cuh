@@ -22,6 +22,12 @@ constexpr unsigned SS_ONE = 0x4B000000u;          // bits of 2^23: an integer si
 constexpr float SS_MAGIC = 8388608.0f;
 constexpr int SS_SUMS_AT = 100 * 1024;            // bytes from an interval's count to its sum in shared memory
 
+// whether (x - min) * inv_w is a number for every x of [min, max]
+__device__ __forceinline__ bool ss_range_fits(const qp_stats_t& st, float inv_w)
+{
+    return st.max - st.min <= 3.4028234663852886e38 && inv_w < __int_as_float(0x7F800000);
+}
+
 template <int HH>
 struct SsPlan {
     float m;                                                  // fp32 mean; y = x - m

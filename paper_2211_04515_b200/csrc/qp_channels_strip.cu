@@ -161,7 +161,8 @@ struct CtDeviations {
             below += __float_as_uint(y) >> 31;
         }
         if (HIST) {                                // bin = floor((x - min) * inv_w), each operation rounded; x = max may give nb
-            const float pos = __fmul_rn(__fsub_rn(v, mn), inv_w);
+            float pos = __fmul_rn(__fsub_rn(v, mn), inv_w);
+            if (GUARD) pos = fminf(fmaxf(pos, 0.f), (float)nb);       // (as the per-tensor kernel)
             const unsigned b = QP_CK(__float_as_uint(__fadd_rd(pos, SS_MAGIC)) - SS_ONE, nb + 1) + SS_ONE;
             asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(b * 4u + base) : "memory");
         }
@@ -299,7 +300,9 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
     } else {
         if ((int)threadIdx.x < nch) s_st[threadIdx.x] = a.st_in[c0 + threadIdx.x];
     }
-    __syncthreads();
+    auto inv_w = [&](const qp_stats_t& q) { return SEARCH && q.max > q.min ? (float)((double)a.nb / (q.max - q.min)) : 0.f; };
+    // a channel whose histogram positions may leave its bins (the caller's statistics may be of another tensor)
+    const bool beyond = __syncthreads_or((int)threadIdx.x < nch && SEARCH && (!STATS || !ss_range_fits(s_st[threadIdx.x], inv_w(s_st[threadIdx.x]))));
     bool odd = false;                                         // a channel with non-finite values: uniform over the cluster
     for (int i = 0; i < nch; ++i) odd |= s_st[i].nonfinite != 0;
 
@@ -311,13 +314,13 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
             CtDeviations<STATS, SEARCH, decltype(guard_tag)::value> d;
             d.m = (float)my.mean;
             d.mn = (float)my.min;
-            d.inv_w = SEARCH && my.max > my.min ? (float)((double)a.nb / (my.max - my.min)) : 0.f;
+            d.inv_w = inv_w(my);
             d.nb = (unsigned)a.nb;
             d.base = (unsigned)__cvta_generic_to_shared(bins + slot * (a.nb + 1)) - SS_ONE * 4u;
             ct_column<T>(mine, m, d);
             v3[0] = d.sd; v3[1] = d.sv; v3[2] = (double)d.below;
         };
-        if (odd) pass(std::true_type{}); else pass(std::false_type{});
+        if (odd || beyond) pass(std::true_type{}); else pass(std::false_type{});
         if constexpr (STATS) {
             ct_reduce<0, 0, 0>(v3, red, rl, nl, w);
             if (rl == 0)

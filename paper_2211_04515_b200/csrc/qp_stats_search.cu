@@ -124,7 +124,9 @@ struct SsMoments {
 
 // ---- phase B: deviations and histogram.  bin = floor((x - min) * inv_w) in fp32, each operation rounded on its
 // own; x = max may come out as bin nb, which is counted with the last one.  The floor is taken by adding 2^23
-// rounding down; the bin number then sits in the low bits, and one multiply-add makes the address.
+// rounding down; the bin number then sits in the low bits, and one multiply-add makes the address.  Positions are in
+// [0, nb] where the range of the tensor and its reciprocal are finite in fp32 and the statistics are this tensor's;
+// GUARD (non-finite elements, or not so) clamps them: NaN, of 0 * inf, to bin 0, what overflows to the last one.
 // The deviations are taken about m, the mean in fp32 (one rounding per element, none where x and m are of a size), and
 // moved to the mean itself by the counts of the two sides: sum |x - mean| = sum |x - m| - dm (N_up - N_down).  Their
 // sums are taken in fp64: the search subtracts nearly all of sum y^2 again, and the conversion and fp64 pipes are idle here.
@@ -137,6 +139,7 @@ struct SsDeviations {
     template <bool GUARD>
     __device__ __forceinline__ void count(float pos, float x) const
     {
+        if (GUARD) pos = fminf(fmaxf(pos, 0.f), (float)nb);
         const unsigned addr = (QP_CK(__float_as_uint(__fadd_rd(pos, SS_MAGIC)) - SS_ONE, nb + 1) + SS_ONE) * hist_mul + hist_base;
         if (!GUARD || qp_is_finite(x)) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory");
     }
@@ -170,7 +173,7 @@ struct SsDeviations {
         below += d < 0.0;
         sd[0] += fabs(d);
         sv[0] = fma(d, d, sv[0]);
-        count<false>(__fmul_rn(__fsub_rn(v, mn), inv_w), v);
+        count<true>(__fmul_rn(__fsub_rn(v, mn), inv_w), v);
     }
 };
 template <bool GUARD>
@@ -659,7 +662,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArg
             d.below = 0u;
             d.nm = qp_pack2(-d.m, -d.m);
             d.nmn = qp_pack2(-d.mn, -d.mn);
-            if (guard) {
+            if (guard || !STATS || !ss_range_fits(s_st, d.inv_w)) {
                 SsDeviationsOf<true> f = {d};
                 SsTiles<T, SS_TILE>::template run<true>(x, a.ntiles, first, step, lane, f);
             } else {

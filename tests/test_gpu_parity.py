@@ -1136,6 +1136,41 @@ def test_stats_and_search_in_one_launch(ctx, bits, bmode, steps, nb, n, data, bf
     assert ctx.qp_get_status() & ~(qp.QP_DEV_NONFINITE | qp.QP_DEV_DEGENERATE) == 0
 
 
+# a histogram over a range that overflows fp32 ("wide": x - min does), or whose reciprocal does ("subnormal": 0 * inf among
+# the positions): every element in a bin, the same one as in the kernels that count by an integer conversion
+@pytest.mark.parametrize("n", [70 * 1024 + 5, (1 << 20) + 77])
+@pytest.mark.parametrize("data", ["wide", "subnormal"])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_histogram_of_a_range_beyond_fp32(ctx, n, data, bf16):
+    x = si.flat_iid(n, 33, "laplace") * np.float32(1e20 if data == "wide" else 1e-40)
+    if data == "wide":
+        x[[3, n // 2, n - 1]] = np.array([-3e38, 3e38, 3e38], np.float32)
+    d = dev(x)
+    if bf16:
+        d = d.to(torch.bfloat16)
+    try:
+        ctx.qp_set_stats_path(qp.QP_STATS_TWO_KERNELS)
+        want = ctx.read_stats(ctx.qp_stats(d, hist_bins=100))
+    finally:
+        ctx.qp_set_stats_path(qp.QP_STATS_AUTO)
+    st = ctx.read_stats(ctx.qp_stats(d, hist_bins=100))
+    assert (st.n, st.nonfinite, st.min, st.max) == (n, 0, want.min, want.max)
+    assert st.hist_bins == 100 and st.hist_peak == want.hist_peak > 0
+    d_plain = ctx.qp_stats(d)                            # no histogram in them: the search counts for itself
+    b_r = []
+    for path in (qp.QP_SEARCH_AUTO, qp.QP_SEARCH_CANDIDATES):
+        ctx.qp_set_search_path(path)
+        try:
+            b_r.append(ctx.read_ds_result(ctx.qp_dsaciq_search(d, d_plain, 2)[0]).b_r)
+        finally:
+            ctx.qp_set_search_path(qp.QP_SEARCH_AUTO)
+    assert b_r[0] == b_r[1]
+    whole, packed = guarded(qp.qp_packed_bytes(n, 2))
+    _, d_qp = ctx.qp_sender_device(d, 2, True, out_packed=packed)
+    assert torch.equal(packed, ctx.qp_quantize_pack(d, 2, d_qp)) and canaries_intact(whole, packed.numel())
+    assert ctx.qp_get_status() & qp.QP_DEV_INDEX_RANGE == 0
+
+
 # ------------------------------------------------------------------ graph replay (execution option)
 
 @pytest.mark.parametrize("n_images,path", [(6, qp.QP_SEARCH_CANDIDATES), (40, qp.QP_SEARCH_AUTO)])
@@ -1489,6 +1524,30 @@ def test_search_channels_strips(ctx, channels, rows, bits):
     a, b = _read_array(want_st, qp.Stats, channels), _read_array(d_stats, qp.Stats, channels)
     assert all((u.mean, u.mad, u.var, u.min, u.max) == (v.mean, v.mad, v.var, v.min, v.max) for u, v in zip(a, b))
     ctx.qp_get_status()
+
+
+@pytest.mark.parametrize("bits", [1, 4])
+def test_search_channels_of_a_range_beyond_fp32(ctx, bits):
+    """A channel whose range overflows fp32, and one whose range has no fp32 reciprocal, beside ordinary ones: the strips'
+    histograms against the kernel that counts by an integer conversion."""
+    channels, rows = 6, 3000
+    x = si.vit_activation((1, rows, channels), 171).reshape(rows, channels).copy()
+    x[:, 1] *= np.float32(1e20)
+    x[[5, 77, 2999], 1] = np.array([-3e38, 3e38, 3e38], np.float32)
+    x[:, 4] *= np.float32(1e-41)
+    d = dev(x.reshape(-1))
+    d_stats = ctx.qp_stats_channels(d, channels)
+    res = []
+    for path in (qp.QP_SEARCH_AUTO, qp.QP_SEARCH_CANDIDATES):
+        ctx.qp_set_search_path(path)
+        try:
+            res.append(_read_array(ctx.qp_dsaciq_search_channels(d, channels, d_stats, bits)[0], qp.DSResult, channels))
+        finally:
+            ctx.qp_set_search_path(qp.QP_SEARCH_AUTO)
+    assert [r.b_r for r in res[0]] == [r.b_r for r in res[1]]
+    packed, d_qp = ctx.qp_sender_channels_device(d, channels, bits, qp.QP_CLIP_DSACIQ)
+    assert torch.equal(packed, ctx.qp_quantize_pack_channels(d, channels, bits, d_qp))
+    assert ctx.qp_get_status() & qp.QP_DEV_INDEX_RANGE == 0
 
 
 @pytest.mark.parametrize("rows", [65535, 65536])
