@@ -184,6 +184,15 @@ struct SsDeviationsOf {                                       // the stream's vi
     __device__ __forceinline__ void end() { d.end(); }
 };
 
+// The guarded pass, out of line: inlined, its code moves the compiler's schedule of the ordinary pass (128-image search sender
+// 117.8 us inlined, 113.1 as a call; 64 images at 4 bits 62.9 and 62.1).
+template <typename T>
+__device__ __noinline__ void ss_guarded_deviations(const T* x, uint64_t ntiles, uint64_t first, uint64_t step, int lane, SsDeviations& d)
+{
+    SsDeviationsOf<true> f = {d};
+    SsTiles<T, SS_TILE>::template run<true>(x, ntiles, first, step, lane, f);
+}
+
 template <int HH, bool GUARD>
 struct SsCounter {
     const SsPlan<HH>& p;
@@ -663,8 +672,9 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArg
             d.nm = qp_pack2(-d.m, -d.m);
             d.nmn = qp_pack2(-d.mn, -d.mn);
             if (guard || !STATS || !ss_range_fits(s_st, d.inv_w)) {
-                SsDeviationsOf<true> f = {d};
-                SsTiles<T, SS_TILE>::template run<true>(x, a.ntiles, first, step, lane, f);
+                SsDeviations g = d;
+                ss_guarded_deviations<T>(x, a.ntiles, first, step, lane, g);
+                d.sd[0] = g.sd[0]; d.sd[1] = g.sd[1]; d.sv[0] = g.sv[0]; d.sv[1] = g.sv[1]; d.below = g.below;
             } else {
                 SsDeviationsOf<false> f = {d};
                 SsTiles<T, SS_TILE>::template run<true>(x, a.ntiles, first, step, lane, f);
