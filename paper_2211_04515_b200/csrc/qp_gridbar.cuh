@@ -68,8 +68,24 @@ __device__ __forceinline__ bool wait(const unsigned* bar, unsigned target, unsig
     return *s_ok != 0;
 }
 
+// A block's way out, by one of its threads, when the block will neither arrive nor poll again.  bar[1] counts the blocks out
+// in its low half and those whose wait ran out in its high half, so that the last one learns both from one atomic (a flag of
+// its own cost the launches 1.9 us at their ends).  The block's own arrivals must have been performed: it has polled since, or
+// fences first.
+constexpr unsigned GAVE_UP = 0x10000u;
+__device__ __forceinline__ unsigned count_out(unsigned* bar, unsigned gave_up = 0u)
+{
+    return atomicAdd(bar + 1, 1u + gave_up);
+}
+// With what count_out returned: whether this was the last block (blocks are below 2^16) ...
+__device__ __forceinline__ bool last_out(unsigned before, unsigned blocks) { return (before & 0xFFFFu) == blocks - 1; }
+// ... which puts the words back to zero.
+__device__ __forceinline__ void reset(unsigned* bar) { bar[0] = bar[1] = 0u; }
+
 // A grid that is one thread-block cluster has the hardware's barrier instead (about 0.4 us against 1.2): all threads
 // arrive, then all wait; it orders global memory like the counter does, and its blocks are resident together by definition.
+// It has no limit and needs none: it waits for threads of the cluster that have not exited, every one of which is running
+// and reaches the same barriers, for no block of a cluster waits for anything else.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 

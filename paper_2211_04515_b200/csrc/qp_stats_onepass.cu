@@ -265,6 +265,9 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
         ++waits;
         return qp_grid::barrier(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
     };
+    auto leave = [&](unsigned gave_up) {
+        if (threadIdx.x == 0 && qp_grid::last_out(qp_grid::count_out(a.bar, gave_up), G)) qp_grid::reset(a.bar);
+    };
     for (int i = threadIdx.x; i < (int)(OP_DYN_BYTES / 16); i += SS_THREADS) reinterpret_cast<uint4*>(raw)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x == 0) s_full = 0;
 
@@ -301,7 +304,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
         if (threadIdx.x == 0)
 #pragma unroll
             for (int j = 0; j < 3; ++j) a.part[(size_t)(2 * G + blockIdx.x) * 8 + j] = v3[j];
-        if (!meet()) return;
+        if (!meet()) { leave(qp_grid::GAVE_UP); return; }
         op_merge<0, 0, 0>(a.part + (size_t)2 * G * 8, G, s_sum);
         // (every sample was counted by its four lanes)
         const double k = s_sum[2] > 0.0 ? s_sum[2] : 1.0, m = s_sum[0] / k, var = s_sum[1] / k - m * m;
@@ -360,7 +363,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
     if (threadIdx.x == 0)
 #pragma unroll
         for (int j = 0; j < 8; ++j) a.part[(size_t)blockIdx.x * 8 + j] = v8[j];
-    if (!meet()) return;
+    if (!meet()) { leave(qp_grid::GAVE_UP); return; }
     op_merge<0, 0, 0, 0, 1, 2, 0, 0>(a.part, G, s_sum);
     qp_stats_t st;
     const double sum_abs = s_sum[1], sum_sq = s_sum[2], below = s_sum[6];
@@ -406,7 +409,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             double* p = a.part + (size_t)(G + blockIdx.x) * 8;
             p[0] = v4[0]; p[1] = v4[1]; p[2] = v4[2]; p[3] = s_full ? 1.0 : 0.0;
         }
-        if (!meet()) return;
+        if (!meet()) { leave(qp_grid::GAVE_UP); return; }
         op_merge<0, 0, 0, 0>(a.part + (size_t)G * 8, G, s_sum);
         const double d = fabs(D), u = (double)delta / 65536.0;
         const double lo = own ? (double)__uint_as_float((unsigned)(own + cell_off) << 17) : 0.0;
@@ -446,7 +449,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             a.part[(size_t)(3 * G + blockIdx.x) * 8] = v2[0];
             a.part[(size_t)(3 * G + blockIdx.x) * 8 + 1] = v2[1];
         }
-        if (!meet()) return;
+        if (!meet()) { leave(qp_grid::GAVE_UP); return; }
         op_merge<0, 0>(a.part + (size_t)3 * G * 8, G, s_sum);
         st.mad = nf > 0.0 ? s_sum[0] / nf : 0.0;
         st.var = nf > 0.0 ? s_sum[1] / nf : 0.0;
@@ -476,7 +479,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
     }
     if (a.cluster) return;
     __syncthreads();
-    if (threadIdx.x == 0 && atomicInc(a.bar + 1, G - 1) == G - 1) atomicExch(a.bar, 0u);       // the last block out
+    leave(0u);
 }
 
 template <typename T>

@@ -539,8 +539,10 @@ __host__ __device__ constexpr int ss_ctile(int hh) { return hh >= 3 ? 512 : 1024
 
 // STATS: phases A and B (otherwise the statistics come with st_in, and B runs only if they lack the histogram).
 // HH: code boundaries above the centre, 2^bits / 2 - 1; -1: statistics only.
+// Returns false where a wait ran out; before (in thread 0): what count_out returned if the block has counted itself out.
+constexpr unsigned SS_IN = 0xFFFFFFFFu;
 template <typename T, bool STATS, int HH>
-__global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArgs a)
+__device__ __forceinline__ bool ss_run(const SsArgs& a, unsigned& before)
 {
     constexpr bool SEARCH = HH >= 0;
     constexpr int H = SEARCH ? HH : 0;
@@ -614,7 +616,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArg
             double* p = a.part + (size_t)blockIdx.x * 8;
             p[0] = v5[0]; p[1] = v5[1]; p[2] = v5[2]; p[3] = v5[3]; p[4] = v5[4];
         }
-        if (!meet()) return;
+        if (!meet()) return false;
         // one warp merges the partials (all loads in flight together), the rest of the block waits at the barrier below
         if (threadIdx.x < 32) {
             double m5[5] = {0.0, 0.0, inf, -inf, 0.0};
@@ -696,13 +698,16 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArg
             if (c) atomicAdd(&a.hist[b], c);
         }
         if constexpr (SEARCH) {
-            if (!meet()) return;
+            if (!meet()) return false;
         } else {                                              // statistics only: the last block out finishes
             __threadfence();
             __syncthreads();
-            if (threadIdx.x == 0) s_last = atomicAdd(a.bar + 1, 1u) == G - 1;
+            if (threadIdx.x == 0) {
+                before = qp_grid::count_out(a.bar);
+                s_last = before == G - 1;                     // (with a block that gave up among those before: no output)
+            }
             __syncthreads();
-            if (!s_last) return;
+            if (!s_last) return true;
             __threadfence();
         }
         if (threadIdx.x < 32) {
@@ -744,10 +749,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArg
             }
         }
         __syncthreads();
-        if constexpr (!SEARCH) {
-            scratch_clean();
-            if (threadIdx.x == 0) { a.bar[0] = 0u; a.bar[1] = 0u; }
-        }
+        if constexpr (!SEARCH) scratch_clean();
     }
 
     // ---- phase C
@@ -848,14 +850,15 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArg
         }
         const int count = hard ? h.M + 1 : 2 * ni;
         if (!cluster) {
-            if (!meet()) return;
+            if (!meet()) return false;
             ss_slices(a, count, raw + SS_TABLE_BYTES);
         }
         arrive();
         if (blockIdx.x == 0) {
             int* pos = reinterpret_cast<int*>(raw + SS_TABLE_BYTES);          // [ncand][H + 2] in the histogram's room (the slices are stored)
             if (!hard) ss_places<H>(s_plan, ncand, ni, s_edge, s_cell, pos);
-            if (!wait((waits + 1) * G)) return;
+            if (!wait((waits + 1) * G)) return false;
+            if (!cluster && !a.packed && threadIdx.x == 0) before = qp_grid::count_out(a.bar);   // (here: the answer comes meanwhile)
             if (cluster) ss_all_slices(a, count);
             if (!hard) {
                 ss_finish<H>(a, s_plan, s_st, ncand, ni, s_cell, pos, s_cand, s_valid, s_curve, s_red, reinterpret_cast<double*>(raw));
@@ -869,30 +872,41 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArg
             }
             ss_pick(a, ncand, s_curve, s_cand, s_valid, s_setup);
             scratch_clean();
-            if (!a.packed) {
-                if (threadIdx.x == 0) a.bar[0] = 0u;          // everybody else has left
-                return;
-            }
+            if (!a.packed) return true;
             arrive();
         } else {
             if (cluster) {
                 wait(0);
                 if (a.packed) arrive();
             }
-            if (!a.packed) return;
+            if (!a.packed) {
+                if (threadIdx.x == 0) __threadfence();        // (the arrival, which nobody here polls for)
+                return true;
+            }
         }
         if constexpr (STATS) {                                // the sender: everybody packs, from the tensor's end
-            if (!wait((waits + 1) * G + 1)) return;
+            if (!wait((waits + 1) * G + 1)) return false;
             const float lo = __ldcg(&a.qp_out->lo), hi = __ldcg(&a.qp_out->hi), inv = __ldcg(&a.qp_out->inv_scale);
             uint32_t* sw = reinterpret_cast<uint32_t*>(raw) + (threadIdx.x >> 5) * 256;
             const uint64_t tiles = (a.n + QP_TILE - 1) / QP_TILE;
             for (uint64_t it = first; it < tiles; it += step)
                 qp_pack_tile<BITS, T, true>(x, a.n, tiles - 1 - it, lane, lo, hi, inv, a.packed, a.nwords, sw);
-            if (cluster) return;
-            __syncthreads();
-            if (threadIdx.x == 0 && atomicInc(a.bar + 1, G - 1) == G - 1) atomicExch(a.bar, 0u);   // the last block out
         }
     }
+    return true;
+}
+
+template <typename T, bool STATS, int HH>
+__global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArgs a)
+{
+    unsigned before = SS_IN;
+    const unsigned gave_up = ss_run<T, STATS, HH>(a, before) ? 0u : qp_grid::GAVE_UP;
+    if (threadIdx.x != 0 || (a.cluster && before == SS_IN)) return;
+    if (before == SS_IN) before = qp_grid::count_out(a.bar, gave_up) | gave_up;
+    if (!qp_grid::last_out(before, gridDim.x)) return;
+    if (before >= qp_grid::GAVE_UP)                           // (only block 0 of an undisturbed launch has cleaned)
+        for (int b = 0; b < a.nb; ++b) a.hist[b] = 0ull;
+    qp_grid::reset(a.bar);
 }
 
 template <typename T>
@@ -979,7 +993,7 @@ int32_t qp_launch_stats_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t
     a.setup = ctx->d_setup;
     a.part = reinterpret_cast<double*>(ctx->d_part);
     unsigned char* f = static_cast<unsigned char*>(ctx->d_fused);
-    a.bar = reinterpret_cast<unsigned*>(f) + 16;              // words 16, 17 (the sender uses 0, 1, the statistics 8..10)
+    a.bar = reinterpret_cast<unsigned*>(f) + 16;              // words 16, 17 (the sender uses 0, 1, the statistics 8..10 and 24, 25)
     a.hist = reinterpret_cast<unsigned long long*>(f + 256);
     a.tot = reinterpret_cast<ulonglong2*>(f + QP_FUSED_TOTALS_AT);
     a.rows = reinterpret_cast<ulonglong2*>(ctx->d_iv_part);

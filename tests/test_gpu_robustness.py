@@ -95,6 +95,47 @@ def test_grid_barrier_that_runs_out_is_reported_and_the_context_stays_usable():
     c.close()
 
 
+# the default launches: statistics (two passes, and one about a pilot centre from 96 MB on), with the histogram, the search
+# with and without the histogram in its statistics, and both senders
+@pytest.mark.parametrize("call,n", [("stats", 300 * 1024 + 5), ("stats", 96 << 18), ("stats_hist", 300 * 1024 + 5),
+                                    ("search", 300 * 1024 + 5), ("search_counts", 300 * 1024 + 5),
+                                    ("sender_search", 300 * 1024 + 5), ("sender", (5 << 19) + 1031)])
+def test_default_launch_whose_barrier_runs_out_leaves_no_trace(call, n):
+    """Every block's wait runs out (as above): no output is written, and the next launch on the context is right although
+    nobody has read the status: the last block out puts the barrier's words and the histogram back to zero."""
+    c = qp.Context(0)
+    d = dev(np.resize(si.vit_activation((1, 1024, 1024), 305).reshape(-1), n))
+    d_stats = c.qp_stats(d, hist_bins=0 if call == "search_counts" else 100)
+    sizes = {"stats": [ctypes.sizeof(qp.Stats)],
+             "search": [ctypes.sizeof(qp.DSResult), ctypes.sizeof(qp.QParams)],
+             "sender": [qp.qp_packed_bytes(n, 2), ctypes.sizeof(qp.QParams), ctypes.sizeof(qp.Stats)]}[call.split("_")[0]]
+
+    def run():
+        out = [torch.full((b,), 0xEE, dtype=torch.uint8, device="cuda") for b in sizes]
+        before = c.qp_launch_count()
+        if call.startswith("stats"):
+            c.qp_stats(d, out=out[0], hist_bins=100 if call == "stats_hist" else 0)
+        elif call.startswith("search"):
+            c.qp_dsaciq_search(d, d_stats, 4, out_result=out[0], out_qp=out[1])
+        else:
+            c.qp_sender_device(d, 2, call == "sender_search", out_packed=out[0], out_qp=out[1], out_stats=out[2])
+        assert c.qp_launch_count() - before == 1
+        torch.cuda.synchronize()
+        return out
+
+    want = run()
+    c.qp_set_wait_limit_for_testing(barrier_polls=500, barrier_extra_arrivals=1)
+    assert all(bool((o == 0xEE).all()) for o in run())
+    c.qp_set_wait_limit_for_testing()
+    assert all(torch.equal(a, b) for a, b in zip(run(), want))
+    with pytest.raises(qp.QuantPipeError) as e:
+        c.qp_get_status()
+    assert e.value.status == qp.QP_ERR_TIMEOUT
+    assert all(torch.equal(a, b) for a, b in zip(run(), want))
+    assert c.qp_get_status() == 0
+    c.close()
+
+
 def test_graph_replay_keeps_calls_with_different_options_apart():
     """Stored graphs are keyed by every argument.  Pairs of calls that differ only in the clip method
     and the histogram's bin count (fields that once shared bits of one key word) must each replay
