@@ -508,6 +508,8 @@ int32_t qp_sender_tokens_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_
  * (d_packed_work 16-byte aligned), d_y_work and h_y >= n elements of out_dtype.
  * Page-locked, 16-byte aligned buffers let qp_receiver_host read and write host memory from the
  * kernel itself (up to 8 bits and 16 MB of elements): up to 1.8 times as fast on a small tensor.
+ * h_packed and h_y may overlap (the elements then take the packed bytes' place): such a call is made
+ * with copies.
  * Errors: as the calls they are made of. */
 /* qp_sender_device: the sender's whole chain on DEVICE buffers in one call, nothing read back
  * to the host: statistics (carrying the histogram along for the search), the clip by

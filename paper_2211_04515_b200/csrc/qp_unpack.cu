@@ -241,6 +241,11 @@ void* mapped(const void* p, uint64_t bytes)
     return ok ? a.devicePointer : nullptr;
 }
 
+bool apart(const void* a, uint64_t na, const void* b, uint64_t nb)
+{
+    return (uintptr_t)a + na <= (uintptr_t)b || (uintptr_t)b + nb <= (uintptr_t)a;
+}
+
 }  // namespace
 
 // The receiver on page-locked, 16-byte aligned buffers in one launch; QP_WARN_INFEASIBLE where it does not apply: copy engines
@@ -255,6 +260,11 @@ int32_t qp_launch_unpack_host(qp_ctx* ctx, const void* h_packed, uint64_t n, int
     const void* in = mapped(h_packed, qp_packed_bytes(n, bits));
     void* out = in ? mapped(h_y, n * esz) : nullptr;
     if (!out) return QP_WARN_INFEASIBLE;
+    // the kernel reads and writes at the same time, the copies one after the other: buffers that overlap are theirs
+    const uint64_t np = qp_packed_bytes(n, bits), ny = n * esz;
+    if (!apart(in, np, out, ny) || !apart(in, np, d_packed, np) || !apart(in, np, d_y, ny) || !apart(out, ny, d_packed, np) ||
+        !apart(out, ny, d_y, ny))
+        return QP_WARN_INFEASIBLE;
     if (out_dtype == QP_F32)
         return unpack_host_typed<float>(ctx, static_cast<const uint32_t*>(in), n, bits, h_qp, static_cast<uint32_t*>(d_packed),
                                         static_cast<float*>(d_y), static_cast<float*>(out), s);

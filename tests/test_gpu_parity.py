@@ -850,6 +850,26 @@ def test_receiver_host_buffers_edges(ctx, n, dtype):
     ctx.qp_get_status()                                  # (one element: degenerate)
 
 
+# the elements take the packed bytes' place, from its start, inside it, and with the packed bytes at their end
+@pytest.mark.parametrize("p_at,y_at", [(0, 0), (0, 1024), (4096, 0), (16 * 1024, 0)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_receiver_host_buffers_that_overlap(ctx, p_at, y_at, dtype):
+    n, bits = 8 * 1024 + 100, 8
+    x = torch.from_numpy(si.vit_activation((1, n, 1), 6).reshape(-1)).cuda()
+    packed, q = ctx.qp_sender_device(x, bits, False)
+    h_qp = ctx.read_qparams(q)
+    want = ctx.qp_unpack_dequantize(packed, n, bits, h_qp, out_dtype=dtype)
+    d_p, d_y = torch.empty_like(packed), torch.empty_like(want)
+    for _ in range(20):                                  # (a race shows itself sometimes)
+        buf = torch.zeros(64 * 1024, dtype=torch.uint8, pin_memory=True)
+        h_p, h_y = buf[p_at:p_at + packed.numel()], buf[y_at:y_at + want.nbytes].view(dtype)
+        h_p.copy_(packed)
+        ctx.qp_receiver_host(h_p, n, bits, h_qp, d_p, d_y, h_y)
+        torch.cuda.synchronize()
+        assert torch.equal(h_y, want.cpu())
+    assert ctx.qp_get_status() == 0
+
+
 # ----------------------------------------------------- full-size configurations
 
 def full_pack_unpack(ctx, x, d, qp_o, bits, label=""):
