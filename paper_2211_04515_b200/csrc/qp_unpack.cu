@@ -14,6 +14,8 @@
 // the work buffer and to page-locked memory, so both directions of the link are busy at once and the two copies around the
 // kernel, 4 us each and in series with it, are gone.  What bounds it: the link, 49 GB/s of stores (a copy engine's 55).  One image
 // at 8 bits: 19 us against 35 (bf16 14.5 / 26), 1.2 M elements 111 / 126 (bf16 65 / 84), 4.2 M 389 / 391 (230 / 246).
+#include <cuda.h>
+
 #include "qp_internal.cuh"
 
 namespace {
@@ -227,18 +229,29 @@ int32_t unpack_host_typed(qp_ctx* ctx, const uint32_t* in, uint64_t n, int bits,
     return qp_check_launch(ctx, "qp_receiver_host");
 }
 
-// the device's address of [p, p + bytes) in page-locked host memory, or NULL
+// The device's address of [p, p + bytes) inside one allocation or registration of page-locked host memory, or NULL.  (The
+// runtime's attributes say nothing of its extent: two registrations with unlocked pages between them look alike at both ends.)
 void* mapped(const void* p, uint64_t bytes)
 {
-    cudaPointerAttributes a, b;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
-        cudaPointerGetAttributes(&b, static_cast<const char*>(p) + bytes - 1) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    const bool ok = a.type == cudaMemoryTypeHost && b.type == cudaMemoryTypeHost && a.devicePointer && b.devicePointer &&
-                    static_cast<char*>(b.devicePointer) - static_cast<char*>(a.devicePointer) == (ptrdiff_t)(bytes - 1);
-    return ok ? a.devicePointer : nullptr;
+    using Get = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+    static const Get get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &f, cudaEnableDefault, &r) != cudaSuccess || r != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Get>(f);
+    }();
+    unsigned type = 0;
+    CUdeviceptr at = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* into[] = {&type, &at, &start, &size};
+    if (!get || get(4, what, into, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return nullptr;
+    const bool ok = type == CU_MEMORYTYPE_HOST && at && at >= start && bytes <= size && at - start <= size - bytes;
+    return ok ? reinterpret_cast<void*>((uintptr_t)at) : nullptr;
 }
 
 bool apart(const void* a, uint64_t na, const void* b, uint64_t nb)

@@ -870,6 +870,45 @@ def test_receiver_host_buffers_that_overlap(ctx, p_at, y_at, dtype):
     assert ctx.qp_get_status() == 0
 
 
+def test_receiver_host_buffer_over_two_registrations(ctx):
+    """A buffer that begins in one registration and ends in another, with pages between them that are not locked, is not the
+    kernel's to read.  The call is captured and never run: one node is the kernel, more are the copies (which may
+    refuse such a buffer)."""
+    cu, rt = ctypes.CDLL("libcuda.so.1"), torch.cuda.cudart()
+    n, bits, page = 48 * 1024, 8, 4096
+    raw = torch.empty(n + 2 * page, dtype=torch.uint8)
+    start = (raw.data_ptr() + page - 1) // page * page
+    h_p = raw[start - raw.data_ptr():][:n]
+    h_y = torch.empty(n, pin_memory=True)
+    d_p, d_y = torch.empty(n, dtype=torch.uint8, device="cuda"), torch.empty(n, device="cuda")
+    h_qp = qp.QParams(-1.0, 1.0, 2.0 / 255, 255.0 / 2, bits, 0)
+    stream = torch.cuda.Stream()
+
+    def nodes():
+        graph, count = ctypes.c_void_p(), ctypes.c_size_t()
+        handle = ctypes.c_void_p(stream.cuda_stream)
+        assert cu.cuStreamBeginCapture_v2(handle, 1) == 0
+        try:
+            with torch.cuda.stream(stream):
+                ctx.qp_receiver_host(h_p, n, bits, h_qp, d_p, d_y, h_y)
+        except qp.QuantPipeError:
+            return None
+        finally:
+            if cu.cuStreamEndCapture(handle, ctypes.byref(graph)) == 0 and graph:
+                assert cu.cuGraphGetNodes(graph, None, ctypes.byref(count)) == 0
+                cu.cuGraphDestroy(graph)
+        return count.value
+
+    for pieces, want in (([(0, n)], (1,)), ([(0, 4 * page), (8 * page, 4 * page)], (None, 3))):
+        for at, size in pieces:
+            assert int(rt.cudaHostRegister(start + at, size, 0)) == 0
+        try:
+            assert nodes() in want
+        finally:
+            for at, _ in pieces:
+                assert int(rt.cudaHostUnregister(start + at)) == 0
+
+
 # ----------------------------------------------------- full-size configurations
 
 def full_pack_unpack(ctx, x, d, qp_o, bits, label=""):
