@@ -88,7 +88,7 @@ class QuantPipeError(RuntimeError):
 
 _lib = None
 _call = _call64 = _tensor_in = None                 # of _qpcall, once load() has run
-_addr: dict = {}                                    # addresses of the entry points called through it
+_addr: dict = {}                                    # numbers of the entry points bound for it
 
 
 def load() -> C.CDLL:
@@ -184,7 +184,18 @@ def _load_call_path(L: C.CDLL) -> None:
     _qpcall.setup(torch.float32, torch.bfloat16)
     _call, _call64, _tensor_in = _qpcall.call, _qpcall.call64, _qpcall.tensor_in
     for name in EXPORTS:
-        _addr[name] = C.cast(getattr(L, name), C.c_void_p).value
+        fn = getattr(L, name)
+        if fn.argtypes and C.c_double not in fn.argtypes:
+            _addr[name] = _qpcall.bind(C.cast(fn, C.c_void_p).value, _kinds(name, fn.argtypes))
+
+
+def _kinds(name: str, argtypes) -> str:
+    """What _qpcall may pass in each place: i an integer, p a buffer, a an address (the context, the stream, host structs and
+    the quantizer that can be one)."""
+    last = len(argtypes) - 1
+    either = {"qp_quantize_pack": 5, "qp_unpack_dequantize": 4}.get(name, 0)
+    return "".join("i" if not (t is C.c_void_p or hasattr(t, "contents")) else
+                   "a" if hasattr(t, "contents") or i in (0, last, either) else "p" for i, t in enumerate(argtypes))
 
 
 # ------------------------------------------------------------- host, pure

@@ -5,33 +5,44 @@
  * the call took 14 us.  Here the arguments go from the vectorcall array straight into registers:
  * about 1 us per call beside the launch itself.
  *
- *   call(address, *args)    calls the function at `address`; returns its int32 status
- *   call64(address, *args)  the same for functions that return uint64
+ *   bind(address, kinds)    makes the function at `address` callable; returns its number for call / call64.  kinds: a
+ *                           letter per parameter,
+ *                             i  an integer: int, or an object that can stand for one (a numpy integer, a tensor of one
+ *                                integer); passed as its low 64 bits
+ *                             p  a buffer: a tensor (its data_ptr()) or None (NULL)
+ *                             a  an address: an int, a tensor or None
+ *   call(number, *args)     calls the function; returns its int32 status
+ *   call64(number, *args)   the same for functions that return uint64
  *   tensor_in(x)            (numel, dtype code) of a contiguous CUDA tensor; AssertionError for others,
  *                           dtype code -1 for a dtype the library does not take
- *   setup(float32, bfloat16)  the two dtype objects that have a code
+ *   setup(float32, bfloat16)  the two dtype objects that have a code; empties the table of bound functions
  *
- * An argument is an int (passed as its low 64 bits), a tensor (its data_ptr()), None (NULL) or a bool.
+ * A tensor of one integer has an address and a value, so which of them is meant has to come from the parameter.
  * Every parameter of the functions called this way is an integer or a pointer, which the 64-bit C
  * calling conventions pass alike, so one function type per argument count covers them all.
  */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
+#include <string.h>
 
 #define MAX_ARGS 16
 
 static PyObject *s_data_ptr, *s_numel, *s_is_contiguous, *s_is_cuda, *s_dtype;
 static PyObject *t_float32, *t_bfloat16;
 
-static int word_of(PyObject* o, uint64_t* out)
+#define MAX_FUNCS 64
+static struct { uint64_t f; Py_ssize_t n; char kinds[MAX_ARGS + 1]; } funcs[MAX_FUNCS];
+static int n_funcs;
+
+static int word_of(PyObject* o, char kind, uint64_t* out)
 {
-    if (PyLong_Check(o)) {                               /* bool is an int */
+    if (PyLong_Check(o) && kind != 'p') {                /* bool is an int */
         *out = PyLong_AsUnsignedLongLongMask(o);
-    } else if (o == Py_None) {
+    } else if (o == Py_None && kind != 'i') {
         *out = 0;
     } else {
-        PyObject* p = PyObject_CallMethodNoArgs(o, s_data_ptr);
+        PyObject* p = kind == 'i' ? PyNumber_Index(o) : PyObject_CallMethodNoArgs(o, s_data_ptr);
         if (!p) return -1;
         *out = PyLong_AsUnsignedLongLongMask(p);
         Py_DECREF(p);
@@ -69,18 +80,36 @@ static u jump(u f, const u* a, Py_ssize_t n)
 
 static int invoke(PyObject* const* args, Py_ssize_t n, u* r)
 {
-    u f, a[MAX_ARGS];
-    if (n < 2 || n - 1 > MAX_ARGS) {
-        PyErr_SetString(PyExc_TypeError, "a function address and 1 to 16 arguments");
+    u a[MAX_ARGS];
+    const long i = n > 0 ? PyLong_AsLong(args[0]) : -1;
+    if (i == -1 && PyErr_Occurred()) return -1;
+    if (i < 0 || i >= n_funcs || n - 1 != funcs[i].n) {
+        PyErr_SetString(PyExc_TypeError, "the number of a bound function and its arguments");
         return -1;
     }
-    if (word_of(args[0], &f)) return -1;
-    for (Py_ssize_t i = 1; i < n; ++i)
-        if (word_of(args[i], &a[i - 1])) return -1;
+    for (Py_ssize_t k = 1; k < n; ++k)
+        if (word_of(args[k], funcs[i].kinds[k - 1], &a[k - 1])) return -1;
     Py_BEGIN_ALLOW_THREADS                               /* a launch may wait for room in the queue */
-    *r = jump(f, a, n - 1);
+    *r = jump(funcs[i].f, a, n - 1);
     Py_END_ALLOW_THREADS
     return 0;
+}
+
+static PyObject* py_bind(PyObject* m, PyObject* args)
+{
+    unsigned long long f;
+    const char* kinds;
+    Py_ssize_t n;
+    (void)m;
+    if (!PyArg_ParseTuple(args, "Ks#", &f, &kinds, &n)) return NULL;
+    if (!f || n < 1 || n > MAX_ARGS || strspn(kinds, "ipa") != (size_t)n || n_funcs == MAX_FUNCS) {
+        PyErr_SetString(PyExc_ValueError, "an address, 1 to 16 kinds of i, p and a, and room in the table");
+        return NULL;
+    }
+    funcs[n_funcs].f = f;
+    funcs[n_funcs].n = n;
+    memcpy(funcs[n_funcs].kinds, kinds, (size_t)n + 1);
+    return PyLong_FromLong(n_funcs++);
 }
 
 static PyObject* py_call(PyObject* m, PyObject* const* args, Py_ssize_t n)
@@ -139,12 +168,14 @@ static PyObject* py_setup(PyObject* m, PyObject* args)
     Py_INCREF(b);
     Py_XSETREF(t_float32, f);
     Py_XSETREF(t_bfloat16, b);
+    n_funcs = 0;
     Py_RETURN_NONE;
 }
 
 static PyMethodDef methods[] = {
-    {"call", (PyCFunction)(void (*)(void))py_call, METH_FASTCALL, "call(address, *args) -> int32 status"},
-    {"call64", (PyCFunction)(void (*)(void))py_call64, METH_FASTCALL, "call64(address, *args) -> uint64"},
+    {"bind", py_bind, METH_VARARGS, "bind(address, kinds) -> number"},
+    {"call", (PyCFunction)(void (*)(void))py_call, METH_FASTCALL, "call(number, *args) -> int32 status"},
+    {"call64", (PyCFunction)(void (*)(void))py_call64, METH_FASTCALL, "call64(number, *args) -> uint64"},
     {"tensor_in", py_tensor_in, METH_O, "tensor_in(x) -> (numel, dtype code)"},
     {"setup", py_setup, METH_VARARGS, "setup(float32, bfloat16)"},
     {NULL, NULL, 0, NULL},

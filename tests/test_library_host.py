@@ -52,6 +52,25 @@ def test_packed_bytes_and_F(lib, bits):
     assert qp.qp_aciq_F(bits, 1) == pytest.approx(oracle.aciq_F(bits, 1), rel=1e-12)
 
 
+def test_call_path_takes_what_each_parameter_can_be(lib):
+    """An integer may be anything that can stand for one (numpy integers, a tensor of one integer: its value, not its address);
+    a buffer only a tensor or None.  Without a context the library refuses the device call, so nothing runs."""
+    import torch
+    from paper_2211_04515_b200 import _qpcall, binding as b
+    for n in (1000, np.int64(1000), np.uint32(1000), torch.tensor(1000)):
+        for bits in (4, np.int32(4), torch.tensor(4, dtype=torch.uint8)):
+            assert _qpcall.call64(b._addr["qp_packed_bytes"], n, bits) == 512
+    x, out, st = torch.zeros(()), torch.zeros(16, dtype=torch.uint8), b._addr["qp_quantize_pack"]
+    args = [None, x, 0, np.int64(1), torch.tensor(8), 0, False, out, 16, 0]
+    assert _qpcall.call(st, *args) == qp.QP_ERR_INVALID_ARG
+    for at, bad in ((1, x.data_ptr()), (7, 16), (7, True), (3, 1.0), (4, None), (4, torch.zeros(2)), (2, "f32")):
+        with pytest.raises((TypeError, AttributeError)):
+            _qpcall.call(st, *args[:at], bad, *args[at + 1:])
+    for few in ((), (st,), (st, *args[:-1]), (st, *args, 0), (-1, *args), (99, *args)):
+        with pytest.raises(TypeError):
+            _qpcall.call(*few)
+
+
 def test_unsupported_bits(lib):
     assert qp.qp_packed_bytes(10, 9) == 0 and qp.qp_packed_bytes(10, 0) == 0
     assert qp.qp_aciq_F(12, 0) == 0.0 and qp.qp_aciq_F(4, 2) == 0.0
