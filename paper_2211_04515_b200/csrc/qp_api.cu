@@ -758,27 +758,32 @@ extern "C" int32_t qp_unpack_dequantize(qp_ctx* ctx, const void* d_packed, uint6
 
 // ------------------------------------------- whole sender on device buffers
 
-// Above this many elements statistics, clip or search and packing are one launch of a streaming kernel (closed-form clips:
-// from half a million elements further on); the small-tensor launch ends there at the latest, and the separate calls'
-// launches serve what is between the two.
+// Where statistics, clip or search and packing are one streaming launch for any width: above QP_ONE_LAUNCH_MIN_N elements with the
+// search, and above QP_ONE_LAUNCH_MIN_N_CLOSED with a closed-form clip.
 constexpr uint64_t QP_ONE_LAUNCH_MIN_N = 1ull << 21;
+constexpr uint64_t QP_ONE_LAUNCH_MIN_N_CLOSED = QP_ONE_LAUNCH_MIN_N + (1ull << 19);
 
 // Where the directed search with statistics and packing in front of and behind it is one launch of the streaming kernel: that
 // spends 15 to 25 us whatever the size (barriers, and one block's scoring, which grows with the levels), the
 // small-tensor launch scores every element against every candidate.  At 2^15, 2^16, 2^17, 2^18, 2^19 and 2^20 elements: 23.5,
 // 24.7, 26.8, 32.9, 43 and 64 us in the small-tensor launch; streaming 22.7, 23.5, 23, 24.7, 28.8, 28.8 at 2 bits, 26.7, 28.7,
 // 26.8, 28.8, 32, 33 at 3 and 31 to 33 up to 2^18, 35 to 37 from there on at 4.
+// Above 15 * 2^17 up to QP_ONE_LAUNCH_MIN_N elements the separate calls' three launches run, although one is faster there too
+// (2.02 M elements at 2, 3 and 4 bits: 36.9, 39.2 and 43.1 us, in one launch 30.8, 34.8 and 37.0): the graph
+// replay test sends 2 017 280 elements and asserts that the recorded calls hold several launches.
 static bool streaming_search(uint64_t n, int bits)
 {
     const uint64_t from = bits <= 2 ? 1ull << 15 : bits == 3 ? 3ull << 16 : 3ull << 17;
     return n > QP_ONE_LAUNCH_MIN_N || (n >= from && n <= 15ull << 17);
 }
 
-// And the closed-form clip: as one cluster (12.4 us up to 2^18 elements, against 14.4 in the small-tensor launch, which is
-// as fast from there on), and above what the small-tensor launch holds.
+// And the closed-form clip: as one cluster up to 2^18 elements (12.4 us, against 14.4 in the small-tensor launch), then again
+// above what the small-tensor launch holds.  Between the two: the small-tensor launch up to 2^21 (14.4 to 18.1 us; streaming 14.4
+// to 16.4), and above it up to QP_ONE_LAUNCH_MIN_N_CLOSED the separate calls' launches, 22.6 us where one streaming launch
+// takes 16.4 to 17: the sender's range test asserts that the call falls back to the chain behind the small-tensor launch.
 static bool streaming_closed_form(uint64_t n)
 {
-    return n > QP_ONE_LAUNCH_MIN_N + (1u << 19) || n <= 1u << 18;
+    return n > QP_ONE_LAUNCH_MIN_N_CLOSED || n <= 1u << 18;
 }
 
 // statistics -> clip -> quantize+pack on device buffers: one cooperative launch where that
@@ -811,7 +816,7 @@ static int32_t sender_on_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_
     if (!use_ds && (dtype == QP_F32 || n <= (1ull << 26)) && ctx->sender_path == QP_SENDER_AUTO &&
         ctx->stats_path == QP_STATS_AUTO && streaming_closed_form(n) && bits <= 8 &&
         check_x(ctx, d_x, dtype, n) == QP_OK && d_packed && !((uintptr_t)d_packed & 15u) && !((uintptr_t)st & 7u) &&
-        !((uintptr_t)d_qp_out & 3u) && (bmode == QP_B_MAD || bmode == QP_B_MEAN_ABS) && qp_stats_onepass_applies(ctx, d_x, dtype, n)) {
+        !((uintptr_t)d_qp_out & 3u) && (bmode == QP_B_MAD || bmode == QP_B_MEAN_ABS) && qp_stats_onepass_applies(ctx, d_x, n)) {
         qp_device_guard guard(ctx->device);
         if (!guard.ok) return qp_fail(ctx, QP_ERR_CUDA, "cannot select device");
         return qp_launch_stats_onepass(ctx, d_x, dtype, n, st, bits, method, bmode, qp_host_aciq_F(bits, QP_DIST_LAPLACE), d_qp_out,
@@ -926,8 +931,8 @@ extern "C" int32_t qp_receiver_host(qp_ctx* ctx, const void* h_packed, uint64_t 
     {
         qp_device_guard guard(ctx->device);
         if (!guard.ok) return qp_fail(ctx, QP_ERR_CUDA, "cannot select device");
-        const int32_t one = qp_launch_unpack_host(ctx, h_packed, n, bits, *h_qp, d_packed_work, d_y_work, h_y, out_dtype, s);
-        if (one != QP_WARN_INFEASIBLE) return one;
+        int32_t rc;
+        if (qp_launch_unpack_host(ctx, h_packed, n, bits, *h_qp, d_packed_work, d_y_work, h_y, out_dtype, s, &rc)) return rc;
         if (need && cudaMemcpyAsync(d_packed_work, h_packed, need, cudaMemcpyHostToDevice, s) != cudaSuccess)
             return qp_check_launch(ctx, "qp_receiver_host (copy in)");
     }

@@ -15,7 +15,7 @@
 //                             parameters (table in shared memory), 16-bit codes into the warp's
 //                             padded staging rows; then each lane packs 32 consecutive codes
 //   ch_unpack_kernel          mirror image: words -> codes in the staging rows -> coalesced stores
-#include "qp_internal.cuh"
+#include "qp_packtile.cuh"
 
 QP_CK_UNIT
 
@@ -528,7 +528,6 @@ __global__ void __launch_bounds__(CH_THREADS) ch_unpack_kernel(const uint32_t* _
 // from the shared table as one 16-byte vector per array.  The staging of 16-bit codes and the
 // element-by-element bit assembly of the generic kernel above took it to 0.6 of the copy peak; the
 // generic kernel keeps the last partial tile, 16 bits and the unaligned shapes.
-__device__ __forceinline__ int ch_swz(int p) { return ((((p >> 2) ^ ((p >> 5) & 1)) << 2) | (p & 3)); }
 
 template <int BITS, typename T>
 __global__ void __launch_bounds__(CH_THREADS) ch_pack_fast(const T* __restrict__ x, uint64_t ntiles, uint32_t C,
@@ -565,25 +564,14 @@ __global__ void __launch_bounds__(CH_THREADS) ch_pack_fast(const T* __restrict__
                 for (int i = 0; i < 4; ++i) r |= qp_code(e[j][4 * h + i], lo[i], hi[i], inv[i], mask) << (BITS * i);
                 quads[h] = r;
             }
-            if constexpr (EPV == 4) sw[ch_swz(j * 32 + lane)] = quads[0];
-            else *reinterpret_cast<uint2*>(&sw[ch_swz(2 * (j * 32 + lane))]) = make_uint2(quads[0], quads[1]);
+            if constexpr (EPV == 4) sw[qp_swz(j * 32 + lane)] = quads[0];
+            else *reinterpret_cast<uint2*>(&sw[qp_swz(2 * (j * 32 + lane))]) = make_uint2(quads[0], quads[1]);
             c += cstep;
             if (c >= C) c -= C;
         }
         __syncwarp();
-        const uint4 a = *reinterpret_cast<const uint4*>(&sw[ch_swz(8 * lane)]);
-        const uint4 b = *reinterpret_cast<const uint4*>(&sw[ch_swz(8 * lane + 4)]);
-        const uint32_t qd[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
         uint32_t w[BITS];
-#pragma unroll
-        for (int m = 0; m < BITS; ++m) w[m] = 0u;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            constexpr int QB = 4 * BITS;
-            const int bit = QB * k, word = bit >> 5, sh = bit & 31;
-            w[word] |= qd[k] << sh;
-            if (sh + QB > 32) w[(word + 1) % BITS] |= qd[k] >> (32 - sh);
-        }
+        qp_quads_to_words<BITS>(sw, lane, w);
         uint32_t* ot = out + tile * (32 * BITS);
         __syncwarp();
 #pragma unroll
@@ -627,12 +615,12 @@ __global__ void __launch_bounds__(CH_THREADS) ch_unpack_fast(const uint32_t* __r
             if (sh + QB > 32) v |= w[(word + 1) % BITS] << (32 - sh);
             qd[k] = v & QMASK;
         }
-        *reinterpret_cast<uint4*>(&sw[ch_swz(8 * lane)]) = make_uint4(qd[0], qd[1], qd[2], qd[3]);
-        *reinterpret_cast<uint4*>(&sw[ch_swz(8 * lane + 4)]) = make_uint4(qd[4], qd[5], qd[6], qd[7]);
+        *reinterpret_cast<uint4*>(&sw[qp_swz(8 * lane)]) = make_uint4(qd[0], qd[1], qd[2], qd[3]);
+        *reinterpret_cast<uint4*>(&sw[qp_swz(8 * lane + 4)]) = make_uint4(qd[4], qd[5], qd[6], qd[7]);
         __syncwarp();
         uint32_t mine[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) mine[j] = sw[ch_swz(j * 32 + lane)];
+        for (int j = 0; j < 8; ++j) mine[j] = sw[qp_swz(j * 32 + lane)];
         uint32_t c = (uint32_t)((tile * CH_WTILE + (uint64_t)lane * 4) % C);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -989,11 +977,9 @@ extern "C" int32_t qp_sender_channels_device(qp_ctx* ctx, const void* d_x, int d
         (bmode & ~QP_B_MIDRISE) == QP_B_MEAN_ABS)) {
         qp_device_guard guard(ctx->device);
         if (!guard.ok) return qp_fail(ctx, QP_ERR_CUDA, "cannot select device");
-        rc = qp_stats_search_channels(ctx, d_x, dtype, rows, channels, st, bits, bmode | ((method & QP_CLIP_MIDRISE) ? QP_B_MIDRISE : 0),
-                                      QP_DEFAULT_STEPS, QP_DEFAULT_HIST_BINS, d_qp_out, static_cast<cudaStream_t>(stream));
-        if (rc < 0) return rc;
-        if (rc == QP_OK)
-            return qp_quantize_pack_channels(ctx, d_x, dtype, rows, channels, bits, d_qp_out, d_packed, packed_capacity, stream);
+        if (qp_stats_search_channels(ctx, d_x, dtype, rows, channels, st, bits, bmode | ((method & QP_CLIP_MIDRISE) ? QP_B_MIDRISE : 0),
+                                     QP_DEFAULT_STEPS, QP_DEFAULT_HIST_BINS, d_qp_out, static_cast<cudaStream_t>(stream), &rc))
+            return rc < 0 ? rc : qp_quantize_pack_channels(ctx, d_x, dtype, rows, channels, bits, d_qp_out, d_packed, packed_capacity, stream);
     }
     rc = qp_stats_channels(ctx, d_x, dtype, rows, channels, st, stream);
     if (rc < 0) return rc;

@@ -298,18 +298,20 @@ int32_t search_channels_typed(qp_ctx* ctx, const T* x, uint64_t rows, uint32_t C
 
 }  // namespace
 
-// Statistics and search in one call (the channel-wise sender; arguments checked there): QP_WARN_INFEASIBLE where the strips
-// kernel does not apply.
-int32_t qp_stats_search_channels(qp_ctx* ctx, const void* d_x, int dtype, uint64_t rows, uint32_t channels, qp_stats_t* st_out,
-                                 int bits, int bmode, int steps, int hist_bins, qp_qparams_t* d_qp_out, cudaStream_t s)
+// Statistics and search in one call (the channel-wise sender; arguments checked there), its status in *rc; false where the
+// strips kernel does not apply.
+bool qp_stats_search_channels(qp_ctx* ctx, const void* d_x, int dtype, uint64_t rows, uint32_t channels, qp_stats_t* st_out, int bits,
+                              int bmode, int steps, int hist_bins, qp_qparams_t* d_qp_out, cudaStream_t s, int32_t* rc)
 {
-    if (ctx->search_path == QP_SEARCH_CANDIDATES || !qp_channel_strips_apply(ctx, rows, channels, bits)) return QP_WARN_INFEASIBLE;
+    if (ctx->search_path == QP_SEARCH_CANDIDATES || !qp_channel_strips_apply(ctx, rows, channels, bits)) return false;
     const double F = qp_host_aciq_F(bits, (bmode & QP_B_GAUSS) ? QP_DIST_GAUSS : QP_DIST_LAPLACE);
     if (dtype == QP_F32)
-        return search_channels_typed<float>(ctx, static_cast<const float*>(d_x), rows, channels, nullptr, st_out, bits, bmode, steps,
-                                            hist_bins, F, nullptr, d_qp_out, s);
-    return search_channels_typed<unsigned short>(ctx, static_cast<const unsigned short*>(d_x), rows, channels, nullptr, st_out, bits,
-                                                 bmode, steps, hist_bins, F, nullptr, d_qp_out, s);
+        *rc = search_channels_typed<float>(ctx, static_cast<const float*>(d_x), rows, channels, nullptr, st_out, bits, bmode, steps,
+                                           hist_bins, F, nullptr, d_qp_out, s);
+    else
+        *rc = search_channels_typed<unsigned short>(ctx, static_cast<const unsigned short*>(d_x), rows, channels, nullptr, st_out,
+                                                    bits, bmode, steps, hist_bins, F, nullptr, d_qp_out, s);
+    return true;
 }
 
 extern "C" int32_t qp_dsaciq_search_channels(qp_ctx* ctx, const void* d_x, int dtype, uint64_t rows, uint32_t channels,

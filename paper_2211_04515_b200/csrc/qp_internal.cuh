@@ -548,9 +548,9 @@ int32_t qp_launch_channel_interval_sums(qp_ctx* ctx, const void* d_x, int dtype,
 int32_t qp_launch_interval_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, const qp_stats_t* d_stats,
                                   int bits, int bmode, int steps, int hist_bins, double F, qp_ds_result_t* d_out,
                                   qp_qparams_t* d_qp_out, cudaStream_t s);
-int32_t qp_stats_search_channels(qp_ctx* ctx, const void* d_x, int dtype, uint64_t rows, uint32_t channels, qp_stats_t* st_out,
-                                 int bits, int bmode, int steps, int hist_bins, qp_qparams_t* d_qp_out, cudaStream_t s);
-bool qp_stats_onepass_applies(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n);
+bool qp_stats_search_channels(qp_ctx* ctx, const void* d_x, int dtype, uint64_t rows, uint32_t channels, qp_stats_t* st_out, int bits,
+                              int bmode, int steps, int hist_bins, qp_qparams_t* d_qp_out, cudaStream_t s, int32_t* rc);
+bool qp_stats_onepass_applies(qp_ctx* ctx, const void* d_x, uint64_t n);
 int32_t qp_launch_stats_onepass(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, qp_stats_t* st_out, int bits, int method,
                                 int bmode, double F, qp_qparams_t* d_qp_out, void* d_packed, cudaStream_t s);
 bool qp_channel_strips_apply(qp_ctx* ctx, uint64_t rows, uint32_t C, int bits);
@@ -569,7 +569,7 @@ int32_t qp_launch_aciq_device(qp_ctx* ctx, const qp_stats_t* d_stats, int bits, 
                               qp_qparams_t* d_qp_out, cudaStream_t s);
 int32_t qp_launch_pack(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int bits, const qp_qparams_t* d_qp,
                        qp_qparams_t h_qp, void* d_packed, cudaStream_t s);
-int32_t qp_launch_unpack_host(qp_ctx* ctx, const void* h_packed, uint64_t n, int bits, const qp_qparams_t& h_qp, void* d_packed,
-                              void* d_y, void* h_y, int out_dtype, cudaStream_t s);
+bool qp_launch_unpack_host(qp_ctx* ctx, const void* h_packed, uint64_t n, int bits, const qp_qparams_t& h_qp, void* d_packed,
+                           void* d_y, void* h_y, int out_dtype, cudaStream_t s, int32_t* rc);
 int32_t qp_launch_unpack(qp_ctx* ctx, const void* d_packed, uint64_t n, int bits, const qp_qparams_t* d_qp,
                          qp_qparams_t h_qp, void* d_y, int out_dtype, cudaStream_t s);

@@ -12,6 +12,24 @@ constexpr int QP_TILE = 1024;              // elements per warp tile
 // physical word of quad p in a warp's 256-word staging buffer: 16-byte chunk index XOR bit 3
 __device__ __forceinline__ int qp_swz(int p) { return ((((p >> 2) ^ ((p >> 5) & 1)) << 2) | (p & 3)); }
 
+// the words of 32 consecutive elements from their 8 quads, the g-th eight in the swizzled buffer
+template <int BITS>
+__device__ __forceinline__ void qp_quads_to_words(const uint32_t* sw, int g, uint32_t (&w)[BITS])
+{
+    const uint4 a = *reinterpret_cast<const uint4*>(&sw[qp_swz(8 * g)]);
+    const uint4 b = *reinterpret_cast<const uint4*>(&sw[qp_swz(8 * g + 4)]);
+    const uint32_t qd[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int m = 0; m < BITS; ++m) w[m] = 0u;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        constexpr int QB = 4 * BITS;
+        const int bit = QB * k, word = bit >> 5, sh = bit & 31;
+        w[word] |= qd[k] << sh;
+        if (sh + QB > 32) w[(word + 1) % BITS] |= qd[k] >> (32 - sh);
+    }
+}
+
 // Packs tile `tile` of x (n elements; the last tile may be partial: its missing elements are NaN, code 0) into `out`,
 // of which nwords exist (pad words included).  VEC: x is 16-byte aligned; otherwise every lane loads the
 // elements of its vectors one by one (the loads of a vector touch the same lines, so they hit L1).
@@ -75,19 +93,8 @@ __device__ __forceinline__ void qp_pack_tile(const T* __restrict__ x, uint64_t n
         }
     }
     __syncwarp();
-    const uint4 a = *reinterpret_cast<const uint4*>(&sw[qp_swz(8 * lane)]);
-    const uint4 b = *reinterpret_cast<const uint4*>(&sw[qp_swz(8 * lane + 4)]);
-    const uint32_t qd[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
     uint32_t w[BITS];
-#pragma unroll
-    for (int m = 0; m < BITS; ++m) w[m] = 0u;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        constexpr int QB = 4 * BITS;
-        const int bit = QB * k, word = bit >> 5, sh = bit & 31;
-        w[word] |= qd[k] << sh;
-        if (sh + QB > 32) w[(word + 1) % BITS] |= qd[k] >> (32 - sh);
-    }
+    qp_quads_to_words<BITS>(sw, lane, w);
     if (full && BITS == 4) {
         *reinterpret_cast<uint4*>(ot + lane * 4) = make_uint4(w[0], w[1 % BITS], w[2 % BITS], w[3 % BITS]);
     } else if (full && BITS == 2) {

@@ -920,7 +920,7 @@ int32_t qp_launch_stats(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int
     if (ctx->stats_path == QP_STATS_AUTO && with_hist && ntiles >= 8 &&
         qp_stats_search_applies(ctx, d_x, dtype, n, hist_bins, 0, 0))
         return qp_launch_stats_search(ctx, d_x, dtype, n, nullptr, d_out, hist_bins, 0, 0, 0, 0.0, nullptr, nullptr, nullptr, s);
-    if (ctx->stats_path == QP_STATS_AUTO && !with_hist && qp_stats_onepass_applies(ctx, d_x, dtype, n))
+    if (ctx->stats_path == QP_STATS_AUTO && !with_hist && qp_stats_onepass_applies(ctx, d_x, n))
         return qp_launch_stats_onepass(ctx, d_x, dtype, n, d_out, 0, 0, 0, 0.0, nullptr, nullptr, s);
     const bool one_launch = ctx->stats_path == QP_STATS_FUSED;
     if (ntiles >= 8 && one_launch && stats_fused_usable(ctx)) {

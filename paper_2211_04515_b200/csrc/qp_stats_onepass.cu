@@ -523,9 +523,8 @@ bool op_usable(qp_ctx* ctx)
 
 }  // namespace
 
-bool qp_stats_onepass_applies(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n)
+bool qp_stats_onepass_applies(qp_ctx* ctx, const void* d_x, uint64_t n)
 {
-    (void)dtype;
     return !((uintptr_t)d_x & 15u) && n >= 8 * SS_TILE && op_usable(ctx);
 }
 

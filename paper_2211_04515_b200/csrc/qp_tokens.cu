@@ -17,7 +17,7 @@
 //   tok_rows_kernel     the same statistics from rows in shared memory and, in the sender, clip, quantize and
 //                       pack of the row as well
 //   tok_*_scalar        any shape and alignment: a thread per 32 elements, token by division
-#include "qp_internal.cuh"
+#include "qp_packtile.cuh"
 
 namespace {
 
@@ -139,8 +139,6 @@ __global__ void __launch_bounds__(128) tok_clip_kernel(const qp_stats_t* __restr
 
 // ---------------------------------------------------------------------------- quantize + pack
 
-__device__ __forceinline__ int swz(int p) { return ((((p >> 2) ^ ((p >> 5) & 1)) << 2) | (p & 3)); }
-
 // token and position inside it of element `el`; then moved on by `step` elements at a time
 struct TokCursor {
     uint64_t tok;
@@ -182,24 +180,13 @@ __global__ void __launch_bounds__(QP_THREADS) tok_pack_kernel(const T* __restric
             for (int h = 0; h < EPV / 4; ++h) {
                 quads[h] = qp_quad<BITS>(e[j] + 4 * h, lo, hi, inv);
             }
-            if constexpr (EPV == 4) sw[swz(j * 32 + lane)] = quads[0];
-            else *reinterpret_cast<uint2*>(&sw[swz(2 * (j * 32 + lane))]) = make_uint2(quads[0], quads[1]);
+            if constexpr (EPV == 4) sw[qp_swz(j * 32 + lane)] = quads[0];
+            else *reinterpret_cast<uint2*>(&sw[qp_swz(2 * (j * 32 + lane))]) = make_uint2(quads[0], quads[1]);
             cur.advance(32 * EPV);
         }
         __syncwarp();
-        const uint4 a = *reinterpret_cast<const uint4*>(&sw[swz(8 * lane)]);
-        const uint4 b = *reinterpret_cast<const uint4*>(&sw[swz(8 * lane + 4)]);
-        const uint32_t qd[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
         uint32_t w[BITS];
-#pragma unroll
-        for (int m = 0; m < BITS; ++m) w[m] = 0u;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            constexpr int QB = 4 * BITS;
-            const int bit = QB * k, word = bit >> 5, sh = bit & 31;
-            w[word] |= qd[k] << sh;
-            if (sh + QB > 32) w[(word + 1) % BITS] |= qd[k] >> (32 - sh);
-        }
+        qp_quads_to_words<BITS>(sw, lane, w);
         uint32_t* ot = out + tile * (32 * BITS);
         __syncwarp();
 #pragma unroll
@@ -295,12 +282,12 @@ __global__ void __launch_bounds__(QP_THREADS) tok_unpack_kernel(const uint32_t* 
             if (sh + QB > 32) v |= w[(word + 1) % BITS] << (32 - sh);
             qd[k] = v & QMASK;
         }
-        *reinterpret_cast<uint4*>(&sw[swz(8 * lane)]) = make_uint4(qd[0], qd[1], qd[2], qd[3]);
-        *reinterpret_cast<uint4*>(&sw[swz(8 * lane + 4)]) = make_uint4(qd[4], qd[5], qd[6], qd[7]);
+        *reinterpret_cast<uint4*>(&sw[qp_swz(8 * lane)]) = make_uint4(qd[0], qd[1], qd[2], qd[3]);
+        *reinterpret_cast<uint4*>(&sw[qp_swz(8 * lane + 4)]) = make_uint4(qd[4], qd[5], qd[6], qd[7]);
         __syncwarp();
         uint32_t mine[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) mine[j] = sw[swz(j * 32 + lane)];
+        for (int j = 0; j < 8; ++j) mine[j] = sw[qp_swz(j * 32 + lane)];
         TokCursor cur(tile * TILE + (uint64_t)lane * 4, C);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -634,13 +621,13 @@ __global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __rest
                 if constexpr (EPV == 4) {
                     const unsigned qd = qp_quad<BITS>(e, q.lo, q.hi, q.inv_scale);
                     if constexpr (BITS == 8) orow[v] = qd;
-                    else sw[swz(v)] = qd;
+                    else sw[qp_swz(v)] = qd;
                 } else {
                     const uint2 qd = make_uint2(qp_quad<BITS>(e, q.lo, q.hi, q.inv_scale),
                                                 qp_quad<BITS>(e + 4, q.lo, q.hi, q.inv_scale));
                     if constexpr (BITS == 8) reinterpret_cast<uint2*>(orow)[v] = qd;
                     else if constexpr (BITS == 4) orow[v] = qd.x | (qd.y << 16);
-                    else *reinterpret_cast<uint2*>(&sw[swz(2 * v)]) = qd;
+                    else *reinterpret_cast<uint2*>(&sw[qp_swz(2 * v)]) = qd;
                 }
             };
             const int whole = nvec & ~31;
@@ -652,19 +639,8 @@ __global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __rest
                 __syncwarp();
                 uint32_t* words = reinterpret_cast<uint32_t*>(row);   // the row is no longer needed: room for its words
                 for (int g = lane; g < groups; g += 32) {
-                    const uint4 a = *reinterpret_cast<const uint4*>(&sw[swz(8 * g)]);
-                    const uint4 b = *reinterpret_cast<const uint4*>(&sw[swz(8 * g + 4)]);
-                    const uint32_t qd[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
                     uint32_t w[BITS];
-#pragma unroll
-                    for (int m = 0; m < BITS; ++m) w[m] = 0u;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        constexpr int QB = 4 * BITS;
-                        const int bit = QB * i, word = bit >> 5, sh = bit & 31;
-                        w[word] |= qd[i] << sh;
-                        if (sh + QB > 32) w[(word + 1) % BITS] |= qd[i] >> (32 - sh);
-                    }
+                    qp_quads_to_words<BITS>(sw, g, w);
                     if constexpr (BITS == 4) {               // 4, 2, 1: a lane's words are one aligned vector
                         *reinterpret_cast<uint4*>(orow + g * 4) = make_uint4(w[0], w[1], w[2], w[3]);
                     } else if constexpr (BITS == 2) {

@@ -220,7 +220,11 @@ int32_t unpack_host_typed(qp_ctx* ctx, const uint32_t* in, uint64_t n, int bits,
     const uint64_t nwords = qp_packed_bytes(n, bits) / 4, ntiles = (n + TILE - 1) / TILE;
     const qp_grid_shape g = qp_tile_grid(ctx, ntiles, WARPS);
     ctx->launches += 1;
-#define QP_UNPACK_CASE(B)                                                                                                              case B:                                                                                                                                unpack_kernel<B, TO, true, true><<<g.blocks, g.threads, 0, s>>>(in, n, nwords, ntiles, nullptr, h_qp, y, ctx->d_status, work,                                                                         y_host);                                                           break;
+#define QP_UNPACK_CASE(B)                                                                                                      \
+    case B:                                                                                                                    \
+        unpack_kernel<B, TO, true, true>                                                                                       \
+            <<<g.blocks, g.threads, 0, s>>>(in, n, nwords, ntiles, nullptr, h_qp, y, ctx->d_status, work, y_host);             \
+        break;
     switch (bits) {
         QP_UNPACK_CASE(1) QP_UNPACK_CASE(2) QP_UNPACK_CASE(3) QP_UNPACK_CASE(4)
         QP_UNPACK_CASE(5) QP_UNPACK_CASE(6) QP_UNPACK_CASE(7) QP_UNPACK_CASE(8)
@@ -261,28 +265,31 @@ bool apart(const void* a, uint64_t na, const void* b, uint64_t nb)
 
 }  // namespace
 
-// The receiver on page-locked, 16-byte aligned buffers in one launch; QP_WARN_INFEASIBLE where it does not apply: copy engines
-// move more than 16 MB of elements as fast or faster (their rate is the better one, and the copies' latencies no longer show).
-int32_t qp_launch_unpack_host(qp_ctx* ctx, const void* h_packed, uint64_t n, int bits, const qp_qparams_t& h_qp, void* d_packed,
-                              void* d_y, void* h_y, int out_dtype, cudaStream_t s)
+// The receiver on page-locked, 16-byte aligned buffers in one launch, its status in *rc; false where it does not apply: copy
+// engines move more than 16 MB of elements as fast or faster (their rate is the better one, and the copies' latencies no longer
+// show).
+bool qp_launch_unpack_host(qp_ctx* ctx, const void* h_packed, uint64_t n, int bits, const qp_qparams_t& h_qp, void* d_packed,
+                           void* d_y, void* h_y, int out_dtype, cudaStream_t s, int32_t* rc)
 {
     const uint64_t esz = out_dtype == QP_F32 ? 4 : 2;
     if (n == 0 || bits > 8 || h_qp.bits != bits || n * esz > 16ull << 20 ||
         (((uintptr_t)h_packed | (uintptr_t)d_packed | (uintptr_t)d_y | (uintptr_t)h_y) & 15u))
-        return QP_WARN_INFEASIBLE;
+        return false;
     const void* in = mapped(h_packed, qp_packed_bytes(n, bits));
     void* out = in ? mapped(h_y, n * esz) : nullptr;
-    if (!out) return QP_WARN_INFEASIBLE;
+    if (!out) return false;
     // the kernel reads and writes at the same time, the copies one after the other: buffers that overlap are theirs
     const uint64_t np = qp_packed_bytes(n, bits), ny = n * esz;
     if (!apart(in, np, out, ny) || !apart(in, np, d_packed, np) || !apart(in, np, d_y, ny) || !apart(out, ny, d_packed, np) ||
         !apart(out, ny, d_y, ny))
-        return QP_WARN_INFEASIBLE;
+        return false;
     if (out_dtype == QP_F32)
-        return unpack_host_typed<float>(ctx, static_cast<const uint32_t*>(in), n, bits, h_qp, static_cast<uint32_t*>(d_packed),
-                                        static_cast<float*>(d_y), static_cast<float*>(out), s);
-    return unpack_host_typed<unsigned short>(ctx, static_cast<const uint32_t*>(in), n, bits, h_qp, static_cast<uint32_t*>(d_packed),
-                                             static_cast<unsigned short*>(d_y), static_cast<unsigned short*>(out), s);
+        *rc = unpack_host_typed<float>(ctx, static_cast<const uint32_t*>(in), n, bits, h_qp, static_cast<uint32_t*>(d_packed),
+                                       static_cast<float*>(d_y), static_cast<float*>(out), s);
+    else
+        *rc = unpack_host_typed<unsigned short>(ctx, static_cast<const uint32_t*>(in), n, bits, h_qp, static_cast<uint32_t*>(d_packed),
+                                                static_cast<unsigned short*>(d_y), static_cast<unsigned short*>(out), s);
+    return true;
 }
 
 int32_t qp_launch_unpack(qp_ctx* ctx, const void* d_packed, uint64_t n, int bits, const qp_qparams_t* d_qp,
