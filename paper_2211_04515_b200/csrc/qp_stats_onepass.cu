@@ -87,7 +87,7 @@ struct OpPass {
     {
         const float a = fabsf(y);
         const int cell = min(max((int)(__float_as_uint(a) >> 17) - cell_off, 0), OP_CELLS - 1);
-        const unsigned addr = (unsigned)cell * mul + base + (__float_as_uint(y) >> 31) * half;
+        const unsigned addr = (unsigned)QP_CK(cell, OP_CELLS) * mul + base + (__float_as_uint(y) >> 31) * half;
         const unsigned d = __float_as_uint(fmaf(a, inv_u, OP_MAGIC)) - OP_ONE;
         asm volatile("{ .reg .pred p; setp.lt.f32 p, %3, %4; @p red.shared.add.u32 [%0], 1; @p red.shared.add.u32 [%0+%2], %1; }"
                      ::"r"(addr), "r"(d), "n"(OP_SUMS_AT), "f"(a), "f"(delta) : "memory");

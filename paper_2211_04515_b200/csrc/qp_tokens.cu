@@ -19,6 +19,8 @@
 //   tok_*_scalar        any shape and alignment: a thread per 32 elements, token by division
 #include "qp_packtile.cuh"
 
+QP_CK_UNIT
+
 namespace {
 
 constexpr int TILE = 1024;
@@ -427,7 +429,7 @@ __device__ __forceinline__ bool tok_row_stats(const T* row, int nvec, uint32_t C
         for (int h = 0; h < 8 / EPV; ++h) {
             const int v = v0 + h * 32 + lane;
             float a[EPV];
-            if (v < nvec) tok_lds<T>(row + v * EPV, a);
+            if (v < nvec) tok_lds<T>(row + QP_CK(v, nvec) * EPV, a);
 #pragma unroll
             for (int i = 0; i < EPV; ++i) e[h * EPV + i] = v < nvec ? a[i] : missing;
         }
@@ -444,7 +446,7 @@ __device__ __forceinline__ bool tok_row_stats(const T* row, int nvec, uint32_t C
 #pragma unroll 2
     for (int v0 = 0; v0 < whole; v0 += STEP) {
         qp_f2 p[4];
-        tok_lds8<T>(row, v0 + lane, p);
+        tok_lds8<T>(row, QP_CK(v0 + lane, nvec - (STEP - 32)), p);
         moments(p);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -527,7 +529,7 @@ __device__ __forceinline__ bool tok_row_stats(const T* row, int nvec, uint32_t C
 #pragma unroll 2
     for (int v0 = 0; v0 < whole; v0 += STEP) {
         qp_f2 p[4];
-        tok_lds8<T>(row, v0 + lane, p);
+        tok_lds8<T>(row, QP_CK(v0 + lane, nvec - (STEP - 32)), p);
         deviations(p, guard);
     }
     if (whole < nvec) {
@@ -578,7 +580,7 @@ __global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __rest
     for (uint64_t t = (uint64_t)blockIdx.x * TR_WARPS + (threadIdx.x >> 5); t < tokens; t += wstride) {
         const T* src = x + t * C;
         auto fetch = [&](int v) {
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(row + v * EPV)),
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(row + QP_CK(v, nvec) * EPV)),
                          "l"(src + (size_t)v * EPV)
                          : "memory");
         };
@@ -617,17 +619,17 @@ __global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __rest
             uint32_t* orow = out + t * (uint64_t)(groups * BITS);
             auto quantize = [&](int v) {                     // vector v: its quads to the output (8 bits: a quad is a word) or to `sw`
                 float e[EPV];
-                tok_lds<T>(row + v * EPV, e);
+                tok_lds<T>(row + QP_CK(v, nvec) * EPV, e);
                 if constexpr (EPV == 4) {
                     const unsigned qd = qp_quad<BITS>(e, q.lo, q.hi, q.inv_scale);
                     if constexpr (BITS == 8) orow[v] = qd;
-                    else sw[qp_swz(v)] = qd;
+                    else sw[QP_CK(qp_swz(v), (int)(C / 4))] = qd;
                 } else {
                     const uint2 qd = make_uint2(qp_quad<BITS>(e, q.lo, q.hi, q.inv_scale),
                                                 qp_quad<BITS>(e + 4, q.lo, q.hi, q.inv_scale));
                     if constexpr (BITS == 8) reinterpret_cast<uint2*>(orow)[v] = qd;
                     else if constexpr (BITS == 4) orow[v] = qd.x | (qd.y << 16);
-                    else *reinterpret_cast<uint2*>(&sw[qp_swz(2 * v)]) = qd;
+                    else *reinterpret_cast<uint2*>(&sw[QP_CK(qp_swz(2 * v), (int)(C / 4) - 1)]) = qd;
                 }
             };
             const int whole = nvec & ~31;
@@ -640,7 +642,7 @@ __global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __rest
                 uint32_t* words = reinterpret_cast<uint32_t*>(row);   // the row is no longer needed: room for its words
                 for (int g = lane; g < groups; g += 32) {
                     uint32_t w[BITS];
-                    qp_quads_to_words<BITS>(sw, g, w);
+                    qp_quads_to_words<BITS>(sw, QP_CK(g, groups), w);
                     if constexpr (BITS == 4) {               // 4, 2, 1: a lane's words are one aligned vector
                         *reinterpret_cast<uint4*>(orow + g * 4) = make_uint4(w[0], w[1], w[2], w[3]);
                     } else if constexpr (BITS == 2) {
@@ -649,12 +651,12 @@ __global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __rest
                         orow[g] = w[0];
                     } else {
 #pragma unroll
-                        for (int m = 0; m < BITS; ++m) words[g * BITS + m] = w[m];
+                        for (int m = 0; m < BITS; ++m) words[QP_CK(g * BITS + m, (int)(C * sizeof(T) / 4))] = w[m];
                     }
                 }
                 if constexpr (BITS != 4 && BITS != 2 && BITS != 1) {
                     __syncwarp();
-                    for (int i = lane; i < groups * BITS; i += 32) orow[i] = words[i];
+                    for (int i = lane; i < groups * BITS; i += 32) orow[i] = words[QP_CK(i, (int)(C * sizeof(T) / 4))];
                 }
             }
             if (t == tokens - 1) {                           // pad words

@@ -48,17 +48,29 @@ def pytest_terminal_summary(terminalreporter):
 
 @pytest.fixture(scope="session", autouse=True)
 def index_checked_build_reports_clean(request):
-    """When the tests run against the library built with index checks (QUANTPIPE_LIB points at it), the
-    session ends by reading the status once more: no index may have been out of range."""
-    yield
+    """When the tests run against the library built with index checks (QUANTPIPE_LIB points at it), no index may
+    have been out of range: the bit is kept from every status that a test reads (reading clears it), and the
+    session ends by reading it once more."""
     if not os.environ.get("QUANTPIPE_LIB"):
+        yield
         return
     import torch
+    import paper_2211_04515_b200 as qp
+    read, seen = qp.Context.qp_get_status, []
+
+    def recording(self):
+        status = read(self)
+        seen.append(status & qp.QP_DEV_INDEX_RANGE)
+        return status
+
+    qp.Context.qp_get_status = recording
+    yield
+    qp.Context.qp_get_status = read
     if not torch.cuda.is_available():
         return
-    import paper_2211_04515_b200 as qp
     assert qp.qp_built_with_index_checks()
     c = qp.Context(0)
     assert c.qp_get_status() & qp.QP_DEV_INDEX_RANGE == 0
     c.close()
+    assert not any(seen)
     _INDEX_CHECK_REPORT.append("index checks: on, no index out of range")

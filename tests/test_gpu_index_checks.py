@@ -5,9 +5,10 @@ No memory checker can be run on the kernels, so the library has a debug build
 kernels' shared-memory tables and scratch rows is range-checked: an index out of range is redirected
 to entry 0 (nothing traps, nothing faults) and raises QP_DEV_INDEX_RANGE in what qp_get_status
 returns.  This test builds that variant, runs the small cases (c1, ragged sizes, degenerate and
-non-finite inputs, searches at 1 to 8 bits, channel-wise and token-wise shapes) in a child process
+non-finite inputs, searches at 1 to 8 bits, channel-wise and token-wise shapes, the streaming launches as
+clusters and as grids, the channel strips and the token rows) in a child process
 that loads it through QUANTPIPE_LIB, and expects them to pass with the bit clear (the child's
-conftest checks the bit once more at the end of the session).
+conftest looks at every status that a test reads, and once more at the end of the session).
 """
 import os
 import subprocess
@@ -22,7 +23,9 @@ pytestmark = pytest.mark.gpu
 SUBSET = ("test_stats_configs or test_stats_ragged or test_stats_special or stats_one_launch or test_pack_unpack_c1 or "
           "test_pack_unpack_ragged or test_pack_special or test_search_c1 or test_search_steps or "
           "test_search_ragged or test_search_degenerate or test_fused_sender_c1 or fused_sender_special or "
-          "test_channels_shapes or test_search_channels_vit or test_tokens_shapes")
+          "test_channels_shapes or test_search_channels_vit or test_tokens_shapes or "
+          "test_stats_streaming or test_sender_search_streaming or test_search_streaming_small or test_search_channels_strips or "
+          "test_tokens_rows_edges or beyond_fp32")
 
 
 def test_small_cases_run_clean_under_the_index_checked_build():
