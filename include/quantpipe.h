@@ -185,7 +185,9 @@ int32_t qp_stats(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int hist_b
 int qp_stats_carries_histogram(const void* d_x, int dtype, uint64_t n, int hist_bins);
 /* How qp_stats runs its passes on 16-byte aligned tensors (an execution option without a
  * counterpart in the paper; min, max, the counts and the histogram's peak are identical on all
- * paths, the other fields agree to ~1e-7 relative):
+ * paths; mean, mean_abs, mad and var are fp64 sums of fp32 partial sums over at most 32 elements,
+ * which the paths group differently: they agree to ~1e-8 relative on continuous data, and to ~2e-7
+ * where a few levels or a few outliers make up the sums, so that the partial sums' roundings repeat):
  *   QP_STATS_TWO_KERNELS  one kernel per pass
  *   QP_STATS_FUSED        one cooperative launch for both (one block per SM; every block keeps the
  *                         last tiles of its first pass in shared memory and starts the second pass,

@@ -184,6 +184,36 @@ def test_stats_one_launch_against_oracle_and_two_kernels(ctx, tiles, tail):
     assert ctx.qp_get_status() == 0
 
 
+@pytest.mark.parametrize("n", [8 * 1024, (1 << 18) + 1, 1500 * 8192 + 77, (96 << 18) + 9])
+@pytest.mark.parametrize("data", ["plain", "two_levels", "outliers"])
+def test_stats_default_path_agrees_with_the_forced_ones(ctx, n, data):
+    """Bounds: an fp32 chain adds at most 16 terms of one sign (u = 2^-24 each), a squared deviation brings 3 u more:
+    19 u a path.  On continuous data the roundings are independent, sqrt(16) u in the root mean square of a chain, n / 16 chains,
+    five sigma; and 1e-8 is what the one pass accepts."""
+    u = 2.0 ** -24
+    x = np.tile(si.flat_iid(min(n, 1 << 20), 32, "laplace"), -(-n // (1 << 20)))[:n] + np.float32(0.25)
+    if data == "two_levels":
+        x = np.where(np.arange(n) % 3 == 0, np.float32(-1.1), np.float32(2.3))
+    elif data == "outliers":
+        x[::9973] *= np.float32(1e4)
+    tol = 2 * 5 * 4 * u / (n / 16) ** 0.5 + 1e-8 if data == "plain" else 2 * 19 * u
+    d = dev(x.astype(np.float32))
+    for nb in (0, 100):
+        st = ctx.read_stats(ctx.qp_stats(d, hist_bins=nb))
+        for path in STATS_PATHS:
+            ctx.qp_set_stats_path(path)
+            try:
+                f = ctx.read_stats(ctx.qp_stats(d, hist_bins=nb))
+            finally:
+                ctx.qp_set_stats_path(qp.QP_STATS_AUTO)
+            assert (st.n, st.nonfinite, st.min, st.max) == (f.n, f.nonfinite, f.min, f.max)
+            assert (st.hist_bins, st.hist_peak) == (f.hist_bins, f.hist_peak)
+            assert abs(st.mean - f.mean) <= tol * f.mean_abs
+            for field in ("mean_abs", "mad", "var"):
+                assert abs(getattr(st, field) - getattr(f, field)) <= tol * getattr(f, field), (field, path, nb)
+    assert ctx.qp_get_status() == 0
+
+
 def test_stats_hard_tensors(sctx):
     """Tensors that are hard on a streaming reduction: sorted (every block sees another level), a third
     of the elements exactly at the mean, constant, two levels, a shifted mixture, a mean far from zero,
@@ -703,7 +733,7 @@ def test_fused_sender_special_values_modes_and_bf16():
 def test_fused_sender_range_and_fallback():
     """Forced, the single launch takes a closed-form clip up to what shared memory holds (millions of
     elements) and the search up to 2^20; beyond that, or beyond 127 steps or 4096 bins, the call runs the
-    kernel chain.  AUTO switches to the chain earlier (2^21), where the chain is the faster one."""
+    kernel chain.  AUTO leaves the single launch earlier (2^21)."""
     c = qp.Context(0)
     x = si.vit_activation((1, 3000000, 1), 33).reshape(-1)
     d = dev(x)
@@ -1124,7 +1154,7 @@ def test_stats_streaming(ctx, n, data, bf16):
     ctx.qp_get_status()
 
 
-# statistics and search in one launch (the default from 2^20 elements on, the sender above 2^21): every width it takes, tile
+# statistics and search in one launch (the default from 8192 elements on, 32768 at 4 bits, the sender by width): every width it takes, tile
 # remainders, the largest and smallest number of steps, tables with few replicas, and the exact-threshold form
 SS_CASES = [(1, 0, 100, 100, (1 << 21) + 1, "vit"), (2, 0, 100, 100, (1 << 21) + 1023, "outliers"), (3, 0, 100, 100, (1 << 21) + 1024, "vit"),
             (4, 0, 100, 100, (1 << 21) + 5, "outliers"), (4, qp.QP_B_MIDRISE, 255, 4096, (1 << 21) + 77, "vit"),
