@@ -14,14 +14,18 @@
 // octave of |y|, so that every cell but the mean's own lies on a known side.  That one is taken as evenly filled, which is
 // accepted where even the worst filling could not change the result by 1e-8; otherwise (and where the mean lies further
 // than delta from c, or a cell's counter might have wrapped) the second pass runs after all.
-// What bounds it: the read, 171 us for 1 GiB of fp32 (6.3 TB/s) of 193 in all, where two passes took 319; the rest is the
-// pilot (3 us for its loads: 64 bytes per sample, one DRAM burst; 16-byte samples took 16 us on 1 GiB), three
-// barriers, and blocks that end up to 8 us apart.  fp32 of 134, 268 and 537 MB: 41, 62 and 102 us against 45, 82 and 157.
+// What bounds it: the read.  1 GiB of fp32, i.i.d. Laplace, by the blocks' time stamps: the pass 177 us in the fastest block and 185 in
+// the slowest (5.8 TB/s), the pilot 7 (3 for its loads: 64 bytes per sample, one DRAM burst; 16-byte samples took 16), the two
+// barriers and merges behind the pass 8, so 194 us in all, where two passes took 319.  Data whose mean lies off the density's
+// peak has fewer elements in the window (channels of different means: 170 to 177 us).  fp32 of 134, 268 and 537 MB: 41, 62 and
+// 102 us against 45, 82 and 157.
 // The window must cost next to nothing: one test per four elements, and behind it one predicated look-up for the lane's hit
 // (all elements through the look-up took 275 us on 1 GiB, four look-ups behind the test 221).
 //
 // Packing here rather than in a launch of its own: 5 to 10 us less (no clip launch, no gaps, and what L2 still holds is not
-// read again), 1 GiB at 8 bits 383 against 394 us, 2^24 fp32 at 2 bits 35 against 44.
+// read again), 2^24 fp32 at 2 bits 35 us against 44; 1 GiB at 8 bits 384 us against 394, of which the packing 173 in the fastest
+// block and 185 in the slowest.  (384 in runs of some milliseconds; in longer ones the GPU draws 975 W and clocks at 1.85 instead
+// of 1.97 GHz: 392 to 410 us.)
 #include "qp_gridbar.cuh"
 #include "qp_packtile.cuh"
 #include "qp_tiles.cuh"

@@ -16,11 +16,13 @@
 // wrap.  Integer sums: the result does not depend on the order.  Tensors whose clip ends are coarse against the quantization
 // step take the "hard" form below, with the exact thresholds.
 //
-// What bounds it, on 129 MB (fp32, 2 bits): phase A the read from DRAM (24 us); B and C the read, most of which L2
-// still holds, together with 9 and 12 instructions and one and two shared atomics per element (18 and 21 us); the packing
-// its read and write (18 us); the rest, 25 us, is barriers, merges and the two serial stretches (candidates; error curve and
-// pick).  On 39 MB at 4 bits, which L2 holds: 9, 5, 12 and 6 us, the rest 28.  113 and 66 us a call, where two kernels for
-// the statistics, five for the search and one for the packing took 171 and 107.
+// What bounds it, by time stamps that the blocks took (each figure from the last block before it to its own last block; the
+// stamps lengthen the launch): on 129 MB (fp32, 2 bits) phase A 25 us, the read from DRAM; barrier and merge 9; B 20 and C 23, the
+// read, most of which L2 still holds, and the instructions (A and B 19 per element together, C 19, at 4 bits 35; one shared
+// atomic in B, two in C); between them barrier, merge and candidates 5; rows, barrier and slices 6; block 0's scoring and
+// pick 9, its result read back 1; packing 21: 119 in all.  On 39 MB at 4 bits, which L2 holds: A 9, then 9, B 6, 5, C 15, 7, 9, 1 and
+// the packing 6: 67.  The calls take 114 and 64 us without the stamps, launch included; two kernels for the statistics, five for the
+// search and one for the packing took 171 and 107.
 #include <type_traits>
 
 #include "qp_affine.cuh"
