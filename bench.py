@@ -43,14 +43,14 @@ MIN_TIMED_S = 0.5              # the K-step region is repeated until this much d
 # digest of the kernel's source files at capture time: when those files have changed since, the entry
 # is stale and the benchmark reports traffic = null.
 NCU_TRAFFIC = {
-    "stats": {"bytes": 176.7e6, "kernel": "stats_fused_kernel<float, 0>", "summary": "profiles/stats_fused_kernel_c4.md",
-              "files": ("qp_stats.cu", "qp_stream.cuh", "qp_gridbar.cuh"), "digest": "6be59a35b2bfd17e"},
-    "clip": {"bytes": 133.1e6, "kernel": "iv_moments2_kernel<float>", "summary": "profiles/kernels_c4_ncu_full.md",
-             "files": ("qp_search_fast.cu",), "digest": "619ca87dc8596b84"},
-    "quantize_pack": {"bytes": 141.5e6, "kernel": "pack_kernel<8, float>", "summary": "profiles/kernels_c4_ncu_full.md",
-                      "files": ("qp_pack.cu",), "digest": "90a28547ba456cdf"},
-    "unpack_dequantize": {"bytes": 99.3e6, "kernel": "unpack_kernel<8, float>", "summary": "profiles/kernels_c4_ncu_full.md",
-                          "files": ("qp_unpack.cu",), "digest": "5b1421f640e0f472"},
+    "stats": {"bytes": 136.5e6, "kernel": "stats_onepass_kernel<float, 0>", "summary": "profiles/streaming_kernels.md",
+              "files": ("qp_stats_onepass.cu", "qp_tiles.cuh", "qp_gridbar.cuh"), "digest": "5f3bd610ce425dbf"},
+    "clip": {"bytes": 133.1e6, "kernel": "stats_search_kernel<float, 0, 1>", "summary": "profiles/streaming_kernels.md",
+             "files": ("qp_stats_search.cu", "qp_affine.cuh", "qp_tiles.cuh", "qp_gridbar.cuh"), "digest": "7833d5085f24c4ee"},
+    "quantize_pack": {"bytes": 146.5e6, "kernel": "pack_kernel<8, float>", "summary": "profiles/streaming_kernels.md",
+                      "files": ("qp_pack.cu", "qp_packtile.cuh"), "digest": "80cc1d90da9d53f0"},
+    "unpack_dequantize": {"bytes": 104.4e6, "kernel": "unpack_kernel<8, float>", "summary": "profiles/streaming_kernels.md",
+                          "files": ("qp_unpack.cu",), "digest": "98f297b6feac2a9c"},
 }
 
 
