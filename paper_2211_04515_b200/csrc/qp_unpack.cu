@@ -59,8 +59,88 @@ __device__ __forceinline__ void store_out(unsigned short* y, uint64_t i4, const 
 __device__ __forceinline__ void store_one(float* y, uint64_t i, float v) { y[i] = v; }
 __device__ __forceinline__ void store_one(unsigned short* y, uint64_t i, float v) { y[i] = qp_f32_to_bf16(v); }
 
-// ntiles counts the last, partial tile too: its words are read up to nwords and its elements written up
-// to n.  VEC: y is aligned for 4-element stores; otherwise the elements are stored one by one.
+// One tile; full: it has all its elements, otherwise its words are read up to nwords and its elements written up to n.  VEC: y
+// is aligned for 4-element stores; otherwise the elements are stored one by one.
+template <int BITS, typename TO, bool VEC, bool HOST>
+__device__ __forceinline__ void unpack_tile(const uint32_t* __restrict__ in, uint64_t n, uint64_t nwords, uint64_t tile, bool full,
+                                            int lane, const DQ& q, uint32_t* sw, TO* __restrict__ y, uint32_t* __restrict__ work,
+                                            TO* __restrict__ y_host)
+{
+    constexpr unsigned MASK = (1u << BITS) - 1u;
+    constexpr int QB = 4 * BITS;
+    constexpr unsigned QMASK = QB >= 32 ? 0xFFFFFFFFu : ((1u << (QB & 31)) - 1u);
+    const uint32_t* it = in + tile * (32 * BITS);
+    uint32_t* wk = HOST ? work + tile * (32 * BITS) : nullptr;
+    uint32_t w[BITS];
+    if (full && BITS == 8) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4*>(it + lane * 8));
+        const uint4 b = __ldg(reinterpret_cast<const uint4*>(it + lane * 8) + 1);
+        w[0] = a.x; w[1 % BITS] = a.y; w[2 % BITS] = a.z; w[3 % BITS] = a.w;
+        w[4 % BITS] = b.x; w[5 % BITS] = b.y; w[6 % BITS] = b.z; w[7 % BITS] = b.w;
+        if constexpr (HOST) {
+            *reinterpret_cast<uint4*>(wk + lane * 8) = a;
+            *(reinterpret_cast<uint4*>(wk + lane * 8) + 1) = b;
+        }
+    } else if (full && BITS == 4) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4*>(it + lane * 4));
+        w[0] = a.x; w[1 % BITS] = a.y; w[2 % BITS] = a.z; w[3 % BITS] = a.w;
+        if constexpr (HOST) *reinterpret_cast<uint4*>(wk + lane * 4) = a;
+    } else if (full && BITS == 2) {
+        const uint2 a = __ldg(reinterpret_cast<const uint2*>(it + lane * 2));
+        w[0] = a.x; w[1 % BITS] = a.y;
+        if constexpr (HOST) *reinterpret_cast<uint2*>(wk + lane * 2) = a;
+    } else {
+        const int room = full ? 32 * BITS : (int)min((uint64_t)(32 * BITS), nwords - tile * (32 * BITS));
+#pragma unroll
+        for (int m = 0; m < BITS; ++m) {
+            const uint32_t v = m * 32 + lane < room ? __ldg(it + m * 32 + lane) : 0u;
+            sw[m * 32 + lane] = v;
+            if (HOST && m * 32 + lane < room) wk[m * 32 + lane] = v;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int m = 0; m < BITS; ++m) w[m] = sw[lane * BITS + m];
+        __syncwarp();
+    }
+    uint32_t qd[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int bit = QB * k, word = bit >> 5, sh = bit & 31;
+        uint32_t v = w[word] >> sh;
+        if (sh + QB > 32) v |= w[(word + 1) % BITS] << (32 - sh);
+        qd[k] = v & QMASK;
+    }
+    *reinterpret_cast<uint4*>(&sw[swz(8 * lane)]) = make_uint4(qd[0], qd[1], qd[2], qd[3]);
+    *reinterpret_cast<uint4*>(&sw[swz(8 * lane + 4)]) = make_uint4(qd[4], qd[5], qd[6], qd[7]);
+    __syncwarp();
+    uint32_t mine[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) mine[j] = sw[swz(j * 32 + lane)];
+    const int have = full ? TILE : (int)(n - tile * TILE);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        float v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = dequant((mine[j] >> (BITS * i)) & MASK, q);
+        const int k = (j * 32 + lane) * 4;
+        if (VEC && (full || k + 4 <= have)) {
+            store_out(y, tile * (TILE / 4) + j * 32 + lane, v);
+            if constexpr (HOST) store_out(y_host, tile * (TILE / 4) + j * 32 + lane, v);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (k + i < have) {
+                    store_one(y, tile * TILE + k + i, v[i]);
+                    if constexpr (HOST) store_one(y_host, tile * TILE + k + i, v[i]);
+                }
+        }
+    }
+    __syncwarp();
+}
+
+// ntiles counts the last, partial tile too.  In the loop's body where a warp writes 4 KB a tile (fp32: 1 to 3 % faster at 2^26 elements
+// and more), behind the loop where it writes 2 KB and the loop is bound by its instructions (bf16: 2^26 elements at 4 bits 51.3 us, 57.4
+// with the partial tile's tests in the loop; 2^28 at 8 bits 169 and 191).
 template <int BITS, typename TO, bool VEC, bool HOST = false>
 __global__ void __launch_bounds__(QP_THREADS) unpack_kernel(const uint32_t* __restrict__ in, uint64_t n, uint64_t nwords,
                                                             uint64_t ntiles, const qp_qparams_t* __restrict__ d_qp,
@@ -74,79 +154,14 @@ __global__ void __launch_bounds__(QP_THREADS) unpack_kernel(const uint32_t* __re
     uint32_t* sw = stage[warp];
     const unsigned warps = blockDim.x >> 5;
     const uint64_t wstride = (uint64_t)gridDim.x * warps;
-    constexpr unsigned MASK = (1u << BITS) - 1u;
-    constexpr int QB = 4 * BITS;
-    constexpr unsigned QMASK = QB >= 32 ? 0xFFFFFFFFu : ((1u << (QB & 31)) - 1u);
-
-    for (uint64_t tile = (uint64_t)blockIdx.x * warps + warp; tile < ntiles; tile += wstride) {
-        const uint32_t* it = in + tile * (32 * BITS);
-        uint32_t* wk = HOST ? work + tile * (32 * BITS) : nullptr;
-        const bool full = (tile + 1) * TILE <= n;                 // warp-uniform
-        uint32_t w[BITS];
-        if (full && BITS == 8) {
-            const uint4 a = __ldg(reinterpret_cast<const uint4*>(it + lane * 8));
-            const uint4 b = __ldg(reinterpret_cast<const uint4*>(it + lane * 8) + 1);
-            w[0] = a.x; w[1 % BITS] = a.y; w[2 % BITS] = a.z; w[3 % BITS] = a.w;
-            w[4 % BITS] = b.x; w[5 % BITS] = b.y; w[6 % BITS] = b.z; w[7 % BITS] = b.w;
-            if constexpr (HOST) {
-                *reinterpret_cast<uint4*>(wk + lane * 8) = a;
-                *(reinterpret_cast<uint4*>(wk + lane * 8) + 1) = b;
-            }
-        } else if (full && BITS == 4) {
-            const uint4 a = __ldg(reinterpret_cast<const uint4*>(it + lane * 4));
-            w[0] = a.x; w[1 % BITS] = a.y; w[2 % BITS] = a.z; w[3 % BITS] = a.w;
-            if constexpr (HOST) *reinterpret_cast<uint4*>(wk + lane * 4) = a;
-        } else if (full && BITS == 2) {
-            const uint2 a = __ldg(reinterpret_cast<const uint2*>(it + lane * 2));
-            w[0] = a.x; w[1 % BITS] = a.y;
-            if constexpr (HOST) *reinterpret_cast<uint2*>(wk + lane * 2) = a;
-        } else {
-            const int room = (int)min((uint64_t)(32 * BITS), nwords - tile * (32 * BITS));
-#pragma unroll
-            for (int m = 0; m < BITS; ++m) {
-                const uint32_t v = m * 32 + lane < room ? __ldg(it + m * 32 + lane) : 0u;
-                sw[m * 32 + lane] = v;
-                if (HOST && m * 32 + lane < room) wk[m * 32 + lane] = v;
-            }
-            __syncwarp();
-#pragma unroll
-            for (int m = 0; m < BITS; ++m) w[m] = sw[lane * BITS + m];
-            __syncwarp();
-        }
-        uint32_t qd[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int bit = QB * k, word = bit >> 5, sh = bit & 31;
-            uint32_t v = w[word] >> sh;
-            if (sh + QB > 32) v |= w[(word + 1) % BITS] << (32 - sh);
-            qd[k] = v & QMASK;
-        }
-        *reinterpret_cast<uint4*>(&sw[swz(8 * lane)]) = make_uint4(qd[0], qd[1], qd[2], qd[3]);
-        *reinterpret_cast<uint4*>(&sw[swz(8 * lane + 4)]) = make_uint4(qd[4], qd[5], qd[6], qd[7]);
-        __syncwarp();
-        uint32_t mine[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) mine[j] = sw[swz(j * 32 + lane)];
-        const int have = full ? TILE : (int)(n - tile * TILE);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            float v[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = dequant((mine[j] >> (BITS * i)) & MASK, q);
-            const int k = (j * 32 + lane) * 4;
-            if (VEC && (full || k + 4 <= have)) {
-                store_out(y, tile * (TILE / 4) + j * 32 + lane, v);
-                if constexpr (HOST) store_out(y_host, tile * (TILE / 4) + j * 32 + lane, v);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (k + i < have) {
-                        store_one(y, tile * TILE + k + i, v[i]);
-                        if constexpr (HOST) store_one(y_host, tile * TILE + k + i, v[i]);
-                    }
-            }
-        }
-        __syncwarp();
+    uint64_t tile = (uint64_t)blockIdx.x * warps + warp;
+    if constexpr (sizeof(TO) == 2) {
+        for (const uint64_t whole = n / TILE; tile < whole; tile += wstride)
+            unpack_tile<BITS, TO, VEC, HOST>(in, n, nwords, tile, true, lane, q, sw, y, work, y_host);
+        if (tile < ntiles) unpack_tile<BITS, TO, VEC, HOST>(in, n, nwords, tile, false, lane, q, sw, y, work, y_host);
+    } else {
+        for (; tile < ntiles; tile += wstride)                    // (warp-uniform)
+            unpack_tile<BITS, TO, VEC, HOST>(in, n, nwords, tile, (tile + 1) * TILE <= n, lane, q, sw, y, work, y_host);
     }
 }
 

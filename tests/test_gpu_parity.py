@@ -330,6 +330,26 @@ def test_pack_bf16_input_and_output(ctx, bits):
         assert np.array_equal(y.view(torch.int16).cpu().numpy().view(np.uint16), y_o)
 
 
+# the partial tile of 1024 behind the loop over whole ones: none, alone, and behind more tiles than the grid has warps
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 8 * 1024 * 64 * 148 + 1024 * 5 + 3])
+def test_pack_unpack_bf16_partial_tile_and_both_directions(ctx, n):
+    x = si.flat_iid(min(n, 1 << 20), 34, "laplace")
+    h = si.to_bf16_bits(np.tile(x, -(-n // x.size))[:n])
+    d = torch.from_numpy(h.view(np.int16)).cuda().view(torch.bfloat16)
+    for bits in (1, 3, 4, 8) if n < 10000 else (3,):
+        _, o = oracle.make_qparams(-4.0, 4.0, bits)
+        want = oracle.quantize_pack(oracle.widen_bf16(h), o)
+        y_o = si.to_bf16_bits(oracle.unpack_dequantize(want, n, o))
+        for _ in range(2):                               # the second call walks the tensor from its end
+            whole, packed = guarded(qp.qp_packed_bytes(n, bits))
+            ctx.qp_quantize_pack(d, bits, to_qp(o), out=packed)
+            assert np.array_equal(packed.cpu().numpy(), want) and canaries_intact(whole, packed.numel())
+        whole, y = guarded(2 * n)
+        ctx.qp_unpack_dequantize(packed, n, bits, to_qp(o), out=y.view(torch.bfloat16))
+        assert np.array_equal(y.cpu().numpy().view(np.uint16), y_o) and canaries_intact(whole, 2 * n)
+    assert ctx.qp_get_status() == 0
+
+
 def test_pack_argument_errors(ctx):
     x = torch.zeros(1000, device="cuda")
     _, qp_h = qp.qp_make_qparams(-1.0, 1.0, 4)
