@@ -423,6 +423,9 @@ uint64_t qp_controller_payload_bytes(const qp_controller_t* h_c, int bits);
  *                                    d_qp_out[0..channels) and, if d_stats_out is not NULL, the
  *                                    statistics (otherwise they stay in a buffer of the context,
  *                                    allocated on first use).
+ * The statistics of one channel are the same bits whichever call takes them, but for tensors beyond L2 (32e6 fp32 or
+ * 1e8 bf16 elements), whose sums qp_stats_channels groups differently from the search in
+ * qp_sender_channels_device (1e-8 relative, as between the paths of qp_stats).
  * d_stats, d_qp: device arrays of `channels` entries.  1 <= channels <= QP_MAX_CHANNELS.
  * Errors: as the per-tensor calls, plus QP_ERR_INVALID_ARG for channels out of range. */
 #define QP_MAX_CHANNELS 4096

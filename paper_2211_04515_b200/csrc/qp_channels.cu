@@ -703,6 +703,16 @@ bool ch_allow_smem(K kernel, size_t bytes)
 
 }  // namespace
 
+// The statistics alone through the strips, whose second walk takes 4 or 2 bytes a lane: while L2 holds the tensor, and a bf16 one, which
+// is bound by its instructions, somewhat beyond.  fp32 of 129 MB (1280 channels), 246 MB (1024) and 492 MB (2048): strips 153, 282 and
+// 548 us, the column reductions 80, 136 and 272; bf16 of 138 MB (1152) and 246 MB (2048): 185 and 409 against 232 and 328.  (Below the
+// line 1280 fp32 channels are the faster in column reductions from 65 MB on, 52 us against 83, and 1024 in strips up to 131 MB, 89
+// against 91.)
+static bool strip_statistics(int dtype, uint64_t rows, uint32_t channels)
+{
+    return dtype == QP_F32 ? rows * channels <= 32000000ull : rows * channels <= 100000000ull;
+}
+
 extern "C" int32_t qp_stats_channels(qp_ctx* ctx, const void* d_x, int dtype, uint64_t rows, uint32_t channels,
                                      qp_stats_t* d_out, void* stream)
 {
@@ -721,7 +731,7 @@ extern "C" int32_t qp_stats_channels(qp_ctx* ctx, const void* d_x, int dtype, ui
             return qp_check_launch(ctx, "qp_stats_channels");
         return QP_OK;
     }
-    if (qp_channel_strips_apply(ctx, rows, channels, 0))
+    if (strip_statistics(dtype, rows, channels) && qp_channel_strips_apply(ctx, rows, channels, 0))
         return qp_launch_channel_strips(ctx, d_x, dtype, rows, channels, nullptr, d_out, 0, 0, QP_DEFAULT_STEPS, 0, 0, 0.0, nullptr,
                                         nullptr, nullptr, nullptr, nullptr, s);
     if (dtype == QP_F32) return stats_channels_typed<float>(ctx, static_cast<const float*>(d_x), rows, channels, d_out, s);

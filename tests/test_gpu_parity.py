@@ -1469,6 +1469,29 @@ def test_channels_full_size_c2_sampled(ctx):
     assert ctx.qp_get_status() == 0
 
 
+@pytest.mark.parametrize("rows,channels,bf16", [(25000, 1280, False), (25001, 1280, False), (65500, 1526, True), (65500, 1527, True)])
+def test_channels_statistics_on_both_sides_of_the_strips_limit(ctx, rows, channels, bf16):
+    """32e6 fp32 and 1e8 bf16 elements are the last that the strips take the statistics of: every channel against sums in 64
+    bits (fp32 chains of at most 16 terms: 16 * 2^-24), and the sender that follows from them."""
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    x = torch.randn(rows, channels, device="cuda", generator=g) * 0.7 + torch.randn(channels, device="cuda", generator=g)
+    x = x.to(torch.bfloat16) if bf16 else x
+    st = _read_array(ctx.qp_stats_channels(x, channels), qp.Stats, channels)
+    for c0 in range(0, channels, 64):                    # (64 bits in pieces)
+        d = x[:, c0:c0 + 64].double()
+        mean, lo, hi = d.mean(0), d.amin(0), d.amax(0)
+        mad, var, ab = (d - mean).abs().mean(0), d.var(0, unbiased=False), d.abs().mean(0)
+        for i, (m, a, v, b, mn, mx) in enumerate(zip(*(t.tolist() for t in (mean, mad, var, ab, lo, hi)))):
+            s = st[c0 + i]
+            assert (s.n, s.nonfinite, s.min, s.max) == (rows, 0, mn, mx)
+            assert abs(s.mean - m) <= 1e-6 * b and abs(s.mad - a) <= 1e-6 * a and abs(s.var - v) <= 1e-6 * v and abs(s.mean_abs - b) <= 1e-6 * b
+    st2 = torch.zeros(ctypes.sizeof(qp.Stats) * channels, dtype=torch.uint8, device="cuda")
+    packed, d_qp = ctx.qp_sender_channels_device(x, channels, 8, qp.QP_CLIP_ACIQ, out_stats=st2)
+    assert all(bytes(a) == bytes(b) for a, b in zip(_read_array(st2, qp.Stats, channels), st))
+    assert torch.equal(packed, ctx.qp_quantize_pack_channels(x, channels, 8, d_qp))
+    assert ctx.qp_get_status() == 0
+
+
 def test_channels_sender_in_one_call(ctx):
     x = si.vit_activation((2, 197, 384), 109, outlier_frac=0.02).reshape(-1)
     d = dev(x)
