@@ -194,7 +194,8 @@ int qp_stats_carries_histogram(const void* d_x, int dtype, uint64_t n, int hist_
  *                         which walks backwards, on them).  Falls back to two kernels on a device
  *                         that cannot hold it.
  *   QP_STATS_AUTO         the streaming launch that the search and the senders use as well: up to 2^18
- *                         elements one thread-block cluster, above that one block per SM (default)
+ *                         elements one thread-block cluster, above that one block per SM; fp32 with the
+ *                         histogram above 2^25 elements as QP_STATS_FUSED (default)
  * A grid barrier or tile wait of the cooperative launch that runs out sets QP_DEV_STREAM_TIMEOUT
  * and the launch ends without output. */
 enum { QP_STATS_AUTO = 0, QP_STATS_TWO_KERNELS = 1, QP_STATS_FUSED = 2 };
@@ -290,7 +291,7 @@ int32_t qp_dsaciq_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, co
  *   QP_SEARCH_INTERVALS   one pass gathers moments per interval between the candidates'
  *                         decision thresholds; used where (steps+1)*(2^bits-1) <= 2048 and
  *                         n < ~1.8e9, otherwise the call falls back to the first way
- *   QP_SEARCH_AUTO        at 1..4 bits, up to 255 steps, 16-byte aligned and n >= 8192 (4 bits: 32768) the
+ *   QP_SEARCH_AUTO        at 1..4 bits, up to 255 steps, 16-byte aligned and n >= 8192 (4 bits: 128 KB) the
  *                         intervals in one streaming launch that numbers them by arithmetic instead of
  *                         looking them up; otherwise for n >= 2^20 the intervals where they apply (default)
  * The pass over x that gathers the moments has two forms with identical results: the plain one

@@ -955,14 +955,16 @@ bool ss_usable(qp_ctx* ctx)
 }  // namespace
 
 // 16-byte aligned tensors; statistics with the histogram from 128 KB on (where qp_stats_carries_histogram says so), the search
-// from 8 tiles on (at 4 bits 32): 11 to 23 us by width up to 2^20 elements, where the candidates scored one by one take 23 us at 2^15,
-// 33 at 2^18 and 60 at 2^20.  At 1..4 bits (each further code boundary costs two instructions per element: at 5 bits and up the
+// from 8 tiles on, at 4 bits from 128 KB: 12 to 23 us by width up to 2^20 elements, where the candidates scored one by one take 23 us at
+// 2^15, 33 at 2^18 and 60 at 2^20.  (Below 128 KB the statistics carry no histogram and the launch counts it as well: 17 to 28 us at 1..3
+// bits, 33 at 4, against 25 to 29.)  At 1..4 bits (each further code boundary costs two instructions per element: at 5 bits and up the
 // interval pass with its table is the cheaper one) and up to 256 candidates (tables that leave a replica to every
 // eighth lane at least).
 bool qp_stats_search_applies(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int hist_bins, int bits, int steps)
 {
     if (((uintptr_t)d_x & 15u) || hist_bins < 1 || hist_bins > SS_MAX_HIST) return false;
-    if (bits ? n < (bits == 4 ? 32 : 8) * SS_TILE : n * (dtype == QP_F32 ? 4 : 2) < 131072) return false;
+    const bool small = n * (dtype == QP_F32 ? 4 : 2) < 131072;
+    if (bits == 0 || bits == 4 ? small : n < 8 * SS_TILE) return false;
     if (bits && (bits > 4 || steps + 1 > QP_SS_MAX_CAND)) return false;
     return ss_usable(ctx);
 }

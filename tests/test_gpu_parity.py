@@ -184,7 +184,7 @@ def test_stats_one_launch_against_oracle_and_two_kernels(ctx, tiles, tail):
     assert ctx.qp_get_status() == 0
 
 
-@pytest.mark.parametrize("n", [8 * 1024, (1 << 18) + 1, 1500 * 8192 + 77, (96 << 18) + 9])
+@pytest.mark.parametrize("n", [8 * 1024, (1 << 18) + 1, 1500 * 8192 + 77, (96 << 18) + 9, 1 << 25, (1 << 25) + 1])
 @pytest.mark.parametrize("data", ["plain", "two_levels", "outliers"])
 def test_stats_default_path_agrees_with_the_forced_ones(ctx, n, data):
     """Bounds: an fp32 chain adds at most 16 terms of one sign (u = 2^-24 each), a squared deviation brings 3 u more:
@@ -1125,6 +1125,14 @@ def test_search_streaming_small(ctx, bits, n):
     assert at > before
     assert bits == 4 and n < 32768 or ctx.qp_launch_count() - at <= 2  # the histogram where the statistics do not carry it
     check_search(ctx, x, d, bits, exact_steps=None if n < 1 << 17 else (0, 50, 100))
+
+
+@pytest.mark.parametrize("n", [(1 << 16) - 8, 1 << 16])    # at 4 bits the line between the candidates and the streaming launch
+def test_search_bf16_at_128_kb(ctx, n):
+    h = si.to_bf16_bits(si.vit_activation((1, n, 1), 65, outlier_frac=0.001).reshape(-1))
+    d = torch.from_numpy(h.view(np.int16)).cuda().view(torch.bfloat16)
+    check_search(ctx, oracle.widen_bf16(h), d, 4)
+    assert ctx.qp_get_status() == 0
 
 
 # statistics about a pilot centre (96 MB and more: 25165824 fp32 elements) and in two streaming passes (below), tiles of 1024
