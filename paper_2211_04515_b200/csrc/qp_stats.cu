@@ -914,15 +914,19 @@ int32_t qp_launch_stats(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int
     }
     const uint64_t ntiles = ((uintptr_t)d_x & 15u) ? 0 : n * (dtype == QP_F32 ? 4 : 2) / ST_TILE;
     // QP_STATS_AUTO takes the streaming launches wherever they apply: 12.4 us at 2^20 fp32 elements against 14.5 in one launch of
-    // bulk-copied tiles and 16.5 in two kernels, 102 against 157 at 2^27; with the histogram 30.6 us for 52 MB.
+    // bulk-copied tiles and 16.5 in two kernels, 102 against 157 at 2^27; with the histogram 30.6 us for 52 MB.  But fp32 with the
+    // histogram above 2^25 elements: there the bulk-copied tiles, the last of which stay in shared memory for the second pass, read
+    // DRAM faster: 2^25, 2^26, 2^27 and 2^28 elements in 53, 90, 165 and 319 us, streaming 53, 97, 185 and 361, two kernels 59,
+    // 98, 177 and 331.  (bf16 is bound by its instructions: streaming 211 us at 2^28, 279 and 233 in the others.)
     // QP_STATS_FUSED and QP_STATS_TWO_KERNELS force the other two.
     const bool with_hist = hist_bins >= 1 && hist_bins <= ST_FUSED_HIST_MAX;
-    if (ctx->stats_path == QP_STATS_AUTO && with_hist && ntiles >= 8 &&
+    const bool tiles = with_hist && dtype == QP_F32 && n > (1ull << 25) && ntiles >= 8 && stats_fused_usable(ctx);
+    if (ctx->stats_path == QP_STATS_AUTO && with_hist && !tiles && ntiles >= 8 &&
         qp_stats_search_applies(ctx, d_x, dtype, n, hist_bins, 0, 0))
         return qp_launch_stats_search(ctx, d_x, dtype, n, nullptr, d_out, hist_bins, 0, 0, 0, 0.0, nullptr, nullptr, nullptr, s);
     if (ctx->stats_path == QP_STATS_AUTO && !with_hist && qp_stats_onepass_applies(ctx, d_x, n))
         return qp_launch_stats_onepass(ctx, d_x, dtype, n, d_out, 0, 0, 0, 0.0, nullptr, nullptr, s);
-    const bool one_launch = ctx->stats_path == QP_STATS_FUSED;
+    const bool one_launch = ctx->stats_path == QP_STATS_FUSED || (ctx->stats_path == QP_STATS_AUTO && tiles);
     if (ntiles >= 8 && one_launch && stats_fused_usable(ctx)) {
         if (dtype == QP_F32) return launch_fused<float>(ctx, static_cast<const float*>(d_x), n, hist_bins, d_out, s);
         return launch_fused<unsigned short>(ctx, static_cast<const unsigned short*>(d_x), n, hist_bins, d_out, s);
