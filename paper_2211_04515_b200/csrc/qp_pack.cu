@@ -58,8 +58,8 @@ __global__ void __launch_bounds__(QP_THREADS) pack_kernel(const T* __restrict__ 
     if constexpr (sizeof(T) == 2) {
         const uint64_t whole = n / TILE;
         for (; it < whole; it += wstride)
-            qp_pack_tile<BITS, T, VEC>(x, n, reverse ? whole - 1 - it : it, true, lane, q.lo, q.hi, q.inv, out, nwords, stage[warp]);
-        if (it < ntiles) qp_pack_tile<BITS, T, VEC>(x, n, it, false, lane, q.lo, q.hi, q.inv, out, nwords, stage[warp]);
+            qp_pack_tile<BITS, T, VEC, true>(x, n, reverse ? whole - 1 - it : it, lane, q.lo, q.hi, q.inv, out, nwords, stage[warp]);
+        if (it < ntiles) qp_pack_tile<BITS, T, VEC>(x, n, it, lane, q.lo, q.hi, q.inv, out, nwords, stage[warp]);
     } else {
         for (; it < ntiles; it += wstride)
             qp_pack_tile<BITS, T, VEC>(x, n, reverse ? ntiles - 1 - it : it, lane, q.lo, q.hi, q.inv, out, nwords, stage[warp]);

@@ -33,14 +33,15 @@ __device__ __forceinline__ void qp_quads_to_words(const uint32_t* sw, int g, uin
 // Packs tile `tile` of x (n elements; the last tile may be partial: its missing elements are NaN, code 0) into `out`,
 // of which nwords exist (pad words included).  VEC: x is 16-byte aligned; otherwise every lane loads the
 // elements of its vectors one by one (the loads of a vector touch the same lines, so they hit L1).
-// sw: 256 words of shared memory of this warp.  full: the tile has all its elements.
-template <int BITS, typename T, bool VEC>
-__device__ __forceinline__ void qp_pack_tile(const T* __restrict__ x, uint64_t n, uint64_t tile, bool full, int lane, float lo,
-                                             float hi, float inv, uint32_t* __restrict__ out, uint64_t nwords, uint32_t* sw)
+// sw: 256 words of shared memory of this warp.  ALL: the caller knows that the tile has all its elements.
+template <int BITS, typename T, bool VEC, bool ALL = false>
+__device__ __forceinline__ void qp_pack_tile(const T* __restrict__ x, uint64_t n, uint64_t tile, int lane, float lo, float hi,
+                                             float inv, uint32_t* __restrict__ out, uint64_t nwords, uint32_t* sw)
 {
     constexpr int EPV = qp_span<T>::EPV;          // 4 (f32) or 8 (bf16) elements per 16-byte vector
     constexpr int NLOAD = QP_TILE / (32 * EPV);   // 8 or 4 vector loads per lane
     const T* xt = x + tile * QP_TILE;
+    const bool full = ALL || (tile + 1) * QP_TILE <= n;          // warp-uniform
     float e[NLOAD][EPV];
     if (full) {
 #pragma unroll
@@ -103,16 +104,10 @@ __device__ __forceinline__ void qp_pack_tile(const T* __restrict__ x, uint64_t n
 #pragma unroll
         for (int m = 0; m < BITS; ++m) sw[lane * BITS + m] = w[m];
         __syncwarp();
-        const int room = full ? 32 * BITS : (int)min((uint64_t)(32 * BITS), nwords - tile * (32 * BITS));
+        const int room = ALL ? 32 * BITS : (int)min((uint64_t)(32 * BITS), nwords - tile * (32 * BITS));
 #pragma unroll
         for (int m = 0; m < BITS; ++m)
             if (m * 32 + lane < room) ot[m * 32 + lane] = sw[m * 32 + lane];
     }
     __syncwarp();
-}
-template <int BITS, typename T, bool VEC>
-__device__ __forceinline__ void qp_pack_tile(const T* __restrict__ x, uint64_t n, uint64_t tile, int lane, float lo, float hi,
-                                             float inv, uint32_t* __restrict__ out, uint64_t nwords, uint32_t* sw)
-{
-    qp_pack_tile<BITS, T, VEC>(x, n, tile, (tile + 1) * QP_TILE <= n, lane, lo, hi, inv, out, nwords, sw);   // (warp-uniform)
 }

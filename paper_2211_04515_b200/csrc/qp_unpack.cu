@@ -59,11 +59,11 @@ __device__ __forceinline__ void store_out(unsigned short* y, uint64_t i4, const 
 __device__ __forceinline__ void store_one(float* y, uint64_t i, float v) { y[i] = v; }
 __device__ __forceinline__ void store_one(unsigned short* y, uint64_t i, float v) { y[i] = qp_f32_to_bf16(v); }
 
-// One tile; full: it has all its elements, otherwise its words are read up to nwords and its elements written up to n.  VEC: y
+// One tile; unless it has all its elements (ALL: the caller knows that it has), its words are read up to nwords and its elements written up to n.  VEC: y
 // is aligned for 4-element stores; otherwise the elements are stored one by one.
-template <int BITS, typename TO, bool VEC, bool HOST>
-__device__ __forceinline__ void unpack_tile(const uint32_t* __restrict__ in, uint64_t n, uint64_t nwords, uint64_t tile, bool full,
-                                            int lane, const DQ& q, uint32_t* sw, TO* __restrict__ y, uint32_t* __restrict__ work,
+template <int BITS, typename TO, bool VEC, bool HOST, bool ALL = false>
+__device__ __forceinline__ void unpack_tile(const uint32_t* __restrict__ in, uint64_t n, uint64_t nwords, uint64_t tile, int lane,
+                                            const DQ& q, uint32_t* sw, TO* __restrict__ y, uint32_t* __restrict__ work,
                                             TO* __restrict__ y_host)
 {
     constexpr unsigned MASK = (1u << BITS) - 1u;
@@ -71,6 +71,7 @@ __device__ __forceinline__ void unpack_tile(const uint32_t* __restrict__ in, uin
     constexpr unsigned QMASK = QB >= 32 ? 0xFFFFFFFFu : ((1u << (QB & 31)) - 1u);
     const uint32_t* it = in + tile * (32 * BITS);
     uint32_t* wk = HOST ? work + tile * (32 * BITS) : nullptr;
+    const bool full = ALL || (tile + 1) * TILE <= n;              // warp-uniform
     uint32_t w[BITS];
     if (full && BITS == 8) {
         const uint4 a = __ldg(reinterpret_cast<const uint4*>(it + lane * 8));
@@ -90,7 +91,7 @@ __device__ __forceinline__ void unpack_tile(const uint32_t* __restrict__ in, uin
         w[0] = a.x; w[1 % BITS] = a.y;
         if constexpr (HOST) *reinterpret_cast<uint2*>(wk + lane * 2) = a;
     } else {
-        const int room = full ? 32 * BITS : (int)min((uint64_t)(32 * BITS), nwords - tile * (32 * BITS));
+        const int room = ALL ? 32 * BITS : (int)min((uint64_t)(32 * BITS), nwords - tile * (32 * BITS));
 #pragma unroll
         for (int m = 0; m < BITS; ++m) {
             const uint32_t v = m * 32 + lane < room ? __ldg(it + m * 32 + lane) : 0u;
@@ -157,11 +158,10 @@ __global__ void __launch_bounds__(QP_THREADS) unpack_kernel(const uint32_t* __re
     uint64_t tile = (uint64_t)blockIdx.x * warps + warp;
     if constexpr (sizeof(TO) == 2) {
         for (const uint64_t whole = n / TILE; tile < whole; tile += wstride)
-            unpack_tile<BITS, TO, VEC, HOST>(in, n, nwords, tile, true, lane, q, sw, y, work, y_host);
-        if (tile < ntiles) unpack_tile<BITS, TO, VEC, HOST>(in, n, nwords, tile, false, lane, q, sw, y, work, y_host);
+            unpack_tile<BITS, TO, VEC, HOST, true>(in, n, nwords, tile, lane, q, sw, y, work, y_host);
+        if (tile < ntiles) unpack_tile<BITS, TO, VEC, HOST>(in, n, nwords, tile, lane, q, sw, y, work, y_host);
     } else {
-        for (; tile < ntiles; tile += wstride)                    // (warp-uniform)
-            unpack_tile<BITS, TO, VEC, HOST>(in, n, nwords, tile, (tile + 1) * TILE <= n, lane, q, sw, y, work, y_host);
+        for (; tile < ntiles; tile += wstride) unpack_tile<BITS, TO, VEC, HOST>(in, n, nwords, tile, lane, q, sw, y, work, y_host);
     }
 }
 
