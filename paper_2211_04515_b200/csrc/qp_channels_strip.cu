@@ -144,7 +144,7 @@ struct CtMomentsGuarded {                          // a column with non-finite v
 };
 
 // Deviations about the fp32 mean, summed in fp64 (as the per-tensor kernel), and the histogram.
-template <bool SUMS, bool HIST, bool GUARD>
+template <bool SUMS, bool HIST, int CARE>                     // CARE: as in the per-tensor kernel
 struct CtDeviations {
     float m, mn, inv_w;
     unsigned base, nb;                             // byte address of the channel's first bin, less what the float's bits bring
@@ -152,7 +152,7 @@ struct CtDeviations {
     unsigned below = 0u;
     __device__ __forceinline__ void one(float v)
     {
-        if (GUARD && !qp_is_finite(v)) return;
+        if (CARE == 2 && !qp_is_finite(v)) return;
         if (SUMS) {
             const float y = __fsub_rn(v, m);
             const double d = (double)y;
@@ -162,9 +162,10 @@ struct CtDeviations {
         }
         if (HIST) {                                // bin = floor((x - min) * inv_w), each operation rounded; x = max may give nb
             float pos = __fmul_rn(__fsub_rn(v, mn), inv_w);
-            if (GUARD) pos = fminf(fmaxf(pos, 0.f), (float)nb);       // (as the per-tensor kernel)
-            const unsigned b = QP_CK(__float_as_uint(__fadd_rd(pos, SS_MAGIC)) - SS_ONE, nb + 1) + SS_ONE;
-            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(b * 4u + base) : "memory");
+            if (CARE == 2) pos = fminf(fmaxf(pos, 0.f), (float)nb);
+            unsigned bin = __float_as_uint(__fadd_rd(pos, SS_MAGIC)) - SS_ONE;
+            if (CARE == 1) bin = min(bin, nb);
+            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"((QP_CK(bin, nb + 1) + SS_ONE) * 4u + base) : "memory");
         }
     }
     __device__ __forceinline__ void fold() {}
@@ -301,8 +302,8 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
         if ((int)threadIdx.x < nch) s_st[threadIdx.x] = a.st_in[c0 + threadIdx.x];
     }
     auto inv_w = [&](const qp_stats_t& q) { return SEARCH && q.max > q.min ? (float)((double)a.nb / (q.max - q.min)) : 0.f; };
-    // a channel whose histogram positions may leave its bins (the caller's statistics may be of another tensor)
-    const bool beyond = __syncthreads_or((int)threadIdx.x < nch && SEARCH && (!STATS || !ss_range_fits(s_st[threadIdx.x], inv_w(s_st[threadIdx.x]))));
+    // a channel whose histogram positions are not all numbers
+    const bool beyond = __syncthreads_or((int)threadIdx.x < nch && SEARCH && !ss_range_fits(s_st[threadIdx.x], inv_w(s_st[threadIdx.x])));
     bool odd = false;                                         // a channel with non-finite values: uniform over the cluster
     for (int i = 0; i < nch; ++i) odd |= s_st[i].nonfinite != 0;
 
@@ -310,8 +311,8 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
     {
         const qp_stats_t& my = s_st[slot < nch ? slot : 0];
         double v3[3];
-        auto pass = [&](auto guard_tag) {
-            CtDeviations<STATS, SEARCH, decltype(guard_tag)::value> d;
+        auto pass = [&](auto care) {
+            CtDeviations<STATS, SEARCH, decltype(care)::value> d;
             d.m = (float)my.mean;
             d.mn = (float)my.min;
             d.inv_w = inv_w(my);
@@ -320,7 +321,7 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
             ct_column<T>(mine, m, d);
             v3[0] = d.sd; v3[1] = d.sv; v3[2] = (double)d.below;
         };
-        if (odd || beyond) pass(std::true_type{}); else pass(std::false_type{});
+        if (odd || beyond) pass(std::integral_constant<int, 2>{}); else pass(std::integral_constant<int, STATS ? 0 : 1>{});
         if constexpr (STATS) {
             ct_reduce<0, 0, 0>(v3, red, rl, nl, w);
             if (rl == 0)

@@ -127,8 +127,9 @@ struct SsMoments {
 // ---- phase B: deviations and histogram.  bin = floor((x - min) * inv_w) in fp32, each operation rounded on its
 // own; x = max may come out as bin nb, which is counted with the last one.  The floor is taken by adding 2^23
 // rounding down; the bin number then sits in the low bits, and one multiply-add makes the address.  Positions are in
-// [0, nb] where the range of the tensor and its reciprocal are finite in fp32 and the statistics are this tensor's;
-// GUARD (non-finite elements, or not so) clamps them: NaN, of 0 * inf, to bin 0, what overflows to the last one.
+// [0, nb] where the range of the tensor and its reciprocal are finite in fp32 and the statistics are this tensor's.
+// CARE 1 (the caller's statistics) keeps the bin's number in range, CARE 2 (non-finite elements, or such a range) clamps the
+// position: NaN, of 0 * inf, to bin 0, what overflows to the last one.
 // The deviations are taken about m, the mean in fp32 (one rounding per element, none where x and m are of a size), and
 // moved to the mean itself by the counts of the two sides: sum |x - mean| = sum |x - m| - dm (N_up - N_down).  Their
 // sums are taken in fp64: the search subtracts nearly all of sum y^2 again, and the conversion and fp64 pipes are idle here.
@@ -138,21 +139,23 @@ struct SsDeviations {
     double sd[2], sv[2];
     unsigned below;                                           // elements below m
     qp_f2 nm, nmn;
-    template <bool GUARD>
+    template <int CARE>
     __device__ __forceinline__ void count(float pos, float x) const
     {
-        if (GUARD) pos = fminf(fmaxf(pos, 0.f), (float)nb);
-        const unsigned addr = (QP_CK(__float_as_uint(__fadd_rd(pos, SS_MAGIC)) - SS_ONE, nb + 1) + SS_ONE) * hist_mul + hist_base;
-        if (!GUARD || qp_is_finite(x)) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory");
+        if (CARE == 2) pos = fminf(fmaxf(pos, 0.f), (float)nb);
+        unsigned bin = __float_as_uint(__fadd_rd(pos, SS_MAGIC)) - SS_ONE;
+        if (CARE == 1) bin = min(bin, nb);
+        const unsigned addr = (QP_CK(bin, nb + 1) + SS_ONE) * hist_mul + hist_base;
+        if (CARE < 2 || qp_is_finite(x)) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory");
     }
     __device__ __forceinline__ void begin() {}
-    template <bool GUARD>
+    template <int CARE>
     __device__ __forceinline__ void take(float a, float b, int)
     {
         float da, db, pa, pb;
         const qp_f2 p = qp_pack2(a, b);
         qp_unpack2(qp_add2(p, nm), da, db);
-        if (GUARD) {
+        if (CARE == 2) {
             da = qp_is_finite(a) ? da : 0.f;
             db = qp_is_finite(b) ? db : 0.f;
         }
@@ -164,8 +167,8 @@ struct SsDeviations {
         below += __float_as_uint(da) >> 31;
         below += __float_as_uint(db) >> 31;
         qp_unpack2(qp_add2(p, nmn), pa, pb);
-        count<GUARD>(__fmul_rn(pa, inv_w), a);
-        count<GUARD>(__fmul_rn(pb, inv_w), b);
+        count<CARE>(__fmul_rn(pa, inv_w), a);
+        count<CARE>(__fmul_rn(pb, inv_w), b);
     }
     __device__ __forceinline__ void end() {}
     __device__ __forceinline__ void one(float v)
@@ -175,14 +178,14 @@ struct SsDeviations {
         below += d < 0.0;
         sd[0] += fabs(d);
         sv[0] = fma(d, d, sv[0]);
-        count<true>(__fmul_rn(__fsub_rn(v, mn), inv_w), v);
+        count<2>(__fmul_rn(__fsub_rn(v, mn), inv_w), v);
     }
 };
-template <bool GUARD>
+template <int CARE>
 struct SsDeviationsOf {                                       // the stream's view of it
     SsDeviations& d;
     __device__ __forceinline__ void begin() { d.begin(); }
-    __device__ __forceinline__ void pair(float a, float b, int i) { d.take<GUARD>(a, b, i); }
+    __device__ __forceinline__ void pair(float a, float b, int i) { d.take<CARE>(a, b, i); }
     __device__ __forceinline__ void end() { d.end(); }
 };
 
@@ -191,7 +194,7 @@ struct SsDeviationsOf {                                       // the stream's vi
 template <typename T>
 __device__ __noinline__ void ss_guarded_deviations(const T* x, uint64_t ntiles, uint64_t first, uint64_t step, int lane, SsDeviations& d)
 {
-    SsDeviationsOf<true> f = {d};
+    SsDeviationsOf<2> f = {d};
     SsTiles<T, SS_TILE>::template run<true>(x, ntiles, first, step, lane, f);
 }
 
@@ -541,10 +544,19 @@ __host__ __device__ constexpr int ss_ctile(int hh) { return hh >= 3 ? 512 : 1024
 
 // STATS: phases A and B (otherwise the statistics come with st_in, and B runs only if they lack the histogram).
 // HH: code boundaries above the centre, 2^bits / 2 - 1; -1: statistics only.
-// Returns false where a wait ran out; before (in thread 0): what count_out returned if the block has counted itself out.
-constexpr unsigned SS_IN = 0xFFFFFFFFu;
+// What the last block out does, with what count_out returned (and whether the block itself gave up): one thread.
+__device__ __forceinline__ void ss_out(const SsArgs& a, unsigned before)
+{
+    if (!qp_grid::last_out(before, gridDim.x)) return;
+    if (before >= qp_grid::GAVE_UP)                           // (block 0 of an undisturbed launch has cleaned)
+        for (int b = 0; b < a.nb; ++b) a.hist[b] = 0ull;
+    qp_grid::reset(a.bar);
+}
+
+// Returns SS_GAVE_UP where a wait ran out, SS_OUT where the block has counted itself out (or is one of a cluster).
+enum { SS_GAVE_UP, SS_DONE, SS_OUT };
 template <typename T, bool STATS, int HH>
-__device__ __forceinline__ bool ss_run(const SsArgs& a, unsigned& before)
+__device__ __forceinline__ int ss_run(const SsArgs& a)
 {
     constexpr bool SEARCH = HH >= 0;
     constexpr int H = SEARCH ? HH : 0;
@@ -618,7 +630,7 @@ __device__ __forceinline__ bool ss_run(const SsArgs& a, unsigned& before)
             double* p = a.part + (size_t)blockIdx.x * 8;
             p[0] = v5[0]; p[1] = v5[1]; p[2] = v5[2]; p[3] = v5[3]; p[4] = v5[4];
         }
-        if (!meet()) return false;
+        if (!meet()) return SS_GAVE_UP;
         // one warp merges the partials (all loads in flight together), the rest of the block waits at the barrier below
         if (threadIdx.x < 32) {
             double m5[5] = {0.0, 0.0, inf, -inf, 0.0};
@@ -675,12 +687,12 @@ __device__ __forceinline__ bool ss_run(const SsArgs& a, unsigned& before)
             d.below = 0u;
             d.nm = qp_pack2(-d.m, -d.m);
             d.nmn = qp_pack2(-d.mn, -d.mn);
-            if (guard || !STATS || !ss_range_fits(s_st, d.inv_w)) {
+            if (guard || !ss_range_fits(s_st, d.inv_w)) {
                 SsDeviations g = d;
                 ss_guarded_deviations<T>(x, a.ntiles, first, step, lane, g);
                 d.sd[0] = g.sd[0]; d.sd[1] = g.sd[1]; d.sv[0] = g.sv[0]; d.sv[1] = g.sv[1]; d.below = g.below;
             } else {
-                SsDeviationsOf<false> f = {d};
+                SsDeviationsOf<STATS ? 0 : 1> f = {d};
                 SsTiles<T, SS_TILE>::template run<true>(x, a.ntiles, first, step, lane, f);
             }
             if (blockIdx.x == G - 1)
@@ -700,16 +712,17 @@ __device__ __forceinline__ bool ss_run(const SsArgs& a, unsigned& before)
             if (c) atomicAdd(&a.hist[b], c);
         }
         if constexpr (SEARCH) {
-            if (!meet()) return false;
+            if (!meet()) return SS_GAVE_UP;
         } else {                                              // statistics only: the last block out finishes
             __threadfence();
             __syncthreads();
             if (threadIdx.x == 0) {
-                before = qp_grid::count_out(a.bar);
+                const unsigned before = qp_grid::count_out(a.bar);
                 s_last = before == G - 1;                     // (with a block that gave up among those before: no output)
+                if (!s_last) ss_out(a, before);
             }
             __syncthreads();
-            if (!s_last) return true;
+            if (!s_last) return SS_OUT;
             __threadfence();
         }
         if (threadIdx.x < 32) {
@@ -751,7 +764,11 @@ __device__ __forceinline__ bool ss_run(const SsArgs& a, unsigned& before)
             }
         }
         __syncthreads();
-        if constexpr (!SEARCH) scratch_clean();
+        if constexpr (!SEARCH) {
+            scratch_clean();
+            if (threadIdx.x == 0) qp_grid::reset(a.bar);
+            return SS_OUT;
+        }
     }
 
     // ---- phase C
@@ -852,15 +869,14 @@ __device__ __forceinline__ bool ss_run(const SsArgs& a, unsigned& before)
         }
         const int count = hard ? h.M + 1 : 2 * ni;
         if (!cluster) {
-            if (!meet()) return false;
+            if (!meet()) return SS_GAVE_UP;
             ss_slices(a, count, raw + SS_TABLE_BYTES);
         }
         arrive();
         if (blockIdx.x == 0) {
             int* pos = reinterpret_cast<int*>(raw + SS_TABLE_BYTES);          // [ncand][H + 2] in the histogram's room (the slices are stored)
             if (!hard) ss_places<H>(s_plan, ncand, ni, s_edge, s_cell, pos);
-            if (!wait((waits + 1) * G)) return false;
-            if (!cluster && !a.packed && threadIdx.x == 0) before = qp_grid::count_out(a.bar);   // (here: the answer comes meanwhile)
+            if (!wait((waits + 1) * G)) return SS_GAVE_UP;
             if (cluster) ss_all_slices(a, count);
             if (!hard) {
                 ss_finish<H>(a, s_plan, s_st, ncand, ni, s_cell, pos, s_cand, s_valid, s_curve, s_red, reinterpret_cast<double*>(raw));
@@ -872,9 +888,11 @@ __device__ __forceinline__ bool ss_run(const SsArgs& a, unsigned& before)
                 ss_reduce<0, 0>(v2, s_red);
                 ss_hard_finish(a, h, s_plan.m, s_st, ncand, v2[0], v2[1], s_cand, s_valid, s_curve, s_red);
             }
+            // (a warp that the pick does not wait for asks meanwhile)
+            if (!cluster && !a.packed && threadIdx.x == SS_THREADS - 1) ss_out(a, qp_grid::count_out(a.bar));
             ss_pick(a, ncand, s_curve, s_cand, s_valid, s_setup);
             scratch_clean();
-            if (!a.packed) return true;
+            if (!a.packed) return SS_OUT;
             arrive();
         } else {
             if (cluster) {
@@ -883,11 +901,11 @@ __device__ __forceinline__ bool ss_run(const SsArgs& a, unsigned& before)
             }
             if (!a.packed) {
                 if (threadIdx.x == 0) __threadfence();        // (the arrival, which nobody here polls for)
-                return true;
+                return SS_DONE;
             }
         }
         if constexpr (STATS) {                                // the sender: everybody packs, from the tensor's end
-            if (!wait((waits + 1) * G + 1)) return false;
+            if (!wait((waits + 1) * G + 1)) return SS_GAVE_UP;
             const float lo = __ldcg(&a.qp_out->lo), hi = __ldcg(&a.qp_out->hi), inv = __ldcg(&a.qp_out->inv_scale);
             uint32_t* sw = reinterpret_cast<uint32_t*>(raw) + (threadIdx.x >> 5) * 256;
             const uint64_t tiles = (a.n + QP_TILE - 1) / QP_TILE;
@@ -895,20 +913,16 @@ __device__ __forceinline__ bool ss_run(const SsArgs& a, unsigned& before)
                 qp_pack_tile<BITS, T, true>(x, a.n, tiles - 1 - it, lane, lo, hi, inv, a.packed, a.nwords, sw);
         }
     }
-    return true;
+    return SS_DONE;
 }
 
 template <typename T, bool STATS, int HH>
 __global__ void __launch_bounds__(SS_THREADS, 1) stats_search_kernel(const SsArgs a)
 {
-    unsigned before = SS_IN;
-    const unsigned gave_up = ss_run<T, STATS, HH>(a, before) ? 0u : qp_grid::GAVE_UP;
-    if (threadIdx.x != 0 || (a.cluster && before == SS_IN)) return;
-    if (before == SS_IN) before = qp_grid::count_out(a.bar, gave_up) | gave_up;
-    if (!qp_grid::last_out(before, gridDim.x)) return;
-    if (before >= qp_grid::GAVE_UP)                           // (only block 0 of an undisturbed launch has cleaned)
-        for (int b = 0; b < a.nb; ++b) a.hist[b] = 0ull;
-    qp_grid::reset(a.bar);
+    const int how = ss_run<T, STATS, HH>(a);
+    if (threadIdx.x != 0 || a.cluster || how == SS_OUT) return;
+    const unsigned gave_up = how == SS_GAVE_UP ? qp_grid::GAVE_UP : 0u;
+    ss_out(a, qp_grid::count_out(a.bar, gave_up) | gave_up);
 }
 
 template <typename T>
