@@ -119,8 +119,10 @@ int32_t qp_destroy(qp_ctx* ctx);
  * qp_last_error gives the whole word). */
 int32_t qp_get_status(qp_ctx* ctx, void* stream);
 /* Test hook for the time-out paths (no counterpart in the paper; not for production use).
- * Every wait inside the kernels is bounded: a wait for a tile copy by a number of clock
- * cycles, a wait at a grid-wide barrier by a number of polls.  This call replaces the limits
+ * Every wait that polls is bounded: a wait for a tile copy by a number of clock
+ * cycles, a wait at a grid-wide barrier by a number of polls.  (The hardware's barrier of a
+ * thread-block cluster waits for blocks that are resident together and needs no bound; with
+ * barrier_extra_arrivals the launches that would use it take the grid-wide one.)  This call replaces the limits
  * of later launches on this context: tile_wait_cycles < 0 and barrier_polls = 0 restore the
  * defaults (about two seconds; a quarter of a second at least); tile_wait_cycles = 0 makes a
  * wait give up at the first attempt that finds the copy still in flight.  (The second wait that
