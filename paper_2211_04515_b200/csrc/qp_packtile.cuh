@@ -41,7 +41,8 @@ __device__ __forceinline__ void qp_pack_tile(const T* __restrict__ x, uint64_t n
     constexpr int EPV = qp_span<T>::EPV;          // 4 (f32) or 8 (bf16) elements per 16-byte vector
     constexpr int NLOAD = QP_TILE / (32 * EPV);   // 8 or 4 vector loads per lane
     const T* xt = x + tile * QP_TILE;
-    const bool full = ALL || (tile + 1) * QP_TILE <= n;          // warp-uniform
+    bool full = (tile + 1) * QP_TILE <= n;                       // warp-uniform
+    if (ALL) full = true;
     float e[NLOAD][EPV];
     if (full) {
 #pragma unroll

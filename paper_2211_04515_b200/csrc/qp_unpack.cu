@@ -71,7 +71,8 @@ __device__ __forceinline__ void unpack_tile(const uint32_t* __restrict__ in, uin
     constexpr unsigned QMASK = QB >= 32 ? 0xFFFFFFFFu : ((1u << (QB & 31)) - 1u);
     const uint32_t* it = in + tile * (32 * BITS);
     uint32_t* wk = HOST ? work + tile * (32 * BITS) : nullptr;
-    const bool full = ALL || (tile + 1) * TILE <= n;              // warp-uniform
+    bool full = (tile + 1) * TILE <= n;                           // warp-uniform
+    if (ALL) full = true;
     uint32_t w[BITS];
     if (full && BITS == 8) {
         const uint4 a = __ldg(reinterpret_cast<const uint4*>(it + lane * 8));
