@@ -3,7 +3,8 @@
 // the same: a block that has polled `spin_limit` times without seeing `target` arrivals raises
 // QP_DEV_STREAM_TIMEOUT in the status word and reports failure, so the kernel can leave and
 // the context stays usable.  The counter must be zero when the launch starts and the kernel
-// resets it when its last block leaves; after a time-out qp_get_status clears it.
+// resets it when its last block leaves; after a time-out too where blocks leave through count_out,
+// by qp_get_status where they do not (the small-tensor sender).
 #pragma once
 
 #include <cuda_runtime.h>
