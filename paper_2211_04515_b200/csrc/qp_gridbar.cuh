@@ -24,6 +24,20 @@ __device__ __forceinline__ void arrive_release(unsigned* p)
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
 }
 
+// One thread polls until `target` arrivals; false when the wait ran out.
+__device__ __forceinline__ bool poll(const unsigned* bar, unsigned target, unsigned spin_limit, unsigned* status)
+{
+    unsigned spins = 0;
+    while (ld_acquire(bar) < target) {
+        if (++spins > spin_limit) {
+            atomicOr(status, QP_DEV_STREAM_TIMEOUT);
+            return false;
+        }
+        if (spins > 64) __nanosleep(64);
+    }
+    return true;
+}
+
 // All blocks arrive, then all leave.  The block's writes are ordered before the arrival by the
 // block barrier and the release; the acquire load orders the other blocks' writes before what
 // follows.  Returns false (for the whole block) when the wait ran out.  s_ok: one int of
@@ -33,40 +47,28 @@ __device__ __forceinline__ bool barrier(unsigned* bar, unsigned target, unsigned
     __syncthreads();
     if (threadIdx.x == 0) {
         arrive_release(bar);
-        int ok = 1;
-        unsigned spins = 0;
-        while (ld_acquire(bar) < target) {
-            if (++spins > spin_limit) {
-                ok = 0;
-                atomicOr(status, QP_DEV_STREAM_TIMEOUT);
-                break;
-            }
-            if (spins > 64) __nanosleep(64);
-        }
-        *s_ok = ok;
+        *s_ok = poll(bar, target, spin_limit, status);
     }
     __syncthreads();
     return *s_ok != 0;
 }
 
-// The wait alone, for a block that has arrived before (arrive_release by one thread behind a block barrier).
-__device__ __forceinline__ bool wait(const unsigned* bar, unsigned target, unsigned spin_limit, unsigned* status, int* s_ok)
+// The same for what warp 0 has written (and what the block had written before its last block barrier), and for what warp 0 reads
+// next; the other warps do not stop here.  By warp 0; the block learns from s_ok, behind its next barrier, whether the wait ran out.
+__device__ __forceinline__ void barrier_warp0(unsigned* bar, unsigned target, unsigned spin_limit, unsigned* status, int* s_ok)
 {
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        unsigned spins = 0;
-        while (ld_acquire(bar) < target) {
-            if (++spins > spin_limit) {
-                ok = 0;
-                atomicOr(status, QP_DEV_STREAM_TIMEOUT);
-                break;
-            }
-            if (spins > 64) __nanosleep(64);
+    __syncwarp();
+    if (threadIdx.x == 0) arrive_release(bar);
+    unsigned spins = 0;
+    while (__any_sync(0xFFFFFFFFu, ld_acquire(bar) < target)) {
+        if (++spins > spin_limit) {
+            if (threadIdx.x == 0) atomicOr(status, QP_DEV_STREAM_TIMEOUT);
+            break;
         }
-        *s_ok = ok;
+        if (spins > 64) __nanosleep(64);
     }
-    __syncthreads();
-    return *s_ok != 0;
+    if (threadIdx.x == 0) *s_ok = spins <= spin_limit;
+    __syncwarp();
 }
 
 // A block's way out, by one of its threads, when the block will neither arrive nor poll again.  bar[1] counts the blocks out

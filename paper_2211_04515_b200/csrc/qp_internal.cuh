@@ -116,11 +116,12 @@ struct qp_ctx {
 };
 
 // Scratch of the cooperative kernels (d_fused): 256 bytes of barrier counters and the histogram (4096 x 8 bytes), both
-// zero between launches, and the interval totals of the search (count and sum, 8 bytes each).
+// zero between launches, and the search's sums per candidate, one set of the sender's, one of the separate search's (the latter
+// zero between launches).
 constexpr int QP_SS_MAX_CAND = 256;              // candidates of the search in one launch with the statistics
-constexpr int QP_SS_TOTALS = 4096;
+constexpr int QP_SS_TOTALS = 4096;               // most intervals of a block's row
 constexpr size_t QP_FUSED_TOTALS_AT = 256 + sizeof(unsigned long long) * 4096;
-constexpr size_t QP_FUSED_BYTES = QP_FUSED_TOTALS_AT + 16 * (size_t)QP_SS_TOTALS;
+constexpr size_t QP_FUSED_BYTES = QP_FUSED_TOTALS_AT + 2 * sizeof(unsigned long long) * (QP_SS_MAX_CAND + 2);
 
 constexpr long long QP_WAIT_CYCLES_DEFAULT = 4000000000ll;   // about two seconds
 constexpr unsigned QP_SPIN_LIMIT_DEFAULT = 1u << 22;          // x 64 ns sleeps: a quarter of a second at least

@@ -6,10 +6,12 @@
 //   phase B   sum |x - mean|, sum (x - mean)^2, histogram over [min, max]
 //   barrier   every block: statistics, histogram peak -> b_R, the candidates
 //   phase C   one pass that gathers, per interval between the candidates' decision thresholds, the count and
-//             the sum of the elements; every block stores its row of interval sums
-//   barrier   every block adds up a slice of the intervals over all rows
-//   exit      block 0 turns the interval sums into the error of every candidate, picks the first minimum and writes
-//             the quantizer; in the sender the other blocks wait for it and all pack
+//             the sum of the elements; every block makes of its own sums its part of the error of every candidate
+//   barrier   the parts are added up in 64-bit integers; every block takes the first minimum, and block 0 writes the result
+//   packing   in the sender, from the tensor's end
+//
+// With one bit a side has one code, so that the statistics tell the errors: the sender packs behind phase B, and the separate search
+// only counts the elements below the centre.
 //
 // Phase C needs no table of thresholds (qp_affine.cuh).  Its tables hold a replica per lane (per two lanes at 4 bits), so a
 // warp's atomics meet neither the same counter nor the same bank.  They are emptied into 64-bit sums before they can
@@ -17,12 +19,14 @@
 // step take the "hard" form below, with the exact thresholds.
 //
 // What bounds it, by time stamps that the blocks took (each figure from the last block before it to its own last block; the
-// stamps lengthen the launch): on 129 MB (fp32, 2 bits) phase A 25 us, the read from DRAM; barrier and merge 9; B 20 and C 23, the
-// read, most of which L2 still holds, and the instructions (A and B 19 per element together, C 19, at 4 bits 35; one shared
-// atomic in B, two in C); between them barrier, merge and candidates 5; rows, barrier and slices 6; block 0's scoring and
-// pick 9, its result read back 1; packing 21: 119 in all.  On 39 MB at 4 bits, which L2 holds: A 9, then 9, B 6, 5, C 15, 7, 9, 1 and
-// the packing 6: 67.  The calls take 114 and 64 us without the stamps, launch included; two kernels for the statistics, five for the
-// search and one for the packing took 171 and 107.
+// stamps lengthen the launch by 2 to 3 us): on 129 MB (fp32, 2 bits) phase A 24 us, the read from DRAM; barrier and merge 3; B 18 and C
+// 21, the read, most of which L2 still holds, and the instructions (A and B 19 per element together, C 19, at 4 bits 35; one shared
+// atomic in B, two in C); between them histogram, barrier, merge and candidates 6; a block's prefix sums and errors 2, barrier and pick
+// 3; packing 20.  On 39 MB at 4 bits, which L2 holds: A 8, then 3, B 5, 6, C 12, 4, 3 and the packing 4: 45 and 3 for the launch.  Both
+// calls took 15 us longer (47 and 99 against 63 and 114) with the blocks' intervals added up by all of them in slices, behind a barrier of their own, the scoring
+// by block 0 alone with the others waiting, and block partials 64 bytes apart.
+// Shuffles by a warp that has not reconverged cost 250 cycles each instead of 30 (the finish 3.6 us instead of 1.3): hence the
+// __syncwarp before them and the grid barrier whose whole warp polls.
 #include <type_traits>
 
 #include "qp_affine.cuh"
@@ -53,10 +57,11 @@ struct SsArgs {
     float4* cand;
     int* valid;
     qp_ds_setup* setup;
-    double* part;                                 // [grid][8]
+    uint4* part;                                  // [4][grid] block partials, 16 bytes each
     unsigned long long* hist;                     // [nb], zero at entry and at exit
-    ulonglong2* rows;                             // [grid][intervals] count, sum
-    ulonglong2* tot;                              // [intervals]
+    ulonglong2* rows;                             // [grid][intervals] count, sum: what a block emptied its tables of on the way
+    unsigned long long* acc;                      // [ncand + 2]: errors of the candidates in fixed point; search only: the elements below the
+                                                  // centre and the others, all zero at entry and at exit
     unsigned* bar;                                // [0] arrivals, [1] blocks that have left; zero at entry and at exit
     unsigned* status;
     unsigned spin_limit, bar_extra;
@@ -70,17 +75,18 @@ struct SsArgs {
 
 // ---- phase A
 struct SsMoments {
-    double s, sa, bad;
+    double s, sa;
     float mn, mx;
+    unsigned bad;
     unsigned odd;                                             // tiles with a non-finite value (or an fp32 overflow)
     qp_f2 s2[2];
     float a4[4], lo, hi;
     __device__ __forceinline__ void clear()
     {
-        s = sa = bad = 0.0;
+        s = sa = 0.0;
         mn = __int_as_float(0x7F800000);
         mx = -mn;
-        odd = 0u;
+        bad = odd = 0u;
     }
     __device__ __forceinline__ void one(float v)              // element by element: skips and counts NaN / Inf
     {
@@ -90,7 +96,7 @@ struct SsMoments {
             mn = fminf(mn, v);
             mx = fmaxf(mx, v);
         } else {
-            bad += 1.0;
+            ++bad;
         }
     }
     __device__ __forceinline__ void begin()
@@ -198,6 +204,22 @@ __device__ __noinline__ void ss_guarded_deviations(const T* x, uint64_t ntiles, 
     SsTiles<T, SS_TILE>::template run<true>(x, ntiles, first, step, lane, f);
 }
 
+// One bit: how many elements lie below m, of how many.
+struct SsSides {
+    float m;
+    bool guard;
+    unsigned down, all;
+    __device__ __forceinline__ void begin() {}
+    __device__ __forceinline__ void pair(float a, float b, int) { one(a, guard); one(b, guard); }
+    __device__ __forceinline__ void end() {}
+    __device__ __forceinline__ void one(float v, bool check = true)
+    {
+        if (check && !qp_is_finite(v)) return;
+        down += __float_as_uint(__fsub_rn(v, m)) >> 31;
+        ++all;
+    }
+};
+
 template <int HH, bool GUARD>
 struct SsCounter {
     const SsPlan<HH>& p;
@@ -211,10 +233,8 @@ struct SsCounter {
     __device__ __forceinline__ void end() {}
 };
 
-// The interval tables' contents go to this block's row (FIRST: set, otherwise added); AGAIN: and the tables back to
-// zero.  A thread takes four replicas of an interval (one 16-byte read of each table, consecutive threads consecutive
-// vectors).
-template <bool AGAIN>
+// The interval tables' contents go to this block's row (first: set, otherwise added) and the tables back to zero.  A thread
+// takes four replicas of an interval (one 16-byte read of each table, consecutive threads consecutive vectors).
 __device__ __forceinline__ void ss_flush(unsigned char* raw, int ni, int rs, ulonglong2* row, bool first)
 {
     const int ts = rs - 2;                                    // log2 of the threads per interval; rs is 2 at least
@@ -228,7 +248,7 @@ __device__ __forceinline__ void ss_flush(unsigned char* raw, int ni, int rs, ulo
             const uint4 c = cnt[u], d = sum[u];
             cn = (unsigned long long)c.x + c.y + ((unsigned long long)c.z + c.w);
             cd = (unsigned long long)d.x + d.y + ((unsigned long long)d.z + d.w);
-            if (AGAIN) cnt[u] = sum[u] = make_uint4(0u, 0u, 0u, 0u);
+            cnt[u] = sum[u] = make_uint4(0u, 0u, 0u, 0u);
         }
         for (int o = 1; o < (1 << ts); o <<= 1) {
             cn += __shfl_xor_sync(0xFFFFFFFFu, cn, o);
@@ -242,182 +262,196 @@ __device__ __forceinline__ void ss_flush(unsigned char* raw, int ni, int rs, ulo
     }
 }
 
-// After the barrier behind the rows: this block's slice of the intervals, added up over all rows.  A warp takes every
-// SS_WARPS-th row (32 consecutive intervals per read), the warps' sums meet in shared memory.  Integers: any order.
-__device__ __forceinline__ void ss_slices(const SsArgs& a, int count, unsigned char* raw)
+// The block's histogram goes into the tensor's; what x = max put into bin nb counts in the last one.
+__device__ __forceinline__ void ss_hist_out(const unsigned* bins, int nb, int shift, unsigned long long* hist)
 {
-    ulonglong2* sh = reinterpret_cast<ulonglong2*>(raw);      // [SS_WARPS][32]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int G = (int)gridDim.x, per = (count + G - 1) / G;
-    const int e0 = blockIdx.x * per, e1 = min(e0 + per, count);
-    for (int e = e0; e < e1; e += 32) {
-        const int i = e + lane;
-        unsigned long long n = 0, s = 0;
-        if (i < e1)
-#pragma unroll 5
-            for (int b = warp; b < G; b += SS_WARPS) {
-                const ulonglong2 v = __ldcg(a.rows + (size_t)b * count + i);
-                n += v.x;
-                s += v.y;
+    const int ts = shift >= 2 ? shift - 2 : 0, units = (nb + 1) << ts;        // a thread takes four replicas of a bin, or all
+    for (int u0 = threadIdx.x & ~31; u0 < units; u0 += SS_THREADS) {
+        const int u = u0 + (threadIdx.x & 31);
+        unsigned c = 0u;
+        if (u < units) {
+            if (shift >= 2) {
+                const uint4 v = reinterpret_cast<const uint4*>(bins)[u];
+                c = v.x + v.y + (v.z + v.w);
+            } else {
+                for (int r = 0; r < (1 << shift); ++r) c += bins[(u << shift) + r];
             }
-        sh[warp * 32 + lane] = make_ulonglong2(n, s);
-        __syncthreads();
-        if (warp == 0 && i < e1) {
-            for (int w = 1; w < SS_WARPS; ++w) { n += sh[w * 32 + lane].x; s += sh[w * 32 + lane].y; }
-            a.tot[i] = make_ulonglong2(n, s);
         }
-        __syncthreads();
+        for (int o = 1; o < (1 << ts); o <<= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
+        if (u < units && (u & ((1 << ts) - 1)) == 0 && c) atomicAdd(&hist[min(u >> ts, nb - 1)], (unsigned long long)c);
     }
 }
 
-// The same for all intervals by one block, for the few rows of a cluster; the block barrier at the end makes them the
-// block's to read.
-__device__ __forceinline__ void ss_all_slices(const SsArgs& a, int count)
+// A side's elements below interval i, this block's: counts and sums of |y| in units of p.u, exclusive prefix sums over the
+// side's intervals, in the place of the interval's own counters (16 bytes of them; an interval has four counters at least).  Half the
+// block per side, a thread takes `per` consecutive intervals.  per is odd, and the order in which a lane reads the vectors of an
+// interval, as well as which of them becomes the slot, turns with the lane and with the interval, so that the eight lanes of a 16-byte
+// access meet no bank twice (1.9 us at 4 bits, 4.3 without the turn, 2.6 with three intervals at a time).  A block's counts stay below 2^32 (the tensor would
+// have to have 6e11 elements).  Returns (to everybody) the elements of the two sides.
+__device__ __forceinline__ ulonglong2* ss_slot(unsigned char* raw, int e, int rs)
 {
-    const int G = (int)gridDim.x;
-    for (int i = threadIdx.x; i < count; i += SS_THREADS) {
-        unsigned long long n = 0, s = 0;
-#pragma unroll 8
-        for (int b = 0; b < G; ++b) {
-            const ulonglong2 v = __ldcg(a.rows + (size_t)b * count + i);
-            n += v.x;
-            s += v.y;
-        }
-        a.tot[i] = make_ulonglong2(n, s);
-    }
-    __syncthreads();
+    return reinterpret_cast<ulonglong2*>(raw + ((size_t)e << (rs + 2)) + (((e >> (5 - rs)) & ((1 << (rs - 2)) - 1)) << 4));
 }
-
-// Exclusive prefix sums of n[0..len), s[0..len) (n[len], s[len]: the totals), by `threads` threads (a multiple of
-// 32) of which this is number t; sh: 2 * threads / 32 doubles.  Block barriers inside: called by all threads.
-__device__ inline void ss_scan(double* n, double* s, int len, int t, int threads, double* sh)
+__device__ __forceinline__ uint2 ss_prefix(unsigned char* raw, int ni, int rs, const ulonglong2* row, const int* s_edge, ulonglong2* sh)
 {
-    const int per = (len + threads - 1) / threads;
-    const int i0 = min(t * per, len), i1 = min(i0 + per, len);
-    double a = 0.0, b = 0.0;
-    for (int i = i0; i < i1; ++i) { a += n[i]; b += s[i]; }
-    double pa = a, pb = b;                                    // inclusive over the warp
-    for (int o = 1; o < 32; o <<= 1) {
-        const double ta = __shfl_up_sync(0xFFFFFFFFu, pa, o), tb = __shfl_up_sync(0xFFFFFFFFu, pb, o);
-        if ((t & 31) >= o) { pa += ta; pb += tb; }
-    }
-    if ((t & 31) == 31) { sh[2 * (t >> 5)] = pa; sh[2 * (t >> 5) + 1] = pb; }
-    __syncthreads();
-    double xa = pa - a, xb = pb - b;
-    for (int w = 0; w < (t >> 5); ++w) { xa += sh[2 * w]; xb += sh[2 * w + 1]; }
+    constexpr int HALF = SS_THREADS / 2, HW = SS_WARPS / 2;
+    static_assert(SS_GRID == 64, "two steps of eight");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, side = threadIdx.x >= HALF, t = threadIdx.x - side * HALF;
+    const int per = ((ni + HALF - 1) / HALF) | 1, vecs = 1 << (rs - 2), turn = lane >> (5 - rs);
+    const int i0 = min(t * per, ni), i1 = min(i0 + per, ni);
+    int cell = 0;                                             // the last cell that starts at or before i0
+#pragma unroll
+    for (int g = 8; g <= 64; g += 8) cell += s_edge[g] <= i0 ? 8 : 0;
+    int more = 0;
+#pragma unroll
+    for (int g = 1; g < 8; ++g) more += s_edge[min(cell + g, SS_GRID)] <= i0 ? 1 : 0;
+    cell = min(cell + more, SS_GRID);
+    unsigned n = 0u;
+    unsigned long long s = 0ull;
     for (int i = i0; i < i1; ++i) {
-        const double vn = n[i], vs = s[i];
-        n[i] = xa; s[i] = xb;
-        xa += vn; xb += vs;
-    }
-    if (t == threads - 1) { n[len] = xa; s[len] = xb; }
-    __syncthreads();
-}
-
-// Block-wide: the error of every candidate is in s_curve[0..ncand); first minimum wins.
-__device__ inline void ss_pick(const SsArgs& a, int ncand, const double* s_curve, const float4* s_cand, const int* s_valid,
-                               const qp_ds_setup& setup)
-{
-    if (threadIdx.x >= 32) {
-        for (int k = threadIdx.x - 32; k < ncand; k += SS_THREADS - 32) {
-            a.curve[k] = s_curve[k];
-            a.cand[k] = s_cand[k];
-            a.valid[k] = s_valid[k];
-        }
-        return;
-    }
-    double bv = __longlong_as_double(0x7FF0000000000000ll);
-    int bk = 1 << 30;
-    for (int k = threadIdx.x; k < ncand; k += 32)
-        if (s_curve[k] < bv) { bv = s_curve[k]; bk = k; }
-    for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_down_sync(0xFFFFFFFFu, bv, o);
-        const int ok = __shfl_down_sync(0xFFFFFFFFu, bk, o);
-        if (ov < bv || (ov == bv && ok < bk)) { bv = ov; bk = ok; }
-    }
-    if (threadIdx.x == 0) {
-        const int best = bk < ncand ? bk : 0;                 // (every error infinite or NaN: keep b_E)
-        qp_ds_write_result(best, s_curve, setup, a.steps, a.nb, a.bits, s_cand[best], a.ds_out, a.qp_out, a.status);
-        *a.setup = setup;
-    }
-}
-
-// Block 0, after its arrival: where the boundaries of every candidate lie among the intervals (in shared memory), while
-// the other blocks are still on their way.  s_cell[i]: grid cell of interval i; pos[k][i]: first interval of
-// code i of a side, i = 0..HH; pos[k][HH + 1] = ni.
-template <int HH>
-__device__ inline void ss_places(const SsPlan<HH>& p, int ncand, int ni, int* s_edge, unsigned char* s_cell, int* pos)
-{
-    constexpr int C = HH + 1;
-    for (int g = threadIdx.x; g <= SS_GRID; g += SS_THREADS) s_edge[g] = ss_cell_start(p, g);
-    const bool flat = !(p.inv_e > 0.f);                       // no width at all: everything has the first code of its side
-    for (int w = threadIdx.x; w < ncand * (C + 1); w += SS_THREADS) {
-        const int k = w / (C + 1), b = w - k * (C + 1);       // boundary b = 1..HH of candidate k
-        pos[w] = QP_CK(b == 0 ? 0 : (b > HH || flat) ? ni : ss_place(p, k, b), ni + 1);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < ni; i += SS_THREADS) {      // cell of an interval: the last one that starts at or before it
-        int lo = 0, hi = SS_GRID;
-        while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (s_edge[mid] <= i) lo = mid; else hi = mid - 1; }
-        s_cell[i] = (unsigned char)lo;
-    }
-}
-
-// Block 0, when the totals are complete: interval totals -> error of every candidate.
-//   sum over one side and code of (|y| - level)^2 = sum y^2 + N level^2 - 2 level sum |y|,
-// sum y^2 of all elements from the statistics, N and sum |y| as differences of prefix sums over the intervals.
-template <int HH>
-__device__ inline void ss_finish(const SsArgs& a, const SsPlan<HH>& p, const qp_stats_t& st, int ncand, int ni, const unsigned char* s_cell,
-                                 const int* pos, const float4* s_cand, const int* s_valid, double* s_curve, double* sh, double* PN)
-{
-    constexpr int C = HH + 1, C2 = 2 * C;                     // codes of a side, of both: 2, 4, 8, 16
-    double* PS = PN + 2 * (ni + 1);                           // PN, PS: [2][ni + 1] counts and sums of |y|, then their prefix sums
-    for (int e0 = threadIdx.x; e0 < 2 * ni; e0 += 4 * SS_THREADS) {
-        ulonglong2 t[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (e0 + j * SS_THREADS < 2 * ni) t[j] = __ldcg(a.tot + e0 + j * SS_THREADS);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int e = e0 + j * SS_THREADS;
-            if (e >= 2 * ni) break;
-            const int side = e >= ni, i = e - side * ni;
-            const double n = (double)t[j].x, ref = (double)s_cell[i] * p.w, s1 = p.u * (double)t[j].y;
-            PN[side * (ni + 1) + i] = n;
-            PS[side * (ni + 1) + i] = s1 + n * ref;
-        }
-    }
-    __syncthreads();
-    {
-        const int side = threadIdx.x >= SS_THREADS / 2;
-        ss_scan(PN + side * (ni + 1), PS + side * (ni + 1), ni, threadIdx.x - side * (SS_THREADS / 2), SS_THREADS / 2,
-                sh + side * SS_WARPS);
-    }
-    const double nf = (double)(st.n - st.nonfinite), dm = st.mean - (double)p.m;
-    const double s_abs = nf * st.mad + dm * (PN[ni] - PN[2 * ni + 1]);        // sum |y|, sum y: the sides are half sum and half difference
-    const double s_sq = nf * (st.var + dm * dm);
-    const double s_up = 0.5 * (s_abs + nf * dm), s_down = 0.5 * (s_abs - nf * dm);
-    // a candidate's codes in C2 neighbouring lanes, added up by a fixed tree
+        const int e = side * ni + i;
+        const uint4* cnt = reinterpret_cast<const uint4*>(raw) + ((size_t)e << (rs - 2));
+        unsigned cn = 0u;                                     // (a flush's counts, and a block's, are below 2^32)
+        unsigned long long cd = 0ull;
 #pragma unroll 4
-    for (int w0 = threadIdx.x & ~31; w0 < ncand * C2; w0 += SS_THREADS) {
-        const int w = w0 + (threadIdx.x & 31), k = w / C2, side = (w / C) & 1, i = w % C;
+        for (int v = 0; v < vecs; ++v) {
+            const int at = (v + turn) & (vecs - 1);
+            const uint4 c = cnt[at], d = cnt[SS_SUMS_AT / 16 + at];
+            cn += c.x + c.y + (c.z + c.w);
+            cd += (unsigned long long)d.x + d.y + ((unsigned long long)d.z + d.w);
+        }
+        while (cell < SS_GRID && s_edge[cell + 1] <= i) ++cell;
+        if (row) { cn += (unsigned)row[e].x; cd += row[e].y; }
+        *ss_slot(raw, e, rs) = make_ulonglong2(n, s);
+        n += cn;
+        s += cd + (((unsigned long long)cn * (unsigned)cell) << SS_UNIT_BITS);
+    }
+    __syncwarp();
+    unsigned pn = n;                                          // inclusive over the warp, then over the warps of the side
+    unsigned long long ps = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned tn = __shfl_up_sync(0xFFFFFFFFu, pn, o);
+        const unsigned long long ts = __shfl_up_sync(0xFFFFFFFFu, ps, o);
+        if (lane >= o) { pn += tn; ps += ts; }
+    }
+    if (lane == 31) sh[warp] = make_ulonglong2(pn, ps);
+    __syncthreads();
+    pn -= n;
+    ps -= s;
+#pragma unroll
+    for (int w = 0; w < HW - 1; ++w) {
+        const ulonglong2 o = sh[side * HW + w];
+        if (w < (warp & (HW - 1))) { pn += (unsigned)o.x; ps += o.y; }
+    }
+#pragma unroll 3
+    for (int i = i0; i < i1; ++i) {
+        ulonglong2* at = ss_slot(raw, side * ni + i, rs);
+        const ulonglong2 v = *at;
+        *at = make_ulonglong2(v.x + pn, v.y + ps);
+    }
+    uint2 all = make_uint2(0u, 0u);
+    for (int w = 0; w < HW; ++w) { all.x += (unsigned)sh[w].x; all.y += (unsigned)sh[HW + w].x; }
+    return all;
+}
+
+// Where the boundaries of every candidate lie among the intervals: pos[k][b - 1], the first interval of code b = 1..HH of a
+// side.  s_edge: the interval that a grid cell starts with.
+template <int HH>
+__device__ __forceinline__ void ss_places(const SsPlan<HH>& p, int ncand, int ni, int* s_edge, int* pos)
+{
+    for (int w = threadIdx.x; w < ncand * HH; w += SS_THREADS) {
+        const int k = w / HH, b = w - k * HH + 1;
+        pos[w] = QP_CK(ss_place(p, k, b), ni);
+    }
+    for (int g = threadIdx.x; g <= SS_GRID; g += SS_THREADS) s_edge[g] = ss_cell_start(p, g);
+}
+
+// The error of candidate k is, over the elements,
+//   sum y^2 + sum over both sides of sum_i (N_i level_i^2 - 2 level_i S_i),   N_i, S_i: count and sum of |y| of code i of the side,
+// and with the prefix sums P(b) at the first interval of code b the sum over the codes i of a side is
+//   N level_HH^2 - 2 S level_HH - sum over b = 1..HH of (P_N(b) (level_b^2 - level_(b-1)^2) - 2 P_S(b) (level_b - level_(b-1))).
+// N and S of the whole sides are known from the statistics; the sum over the boundaries is a sum over the blocks, which they add up
+// in 64-bit integers (any order, the same bits) with the unit 2^-fix.  It is below 2^62 units: the sides together come to less than
+// 4 n E^2, E the power of two above the widest clip and every level.  A block's rounding to a unit is 2^-60 of that bound.
+__device__ __forceinline__ int ss_fix(uint64_t n, int e) { return 60 - (64 - __clzll((long long)n)) - 2 * e; }
+template <int HH>
+__device__ __forceinline__ void ss_errors(const SsPlan<HH>& p, int ncand, int ni, int rs, int fix, unsigned char* raw, const int* pos,
+                                          const float4* s_cand, const int* s_valid, unsigned long long* acc)
+{
+    constexpr int TPC = HH == 1 ? 2 : 4, RUN = (2 * HH + TPC - 1) / TPC;     // threads per candidate: one or two per side
+    const double unit = ldexp(1.0, fix);
+    for (int w0 = threadIdx.x & ~31; w0 < ncand * TPC; w0 += SS_THREADS) {
+        const int w = w0 + (threadIdx.x & 31), k = w / TPC, part = w % TPC;
+        const int side = part / (TPC / 2), b0 = 1 + (part % (TPC / 2)) * RUN;
         double v = 0.0;
         if (k < ncand && s_valid[k]) {
-            const int p0 = pos[k * (C + 1) + i], p1 = pos[k * (C + 1) + i + 1];
-            const double* N = PN + side * (ni + 1);
-            const double* S = PS + side * (ni + 1);
-            const double s_side = side ? s_down : s_up;
-            const double cn = N[p1] - N[p0], cs = (p1 == ni ? s_side : S[p1]) - (p0 == ni ? s_side : S[p0]);
-            double lv = ss_level(s_cand[k], side ? HH - i : HH + 1 + i, p.m);
-            if (side) lv = -lv;                               // distance from the centre, as |y|
-            v = cn * lv * lv - 2.0 * lv * cs;
+            const float4 c = s_cand[k];
+            auto level = [&](int b) { const double l = ss_level(c, side ? HH - b : HH + 1 + b, p.m); return side ? -l : l; };
+            double below = level(b0 - 1);
+#pragma unroll
+            for (int j = 0; j < RUN; ++j) {
+                const int b = b0 + j;
+                if (b > HH) break;
+                const ulonglong2 P = *ss_slot(raw, side * ni + pos[k * HH + b - 1], rs);
+                const double lv = level(b), step = lv - below;
+                v += step * (2.0 * p.u * (double)P.y - (lv + below) * (double)P.x);
+                below = lv;
+            }
         }
 #pragma unroll
-        for (int o = C2 / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-        if (k < ncand && w % C2 == 0)
-            s_curve[k] = !s_valid[k] ? __longlong_as_double(0x7FF0000000000000ll) : (nf > 0.0 ? (s_sq + v) / nf : 0.0);
+        for (int o = TPC / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+        if (k < ncand && part == 0) atomicAdd(acc + k, (unsigned long long)__double2ll_rn(v * unit));
+    }
+}
+
+// What the finish needs of the hard form: levels of the codes that hold the elements beyond the ends, their sums.
+struct SsBeyond { const double *lv_lo, *lv_hi; double e_lo, e_hi; };
+
+// Every block, when the sums are complete: the error of every candidate into s_curve, the first minimum as the result (every block the
+// same).  A thread per candidate, a warp's minimum by shuffles, the warps' through s_min, s_at [SS_WARPS].
+template <int HH>
+__device__ __forceinline__ int ss_finish(const SsArgs& a, float m, bool flat, const qp_stats_t& st, double n_up, double n_down, int ncand, int fix,
+                                         const float4* s_cand, const int* s_valid, double* s_curve, const SsBeyond* hard, double* s_min, int* s_at)
+{
+    static_assert(QP_SS_MAX_CAND <= SS_THREADS, "a thread per candidate");
+    const double inf = __longlong_as_double(0x7FF0000000000000ll);
+    const int k = threadIdx.x, lane = threadIdx.x & 31, warps = (ncand + 31) >> 5;
+    if ((k >> 5) < warps) {
+        const double nf = (double)(st.n - st.nonfinite), dm = st.mean - (double)m;
+        const double s_abs = nf * st.mad + dm * (n_up - n_down);              // sum |y|, sum y: the sides are half sum and half difference
+        const double s_sq = nf * (st.var + dm * dm);
+        const double s_up = 0.5 * (s_abs + nf * dm), s_down = 0.5 * (s_abs - nf * dm);
+        double best = inf;
+        if (k < ncand) {
+            double v = HH || hard ? ldexp((double)(long long)__ldcg(a.acc + k), -fix) : 0.0;
+            if (hard) {
+                v -= 2.0 * (hard->lv_lo[k] * hard->e_lo + hard->lv_hi[k] * hard->e_hi);
+            } else {
+                const int top = flat ? 0 : HH;                // (flat: everything has the first code of its side)
+                const double lu = ss_level(s_cand[k], HH + 1 + top, m), ld = -ss_level(s_cand[k], HH - top, m);
+                v += n_up * lu * lu - 2.0 * lu * s_up + (n_down * ld * ld - 2.0 * ld * s_down);
+            }
+            v = !s_valid[k] ? inf : (nf > 0.0 ? (s_sq + v) / nf : 0.0);
+            s_curve[k] = v;
+            if (v < best) best = v;
+        }
+        __syncwarp();
+        int at = best < inf ? k : 1 << 30;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double ov = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+            const int ok = __shfl_xor_sync(0xFFFFFFFFu, at, o);
+            if (ov < best || (ov == best && ok < at)) { best = ov; at = ok; }
+        }
+        if (lane == 0) { s_min[k >> 5] = best; s_at[k >> 5] = at; }
     }
     __syncthreads();
+    double best = inf;
+    int at = 0;                                               // (every error infinite or NaN: keep b_E)
+    for (int w = 0; w < warps; ++w)
+        if (s_min[w] < best) { best = s_min[w]; at = s_at[w]; }
+    return at;
 }
 
 // ---- the hard form: exact thresholds T(k, j) = smallest float with code >= j, found by bisection with the
@@ -504,24 +538,54 @@ __device__ inline void ss_hard_flush(const SsHard& h, ulonglong2* row, bool firs
         row[i] = make_ulonglong2(cn, cd);
     }
 }
-__device__ inline void ss_hard_finish(const SsArgs& a, const SsHard& h, float m, const qp_stats_t& st, int ncand, double e_lo,
-                                      double e_hi, const float4* s_cand, const int* s_valid, double* s_curve, double* sh)
+// Exclusive prefix sums of n[0..len), s[0..len) (n[len], s[len]: the totals); sh: 2 * SS_WARPS doubles.
+__device__ inline void ss_scan(double* n, double* s, int len, double* sh)
+{
+    const int t = threadIdx.x, per = (len + SS_THREADS - 1) / SS_THREADS;
+    const int i0 = min(t * per, len), i1 = min(i0 + per, len);
+    double a = 0.0, b = 0.0;
+    for (int i = i0; i < i1; ++i) { a += n[i]; b += s[i]; }
+    double pa = a, pb = b;                                    // inclusive over the warp
+    for (int o = 1; o < 32; o <<= 1) {
+        const double ta = __shfl_up_sync(0xFFFFFFFFu, pa, o), tb = __shfl_up_sync(0xFFFFFFFFu, pb, o);
+        if ((t & 31) >= o) { pa += ta; pb += tb; }
+    }
+    if ((t & 31) == 31) { sh[2 * (t >> 5)] = pa; sh[2 * (t >> 5) + 1] = pb; }
+    __syncthreads();
+    double xa = pa - a, xb = pb - b;
+    for (int w = 0; w < (t >> 5); ++w) { xa += sh[2 * w]; xb += sh[2 * w + 1]; }
+    for (int i = i0; i < i1; ++i) {
+        const double vn = n[i], vs = s[i];
+        n[i] = xa; s[i] = xb;
+        xa += vn; xb += vs;
+    }
+    if (t == SS_THREADS - 1) { n[len] = xa; s[len] = xb; }
+    __syncthreads();
+}
+// This block's part of the errors, as ss_errors; lv_lo, lv_hi [ncand]: levels of the codes of the two ends.  Returns fix.
+__device__ inline int ss_hard_errors(const SsArgs& a, const SsHard& h, float m, int ncand, const ulonglong2* row, const float4* s_cand,
+                                     const int* s_valid, double* lv_lo, double* lv_hi, double* sh)
 {
     // (behind the thresholds: the tables are done with)
     double* PN = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(h.thr) + ((size_t)8 * h.M + 15) / 16 * 16);
     double* PS = PN + (h.M + 2);
     for (int i = threadIdx.x; i <= h.M; i += SS_THREADS) {
-        const ulonglong2 t = __ldcg(a.tot + i);
+        const ulonglong2 t = row[i];
         PN[i] = (double)t.x;
         PS[i] = (double)t.x * ((double)h.g_lo - (double)m) + h.u * (double)t.y;
     }
     __syncthreads();
-    ss_scan(PN, PS, h.M + 1, threadIdx.x, SS_THREADS, sh);
-    const double nf = (double)(st.n - st.nonfinite), dm = st.mean - (double)m;
+    ss_scan(PN, PS, h.M + 1, sh);
+    const double most = fmax(fabs((double)h.g_lo - (double)m), fabs((double)h.g_hi - (double)m));   // of levels and elements
+    int e = 0;
+    frexp(most, &e);
+    const int fix = ss_fix(a.n, e);
+    const double unit = most < __longlong_as_double(0x7FF0000000000000ll) ? ldexp(1.0, fix) : 0.0;
     const int L1 = (1 << a.bits) - 1;
     for (int k = threadIdx.x; k < ncand; k += SS_THREADS) {
-        double t = nf * (st.var + dm * dm);
+        double t = 0.0;
         int p0 = 0;
+        lv_lo[k] = lv_hi[k] = 0.0;
         for (int j = 0; s_valid[k] && j <= L1; ++j) {
             int p1 = h.M + 1;
             if (j < L1) {
@@ -529,30 +593,34 @@ __device__ inline void ss_hard_finish(const SsArgs& a, const SsHard& h, float m,
                 if (T < __int_as_float(0x7F800000)) p1 = max(ss_hard_at(h, T), p0);
             }
             const double lv = ss_level(s_cand[k], j, m);
-            double sum = PS[p1] - PS[p0];
-            if (p0 == 0 && p1 > 0) sum += e_lo;
-            if (p1 == h.M + 1 && p0 < h.M + 1) sum += e_hi;
-            t += (PN[p1] - PN[p0]) * lv * lv - 2.0 * lv * sum;
+            if (p0 == 0 && p1 > 0) lv_lo[k] = lv;
+            if (p1 == h.M + 1 && p0 < h.M + 1) lv_hi[k] = lv;
+            t += (PN[p1] - PN[p0]) * lv * lv - 2.0 * lv * (PS[p1] - PS[p0]);
             p0 = p1;
         }
-        s_curve[k] = !s_valid[k] ? __longlong_as_double(0x7FF0000000000000ll) : (nf > 0.0 ? t / nf : 0.0);
+        // (ends that are not finite: the levels carry the infinity into the curve)
+        if (unit > 0.0 && fabs(t) < 1e300) atomicAdd(a.acc + k, (unsigned long long)__double2ll_rn(t * unit));
+        else lv_lo[k] = lv_hi[k] = __longlong_as_double(0x7FF8000000000000ll);
     }
-    __syncthreads();
+    return fix;
 }
 
 __host__ __device__ constexpr int ss_ctile(int hh) { return hh >= 3 ? 512 : 1024; }   // phase C's tile: long code per element, short tile (instruction cache)
 
-// STATS: phases A and B (otherwise the statistics come with st_in, and B runs only if they lack the histogram).
-// HH: code boundaries above the centre, 2^bits / 2 - 1; -1: statistics only.
 // What the last block out does, with what count_out returned (and whether the block itself gave up): one thread.
 __device__ __forceinline__ void ss_out(const SsArgs& a, unsigned before)
 {
     if (!qp_grid::last_out(before, gridDim.x)) return;
-    if (before >= qp_grid::GAVE_UP)                           // (block 0 of an undisturbed launch has cleaned)
+    if (before >= qp_grid::GAVE_UP) {                         // (block 0 of an undisturbed launch has cleaned)
         for (int b = 0; b < a.nb; ++b) a.hist[b] = 0ull;
+        if (a.bits)
+            for (int k = 0; k < a.steps + 3; ++k) a.acc[k] = 0ull;
+    }
     qp_grid::reset(a.bar);
 }
 
+// STATS: phases A and B (otherwise the statistics come with st_in, and B runs only if they lack the histogram).
+// HH: code boundaries above the centre, 2^bits / 2 - 1; -1: statistics only.
 // Returns SS_GAVE_UP where a wait ran out, SS_OUT where the block has counted itself out (or is one of a cluster).
 enum { SS_GAVE_UP, SS_DONE, SS_OUT };
 template <typename T, bool STATS, int HH>
@@ -561,10 +629,12 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
     constexpr bool SEARCH = HH >= 0;
     constexpr int H = SEARCH ? HH : 0;
     extern __shared__ __align__(16) unsigned char raw[];
-    __shared__ double s_red[SS_WARPS * 5];
+    __shared__ SsBlock s_block[2];
+    __shared__ __align__(16) double s_red[SS_WARPS * 2];
     __shared__ int s_ok;
     __shared__ bool s_last;
     __shared__ qp_stats_t s_st;
+    __shared__ double s_down;                                 // elements below the fp32 mean
     __shared__ qp_ds_setup s_setup;
     __shared__ SsPlan<H> s_plan;
     const T* x = static_cast<const T*>(a.x);
@@ -572,8 +642,8 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
     const unsigned G = gridDim.x;
     const uint64_t first = (uint64_t)blockIdx.x * SS_WARPS + (threadIdx.x >> 5), step = (uint64_t)G * SS_WARPS;
     const uint64_t tail0 = a.ntiles * SS_TILE;
-    const double inf = __longlong_as_double(0x7FF0000000000000ll);
     unsigned* bins = reinterpret_cast<unsigned*>(raw + SS_TABLE_BYTES);
+    uint4* part = a.part + blockIdx.x;                        // this block's: row r at part[r * G]
     unsigned waits = 0;
     const bool cluster = a.cluster;
     auto meet = [&]() {
@@ -585,33 +655,30 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
         ++waits;
         return qp_grid::barrier(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
     };
-    auto arrive = [&]() {
-        __syncthreads();
+    // for what warp 0 wrote and reads next; the others learn from s_ok behind the next block barrier
+    auto meet_warp0 = [&]() {
+        ++waits;
         if (cluster) {
             qp_grid::cluster_arrive();
-            return;
-        }
-        if (threadIdx.x == 0) qp_grid::arrive_release(a.bar);
-    };
-    auto wait = [&](unsigned target) {                        // behind arrive
-        if (cluster) {
             qp_grid::cluster_wait();
-            return true;
+            if (threadIdx.x == 0) s_ok = 1;
+        } else if (threadIdx.x < 32) {
+            qp_grid::barrier_warp0(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
         }
-        return qp_grid::wait(a.bar, target + a.bar_extra, a.spin_limit, a.status, &s_ok);
     };
-    auto scratch_clean = [&]() {                              // one block, when nobody needs the scratch any more
-        for (int b = threadIdx.x; b < a.nb; b += SS_THREADS) a.hist[b] = 0ull;
+    auto empty = [&](int t, int threads) {                    // the tables, by threads t = 0 .. threads - 1
+        for (int i = t; i < ((a.nb + 1) << a.hist_shift); i += threads) bins[i] = 0u;
+        if constexpr (H > 0) {                                // (2 ni words << rep_shift are a multiple of 16 bytes)
+            const int vecs = (SS_GRID + 1 + H * (a.steps + 1)) << a.rep_shift >> 1;
+            for (int i = t; i < vecs; i += threads)
+                reinterpret_cast<uint4*>(raw)[i] = reinterpret_cast<uint4*>(raw + SS_SUMS_AT)[i] = make_uint4(0u, 0u, 0u, 0u);
+        }
     };
-    for (int i = threadIdx.x; i < ((a.nb + 1) << a.hist_shift); i += SS_THREADS) bins[i] = 0u;
-    if constexpr (SEARCH) {                                   // (2 ni words << rep_shift are a multiple of 16 bytes)
-        const int vecs = (SS_GRID + 1 + H * (a.steps + 1)) << a.rep_shift >> 1;
-        for (int i = threadIdx.x; i < vecs; i += SS_THREADS)
-            reinterpret_cast<uint4*>(raw)[i] = reinterpret_cast<uint4*>(raw + SS_SUMS_AT)[i] = make_uint4(0u, 0u, 0u, 0u);
-    }
 
     // ---- phase A
     if constexpr (STATS) {
+        if (SEARCH && blockIdx.x == 0)                        // (their first use is behind the barrier)
+            for (int k = threadIdx.x; k <= a.steps; k += SS_THREADS) a.acc[k] = 0ull;
         using Tiles = SsTiles<T, SS_TILE>;
         SsMoments acc;
         acc.clear();
@@ -624,57 +691,57 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
         }
         if (blockIdx.x == G - 1)
             for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) acc.one(qp_load_one(x + i));
-        double v5[5] = {acc.s, acc.sa, (double)acc.mn, (double)acc.mx, acc.bad};
-        ss_reduce<0, 0, 1, 2, 0>(v5, s_red);
+        const SsParts v = ss_block_parts<true>({acc.s, acc.sa, acc.mn, acc.mx, acc.bad}, s_block[0]);
         if (threadIdx.x == 0) {
-            double* p = a.part + (size_t)blockIdx.x * 8;
-            p[0] = v5[0]; p[1] = v5[1]; p[2] = v5[2]; p[3] = v5[3]; p[4] = v5[4];
+            part[0] = ss_row(v.a, v.b);
+            part[G] = make_uint4(__float_as_uint(v.lo), __float_as_uint(v.hi), v.count, 0u);
         }
-        if (!meet()) return SS_GAVE_UP;
-        // one warp merges the partials (all loads in flight together), the rest of the block waits at the barrier below
+        if (threadIdx.x >= 32) empty(threadIdx.x - 32, SS_THREADS - 32);          // while warp 0 waits and merges
+        meet_warp0();
         if (threadIdx.x < 32) {
-            double m5[5] = {0.0, 0.0, inf, -inf, 0.0};
-            for (unsigned b0 = lane; b0 < G; b0 += 32 * SS_MERGE) {
-                double p[SS_MERGE][5];
-#pragma unroll
-                for (int u = 0; u < SS_MERGE; ++u)
-#pragma unroll
-                    for (int j = 0; j < 5; ++j)
-                        p[u][j] = b0 + 32 * u < G ? __ldcg(a.part + (size_t)(b0 + 32 * u) * 8 + j) : (j == 2 ? inf : j == 3 ? -inf : 0.0);
-#pragma unroll
-                for (int u = 0; u < SS_MERGE; ++u) {
-                    m5[0] += p[u][0];
-                    m5[1] += p[u][1];
-                    m5[2] = fmin(m5[2], p[u][2]);
-                    m5[3] = fmax(m5[3], p[u][3]);
-                    m5[4] += p[u][4];                         // exact: counts are far below 2^53
-                }
-            }
-            ss_warp_reduce<0, 0, 1, 2, 0>(m5);
+            double s = 0.0, sa = 0.0, bad = 0.0;
+            float mn = __int_as_float(0x7F800000), mx = -mn;
+            ss_merge<2>(a.part, G, [&](const uint4 (&p)[2]) {
+                s += ss_row_first(p[0]);
+                sa += ss_row_second(p[0]);
+                mn = fminf(mn, __uint_as_float(p[1].x));
+                mx = fmaxf(mx, __uint_as_float(p[1].y));
+                bad += (double)p[1].z;                        // exact: counts are far below 2^53
+            });
+            __syncwarp();
+            s = ss_pair_sum(s, sa);
+            mn = ss_pair_min(mn, -mx);
+            bad = ss_pair_sum(bad, 0.0);
+            sa = __shfl_sync(0xFFFFFFFFu, s, 16);
+            mx = -__shfl_sync(0xFFFFFFFFu, mn, 16);
             if (lane == 0) {
-                const unsigned long long bad = (unsigned long long)m5[4], nf = a.n - bad;
+                const unsigned long long nbad = (unsigned long long)bad, nf = a.n - nbad;
                 s_st.n = a.n;
-                s_st.nonfinite = bad;
-                s_st.mean = nf ? m5[0] / (double)nf : 0.0;
-                s_st.mean_abs = nf ? m5[1] / (double)nf : 0.0;
-                s_st.min = nf ? m5[2] : 0.0;
-                s_st.max = nf ? m5[3] : 0.0;
+                s_st.nonfinite = nbad;
+                s_st.mean = nf ? s / (double)nf : 0.0;
+                s_st.mean_abs = nf ? sa / (double)nf : 0.0;
+                s_st.min = nf ? (double)mn : 0.0;
+                s_st.max = nf ? (double)mx : 0.0;
                 s_st.mad = s_st.var = 0.0;
                 s_st.hist_peak = 0;
                 s_st.hist_bins = 0;
                 s_st.reserved = 0;
             }
         }
+        __syncthreads();
+        if (!s_ok) return SS_GAVE_UP;
     } else {
+        empty(threadIdx.x, SS_THREADS);
         if (threadIdx.x == 0) s_st = *a.st_in;
+        __syncthreads();
     }
-    __syncthreads();
 
     // ---- phase B
     const bool guard = s_st.nonfinite != 0;
     const bool counting = STATS || (!a.promised && s_st.hist_bins != a.nb);
     if (counting) {
         const bool hist_on = s_st.max > s_st.min;
+        SsParts v = {0.0, 0.0, 0.f, 0.f, 0u};
         {
             SsDeviations d;
             d.m = (float)s_st.mean;
@@ -697,22 +764,16 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
             }
             if (blockIdx.x == G - 1)
                 for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) d.one(qp_load_one(x + i));
-            double v3[3] = {d.sd[0] + d.sd[1], d.sv[0] + d.sv[1], (double)d.below};
-            ss_reduce<0, 0, 0>(v3, s_red);                    // (its barriers also order the counters)
-            if (STATS && threadIdx.x == 0)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) a.part[(size_t)blockIdx.x * 8 + 5 + j] = v3[j];
+            v = ss_block_parts<false>({d.sd[0] + d.sd[1], d.sv[0] + d.sv[1], 0.f, 0.f, d.below}, s_block[1]);   // (its barrier orders the counters)
+            if (STATS && threadIdx.x == 0) {
+                part[2 * G] = ss_row(v.a, v.b);
+                part[3 * G] = make_uint4(v.count, 0u, 0u, 0u);
+            }
         }
-        const int reps = 1 << a.hist_shift;
-        for (int b = threadIdx.x; hist_on && b < a.nb; b += SS_THREADS) {
-            unsigned long long c = 0;
-            for (int r = 0; r < reps; ++r) c += bins[(b << a.hist_shift) + ((r + threadIdx.x) & (reps - 1))];
-            if (b == a.nb - 1)
-                for (int r = 0; r < reps; ++r) c += bins[(a.nb << a.hist_shift) + r];
-            if (c) atomicAdd(&a.hist[b], c);
-        }
+        if (hist_on) ss_hist_out(bins, a.nb, a.hist_shift, a.hist);
         if constexpr (SEARCH) {
-            if (!meet()) return SS_GAVE_UP;
+            __syncthreads();
+            meet_warp0();
         } else {                                              // statistics only: the last block out finishes
             __threadfence();
             __syncthreads();
@@ -726,36 +787,35 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
             __threadfence();
         }
         if (threadIdx.x < 32) {
-            double v3[4] = {0.0, 0.0, 0.0, 0.0};              // sum |x - m|, sum (x - m)^2, elements below m; largest bin
+            double sd = 0.0, sv = 0.0, below = 0.0, peak = 0.0;
+            unsigned long long c[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) c[u] = hist_on && lane + 32 * u < a.nb ? __ldcg(&a.hist[lane + 32 * u]) : 0ull;
             if (STATS)
-                for (unsigned b0 = lane; b0 < G; b0 += 32 * SS_MERGE) {
-                    double p[SS_MERGE][3];
+                ss_merge<2>(a.part + 2 * G, G, [&](const uint4 (&p)[2]) {
+                    sd += ss_row_first(p[0]);
+                    sv += ss_row_second(p[0]);
+                    below += (double)p[1].x;
+                });
 #pragma unroll
-                    for (int u = 0; u < SS_MERGE; ++u)
-#pragma unroll
-                        for (int j = 0; j < 3; ++j)
-                            p[u][j] = b0 + 32 * u < G ? __ldcg(a.part + (size_t)(b0 + 32 * u) * 8 + 5 + j) : 0.0;
-#pragma unroll
-                    for (int u = 0; u < SS_MERGE; ++u)
-#pragma unroll
-                        for (int j = 0; j < 3; ++j) v3[j] += p[u][j];
-                }
+            for (int u = 0; u < 4; ++u) peak = fmax(peak, (double)c[u]);
             if (hist_on)
-                for (int b0 = lane; b0 < a.nb; b0 += 32 * 4) {
-                    unsigned long long c[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) c[u] = b0 + 32 * u < a.nb ? __ldcg(&a.hist[b0 + 32 * u]) : 0ull;
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) v3[3] = fmax(v3[3], (double)c[u]);
-                }
-            ss_warp_reduce<0, 0, 0, 2>(v3);
+                for (int b = lane + 128; b < a.nb; b += 32) peak = fmax(peak, (double)__ldcg(&a.hist[b]));
+            __syncwarp();
+            if (STATS) {
+                sd = ss_pair_sum(sd, sv);
+                below = ss_pair_sum(below, 0.0);
+                sv = __shfl_sync(0xFFFFFFFFu, sd, 16);
+            }
+            for (int o = 16; o > 0; o >>= 1) peak = fmax(peak, __shfl_xor_sync(0xFFFFFFFFu, peak, o));
             if (lane == 0) {
                 if (STATS) {
                     const double nf = (double)(a.n - s_st.nonfinite), dm = s_st.mean - (double)(float)s_st.mean;
-                    s_st.mad = nf > 0.0 ? fmax(0.0, v3[0] - dm * (nf - 2.0 * v3[2])) / nf : 0.0;
-                    s_st.var = nf > 0.0 ? fmax(0.0, v3[1] / nf - dm * dm) : 0.0;
+                    s_st.mad = nf > 0.0 ? fmax(0.0, sd - dm * (nf - 2.0 * below)) / nf : 0.0;
+                    s_st.var = nf > 0.0 ? fmax(0.0, sv / nf - dm * dm) : 0.0;
+                    s_down = below;
                 }
-                s_st.hist_peak = (unsigned long long)v3[3];
+                s_st.hist_peak = (unsigned long long)peak;
                 s_st.hist_bins = a.nb;
                 if (STATS && (!SEARCH || blockIdx.x == 0)) {
                     *a.st_out = s_st;
@@ -765,9 +825,11 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
         }
         __syncthreads();
         if constexpr (!SEARCH) {
-            scratch_clean();
+            for (int b = threadIdx.x; b < a.nb; b += SS_THREADS) a.hist[b] = 0ull;
             if (threadIdx.x == 0) qp_grid::reset(a.bar);
             return SS_OUT;
+        } else if (!s_ok) {
+            return SS_GAVE_UP;
         }
     }
 
@@ -779,7 +841,6 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
         __shared__ int s_valid[QP_SS_MAX_CAND];
         __shared__ double s_curve[QP_SS_MAX_CAND];
         __shared__ int s_edge[SS_GRID + 1];                   // interval that a grid cell starts with
-        __shared__ unsigned char s_cell[SS_GRID + 1 + H * QP_SS_MAX_CAND];
         {                                                     // every thread the same set-up, then its part of the plan and its candidates
             const bool have = s_st.hist_bins == a.nb;
             if (!have && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, QP_DEV_HIST_MISSING);
@@ -802,10 +863,26 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
             }
         }
         __syncthreads();
-        const bool hard = s_plan.hard;
-        SsHard h;
-        h.M = 0;
-        if (!hard) {
+        const bool hard = s_plan.hard, flat = !(s_plan.inv_e > 0.f);
+        int* pos = reinterpret_cast<int*>(bins);              // [ncand][H], or the hard form's levels [2][ncand]: the histogram is out
+        double* lv = reinterpret_cast<double*>(bins);
+        int fix = ss_fix(a.n, 127 - (int)(__float_as_uint(s_plan.inv_e) >> 23));  // (1 / E is a power of two)
+        if constexpr (H == 0) {
+            // one bit: a side has one code, and the statistics say what its elements come to; how many they are is the
+            // one thing that the caller's statistics do not say
+            if constexpr (!STATS) {
+                const SsPlan<H> p = s_plan;
+                SsSides f = {p.m, guard, 0u, 0u};
+                SsTiles<T, SS_TILE>::template run<false>(x, a.ntiles, first, step, lane, f);
+                if (blockIdx.x == G - 1)
+                    for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) f.one(qp_load_one(x + i));
+                const SsParts v = ss_block_parts<false>({(double)f.all, 0.0, 0.f, 0.f, f.down}, s_block[0]);
+                if (threadIdx.x == 0) {
+                    atomicAdd(a.acc + ncand, (unsigned long long)v.count);
+                    atomicAdd(a.acc + ncand + 1, (unsigned long long)v.a - v.count);
+                }
+            }
+        } else if (!hard) {
             constexpr int CT = ss_ctile(H);
             const SsPlan<H> p = s_plan;
             SsTable tb;
@@ -822,7 +899,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
                 const uint64_t t1 = ntiles - t0 < per ? ntiles : t0 + per;
                 if (t0) {
                     __syncthreads();
-                    ss_flush<true>(raw, ni, a.rep_shift, row, t0 == per);
+                    ss_flush(raw, ni, a.rep_shift, row, t0 == per);
                     __syncthreads();
                 }
                 if (guard) {
@@ -838,9 +915,17 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
                     const float v = qp_load_one(x + i);
                     if (qp_is_finite(v)) ss_count<H>(p, tb, v);
                 }
+            ss_places<H>(s_plan, ncand, ni, s_edge, pos);
             __syncthreads();
-            ss_flush<false>(raw, ni, a.rep_shift, row, ntiles <= per);
+            const uint2 sides = ss_prefix(raw, ni, a.rep_shift, ntiles > per ? row : nullptr, s_edge, reinterpret_cast<ulonglong2*>(s_red));
+            __syncthreads();
+            if (!flat) ss_errors<H>(s_plan, ncand, ni, a.rep_shift, fix, raw, pos, s_cand, s_valid, a.acc);
+            if (!STATS && threadIdx.x == 0) {
+                atomicAdd(a.acc + ncand, (unsigned long long)sides.y);
+                atomicAdd(a.acc + ncand + 1, (unsigned long long)sides.x);
+            }
         } else {
+            SsHard h;
             double e2[2] = {0.0, 0.0};
             ss_hard_setup(a, ncand, s_cand, s_valid, raw, s_red, h);
             ulonglong2* row = a.rows + (size_t)blockIdx.x * (h.M + 1);
@@ -860,57 +945,68 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
             }
             if (blockIdx.x == G - 1)
                 for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) ss_hard_one(h, qp_load_one(x + i), e2[0], e2[1]);
-            ss_reduce<0, 0>(e2, s_red);
-            if (threadIdx.x == 0) {
-                a.part[(size_t)blockIdx.x * 8] = e2[0];
-                a.part[(size_t)blockIdx.x * 8 + 1] = e2[1];
-            }
+            const SsParts e = ss_block_parts<false>({e2[0], e2[1], 0.f, 0.f, 0u}, s_block[0]);
+            if (threadIdx.x == 0) part[0] = ss_row(e.a, e.b);         // (every block is done with the first rows)
             ss_hard_flush(h, row, fresh);
+            __syncthreads();
+            fix = ss_hard_errors(a, h, s_plan.m, ncand, row, s_cand, s_valid, lv, lv + ncand, s_red);
         }
-        const int count = hard ? h.M + 1 : 2 * ni;
-        if (!cluster) {
-            if (!meet()) return SS_GAVE_UP;
-            ss_slices(a, count, raw + SS_TABLE_BYTES);
-        }
-        arrive();
-        if (blockIdx.x == 0) {
-            int* pos = reinterpret_cast<int*>(raw + SS_TABLE_BYTES);          // [ncand][H + 2] in the histogram's room (the slices are stored)
-            if (!hard) ss_places<H>(s_plan, ncand, ni, s_edge, s_cell, pos);
-            if (!wait((waits + 1) * G)) return SS_GAVE_UP;
-            if (cluster) ss_all_slices(a, count);
-            if (!hard) {
-                ss_finish<H>(a, s_plan, s_st, ncand, ni, s_cell, pos, s_cand, s_valid, s_curve, s_red, reinterpret_cast<double*>(raw));
-            } else {
-                double v2[2] = {0.0, 0.0};
-                for (unsigned b = threadIdx.x; b < G; b += SS_THREADS)
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) v2[j] += __ldcg(a.part + (size_t)b * 8 + j);
-                ss_reduce<0, 0>(v2, s_red);
-                ss_hard_finish(a, h, s_plan.m, s_st, ncand, v2[0], v2[1], s_cand, s_valid, s_curve, s_red);
-            }
-            // (a warp that the pick does not wait for asks meanwhile)
-            if (!cluster && !a.packed && threadIdx.x == SS_THREADS - 1) ss_out(a, qp_grid::count_out(a.bar));
-            ss_pick(a, ncand, s_curve, s_cand, s_valid, s_setup);
-            scratch_clean();
-            if (!a.packed) return SS_OUT;
-            arrive();
-        } else {
-            if (cluster) {
-                wait(0);
-                if (a.packed) arrive();
-            }
-            if (!a.packed) {
-                if (threadIdx.x == 0) __threadfence();        // (the arrival, which nobody here polls for)
+        if constexpr (H > 0 || !STATS) {
+            __syncthreads();
+            if (!a.packed && blockIdx.x != 0) {               // nobody waits for the result but block 0
+                if (cluster) {
+                    qp_grid::cluster_arrive();
+                    qp_grid::cluster_wait();
+                } else if (threadIdx.x == 0) {
+                    qp_grid::arrive_release(a.bar);
+                    __threadfence();                          // (the arrival, which nobody here polls for)
+                }
                 return SS_DONE;
             }
+            if (!meet()) return SS_GAVE_UP;
+            // (block 0 of a separate search: a warp that the rest does not wait for asks meanwhile who is out)
+            if (!a.packed && !cluster && threadIdx.x == SS_THREADS - 1) ss_out(a, qp_grid::count_out(a.bar));
         }
+        SsBeyond beyond = {lv, lv + ncand, 0.0, 0.0};
+        if (hard && H > 0) {
+            if (threadIdx.x < 32) {
+                ss_merge<1>(a.part, G, [&](const uint4 (&p)[1]) {
+                    beyond.e_lo += ss_row_first(p[0]);
+                    beyond.e_hi += ss_row_second(p[0]);
+                });
+                __syncwarp();
+                const double e = ss_pair_sum(beyond.e_lo, beyond.e_hi);
+                if ((lane & 15) == 0) s_red[lane >> 4] = e;
+            }
+            __syncthreads();
+            beyond.e_lo = s_red[0];
+            beyond.e_hi = s_red[1];
+        }
+        const double down = STATS ? s_down : (double)__ldcg(a.acc + ncand);
+        const double up = STATS ? (double)(s_st.n - s_st.nonfinite) - down : (double)__ldcg(a.acc + ncand + 1);
+        const int best = ss_finish<H>(a, s_plan.m, flat, s_st, up, down, ncand, fix, s_cand, s_valid, s_curve, hard && H > 0 ? &beyond : nullptr,
+                                      s_block[0].sum, reinterpret_cast<int*>(s_block[0].count));
+        if (blockIdx.x == 0) {
+            if (threadIdx.x == 0) {
+                qp_ds_write_result(best, s_curve, s_setup, a.steps, a.nb, BITS, s_cand[best], a.ds_out, a.qp_out, a.status);
+                *a.setup = s_setup;
+            }
+            for (int k = threadIdx.x; k < ncand; k += SS_THREADS) {
+                a.curve[k] = s_curve[k];
+                a.cand[k] = s_cand[k];
+                a.valid[k] = s_valid[k];
+            }
+            for (int b = threadIdx.x; b < a.nb; b += SS_THREADS) a.hist[b] = 0ull;       // (nobody needs it any more)
+            if (!STATS)
+                for (int k = threadIdx.x; k < ncand + 2; k += SS_THREADS) a.acc[k] = 0ull;
+        }
+        if constexpr (!STATS) return SS_OUT;
         if constexpr (STATS) {                                // the sender: everybody packs, from the tensor's end
-            if (!wait((waits + 1) * G + 1)) return SS_GAVE_UP;
-            const float lo = __ldcg(&a.qp_out->lo), hi = __ldcg(&a.qp_out->hi), inv = __ldcg(&a.qp_out->inv_scale);
+            const float4 q = s_cand[best];
             uint32_t* sw = reinterpret_cast<uint32_t*>(raw) + (threadIdx.x >> 5) * 256;
             const uint64_t tiles = (a.n + QP_TILE - 1) / QP_TILE;
             for (uint64_t it = first; it < tiles; it += step)
-                qp_pack_tile<BITS, T, true>(x, a.n, tiles - 1 - it, lane, lo, hi, inv, a.packed, a.nwords, sw);
+                qp_pack_tile<BITS, T, true>(x, a.n, tiles - 1 - it, lane, q.x, q.y, q.w, a.packed, a.nwords, sw);
         }
     }
     return SS_DONE;
@@ -944,7 +1040,7 @@ bool ss_usable(qp_ctx* ctx)
         // the scratch that other forms own: block partials, and the interval path's rows
         bool ok = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device) == cudaSuccess && coop &&
                   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device) == cudaSuccess &&
-                  (size_t)ctx->sm_count * 8 * sizeof(double) <= sizeof(qp_stats_partial) * QP_MAX_BLOCKS &&
+                  (size_t)ctx->sm_count * 4 * sizeof(uint4) <= sizeof(qp_stats_partial) * QP_MAX_BLOCKS &&
                   (size_t)ctx->sm_count * QP_SS_TOTALS * 2 <= (size_t)ctx->iv_blocks * (QP_IV_MAXB + 1);
         for (int bits = 0; ok && bits <= 4; ++bits)
             for (int v = 0; ok && v < (bits ? 4 : 2); ++v) {
@@ -990,7 +1086,7 @@ int32_t qp_launch_stats_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t
                                qp_qparams_t* d_qp_out, void* d_packed, cudaStream_t s)
 {
     static_assert(2 * (SS_GRID + 1 + 7 * QP_SS_MAX_CAND) <= QP_SS_TOTALS && 15 * QP_SS_MAX_CAND + 1 <= QP_SS_TOTALS, "interval totals");
-    static_assert(QP_SS_MAX_CAND * 9 * sizeof(int) <= SS_HIST_BYTES && SS_WARPS * 32 * 16 <= SS_HIST_BYTES, "the histogram's room is used again");
+    static_assert(QP_SS_MAX_CAND * 7 * sizeof(int) <= SS_HIST_BYTES && QP_SS_MAX_CAND * 2 * sizeof(double) <= SS_HIST_BYTES, "the histogram's room is used again");
     SsArgs a;
     a.x = d_x;
     a.n = n;
@@ -1009,11 +1105,11 @@ int32_t qp_launch_stats_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t
     a.cand = ctx->d_cand;
     a.valid = ctx->d_valid;
     a.setup = ctx->d_setup;
-    a.part = reinterpret_cast<double*>(ctx->d_part);
+    a.part = reinterpret_cast<uint4*>(ctx->d_part);
     unsigned char* f = static_cast<unsigned char*>(ctx->d_fused);
     a.bar = reinterpret_cast<unsigned*>(f) + 16;              // words 16, 17 (the sender uses 0, 1, the statistics 8..10 and 24, 25)
     a.hist = reinterpret_cast<unsigned long long*>(f + 256);
-    a.tot = reinterpret_cast<ulonglong2*>(f + QP_FUSED_TOTALS_AT);
+    a.acc = reinterpret_cast<unsigned long long*>(f + QP_FUSED_TOTALS_AT) + (st_in ? QP_SS_MAX_CAND + 2 : 0);
     a.rows = reinterpret_cast<ulonglong2*>(ctx->d_iv_part);
     a.status = ctx->d_status;
     a.spin_limit = ctx->spin_limit;

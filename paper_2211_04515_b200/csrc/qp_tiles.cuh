@@ -48,6 +48,91 @@ __device__ __forceinline__ void ss_reduce(double (&v)[sizeof...(OPS)], double* s
     }
 }
 
+// Two values at once over a warp, in one shuffle more than one takes: lanes 0..15 get a's result, lanes 16..31 b's.
+__device__ __forceinline__ double ss_pair_sum(double a, double b)
+{
+    const bool upper = (threadIdx.x & 16) != 0;
+    double v = upper ? b : a;
+    v += __shfl_xor_sync(0xFFFFFFFFu, upper ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+}
+__device__ __forceinline__ float ss_pair_min(float a, float b)
+{
+    const bool upper = (threadIdx.x & 16) != 0;
+    float v = upper ? b : a;
+    v = fminf(v, __shfl_xor_sync(0xFFFFFFFFu, upper ? a : b, 16));
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    return v;
+}
+
+// Two sums, a smallest and a largest value and a count over the block, for the lanes of warp 0 (the warps' results in a fixed
+// order); the other warps have stored theirs and are behind the block barrier.  RANGE: lo and hi are wanted.
+struct SsBlock { double sum[2 * SS_WARPS]; float least[2 * SS_WARPS]; unsigned count[SS_WARPS]; };
+struct SsParts { double a, b; float lo, hi; unsigned count; };
+template <bool RANGE>
+__device__ __forceinline__ SsParts ss_block_parts(SsParts v, SsBlock& sh)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double s = ss_pair_sum(v.a, v.b);
+    float l = 0.f;
+    if (RANGE) l = ss_pair_min(v.lo, -v.hi);
+    const unsigned c = __reduce_add_sync(0xFFFFFFFFu, v.count);
+    if ((lane & 15) == 0) {
+        sh.sum[lane + warp] = s;
+        if (RANGE) sh.least[lane + warp] = l;
+        if (lane == 0) sh.count[warp] = c;
+    }
+    static_assert(SS_WARPS == 16, "a lane per warp's sum and half");
+    __syncthreads();
+    if (warp == 0) {
+        double t = sh.sum[lane];
+        float m = RANGE ? sh.least[lane] : 0.f;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+            if (RANGE) m = fminf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+        }
+        v.a = __shfl_sync(0xFFFFFFFFu, t, 0);
+        v.b = __shfl_sync(0xFFFFFFFFu, t, 16);
+        if (RANGE) {
+            v.lo = __shfl_sync(0xFFFFFFFFu, m, 0);
+            v.hi = -__shfl_sync(0xFFFFFFFFu, m, 16);
+        }
+        v.count = __reduce_add_sync(0xFFFFFFFFu, lane < SS_WARPS ? sh.count[lane] : 0u);
+    }
+    return v;
+}
+
+// Block partials: rows of 16 bytes per block.  All blocks read all of them at the same time, so what counts is how few sectors of
+// L2 a merge asks for: with a partial's five doubles 64 bytes apart from the next block's, the slowest of 148 blocks had the sums of
+// phase A 6 us after the fastest; with two rows of 16 bytes it is within 1 us.  One warp, SS_MERGE blocks per lane in flight;
+// take(u): the ROWS vectors of a block, in order of its number per lane.
+__device__ __forceinline__ uint4 ss_row(double a, double b)
+{
+    const unsigned long long u = (unsigned long long)__double_as_longlong(a), v = (unsigned long long)__double_as_longlong(b);
+    return make_uint4((unsigned)u, (unsigned)(u >> 32), (unsigned)v, (unsigned)(v >> 32));
+}
+__device__ __forceinline__ double ss_row_first(const uint4& r) { return __hiloint2double((int)r.y, (int)r.x); }
+__device__ __forceinline__ double ss_row_second(const uint4& r) { return __hiloint2double((int)r.w, (int)r.z); }
+template <int ROWS, typename F>
+__device__ __forceinline__ void ss_merge(const uint4* part, unsigned G, F&& take)
+{
+    for (unsigned b0 = threadIdx.x & 31; b0 < G; b0 += 32 * SS_MERGE) {
+        uint4 p[SS_MERGE][ROWS];
+#pragma unroll
+        for (int u = 0; u < SS_MERGE; ++u)
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r)
+                if (b0 + 32 * u < G) p[u][r] = __ldcg(part + (size_t)r * G + b0 + 32 * u);
+#pragma unroll
+        for (int u = 0; u < SS_MERGE; ++u)
+            if (b0 + 32 * u < G) take(p[u]);
+    }
+}
+
 // ---- streaming.  A warp works on tiles of N 16-byte vectors per lane, held in registers; a vector's registers are
 // reloaded from the warp's next tile as soon as its elements have been taken out, so the loads of a whole tile are
 // in flight all the time without a second set of registers or moves between the two.

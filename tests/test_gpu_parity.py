@@ -1253,6 +1253,27 @@ def test_stats_and_search_in_one_launch(ctx, bits, bmode, steps, nb, n, data, bf
     assert ctx.qp_get_status() & ~(qp.QP_DEV_NONFINITE | qp.QP_DEV_DEGENERATE) == 0
 
 
+# the blocks add up their parts of the candidates' errors in integers: tables emptied on the way (few replicas: after three tiles
+# of 512 elements per warp; one tile less, and one element more), every number of intervals per thread of the prefix sums, one bit with
+# elements that do not count; the separate search and the sender score alike
+@pytest.mark.parametrize("bits,steps,n,data", [(4, 255, 3 * 148 * 16 * 512, "vit"), (4, 255, 3 * 148 * 16 * 512 + 1025, "outliers"),
+                                               (3, 255, 40 * 1024 + 3, "vit"), (4, 170, 70 * 1024, "vit"), (2, 255, 33 * 1024, "vit"),
+                                               (1, 100, 40 * 1024 + 3, "nonfinite"), (4, 100, (1 << 18) + 5, "nonfinite")])
+def test_search_block_sums(ctx, bits, steps, n, data):
+    x = si.vit_activation((1, n // 256 + 1, 256), 800 + bits, outlier_frac=0.02 if data == "outliers" else 0.0).reshape(-1)[:n].copy()
+    if data == "nonfinite":
+        x[[0, 1023, n // 2, n - 1]] = [np.nan, np.inf, -np.inf, np.nan]
+    d = dev(x)
+    check_search(ctx, x, d, bits, 0, steps, 100, exact_steps=[0, steps // 2, steps])
+    separate = np.array(ctx.qp_dsaciq_curve(steps))
+    for _ in range(2):                                        # (the second launch finds the sums as the first one left them)
+        ctx.qp_sender_device(d, bits, True, steps=steps)
+        curve = np.array(ctx.qp_dsaciq_curve(steps))
+        fin = np.isfinite(separate)
+        assert np.array_equal(np.isfinite(curve), fin) and np.all(np.abs(curve - separate)[fin] <= 1e-7 * separate[fin])
+    ctx.qp_get_status()
+
+
 # a histogram over a range that overflows fp32 ("wide": x - min does), or whose reciprocal does ("subnormal": 0 * inf among
 # the positions): every element in a bin, the same one as in the kernels that count by an integer conversion
 @pytest.mark.parametrize("n", [70 * 1024 + 5, (1 << 20) + 77])
