@@ -6,17 +6,18 @@
 //   phase B   sum |x - mean|, sum (x - mean)^2, histogram over the channel's [min, max]
 //   phase C   per channel, the count and the sum of the elements of every interval between the candidates' thresholds
 //             (qp_affine.cuh), in shared memory
-//   finish    a team of four warps per channel (the first two scan a side each): prefix sums over the intervals, the error of every candidate from 2^bits
-//             differences, first minimum, quantizer
+//   finish    a team of four warps per channel (two scan a side each): prefix sums over the intervals, the error of every candidate from 2^bits
+//             differences (a thread each), first minimum, quantizer
 // Between the phases the blocks of a cluster add up their parts through distributed shared memory.  A thread stays with one
 // channel and walks its rows, eight loads ahead; the first pass takes the strip from DRAM, the others from L2.
 //
-// What bounds it: the loads of 4 bytes per lane (a strip's row is 4 w bytes, so a warp's load touches several lines; the load
-// queue and the latency behind it are two thirds of the stalls), the instructions (A 4, B 11, C 14 + 2 per code
-// boundary and element), and the finish.  12608 x 1024 fp32 at 4 bits (52 MB): 105 us, of which A 18, B 12, C 19, sums across the
-// cluster 17, finish 27, plans 4; the ten kernels before (four for the statistics, histogram, set-up, thresholds sorted per
-// channel, a pass with binary searches, error curves, pick) took 255 us.  Gathering the interval sums entry by entry
-// through distributed shared memory took 32 us instead of 10, one warp per side for all of a channel's candidates 16 instead of 5.
+// What bounds it: the 32-byte sectors that a strip's rows touch (ct_choose), the instructions (A 4, B 11, C 14 + 2 per code
+// boundary and element) with their shared atomics, and the chain of small steps around the passes.  12608 x 1024 fp32 at 4 bits (52 MB), by
+// time stamps: A 15 us, its sums across the cluster 3, B 13 and 3, peaks and plans 5, C 19, interval sums across the cluster 6 (16
+// bytes a load; 8 with 4 bytes), prefix sums 4 (13 without a branch per interval and with a warp per side), errors 7, pick 1: 77, and
+// the whole stage (receiver, this, packing) 110; strips of 14 channels, whose rows start anywhere in a sector, and those
+// two forms took 101 and 134.  The ten kernels before (four for the statistics, histogram, set-up, thresholds sorted per
+// channel, a pass with binary searches, error curves, pick) took 255 us.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -32,6 +33,7 @@ namespace {
 constexpr int CT_THREADS = 1024;
 constexpr int CT_TEAMS = 8;                        // teams of the finish: a channel each
 constexpr int CT_TEAM = CT_THREADS / CT_TEAMS;     // threads of a team (two warps at least: a side each)
+constexpr int CT_PEAK = 64;                        // threads that look for a histogram's peak
 constexpr int CT_MAX_W = 16;                       // channels of a strip
 constexpr int CT_MAX_S = 8;                        // blocks of a cluster
 constexpr int CT_AHEAD = 8;                        // loads in flight per thread: a batch
@@ -48,6 +50,7 @@ struct CtArgs {
     int w;                                         // channels per strip
     uint64_t rows_pb;                              // rows per block of a cluster
     int nb, steps, bmode, ncp, ub;
+    int len;                                       // words of a channel's intervals, both sides, up to the next 16 bytes
     double F;
     const qp_stats_t* st_in;                       // search only: the caller's statistics
     qp_stats_t* st_out;
@@ -182,31 +185,36 @@ struct CtCounter {
     __device__ __forceinline__ void fold() {}
 };
 
-// N quantities of every thread added up (OPS: 0 sum, 1 min, 2 max) over the row lanes of its channel: a fixed tree; the
-// result is in the threads of row lane 0.  red: N * CT_THREADS doubles.
+// N quantities of every thread added up (OPS: 0 sum, 1 min, 2 max) over the row lanes of its channel: a warp takes a
+// channel, in a fixed tree, and leaves the results in out[channel].  red: N * w * (nl | 1) doubles, a channel's values side by side.
 template <int... OPS>
-__device__ __forceinline__ void ct_reduce(double (&v)[sizeof...(OPS)], double* red, int rl, int nl, int w)
+__device__ __forceinline__ void ct_reduce(const double (&v)[sizeof...(OPS)], double* red, int slot, int rl, int nl, int w,
+                                          double (*out)[sizeof...(OPS)])
 {
     constexpr int N = sizeof...(OPS);
     constexpr int ops[N] = {OPS...};
+    const int pitch = nl | 1, lane = threadIdx.x & 31;
+    if (rl < nl)
 #pragma unroll
-    for (int j = 0; j < N; ++j) red[j * CT_THREADS + threadIdx.x] = v[j];
+        for (int j = 0; j < N; ++j) red[(j * w + slot) * pitch + rl] = v[j];
     __syncthreads();
-    int off = 1;
-    while (off < nl) off <<= 1;
-    for (off >>= 1; off > 0; off >>= 1) {
-        if (rl < off && rl + off < nl) {
+    for (int c = threadIdx.x >> 5; c < w; c += CT_THREADS / 32) {
 #pragma unroll
-            for (int j = 0; j < N; ++j) {
-                const double t = red[j * CT_THREADS + threadIdx.x + off * w];
-                v[j] = ops[j] == 0 ? v[j] + t : (ops[j] == 1 ? fmin(v[j], t) : fmax(v[j], t));
-                red[j * CT_THREADS + threadIdx.x] = v[j];
-            }
+        for (int j = 0; j < N; ++j) {
+            const double* at = red + (j * w + c) * pitch;
+            auto both = [&](double a, double b) { return ops[j] == 0 ? a + b : (ops[j] == 1 ? fmin(a, b) : fmax(a, b)); };
+            double t = ops[j] == 0 ? 0.0 : (ops[j] == 1 ? (double)CT_INF : -(double)CT_INF);
+            for (int i = lane; i < nl; i += 32) t = both(t, at[i]);
+            __syncwarp();
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t = both(t, __shfl_xor_sync(0xFFFFFFFFu, t, o));
+            if (lane == 0) out[c][j] = t;
         }
-        __syncthreads();
     }
 }
 
+__device__ __forceinline__ void ct_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void ct_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void ct_team_sync(int team) { asm volatile("barrier.sync %0, %1;" ::"r"(team + 1), "n"(CT_TEAM) : "memory"); }
 
 // STATS: phases A and B (otherwise the statistics come with st_in and B only counts the histogram).  HH: code boundaries above
@@ -270,10 +278,7 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
                 v5[0] = g.s; v5[1] = g.sa; v5[2] = (double)g.mn; v5[3] = (double)g.mx; v5[4] = g.bad;
             }
         }
-        ct_reduce<0, 0, 1, 2, 0>(v5, red, rl, nl, w);
-        if (rl == 0)
-#pragma unroll
-            for (int j = 0; j < 5; ++j) s_a[slot][j] = v5[j];
+        ct_reduce<0, 0, 1, 2, 0>(v5, red, slot, rl, nl, w, s_a);
         cluster.sync();
         if ((int)threadIdx.x < nch) {                         // every block the same sums, in rank order
             double t[5] = {0.0, 0.0, inf, -inf, 0.0};
@@ -323,12 +328,14 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
         };
         if (odd || beyond) pass(std::integral_constant<int, 2>{}); else pass(std::integral_constant<int, STATS ? 0 : 1>{});
         if constexpr (STATS) {
-            ct_reduce<0, 0, 0>(v3, red, rl, nl, w);
-            if (rl == 0)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) s_b[slot][j] = v3[j];
+            ct_reduce<0, 0, 0>(v3, red, slot, rl, nl, w, s_b);
+            if (SEARCH) __syncthreads();                      // (the interval tables lie where red is)
         }
-        cluster.sync();                                       // (orders the histogram counters of the cluster, too)
+        ct_arrive();                                          // (orders the histogram counters of the cluster, too)
+        if constexpr (SEARCH)
+            for (int i = threadIdx.x; i < w * a.len / 4; i += CT_THREADS)
+                reinterpret_cast<uint4*>(raw)[i] = reinterpret_cast<uint4*>(raw + SS_SUMS_AT)[i] = make_uint4(0u, 0u, 0u, 0u);
+        ct_wait();
         if (STATS && (int)threadIdx.x < nch) {
             double t[3] = {0.0, 0.0, 0.0};
             for (int r = 0; r < S; ++r) {
@@ -354,23 +361,28 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
         __shared__ qp_ds_setup s_setup[CT_MAX_W];
         // (in the histogram's room, which is free by then)
         double (*s_v)[CT_MAX_CAND] = reinterpret_cast<double (*)[CT_MAX_CAND]>(raw + CT_TABLE_BYTES);
-        int (*s_edge)[SS_GRID + 1] = reinterpret_cast<int (*)[SS_GRID + 1]>(raw + CT_TABLE_BYTES + sizeof(double) * (CT_TEAMS) * CT_MAX_CAND);
-        static_assert((CT_TEAMS) * (CT_MAX_CAND * sizeof(double) + (SS_GRID + 1) * sizeof(int)) <= CT_DYN_BYTES - CT_TABLE_BYTES, "room");
-        __shared__ unsigned s_n[CT_TEAMS][2];
+        int (*s_edge)[SS_GRID + 2] = reinterpret_cast<int (*)[SS_GRID + 2]>(raw + CT_TABLE_BYTES + sizeof(double) * CT_TEAMS * CT_MAX_CAND);
+        static_assert(CT_TEAMS * (CT_MAX_CAND * sizeof(double) + (SS_GRID + 2) * sizeof(int)) <= CT_DYN_BYTES - CT_TABLE_BYTES, "room");
+        static_assert(CT_MAX_CAND <= CT_TEAM, "a thread per candidate");
+        __shared__ uint2 s_n[CT_TEAMS][4];                    // per warp: elements, and the first candidate of the smallest error
+        __shared__ unsigned long long s_sum[CT_TEAMS][4];
         const int ncand = a.steps + 1, ni = SS_GRID + 1 + H * ncand;
         if (threadIdx.x < CT_MAX_W) s_top[threadIdx.x] = 0u;
-        for (int i = threadIdx.x; i < w * ni; i += CT_THREADS)                     // w * 2 ni words of counts and of sums
-            reinterpret_cast<uint2*>(raw)[i] = reinterpret_cast<uint2*>(raw + SS_SUMS_AT)[i] = make_uint2(0u, 0u);
         __syncthreads();
-        for (int i = threadIdx.x; i < nch * a.nb; i += CT_THREADS) {               // peak of the histogram
-            const int sl = i / a.nb, b = i - sl * a.nb;
-            unsigned c = 0u;
-            for (int r = 0; r < S; ++r) {
-                const unsigned* q = cluster.map_shared_rank(bins, r) + sl * (a.nb + 1) + b;
-                c += q[0];
-                if (b == a.nb - 1) c += q[1];
+        for (int sl = threadIdx.x / CT_PEAK; sl < nch; sl += CT_THREADS / CT_PEAK) {          // peak of the histogram
+            unsigned top = 0u;
+            for (int b = threadIdx.x % CT_PEAK; b < a.nb; b += CT_PEAK) {
+                unsigned c = 0u;
+                for (int r = 0; r < S; ++r) {
+                    const unsigned* q = cluster.map_shared_rank(bins, r) + sl * (a.nb + 1) + b;
+                    c += q[0];
+                    if (b == a.nb - 1) c += q[1];
+                }
+                top = max(top, c);
             }
-            atomicMax(&s_top[sl], c);
+            __syncwarp();
+            top = __reduce_max_sync(0xFFFFFFFFu, top);
+            if (lane == 0) atomicMax(&s_top[sl], top);
         }
         __syncthreads();
         if ((int)threadIdx.x < nch * 8) {                     // eight threads per channel: the common part, and a boundary each
@@ -389,7 +401,7 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
             const SsPlan<H> p = s_plan[slot < nch ? slot : 0];
             SsTable tb;
             tb.mul = 4u;
-            tb.base = (unsigned)__cvta_generic_to_shared(raw) + (unsigned)(slot * 2 * ni) * 4u - SS_ONE * 4u;
+            tb.base = (unsigned)__cvta_generic_to_shared(raw) + (unsigned)(slot * a.len) * 4u - SS_ONE * 4u;
             tb.half = (unsigned)ni * 4u;
             tb.ni = (unsigned)ni;
             tb.ub = (unsigned)a.ub;
@@ -406,101 +418,118 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
         cluster.sync();
 
         // ---- finish: channel slots rank, rank + S, ... of the strip are this block's.  Their totals over the cluster, in place:
-        // count | high bits of the sum << 24 (rows <= 65535, at most 8 sums of 32 bits); eight entries' loads in flight.
+        // count | high bits of the sum << 24 (rows <= 65535, at most 8 sums of 32 bits); 16 bytes a load, the peers one after another
+        // from the next one on.
         if (S > 1) {
-            const int own = (nch - rank + S - 1) / S, len = 2 * ni;
-            unsigned* cnt = reinterpret_cast<unsigned*>(raw);
-            unsigned* sum = reinterpret_cast<unsigned*>(raw + SS_SUMS_AT);
-            for (int e0 = threadIdx.x; e0 < own * len; e0 += 8 * CT_THREADS) {
-                unsigned n[8];
-                unsigned long long t[8];
-                int at[8];
+            const int own = (nch - rank + S - 1) / S, len = a.len / 4;
+            uint4* cnt = reinterpret_cast<uint4*>(raw);
+            uint4* sum = reinterpret_cast<uint4*>(raw + SS_SUMS_AT);
+            for (int e0 = threadIdx.x; e0 < own * len; e0 += 2 * CT_THREADS) {
+                uint4 n[2];
+                unsigned long long t[2][4];
+                int at[2];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int e = e0 + j * CT_THREADS, sl = e / len;
-                    at[j] = e < own * len ? (rank + sl * S) * len + (e - sl * len) : 0;
-                    n[j] = 0u;
-                    t[j] = 0ull;
+                for (int j = 0; j < 2; ++j) {
+                    const int e = min(e0 + j * CT_THREADS, own * len - 1), sl = e / len;
+                    at[j] = (rank + sl * S) * len + (e - sl * len);
+                    n[j] = cnt[at[j]];
+                    const uint4 d = sum[at[j]];
+                    t[j][0] = d.x; t[j][1] = d.y; t[j][2] = d.z; t[j][3] = d.w;
                 }
-                for (int r = 0; r < S; ++r) {
-                    const unsigned* rc = cluster.map_shared_rank(cnt, r);
-                    const unsigned* rs = cluster.map_shared_rank(sum, r);
+                for (int o = 1; o < S; ++o) {
+                    const int r = rank + o < S ? rank + o : rank + o - S;
+                    const uint4* rc = cluster.map_shared_rank(cnt, r);
+                    const uint4* rs = cluster.map_shared_rank(sum, r);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        n[j] += rc[at[j]];
-                        t[j] += rs[at[j]];
+                    for (int j = 0; j < 2; ++j) {
+                        const uint4 c = rc[at[j]], d = rs[at[j]];
+                        n[j].x += c.x; n[j].y += c.y; n[j].z += c.z; n[j].w += c.w;
+                        t[j][0] += d.x; t[j][1] += d.y; t[j][2] += d.z; t[j][3] += d.w;
                     }
                 }
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
+                for (int j = 0; j < 2; ++j)
                     if (e0 + j * CT_THREADS < own * len) {
-                        cnt[at[j]] = n[j] | (unsigned)(t[j] >> 32) << 24;
-                        sum[at[j]] = (unsigned)t[j];
+                        cnt[at[j]] = make_uint4(n[j].x | (unsigned)(t[j][0] >> 32) << 24, n[j].y | (unsigned)(t[j][1] >> 32) << 24,
+                                                n[j].z | (unsigned)(t[j][2] >> 32) << 24, n[j].w | (unsigned)(t[j][3] >> 32) << 24);
+                        sum[at[j]] = make_uint4((unsigned)t[j][0], (unsigned)t[j][1], (unsigned)t[j][2], (unsigned)t[j][3]);
                     }
             }
             __syncthreads();
         }
-        // a team takes a channel: its first two warps a side each for the prefix sums, then all of it the candidates
-        const int team = threadIdx.x / CT_TEAM, tt = threadIdx.x % CT_TEAM, side = tt >> 5;
-        for (int sl = rank + team * S; sl < nch; sl += (CT_TEAMS) * S) {
+        // a team takes a channel: two warps a side for the prefix sums, then a thread per candidate
+        const int team = threadIdx.x / CT_TEAM, tt = threadIdx.x % CT_TEAM, part = tt >> 5, side = part >> 1;
+        for (int sl = rank + team * S; sl < nch; sl += CT_TEAMS * S) {
             const SsPlan<H>& p = s_plan[sl];
             if (p.hard) continue;                             // uniform over the team
             const uint32_t c = c0 + sl;
-            for (int g = tt; g <= SS_GRID; g += CT_TEAM) s_edge[team][g] = ss_cell_start(p, g);
+            unsigned* c_up = reinterpret_cast<unsigned*>(raw) + sl * a.len;
+            unsigned* t_up = reinterpret_cast<unsigned*>(raw + SS_SUMS_AT) + sl * a.len;
+            for (int g = tt; g <= SS_GRID + 1; g += CT_TEAM) s_edge[team][g] = g <= SS_GRID ? ss_cell_start(p, g) : 1 << 30;
             ct_team_sync(team);
-            if (side < 2) {
-                unsigned* cnt = reinterpret_cast<unsigned*>(raw) + (2 * sl + side) * ni;
-                unsigned* sum = reinterpret_cast<unsigned*>(raw + SS_SUMS_AT) + (2 * sl + side) * ni;
-                const int per = (ni + 31) / 32, i0 = min(lane * per, ni), i1 = min(i0 + per, ni);
-                int cell = 0;
-                {
-                    int hi = SS_GRID;                             // grid cell of interval i0
-                    while (cell < hi) { const int mid = (cell + hi + 1) >> 1; if (s_edge[team][mid] <= i0) cell = mid; else hi = mid - 1; }
-                }
-                const int cell0 = cell;
+            {
+                // Consecutive intervals per thread, an odd number of them (no bank twice); an interval is in the cell of the one before
+                // it or in the next, as every cell starts an interval.  No branch may part the lanes here: 25 intervals a lane behind a
+                // `while` over the cells took 12 us.
+                constexpr int HALF = CT_TEAM / 2;
+                unsigned* cnt = c_up + side * ni;
+                unsigned* sum = t_up + side * ni;
+                const int* edge = s_edge[team];
+                const int per = ((ni + HALF - 1) / HALF) | 1, i0 = min((tt & (HALF - 1)) * per, ni), i1 = min(i0 + per, ni);
+                int cell0 = 0;                                // grid cell of interval i0
+#pragma unroll
+                for (int o = SS_GRID; o > 0; o >>= 1) cell0 += edge[min(cell0 + o, SS_GRID + 1)] <= i0 ? o : 0;
                 unsigned n_all = 0u;
                 unsigned long long s_all = 0ull;
+                int cell = cell0, next = edge[cell + 1];
                 for (int i = i0; i < i1; ++i) {
-                    while (cell < SS_GRID && s_edge[team][cell + 1] <= i) ++cell;
-                    const unsigned n = cnt[i] & 0xFFFFFFu;
+                    cell += next <= i ? 1 : 0;
+                    next = edge[cell + 1];
+                    const unsigned cn = cnt[i], n = cn & 0xFFFFFFu;
                     n_all += n;
-                    s_all += ((unsigned long long)(cnt[i] >> 24) << 32 | sum[i]) + ((unsigned long long)n * (unsigned)cell << a.ub);
+                    s_all += ((unsigned long long)(cn >> 24) << 32 | sum[i]) + ((unsigned long long)n * (unsigned)cell << a.ub);
                 }
+                __syncwarp();
                 // exclusive prefix sums, in place: count in 17 bits | high bits of the sum << 17, low word of the sum
                 unsigned np = n_all;
                 unsigned long long sp = s_all;
+#pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const unsigned tn = __shfl_up_sync(0xFFFFFFFFu, np, o);
                     const unsigned long long ts = __shfl_up_sync(0xFFFFFFFFu, sp, o);
                     if (lane >= o) { np += tn; sp += ts; }
                 }
-                const unsigned n_side = __shfl_sync(0xFFFFFFFFu, np, 31);
+                if (lane == 31) { s_n[team][part].x = np; s_sum[team][part] = sp; }
+                ct_team_sync(team);
                 np -= n_all;
                 sp -= s_all;
+                if (part & 1) { np += s_n[team][part - 1].x; sp += s_sum[team][part - 1]; }
                 cell = cell0;
+                next = edge[cell + 1];
                 for (int i = i0; i < i1; ++i) {
-                    while (cell < SS_GRID && s_edge[team][cell + 1] <= i) ++cell;
-                    const unsigned n = cnt[i] & 0xFFFFFFu;
-                    const unsigned long long s = (unsigned long long)(cnt[i] >> 24) << 32 | sum[i];
+                    cell += next <= i ? 1 : 0;
+                    next = edge[cell + 1];
+                    const unsigned cn = cnt[i], n = cn & 0xFFFFFFu;
+                    const unsigned long long s = (unsigned long long)(cn >> 24) << 32 | sum[i];
                     cnt[i] = np | (unsigned)(sp >> 32) << 17;
                     sum[i] = (unsigned)sp;
                     np += n;
                     sp += s + ((unsigned long long)n * (unsigned)cell << a.ub);
                 }
-                if (lane == 0) s_n[team][side] = n_side;
             }
             ct_team_sync(team);
 
             const qp_stats_t& q = s_st[sl];
-            const qp_ds_setup su = s_setup[sl];
+            const qp_ds_setup& su = s_setup[sl];
             const double nf = (double)(q.n - q.nonfinite), dm = q.mean - (double)p.m;
-            const double s_abs = nf * q.mad + dm * ((double)s_n[team][0] - (double)s_n[team][1]);
+            const double up = (double)(s_n[team][0].x + s_n[team][1].x), down = (double)(s_n[team][2].x + s_n[team][3].x);
+            const double s_abs = nf * q.mad + dm * (up - down);
             const double s_up = 0.5 * (s_abs + nf * dm), s_down = 0.5 * (s_abs - nf * dm);     // sum |y| of each side
             const bool flat = !(p.inv_e > 0.f);
-            const unsigned* c_up = reinterpret_cast<unsigned*>(raw) + 2 * sl * ni;
-            const unsigned* t_up = reinterpret_cast<unsigned*>(raw + SS_SUMS_AT) + 2 * sl * ni;
-            for (int k = tt; k < ncand; k += CT_TEAM) {
-                float4 cd;
+            const int k = tt;
+            float4 cd = make_float4(0.f, 0.f, 0.f, 0.f);
+            double mse = inf;
+            if (k < ncand) {
                 int ok;
                 qp_ds_candidate(su, k, a.steps, BITS, a.bmode & QP_B_MIDRISE, cd, ok);
                 a.cand[(size_t)c * a.ncp + k] = cd;
@@ -508,7 +537,7 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
                 double v = 0.0, n_up = 0.0, n_down = 0.0, x_up = 0.0, x_down = 0.0;
                 for (int i = 0; ok && i <= H; ++i) {          // code i of both sides, outwards
                     const int p1 = i == H || flat ? ni : QP_CK(ss_place(p, k, i + 1), ni);
-                    double n1 = (double)s_n[team][0], n2 = (double)s_n[team][1], x1 = s_up, x2 = s_down;
+                    double n1 = up, n2 = down, x1 = s_up, x2 = s_down;
                     if (p1 < ni) {
                         const unsigned w1 = c_up[p1], w2 = c_up[ni + p1];
                         n1 = (double)(w1 & 0x1FFFFu);
@@ -520,31 +549,34 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
                     v += ((n1 - n_up) * l1 * l1 - 2.0 * l1 * (x1 - x_up)) + ((n2 - n_down) * l2 * l2 - 2.0 * l2 * (x2 - x_down));
                     n_up = n1; n_down = n2; x_up = x1; x_down = x2;
                 }
-                const double mse = !ok ? inf : nf > 0.0 ? (nf * (q.var + dm * dm) + v) / nf : 0.0;
+                mse = !ok ? inf : nf > 0.0 ? (nf * (q.var + dm * dm) + v) / nf : 0.0;
                 a.curve[(size_t)c * a.ncp + k] = mse;
                 s_v[team][k] = mse;
             }
-            ct_team_sync(team);
-            if (side == 0) {                                  // the first minimum
-                double bv = inf;
-                int bk = 1 << 30;
-                for (int k = lane; k < ncand; k += 32)
-                    if (s_v[team][k] < bv) { bv = s_v[team][k]; bk = k; }
+            {                                                 // the first minimum, by all of the team
+                double bv = mse < inf ? mse : inf;            // (NaN: not below anything)
+                int bk = mse < inf ? k : 1 << 30;
+                __syncwarp();
+#pragma unroll
                 for (int o = 16; o > 0; o >>= 1) {
-                    const double ov = __shfl_down_sync(0xFFFFFFFFu, bv, o);
-                    const int ok = __shfl_down_sync(0xFFFFFFFFu, bk, o);
+                    const double ov = __shfl_xor_sync(0xFFFFFFFFu, bv, o);
+                    const int ok = __shfl_xor_sync(0xFFFFFFFFu, bk, o);
                     if (ov < bv || (ov == bv && ok < bk)) { bv = ov; bk = ok; }
                 }
-                if (lane == 0) {
-                    const int best = bk < ncand ? bk : 0;     // (every error infinite or NaN: keep b_E)
-                    float4 cd;
-                    int ok;
-                    qp_ds_candidate(su, best, a.steps, BITS, a.bmode & QP_B_MIDRISE, cd, ok);
+                if (lane == 0) s_n[team][part].y = (unsigned)bk;
+                ct_team_sync(team);
+                double least = inf;
+                int best = 0;                                 // (every error infinite or NaN: keep b_E)
+#pragma unroll
+                for (int j = 0; j < CT_TEAM / 32; ++j) {
+                    const unsigned at = s_n[team][j].y;
+                    if (at < (unsigned)ncand && s_v[team][at] < least) { least = s_v[team][at]; best = (int)at; }
+                }
+                if (k == best)
                     qp_ds_write_result(best, s_v[team], su, a.steps, a.nb, BITS, cd, a.ds_out ? a.ds_out + c : nullptr,
                                        a.qp_out + c, a.status);
-                }
             }
-            ct_team_sync(team);                               // s_v, s_edge and s_n are free again
+            ct_team_sync(team);                               // s_v, s_edge, s_n and s_sum are free again
         }
 
         // ---- hard channels (clip ends coarse against the step): every candidate scored on every element
@@ -676,19 +708,23 @@ bool ct_usable(qp_ctx* ctx)
     return ctx->ct_ok != 0;
 }
 
-// Strip width w and cluster size S: the fewest row-elements on the busiest SM, counting 2 more elements per row of a strip
-// (its cache lines are looked up one by one) and 6000 per wave (prologue, plan and finish, ~20 us).  A block's part stays
-// below 8192 rows where clusters allow it, so that offsets keep 19 bits.
-void ct_choose(const qp_ctx* ctx, uint64_t rows, uint32_t C, int max_w, int& w, int& S)
+// Strip width w and cluster size S by the time of the busiest SM, in ns: of a row, 0.18 per element, 1.5 per 32-byte sector (what a
+// load fetches: a strip that starts and ends inside sectors fetches half as much again, and the neighbours fetch it, too) and 2
+// whatever its width; and 20 us per wave (prologue, plan and finish).  Measured on 12608 x 1024 fp32 at 4 bits: w 14, S 2 (148 blocks,
+// 2.6 sectors a row) 134 us, w 16, S 2 (128 blocks, 2 sectors) 124, w 8, S 1 (128 blocks, 1 sector, four lines a load) 126.  A
+// block's part stays below 8192 rows where clusters allow it, so that offsets keep 19 bits.
+void ct_choose(const qp_ctx* ctx, const void* x, int size, uint64_t rows, uint32_t C, int max_w, int& w, int& S)
 {
     double best = 1e300;
     w = S = 1;
+    const bool whole = (((uintptr_t)x | (uint64_t)C * size) & 31u) == 0;          // every row starts with a sector
     for (int s = 1; s <= CT_MAX_S; ++s) {
         if (ctx->ct_clusters[s] < 1 || (s > 1 && (uint64_t)s > rows)) continue;
         for (int v = 1; v <= max_w && (uint32_t)v <= C; ++v) {
             const uint64_t strips = (C + v - 1) / v, waves = (strips + ctx->ct_clusters[s] - 1) / ctx->ct_clusters[s];
             const uint64_t rows_pb = (rows + s - 1) / s;
-            double cost = (double)waves * ((double)rows_pb * (v + 2) + 6000.0);
+            const double sectors = (v * size + (whole && v * size % 32 == 0 ? 0 : 32 - size)) / 32.0;
+            double cost = (double)waves * ((double)rows_pb * (0.18 * v + 1.5 * sectors + 2.0) + 20000.0);
             if (rows_pb > 8191) cost *= 4.0;
             if (cost < best) { best = cost; w = v; S = s; }
         }
@@ -711,11 +747,13 @@ int32_t qp_launch_channel_strips(qp_ctx* ctx, const void* d_x, int dtype, uint64
     // (statistics always with the strips of the default search, so that they come out the same with and without it)
     const int hh = bits ? (1 << bits) / 2 - 1 : 0;
     const int ni = SS_GRID + 1 + hh * (steps + 1);
+    const int len = (2 * ni + 3) & ~3;
     int max_w = CT_MAX_W;
-    while (max_w > 1 && (size_t)max_w * 2 * ni * sizeof(unsigned) > (size_t)SS_SUMS_AT) --max_w;
+    while (max_w > 1 && (size_t)max_w * len * sizeof(unsigned) > (size_t)SS_SUMS_AT) --max_w;
     int w, S;
-    ct_choose(ctx, rows, C, max_w, w, S);
+    ct_choose(ctx, d_x, dtype == QP_F32 ? 4 : 2, rows, C, max_w, w, S);
     CtArgs a;
+    a.len = len;
     a.x = d_x;
     a.rows = rows;
     a.C = C;

@@ -1687,6 +1687,18 @@ def test_search_channels_strips(ctx, channels, rows, bits):
     ctx.qp_get_status()
 
 
+# whole sectors per row and rows that start inside one (by the width, or by the pointer), a last strip of one channel, the most candidates
+@pytest.mark.parametrize("channels,rows,bits,skip,steps", [(1024, 300, 4, 0, 100), (1024, 300, 4, 1, 100), (1281, 150, 2, 0, 100),
+                                                           (16, 4097, 3, 0, 127), (40, 700, 4, 2, 127), (24, 65535, 4, 0, 20)])
+def test_search_channels_strips_and_sectors(ctx, channels, rows, bits, skip, steps):
+    x = si.vit_activation((1, rows, channels), 180 + channels % 7, outlier_frac=0.02).reshape(-1)
+    room = torch.empty(x.size + 8, device="cuda")
+    d = room[skip:skip + x.size]
+    d.copy_(torch.from_numpy(x))
+    check_search_channels(ctx, x, d, channels, bits, steps=steps)
+    ctx.qp_get_status()
+
+
 @pytest.mark.parametrize("bits", [1, 4])
 def test_search_channels_of_a_range_beyond_fp32(ctx, bits):
     """A channel whose range overflows fp32, and one whose range has no fp32 reciprocal, beside ordinary ones: the strips'
