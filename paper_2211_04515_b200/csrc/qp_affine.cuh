@@ -47,16 +47,16 @@ __device__ inline void ss_make_plan(SsPlan<HH>& p, int i, double mean, double a0
     const double a_min = fmin(a0, a1), R = fmax(a0, a1), L1 = (double)((1 << bits) - 1);
     const bool any = R > 1e-30 && R < 1e30;
     if (i < 0) {
-        int e = 0;
-        if (any) frexp(R, &e);                                // R < 2^e
+        const int e = any ? (int)((unsigned)__double2hiint(R) >> 20) - 1022 : 0;            // R < 2^e, a normal number
+        auto two_to = [](int k) { return __hiloint2double((k + 1023) << 20, 0); };
         p.m = (float)mean;
         p.ncand = ncand;
         p.kf = (float)ncand;
         p.down = a1 < a0;
-        p.inv_e = any ? (float)ldexp(1.0, -e) : 0.f;
-        p.w = any ? ldexp(1.0, e - 6) : 0.0;
+        p.inv_e = any ? (float)two_to(-e) : 0.f;
+        p.w = any ? two_to(e - 6) : 0.0;
         p.cell = (float)p.w;
-        p.u = any ? ldexp(1.0, e - 6 - ub) : 1.0;
+        p.u = any ? two_to(e - 6 - ub) : 1.0;
         // clip ends that are coarse against the smallest step (an ulp of the mean beyond 2^-15 of it, where a candidate's
         // error would move by 1e-8), or clips beyond what the formula's fp32 constants hold: the exact thresholds
         p.hard = HH > 0 && R > 0.0 && (!any || fabs(mean) * 1.1920928955078125e-7 > 3.0517578125e-5 * (2.0 * a_min / L1));

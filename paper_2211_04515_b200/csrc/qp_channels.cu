@@ -704,10 +704,10 @@ bool ch_allow_smem(K kernel, size_t bytes)
 }  // namespace
 
 // The statistics alone through the strips, whose second walk takes 4 or 2 bytes a lane: while L2 holds the tensor, and a bf16 one, which
-// is bound by its instructions, somewhat beyond.  fp32 of 129 MB (1280 channels), 246 MB (1024) and 492 MB (2048): strips 153, 282 and
-// 548 us, the column reductions 80, 136 and 272; bf16 of 138 MB (1152) and 246 MB (2048): 185 and 409 against 232 and 328.  (Below the
-// line 1280 fp32 channels are the faster in column reductions from 65 MB on, 52 us against 83, and 1024 in strips up to 131 MB, 89
-// against 91.)
+// is bound by its instructions, somewhat beyond.  fp32 of 246 MB (1024 and 1280 channels) and 492 MB (2048): strips 211, 204 and
+// 404 us, the column reductions 135, 114 and 270; bf16 of 138 MB (1152) and 246 MB (2048): 181 and 312 against 232 and 326.  (Below the
+// line 52 and 103 MB of 1024 channels take 31 and 66 us in strips, 56 and 80 in column reductions; 1280 channels, whose 80 strips of 16
+// leave SMs idle, 51 and 52 at 65 MB, 105 and 80 at the line itself.)
 static bool strip_statistics(int dtype, uint64_t rows, uint32_t channels)
 {
     return dtype == QP_F32 ? rows * channels <= 32000000ull : rows * channels <= 100000000ull;

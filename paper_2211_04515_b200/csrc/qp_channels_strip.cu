@@ -13,10 +13,11 @@
 //
 // What bounds it: the 32-byte sectors that a strip's rows touch (ct_choose), the instructions (A 4, B 11, C 14 + 2 per code
 // boundary and element) with their shared atomics, and the chain of small steps around the passes.  12608 x 1024 fp32 at 4 bits (52 MB), by
-// time stamps: A 15 us, its sums across the cluster 3, B 13 and 3, peaks and plans 5, C 19, interval sums across the cluster 6 (16
-// bytes a load; 8 with 4 bytes), prefix sums 4 (13 without a branch per interval and with a warp per side), errors 7, pick 1: 77, and
-// the whole stage (receiver, this, packing) 110; strips of 14 channels, whose rows start anywhere in a sector, and those
-// two forms took 101 and 134.  The ten kernels before (four for the statistics, histogram, set-up, thresholds sorted per
+// time stamps: A 14 us, its sums across the cluster 3, B 10 and 4, peaks and plans 5, C 20, interval sums across the cluster 6 (16
+// bytes a load; 8 with 4 bytes), prefix sums 3 (13 with a `while` over the cells per interval and a warp per side), errors 7, pick 1:
+// 74, and the whole stage (receiver, this, packing) 106; with strips of 14 channels, whose rows start anywhere in a sector, and
+// those two forms 101 and 134.  Unrolling the errors' loop or three vectors of the interval sums at a time costs 2 us each (straight
+// code that runs once).  The ten kernels before (four for the statistics, histogram, set-up, thresholds sorted per
 // channel, a pass with binary searches, error curves, pick) took 255 us.
 #include <cooperative_groups.h>
 
@@ -41,6 +42,9 @@ constexpr int CT_PREFETCH = 4;                     // batches that the first pas
 constexpr float CT_INF = __builtin_huge_valf();
 constexpr int CT_MAX_CAND = QP_CH_MAX_STEPS + 1;
 constexpr size_t CT_TABLE_BYTES = 2 * SS_SUMS_AT;  // interval tables (counts, then sums) of the strip
+constexpr int CT_HIST_AT = 64 * 1024;              // phase B: the histogram with a replica per lane, where the interval tables will be
+static_assert(5 * CT_MAX_W * (CT_THREADS / CT_MAX_W + 1) * sizeof(double) <= CT_HIST_AT && 5 * (CT_THREADS + 1) * sizeof(double) <= CT_HIST_AT, "sums before it");
+static_assert(CT_HIST_AT + (QP_CH_MAX_HIST_BINS + 1) * 64 * sizeof(unsigned) <= CT_TABLE_BYTES, "room");
 constexpr size_t CT_DYN_BYTES = CT_TABLE_BYTES + (size_t)CT_MAX_W * (QP_CH_MAX_HIST_BINS + 1) * sizeof(unsigned);
 
 struct CtArgs {
@@ -150,7 +154,7 @@ struct CtMomentsGuarded {                          // a column with non-finite v
 template <bool SUMS, bool HIST, int CARE>                     // CARE: as in the per-tensor kernel
 struct CtDeviations {
     float m, mn, inv_w;
-    unsigned base, nb;                             // byte address of the channel's first bin, less what the float's bits bring
+    unsigned base, mul, nb;                        // byte address of the lane's first bin, less what the float's bits bring; from bin to bin
     double sd = 0.0, sv = 0.0;
     unsigned below = 0u;
     __device__ __forceinline__ void one(float v)
@@ -168,7 +172,7 @@ struct CtDeviations {
             if (CARE == 2) pos = fminf(fmaxf(pos, 0.f), (float)nb);
             unsigned bin = __float_as_uint(__fadd_rd(pos, SS_MAGIC)) - SS_ONE;
             if (CARE == 1) bin = min(bin, nb);
-            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"((QP_CK(bin, nb + 1) + SS_ONE) * 4u + base) : "memory");
+            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"((QP_CK(bin, nb + 1) + SS_ONE) * mul + base) : "memory");
         }
     }
     __device__ __forceinline__ void fold() {}
@@ -242,10 +246,13 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
                          (unsigned)nl * a.C * (unsigned)sizeof(T)};
     const double inf = __longlong_as_double(0x7FF0000000000000ll);
     double* red = reinterpret_cast<double*>(raw);
-    unsigned* bins = reinterpret_cast<unsigned*>(raw + CT_TABLE_BYTES);            // [w][nb + 1]
-
+    unsigned* bins = reinterpret_cast<unsigned*>(raw + CT_TABLE_BYTES);            // [w][nb]
+    // Phase B counts with a counter per bin and lane: 32 neighbouring threads meet 32 banks (as w divides 32, otherwise a few twice),
+    // whatever their bins (12608 x 1024: 12.5 us with a channel's bins side by side, 10.4 so).
+    unsigned* lane_bins = reinterpret_cast<unsigned*>(raw + CT_HIST_AT);           // [nb + 1][pitch], w * copies of the pitch used
+    const int copies = (31 + w) / w, pitch = (w * copies + 31) & ~31;
     if constexpr (SEARCH)
-        for (int i = threadIdx.x; i < w * (a.nb + 1); i += CT_THREADS) bins[i] = 0u;
+        for (int i = threadIdx.x; i < (a.nb + 1) * pitch / 4; i += CT_THREADS) reinterpret_cast<uint4*>(lane_bins)[i] = make_uint4(0u, 0u, 0u, 0u);
 
     // ---- phase A
     if constexpr (STATS) {
@@ -322,14 +329,27 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
             d.mn = (float)my.min;
             d.inv_w = inv_w(my);
             d.nb = (unsigned)a.nb;
-            d.base = (unsigned)__cvta_generic_to_shared(bins + slot * (a.nb + 1)) - SS_ONE * 4u;
+            d.mul = 4u * (unsigned)pitch;
+            d.base = (unsigned)__cvta_generic_to_shared(lane_bins + threadIdx.x % (w * copies)) - SS_ONE * d.mul;
             ct_column<T>(mine, m, d);
             v3[0] = d.sd; v3[1] = d.sv; v3[2] = (double)d.below;
         };
         if (odd || beyond) pass(std::integral_constant<int, 2>{}); else pass(std::integral_constant<int, STATS ? 0 : 1>{});
         if constexpr (STATS) {
             ct_reduce<0, 0, 0>(v3, red, slot, rl, nl, w, s_b);
-            if (SEARCH) __syncthreads();                      // (the interval tables lie where red is)
+        }
+        if constexpr (SEARCH) {                               // this block's bins; what x = max put into bin nb counts in the last one
+            if (!STATS) __syncthreads();                      // (ct_reduce has one)
+            for (int b = rl; b < a.nb && rl < nl; b += nl) {
+                unsigned c = 0u;
+                for (int j = 0; j < copies; ++j) {
+                    const unsigned* at = lane_bins + b * pitch + j * w + slot;
+                    c += at[0];
+                    if (b == a.nb - 1) c += at[pitch];
+                }
+                bins[slot * a.nb + b] = c;
+            }
+            __syncthreads();                                  // (the interval tables lie where all this is)
         }
         ct_arrive();                                          // (orders the histogram counters of the cluster, too)
         if constexpr (SEARCH)
@@ -373,11 +393,7 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
             unsigned top = 0u;
             for (int b = threadIdx.x % CT_PEAK; b < a.nb; b += CT_PEAK) {
                 unsigned c = 0u;
-                for (int r = 0; r < S; ++r) {
-                    const unsigned* q = cluster.map_shared_rank(bins, r) + sl * (a.nb + 1) + b;
-                    c += q[0];
-                    if (b == a.nb - 1) c += q[1];
-                }
+                for (int r = 0; r < S; ++r) c += cluster.map_shared_rank(bins, r)[sl * a.nb + b];
                 top = max(top, c);
             }
             __syncwarp();
@@ -479,18 +495,21 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
                 int cell0 = 0;                                // grid cell of interval i0
 #pragma unroll
                 for (int o = SS_GRID; o > 0; o >>= 1) cell0 += edge[min(cell0 + o, SS_GRID + 1)] <= i0 ? o : 0;
-                unsigned n_all = 0u;
+                // Exclusive prefix sums, in place: count in 17 bits | high bits of the sum << 17, low word of the sum.  First those of
+                // the thread's own intervals, then what lies before them.
+                unsigned n_all = 0u, at = (unsigned)cell0 << a.ub;
                 unsigned long long s_all = 0ull;
                 int cell = cell0, next = edge[cell + 1];
                 for (int i = i0; i < i1; ++i) {
-                    cell += next <= i ? 1 : 0;
+                    if (next <= i) { ++cell; at += 1u << a.ub; }
                     next = edge[cell + 1];
-                    const unsigned cn = cnt[i], n = cn & 0xFFFFFFu;
+                    const unsigned cn = cnt[i], n = cn & 0xFFFFFFu, lo = sum[i];
+                    cnt[i] = n_all | (unsigned)(s_all >> 32) << 17;
+                    sum[i] = (unsigned)s_all;
                     n_all += n;
-                    s_all += ((unsigned long long)(cn >> 24) << 32 | sum[i]) + ((unsigned long long)n * (unsigned)cell << a.ub);
+                    s_all += (unsigned long long)n * at + ((unsigned long long)(cn >> 24) << 32 | lo);
                 }
                 __syncwarp();
-                // exclusive prefix sums, in place: count in 17 bits | high bits of the sum << 17, low word of the sum
                 unsigned np = n_all;
                 unsigned long long sp = s_all;
 #pragma unroll
@@ -504,17 +523,11 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
                 np -= n_all;
                 sp -= s_all;
                 if (part & 1) { np += s_n[team][part - 1].x; sp += s_sum[team][part - 1]; }
-                cell = cell0;
-                next = edge[cell + 1];
+                const unsigned before = np | (unsigned)(sp >> 32) << 17, low = (unsigned)sp;
                 for (int i = i0; i < i1; ++i) {
-                    cell += next <= i ? 1 : 0;
-                    next = edge[cell + 1];
-                    const unsigned cn = cnt[i], n = cn & 0xFFFFFFu;
-                    const unsigned long long s = (unsigned long long)(cn >> 24) << 32 | sum[i];
-                    cnt[i] = np | (unsigned)(sp >> 32) << 17;
-                    sum[i] = (unsigned)sp;
-                    np += n;
-                    sp += s + ((unsigned long long)n * (unsigned)cell << a.ub);
+                    const unsigned lo = sum[i] + low;
+                    cnt[i] += before + (lo < low ? 1u << 17 : 0u);
+                    sum[i] = lo;
                 }
             }
             ct_team_sync(team);
@@ -535,19 +548,24 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
                 a.cand[(size_t)c * a.ncp + k] = cd;
                 a.valid[(size_t)c * a.ncp + k] = ok;
                 double v = 0.0, n_up = 0.0, n_down = 0.0, x_up = 0.0, x_down = 0.0;
-                for (int i = 0; ok && i <= H; ++i) {          // code i of both sides, outwards
-                    const int p1 = i == H || flat ? ni : QP_CK(ss_place(p, k, i + 1), ni);
-                    double n1 = up, n2 = down, x1 = s_up, x2 = s_down;
-                    if (p1 < ni) {
-                        const unsigned w1 = c_up[p1], w2 = c_up[ni + p1];
-                        n1 = (double)(w1 & 0x1FFFFu);
-                        n2 = (double)(w2 & 0x1FFFFu);
-                        x1 = p.u * (double)((unsigned long long)(w1 >> 17) << 32 | t_up[p1]);
-                        x2 = p.u * (double)((unsigned long long)(w2 >> 17) << 32 | t_up[ni + p1]);
+                // integers below 2^52 to fp64 by the exponent of 2^52 (the conversion unit is a quarter of the fp64 one's rate)
+                auto whole = [](unsigned hi, unsigned lo) { return __hiloint2double((int)(0x43300000u | hi), (int)lo) - 4503599627370496.0; };
+                if (ok) {
+#pragma unroll 1
+                    for (int i = 0; i <= H; ++i) {            // code i of both sides, outwards
+                        const int p1 = i == H || flat ? ni : QP_CK(ss_place(p, k, i + 1), ni);
+                        double n1 = up, n2 = down, x1 = s_up, x2 = s_down;
+                        if (p1 < ni) {
+                            const unsigned w1 = c_up[p1], w2 = c_up[ni + p1];
+                            n1 = whole(0u, w1 & 0x1FFFFu);
+                            n2 = whole(0u, w2 & 0x1FFFFu);
+                            x1 = p.u * whole(w1 >> 17, t_up[p1]);
+                            x2 = p.u * whole(w2 >> 17, t_up[ni + p1]);
+                        }
+                        const double l1 = ss_level(cd, H + 1 + i, p.m), l2 = -ss_level(cd, H - i, p.m);   // distances from the centre
+                        v += ((n1 - n_up) * l1 * l1 - 2.0 * l1 * (x1 - x_up)) + ((n2 - n_down) * l2 * l2 - 2.0 * l2 * (x2 - x_down));
+                        n_up = n1; n_down = n2; x_up = x1; x_down = x2;
                     }
-                    const double l1 = ss_level(cd, H + 1 + i, p.m), l2 = -ss_level(cd, H - i, p.m);   // distances from the centre
-                    v += ((n1 - n_up) * l1 * l1 - 2.0 * l1 * (x1 - x_up)) + ((n2 - n_down) * l2 * l2 - 2.0 * l2 * (x2 - x_down));
-                    n_up = n1; n_down = n2; x_up = x1; x_down = x2;
                 }
                 mse = !ok ? inf : nf > 0.0 ? (nf * (q.var + dm * dm) + v) / nf : 0.0;
                 a.curve[(size_t)c * a.ncp + k] = mse;
