@@ -3,8 +3,12 @@
 //
 // Two passes, while L2 still holds the tensor when the second one comes (which walks it backwards): sum x, sum |x|, min and
 // max; a grid barrier; sum |x - mean| and sum (x - mean)^2; a second barrier, and every block knows the clip and packs.
-// What bounds it: two barriers and merges of 2.5 us each, then L2 and the instructions.  Against one launch of 32 KB
-// tiles copied by TMA: 12.5 against 14.5 us at 2^20 elements, 20.4 / 21.7 at 2^23, 26.7 / 28.6 at 2^24 fp32.
+// What bounds it: L2 and the instructions, then the barriers.  27 M bf16 elements at 6 bits (54 MB), by block 0's time stamps: first pass
+// 10.5 us, parts, barrier and merge 3.8, second pass 6.2, 2.5, clip 0.5, packing 9.6: 34, and 37 between launches.  One image at 8 bits (10
+// blocks, a cluster): passes 0.9 and 1.1, the steps between them 2.2 and 1.9, clip 0.5, packing 1.2: 8.6, and 10.3 between launches.
+// With the blocks' partials 64 bytes apart, every quantity in a reduction of its own and every thread adding up the warps' sums
+// they took 40 and 12.3.  (Lanes that have parted take a shuffle one after another: a __syncwarp less in front of the
+// reductions and the image takes 16.4.)
 //
 // One pass above that.  sum |x - mean| needs the mean first, so the deviations are taken about a pilot centre c, y = x - c,
 // and the split point is moved to the mean afterwards: with D = mean - c > 0
@@ -45,6 +49,10 @@ constexpr unsigned OP_ONE = 0x4B000000u;
 constexpr size_t OP_DYN_BYTES = (size_t)(2 * OP_CELLS * 2 << OP_REPS) * sizeof(unsigned);   // >= 16 KB: the packer's staging
 constexpr int OP_SUMS_AT = (int)(OP_DYN_BYTES / 2);
 
+// rows of block partials: of the pass (sum y, |x|; min, max, non-finite, below c; sum |y|, y^2), of the pilot (two), of the window
+// (two), of the second pass (a slow block may still read an earlier one's)
+enum { OP_PASS = 0, OP_PILOT = 3, OP_WINDOW = 5, OP_SECOND = 7, OP_ROWS = 8 };
+
 struct OpArgs {
     const void* x;
     uint64_t n, ntiles;                            // ntiles: whole tiles
@@ -56,7 +64,7 @@ struct OpArgs {
     double F;
     int one;                                       // one pass, or two
     int sample;                                    // pilot vectors per thread
-    double* part;                                  // [4][grid][8]
+    uint4* part;                                   // [OP_ROWS][grid] block partials, 16 bytes each
     unsigned* bar;                                 // [0] arrivals, [1] blocks that have left; zero at entry and at exit
     unsigned* status;
     unsigned spin_limit, bar_extra;
@@ -157,17 +165,18 @@ struct OpPass {
 };
 // element by element: a lane's share with non-finite values, and what is behind the last tile
 struct OpOnes {
-    double sy = 0.0, sa = 0.0, sv = 0.0, sx = 0.0, below = 0.0, bad = 0.0;
+    double sy = 0.0, sa = 0.0, sv = 0.0, sx = 0.0;
+    unsigned below = 0u, bad = 0u;
     float mn, mx;
     __device__ __forceinline__ void one(float v, float c)
     {
-        if (!qp_is_finite(v)) { bad += 1.0; return; }
+        if (!qp_is_finite(v)) { ++bad; return; }
         const double y = (double)__fsub_rn(v, c);
         sy += y;
         sa += fabs(y);
         sv += y * y;
         sx += (double)fabsf(v);
-        below += y < 0.0 ? 1.0 : 0.0;
+        below += y < 0.0 ? 1u : 0u;
         mn = fminf(mn, v);
         mx = fmaxf(mx, v);
     }
@@ -207,39 +216,6 @@ struct OpDeviations {
     }
 };
 
-// N partials of every block, in order, by one warp with all loads in flight; the result in s (shared), for everybody
-// behind the block barrier at the end.  OPS: 0 sum, 1 min, 2 max.
-template <int... OPS>
-__device__ __forceinline__ void op_merge(const double* part, unsigned G, double* s)
-{
-    constexpr int N = sizeof...(OPS);
-    constexpr int ops[N] = {OPS...};
-    const double inf = __longlong_as_double(0x7FF0000000000000ll);
-    if (threadIdx.x < 32) {
-        double m[N];
-#pragma unroll
-        for (int j = 0; j < N; ++j) m[j] = ops[j] == 0 ? 0.0 : ops[j] == 1 ? inf : -inf;
-        for (unsigned b0 = threadIdx.x; b0 < G; b0 += 32 * SS_MERGE) {
-            double p[SS_MERGE][N];
-#pragma unroll
-            for (int u = 0; u < SS_MERGE; ++u)
-#pragma unroll
-                for (int j = 0; j < N; ++j)
-                    p[u][j] = b0 + 32 * u < G ? __ldcg(part + (size_t)(b0 + 32 * u) * 8 + j) : (ops[j] == 0 ? 0.0 : ops[j] == 1 ? inf : -inf);
-#pragma unroll
-            for (int u = 0; u < SS_MERGE; ++u)
-#pragma unroll
-                for (int j = 0; j < N; ++j)
-                    m[j] = ops[j] == 0 ? m[j] + p[u][j] : (ops[j] == 1 ? fmin(m[j], p[u][j]) : fmax(m[j], p[u][j]));
-        }
-        ss_warp_reduce<OPS...>(m);
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int j = 0; j < N; ++j) s[j] = m[j];
-    }
-    __syncthreads();
-}
-
 // BITS = 0: statistics only; 1..8: the sender.
 template <typename T, int BITS>
 __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpArgs a)
@@ -247,31 +223,38 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
     extern __shared__ __align__(16) unsigned char raw[];
     using Tiles = SsTiles<T, SS_TILE>;
     constexpr int EPV = Tiles::EPV;
-    __shared__ double s_red[SS_WARPS * 8];
-    __shared__ double s_sum[8];
-    __shared__ int s_ok, s_full;
+    __shared__ SsBlock s_block[3];
+    __shared__ int s_ok, s_full, s_again;
+    __shared__ float s_c, s_delta;
+    __shared__ double s_D, s_abs, s_below;
+    __shared__ qp_stats_t s_st;
     __shared__ qp_qparams_t s_qp;
     const T* x = static_cast<const T*>(a.x);
     const int lane = threadIdx.x & 31;
     const unsigned G = gridDim.x;
-    const uint64_t first = (uint64_t)blockIdx.x * SS_WARPS + (threadIdx.x >> 5), step = (uint64_t)G * SS_WARPS;
+    const uint64_t first = (uint64_t)(threadIdx.x >> 5) * G + blockIdx.x, step = (uint64_t)G * SS_WARPS;
     const uint64_t tail0 = a.ntiles * SS_TILE;
     const double inf = __longlong_as_double(0x7FF0000000000000ll);
     unsigned* table = reinterpret_cast<unsigned*>(raw);
+    uint4* part = a.part + blockIdx.x;             // this block's: row r at part[r * G]
     unsigned waits = 0;
-    auto meet = [&]() {
+    // for what warp 0 wrote and merges next; the others wait at the block barrier behind, and learn from s_ok
+    auto meet_warp0 = [&]() {
+        ++waits;
         if (a.cluster) {
             qp_grid::cluster_arrive();
             qp_grid::cluster_wait();
-            return true;
+            if (threadIdx.x == 0) s_ok = 1;
+            __syncwarp();
+        } else if (threadIdx.x < 32) {
+            qp_grid::barrier_warp0(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
         }
-        ++waits;
-        return qp_grid::barrier(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
     };
     auto leave = [&](unsigned gave_up) {
         if (threadIdx.x == 0 && qp_grid::last_out(qp_grid::count_out(a.bar, gave_up), G)) qp_grid::reset(a.bar);
     };
-    for (int i = threadIdx.x; i < (int)(OP_DYN_BYTES / 16); i += SS_THREADS) reinterpret_cast<uint4*>(raw)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (a.one)                                                // the window's table
+        for (int i = threadIdx.x; i < (int)(OP_DYN_BYTES / 16); i += SS_THREADS) reinterpret_cast<uint4*>(raw)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x == 0) s_full = 0;
 
     // ---- pilot: sample i, four neighbouring vectors (the bytes of one DRAM burst) by four lanes, lies at a random place of
@@ -280,17 +263,18 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
     if (a.one) {
         const uint64_t nv4 = a.n / (4 * EPV);
         const unsigned total = (unsigned)a.sample * G * (SS_THREADS / 4);
-        const uint64_t part = nv4 / total;                    // >= 1
+        const uint64_t each = nv4 / total;                    // >= 1
         float e[OP_SAMPLE][EPV];
 #pragma unroll
         for (int j = 0; j < OP_SAMPLE; ++j) {
             const unsigned i = ((unsigned)j * G + blockIdx.x) * (SS_THREADS / 4) + threadIdx.x / 4;
-            const uint64_t v = (i * part + ((uint64_t)op_place(i) * part >> 32)) * 4 + (lane & 3);
+            const uint64_t v = (i * each + ((uint64_t)op_place(i) * each >> 32)) * 4 + (lane & 3);
             if (j < a.sample) qp_load_vec(x + v * EPV, e[j]);
         }
         float x0 = qp_load_one(x);                            // (any value near the tensor's: the sums are taken about it)
         if (!qp_is_finite(x0)) x0 = 0.f;
-        float p1 = 0.f, p2 = 0.f, pn = 0.f;
+        float p1 = 0.f, p2 = 0.f;
+        unsigned pn = 0u;
 #pragma unroll
         for (int j = 0; j < OP_SAMPLE; ++j) {
             if (j >= a.sample) break;
@@ -300,25 +284,42 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             m *= 0.25f / EPV;
             m += __shfl_xor_sync(0xFFFFFFFFu, m, 1);
             m += __shfl_xor_sync(0xFFFFFFFFu, m, 2);
-            if (m * m < __int_as_float(0x7F800000)) { p1 += m; p2 = fmaf(m, m, p2); pn += 1.f; }
+            if (m * m < __int_as_float(0x7F800000)) { p1 += m; p2 = fmaf(m, m, p2); ++pn; }
         }
-        double v3[3] = {(double)p1, (double)p2, (double)pn};
-        ss_reduce<0, 0, 0>(v3, s_red);
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) a.part[(size_t)(2 * G + blockIdx.x) * 8 + j] = v3[j];
-        if (!meet()) { leave(qp_grid::GAVE_UP); return; }
-        op_merge<0, 0, 0>(a.part + (size_t)2 * G * 8, G, s_sum);
-        // (every sample was counted by its four lanes)
-        const double k = s_sum[2] > 0.0 ? s_sum[2] : 1.0, m = s_sum[0] / k, var = s_sum[1] / k - m * m;
-        c = (float)((double)x0 + m);
-        if (!qp_is_finite(c)) c = 0.f;
-        const double want = fmax(fmax(12.0 * sqrt(fmax(var, 0.0) / k), fabs((double)c) * 3.814697265625e-6), 1e-30);
-        delta = (float)fmin(want, 1e30);
+        const SsParts v = ss_block_parts<false>({(double)p1, (double)p2, 0.f, 0.f, pn}, s_block[0]);
+        if (threadIdx.x == 0) {
+            part[OP_PILOT * G] = ss_row(v.a, v.b);
+            part[(OP_PILOT + 1) * G] = make_uint4(v.count, 0u, 0u, 0u);
+        }
+        meet_warp0();
+        if (threadIdx.x < 32) {
+            double t1 = 0.0, t2 = 0.0, tn = 0.0;
+            ss_merge<2>(a.part + OP_PILOT * G, G, [&](const uint4 (&p)[2]) {
+                t1 += ss_row_first(p[0]);
+                t2 += ss_row_second(p[0]);
+                tn += (double)p[1].x;
+            });
+            __syncwarp();
+            t1 = ss_pair_sum(t1, t2);
+            tn = ss_pair_sum(tn, 0.0);
+            t2 = __shfl_sync(0xFFFFFFFFu, t1, 16);
+            if (lane == 0) {                                  // (every sample was counted by its four lanes)
+                const double k = tn > 0.0 ? tn : 1.0, m = t1 / k, var = t2 / k - m * m;
+                float centre = (float)((double)x0 + m);
+                if (!qp_is_finite(centre)) centre = 0.f;
+                const double want = fmax(fmax(12.0 * sqrt(fmax(var, 0.0) / k), fabs((double)centre) * 3.814697265625e-6), 1e-30);
+                s_c = centre;
+                s_delta = (float)fmin(want, 1e30);
+            }
+        }
+        __syncthreads();
+        if (!s_ok) { leave(qp_grid::GAVE_UP); return; }
+        c = s_c;
+        delta = s_delta;
     }
 
     // ---- the pass
-    double v8[8];
+    OpOnes o;
     const int cell_off = (int)(__float_as_uint(delta) >> 17) - (OP_CELLS - 1);   // delta's own cell is the last
     auto pass = [&](auto& f) {
         f.c = c;
@@ -334,7 +335,6 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
         f.below = f.odd = 0u;
         f.nc = qp_pack2(-c, -c);
         Tiles::template run<false>(x, a.ntiles, first, step, lane, f);
-        OpOnes o;
         o.mn = f.mn;
         o.mx = f.mx;
         if (f.odd) {                                          // rare: this lane's share again (its window counts stand)
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
                     for (int i = 0; i < EPV; ++i) o.one(qp_load_one(x + t * SS_TILE + (j * 32 + lane) * EPV + i), c);
         } else {
             o.sy = f.sy; o.sa = f.sa; o.sv = f.sv; o.sx = f.sx;
-            o.below = (double)f.below;
+            o.below = f.below;
         }
         if (blockIdx.x == G - 1)
             for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) {
@@ -353,7 +353,6 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
                 o.one(v, c);
                 if (a.one && qp_is_finite(v)) f.window(__fsub_rn(v, c));
             }
-        v8[0] = o.sy; v8[1] = o.sa; v8[2] = o.sv; v8[3] = o.sx; v8[4] = (double)o.mn; v8[5] = (double)o.mx; v8[6] = o.below; v8[7] = o.bad;
     };
     if (a.one) {
         OpPass<true> f;
@@ -362,38 +361,80 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
         OpPass<false> f;
         pass(f);
     }
-    ss_reduce<0, 0, 0, 0, 1, 2, 0, 0>(v8, s_red);             // (its barriers also order the window's counters)
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) a.part[(size_t)blockIdx.x * 8 + j] = v8[j];
-    if (!meet()) { leave(qp_grid::GAVE_UP); return; }
-    op_merge<0, 0, 0, 0, 1, 2, 0, 0>(a.part, G, s_sum);
-    qp_stats_t st;
-    const double sum_abs = s_sum[1], sum_sq = s_sum[2], below = s_sum[6];
-    double D, nf;
     {
-        const unsigned long long bad = (unsigned long long)s_sum[7];
-        nf = (double)(a.n - bad);
-        D = nf > 0.0 ? s_sum[0] / nf : 0.0;
-        st.n = a.n;
-        st.nonfinite = bad;
-        st.mean = nf > 0.0 ? (double)c + D : 0.0;
-        st.mean_abs = nf > 0.0 ? s_sum[3] / nf : 0.0;
-        st.min = nf > 0.0 ? s_sum[4] : 0.0;
-        st.max = nf > 0.0 ? s_sum[5] : 0.0;
-        st.hist_peak = 0;
-        st.hist_bins = 0;
-        st.reserved = 0;
-        st.var = nf > 0.0 ? fmax(0.0, sum_sq / nf - D * D) : 0.0;
-        st.mad = 0.0;
+        const SsParts v = ss_block_parts<true>({o.sy, o.sx, o.mn, o.mx, o.bad}, s_block[1]);       // (its barrier also orders the window's counters)
+        SsParts u = {0.0, 0.0, 0.f, 0.f, 0u};
+        if (a.one) u = ss_block_parts<false>({o.sa, o.sv, 0.f, 0.f, o.below}, s_block[2]);
+        if (threadIdx.x == 0) {
+            part[OP_PASS * G] = ss_row(v.a, v.b);
+            part[(OP_PASS + 1) * G] = make_uint4(__float_as_uint(v.lo), __float_as_uint(v.hi), v.count, u.count);
+            if (a.one) part[(OP_PASS + 2) * G] = ss_row(u.a, u.b);
+        }
     }
-    bool again = !a.one || !(fabs(D) < (double)delta) || !(sum_sq < inf);
+    meet_warp0();
+    if (threadIdx.x < 32) {
+        double sy = 0.0, sx = 0.0, sa = 0.0, sv = 0.0, bad = 0.0, below = 0.0;
+        float mn = __int_as_float(0x7F800000), mx = -mn;
+        auto first_two = [&](const uint4& p, const uint4& q) {
+            sy += ss_row_first(p);
+            sx += ss_row_second(p);
+            mn = fminf(mn, __uint_as_float(q.x));
+            mx = fmaxf(mx, __uint_as_float(q.y));
+            bad += (double)q.z;                               // exact: counts are far below 2^53
+        };
+        if (a.one) {
+            ss_merge<3>(a.part + OP_PASS * G, G, [&](const uint4 (&p)[3]) {
+                first_two(p[0], p[1]);
+                below += (double)p[1].w;
+                sa += ss_row_first(p[2]);
+                sv += ss_row_second(p[2]);
+            });
+        } else {
+            ss_merge<2>(a.part + OP_PASS * G, G, [&](const uint4 (&p)[2]) { first_two(p[0], p[1]); });
+        }
+        __syncwarp();
+        sy = ss_pair_sum(sy, sx);
+        mn = ss_pair_min(mn, -mx);
+        bad = ss_pair_sum(bad, below);
+        sx = __shfl_sync(0xFFFFFFFFu, sy, 16);
+        mx = -__shfl_sync(0xFFFFFFFFu, mn, 16);
+        if (a.one) {
+            sa = ss_pair_sum(sa, sv);
+            sv = __shfl_sync(0xFFFFFFFFu, sa, 16);
+            below = __shfl_sync(0xFFFFFFFFu, bad, 16);
+        }
+        if (lane == 0) {
+            const unsigned long long nbad = (unsigned long long)bad;
+            const double nf = (double)(a.n - nbad), D = nf > 0.0 ? sy / nf : 0.0;
+            s_st.n = a.n;
+            s_st.nonfinite = nbad;
+            s_st.mean = nf > 0.0 ? (double)c + D : 0.0;
+            s_st.mean_abs = nf > 0.0 ? sx / nf : 0.0;
+            s_st.min = nf > 0.0 ? (double)mn : 0.0;
+            s_st.max = nf > 0.0 ? (double)mx : 0.0;
+            s_st.mad = s_st.var = 0.0;
+            s_st.hist_peak = 0;
+            s_st.hist_bins = 0;
+            s_st.reserved = 0;
+            if (a.one) {
+                s_st.var = nf > 0.0 ? fmax(0.0, sv / nf - D * D) : 0.0;
+                s_D = D;
+                s_abs = sa;
+                s_below = below;
+            }
+            s_again = !a.one || !(fabs(D) < (double)delta) || !(sv < inf);
+        }
+    }
+    __syncthreads();
+    if (!s_ok) { leave(qp_grid::GAVE_UP); return; }
     // ---- this block's share of the elements between c and the mean
-    if (!again) {                                             // uniform over the grid
+    if (!s_again) {                                           // uniform over the grid
+        const double D = s_D;
         const int side = D < 0.0;
         const float aD = (float)fabs(D);
         const int own = max((int)(__float_as_uint(aD) >> 17) - cell_off, 0);
-        double v4[4] = {0.0, 0.0, 0.0, 0.0};                  // count and sum below the mean's cell, count in it, overflow
+        double vn = 0.0, vs = 0.0;                            // count and sum below the mean's cell
+        unsigned in_own = 0u;                                 // count in it (a block's: below 2^32)
         for (int i = threadIdx.x; i < OP_CELLS; i += SS_THREADS) {
             const unsigned* cnt = table + ((size_t)(side * OP_CELLS + i) << OP_REPS);
             const unsigned* sum = reinterpret_cast<const unsigned*>(raw + OP_SUMS_AT) + ((size_t)(side * OP_CELLS + i) << OP_REPS);
@@ -404,61 +445,88 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
                 cs += sum[rr];
                 if (cnt[rr] > OP_FULL) s_full = 1;            // benign race: every writer writes 1
             }
-            if (i < own) { v4[0] += (double)cn; v4[1] += (double)cs; }
-            if (i == own) v4[2] += (double)cn;
+            if (i < own) { vn += (double)cn; vs += (double)cs; }
+            if (i == own) in_own += (unsigned)cn;
         }
-        ss_reduce<0, 0, 0, 0>(v4, s_red);
+        const SsParts v = ss_block_parts<false>({vn, vs, 0.f, 0.f, in_own}, s_block[0]);
         if (threadIdx.x == 0) {
-            double* p = a.part + (size_t)(G + blockIdx.x) * 8;
-            p[0] = v4[0]; p[1] = v4[1]; p[2] = v4[2]; p[3] = s_full ? 1.0 : 0.0;
+            part[OP_WINDOW * G] = ss_row(v.a, v.b);
+            part[(OP_WINDOW + 1) * G] = make_uint4(v.count, (unsigned)s_full, 0u, 0u);
         }
-        if (!meet()) { leave(qp_grid::GAVE_UP); return; }
-        op_merge<0, 0, 0, 0>(a.part + (size_t)G * 8, G, s_sum);
-        const double d = fabs(D), u = (double)delta / 65536.0;
-        const double lo = own ? (double)__uint_as_float((unsigned)(own + cell_off) << 17) : 0.0;
-        const double hi = (double)__uint_as_float((unsigned)(own + 1 + cell_off) << 17), w = hi - lo;
-        const double own_part = s_sum[2] * (d - lo) * (d - lo) / (2.0 * w);       // evenly filled
-        const double between = d * s_sum[0] - u * s_sum[1] + own_part;
-        const double neg = side ? nf - below : below;         // elements on the other side of c
-        const double sd = sum_abs + d * (neg - (nf - neg)) + 2.0 * between;
-        st.mad = nf > 0.0 ? fmax(0.0, sd) / nf : 0.0;
-        again = s_sum[3] > 0.0 || !(s_sum[2] * w * 0.5 <= 1e-8 * sum_abs);
-        if (sum_abs == 0.0) again = false;                    // (every element is c)
-    }
-    if (again) {                                              // uniform over the grid
+        meet_warp0();
+        if (threadIdx.x < 32) {
+            double tn = 0.0, ts = 0.0, to = 0.0, full = 0.0;
+            ss_merge<2>(a.part + OP_WINDOW * G, G, [&](const uint4 (&p)[2]) {
+                tn += ss_row_first(p[0]);
+                ts += ss_row_second(p[0]);
+                to += (double)p[1].x;
+                full += (double)p[1].y;
+            });
+            __syncwarp();
+            tn = ss_pair_sum(tn, ts);
+            to = ss_pair_sum(to, full);
+            ts = __shfl_sync(0xFFFFFFFFu, tn, 16);
+            full = __shfl_sync(0xFFFFFFFFu, to, 16);
+            if (lane == 0) {
+                const double nf = (double)(a.n - s_st.nonfinite), sum_abs = s_abs;
+                const double d = fabs(D), u = (double)delta / 65536.0;
+                const double lo = own ? (double)__uint_as_float((unsigned)(own + cell_off) << 17) : 0.0;
+                const double hi = (double)__uint_as_float((unsigned)(own + 1 + cell_off) << 17), w = hi - lo;
+                const double own_part = to * (d - lo) * (d - lo) / (2.0 * w);         // evenly filled
+                const double between = d * tn - u * ts + own_part;
+                const double neg = side ? nf - s_below : s_below;                     // elements on the other side of c
+                const double sd = sum_abs + d * (neg - (nf - neg)) + 2.0 * between;
+                s_st.mad = nf > 0.0 ? fmax(0.0, sd) / nf : 0.0;
+                // (sum_abs 0: every element is c)
+                s_again = sum_abs != 0.0 && (full > 0.0 || !(to * w * 0.5 <= 1e-8 * sum_abs));
+            }
+        }
         __syncthreads();
-        const float m_hi = (float)st.mean, m_lo = (float)(st.mean - (double)m_hi);    // the mean as an unevaluated fp32 pair
+        if (!s_ok) { leave(qp_grid::GAVE_UP); return; }
+    }
+    if (s_again) {                                            // uniform over the grid
+        const float m_hi = (float)s_st.mean, m_lo = (float)(s_st.mean - (double)m_hi);    // the mean as an unevaluated fp32 pair
         const qp_f2 nhi = qp_pack2(-m_hi, -m_hi), nlo = qp_pack2(-m_lo, -m_lo);
-        double v2[2];
-        if (st.nonfinite) {
+        double sd, sv;
+        if (s_st.nonfinite) {
             OpDeviations<true> f = {nhi, nlo, 0.0, 0.0};
             Tiles::template run<true>(x, a.ntiles, first, step, lane, f);
-            v2[0] = f.sd; v2[1] = f.sv;
+            sd = f.sd; sv = f.sv;
         } else {
             OpDeviations<false> f = {nhi, nlo, 0.0, 0.0};
             Tiles::template run<true>(x, a.ntiles, first, step, lane, f);
-            v2[0] = f.sd; v2[1] = f.sv;
+            sd = f.sd; sv = f.sv;
         }
         if (blockIdx.x == G - 1)
             for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) {
                 const float v = qp_load_one(x + i);
                 if (!qp_is_finite(v)) continue;
                 const float dd = __fsub_rn(__fsub_rn(v, m_hi), m_lo);
-                v2[0] += (double)fabsf(dd);
-                v2[1] += (double)(dd * dd);
+                sd += (double)fabsf(dd);
+                sv += (double)(dd * dd);
             }
-        ss_reduce<0, 0>(v2, s_red);
-        if (threadIdx.x == 0) {                               // (rows of their own: a slow block may still read the others)
-            a.part[(size_t)(3 * G + blockIdx.x) * 8] = v2[0];
-            a.part[(size_t)(3 * G + blockIdx.x) * 8 + 1] = v2[1];
+        const SsParts v = ss_block_parts<false>({sd, sv, 0.f, 0.f, 0u}, s_block[2]);
+        if (threadIdx.x == 0) part[OP_SECOND * G] = ss_row(v.a, v.b);
+        meet_warp0();
+        if (threadIdx.x < 32) {
+            double td = 0.0, tv = 0.0;
+            ss_merge<1>(a.part + OP_SECOND * G, G, [&](const uint4 (&p)[1]) {
+                td += ss_row_first(p[0]);
+                tv += ss_row_second(p[0]);
+            });
+            __syncwarp();
+            td = ss_pair_sum(td, tv);
+            tv = __shfl_sync(0xFFFFFFFFu, td, 16);
+            if (lane == 0) {
+                const double nf = (double)(a.n - s_st.nonfinite);
+                s_st.mad = nf > 0.0 ? td / nf : 0.0;
+                s_st.var = nf > 0.0 ? tv / nf : 0.0;
+            }
         }
-        if (!meet()) { leave(qp_grid::GAVE_UP); return; }
-        op_merge<0, 0>(a.part + (size_t)3 * G * 8, G, s_sum);
-        st.mad = nf > 0.0 ? s_sum[0] / nf : 0.0;
-        st.var = nf > 0.0 ? s_sum[1] / nf : 0.0;
     }
-    if (threadIdx.x == 0) {
-        if (blockIdx.x == 0) {
+    if (threadIdx.x == 0) {                                   // (it has written s_st itself)
+        const qp_stats_t st = s_st;
+        if (blockIdx.x == 0 && s_ok) {
             *a.st_out = st;
             if (st.nonfinite) atomicOr(a.status, QP_DEV_NONFINITE);
         }
@@ -466,13 +534,14 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             double lo, hi;
             qp_clip_ends(st, a.method, QP_DIST_LAPLACE, a.bmode, BITS, a.F, lo, hi);
             const int rc = qp_fill_qparams(lo, hi, BITS, &s_qp);
-            if (blockIdx.x == 0) {
+            if (blockIdx.x == 0 && s_ok) {
                 *a.qp_out = s_qp;
                 if (rc == QP_WARN_DEGENERATE) atomicOr(a.status, QP_DEV_DEGENERATE);
             }
         }
     }
     __syncthreads();
+    if (!s_ok) { leave(qp_grid::GAVE_UP); return; }
     if constexpr (BITS > 0) {                                 // from the tensor's end, which L2 holds
         uint32_t* sw = reinterpret_cast<uint32_t*>(raw) + (threadIdx.x >> 5) * 256;
         const float lo = s_qp.lo, hi = s_qp.hi, inv = s_qp.inv_scale;
@@ -507,7 +576,7 @@ bool op_usable(qp_ctx* ctx)
         ctx->op_checked = 1;
         int coop = 0;
         bool ok = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device) == cudaSuccess && coop &&
-                  (size_t)ctx->sm_count * 32 * sizeof(double) <= sizeof(qp_stats_partial) * QP_MAX_BLOCKS;
+                  (size_t)ctx->sm_count * OP_ROWS * sizeof(uint4) <= sizeof(qp_stats_partial) * QP_MAX_BLOCKS;
         for (int bits = 0; ok && bits <= 8; ++bits)
             for (int v = 0; ok && v < 2; ++v) {
                 void* k = v ? op_kernel<unsigned short>(bits) : op_kernel<float>(bits);
@@ -548,15 +617,13 @@ int32_t qp_launch_stats_onepass(qp_ctx* ctx, const void* d_x, int dtype, uint64_
     a.method = method;
     a.bmode = bmode;
     a.F = F;
-    a.part = reinterpret_cast<double*>(ctx->d_part);
+    a.part = reinterpret_cast<uint4*>(ctx->d_part);
     a.bar = reinterpret_cast<unsigned*>(ctx->d_fused) + 24;   // words 24, 25 of the barrier scratch
     a.status = ctx->d_status;
     a.spin_limit = ctx->spin_limit;
     a.bar_extra = (unsigned)ctx->bar_extra;
-    const uint64_t want = (a.ntiles + SS_WARPS - 1) / SS_WARPS;
     a.cluster = qp_cluster_wanted(ctx, ctx->op_cluster, n);
-    const unsigned most = a.cluster ? QP_CLUSTER_BLOCKS : (unsigned)ctx->sm_count;
-    const unsigned G = (unsigned)(want < most ? want : most);
+    const unsigned G = qp_together_blocks(ctx, a.cluster, a.ntiles);
     const uint64_t share = n / (dtype == QP_F32 ? 4 : 8) / ((uint64_t)G * SS_THREADS * 16);   // a sixteenth of the tensor
     // Two passes while the second one finds the tensor in L2, where it costs less than the pilot and the window; fp32 of 67, 134
     // and 268 MB: 30.6, 41 and 62 us in one pass, 28.6, 45 and 82 us in two; bf16 of 34, 67 and 134 MB: 28.8, 38.9 and 57,

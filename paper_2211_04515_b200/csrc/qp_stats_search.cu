@@ -640,7 +640,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
     const T* x = static_cast<const T*>(a.x);
     const int lane = threadIdx.x & 31;
     const unsigned G = gridDim.x;
-    const uint64_t first = (uint64_t)blockIdx.x * SS_WARPS + (threadIdx.x >> 5), step = (uint64_t)G * SS_WARPS;
+    const uint64_t first = (uint64_t)(threadIdx.x >> 5) * G + blockIdx.x, step = (uint64_t)G * SS_WARPS;
     const uint64_t tail0 = a.ntiles * SS_TILE;
     unsigned* bins = reinterpret_cast<unsigned*>(raw + SS_TABLE_BYTES);
     uint4* part = a.part + blockIdx.x;                        // this block's: row r at part[r * G]
@@ -1127,10 +1127,8 @@ int32_t qp_launch_stats_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t
     // for the elements behind the last tile
     a.flush_tiles = ((8191 - 64) << a.rep_shift) / (SS_WARPS * ss_ctile(hh));
     if (a.flush_tiles < 1) return qp_fail(ctx, QP_ERR_INVALID_ARG, "statistics and search: tables too small");
-    const uint64_t want = (a.ntiles + SS_WARPS - 1) / SS_WARPS;
     a.cluster = qp_cluster_wanted(ctx, ctx->ss_cluster, n);
-    const unsigned most = a.cluster ? QP_CLUSTER_BLOCKS : (unsigned)ctx->sm_count;
-    const unsigned G = (unsigned)(want < most ? want : most);
+    const unsigned G = qp_together_blocks(ctx, a.cluster, a.ntiles);
     void* k = dtype == QP_F32 ? ss_kernel<float>(st_in == nullptr, bits) : ss_kernel<unsigned short>(st_in == nullptr, bits);
     void* params[] = {&a};
     if (qp_launch_together(k, G, SS_THREADS, params, SS_DYN_BYTES, a.cluster, s) != cudaSuccess)
