@@ -758,33 +758,24 @@ extern "C" int32_t qp_unpack_dequantize(qp_ctx* ctx, const void* d_packed, uint6
 
 // ------------------------------------------- whole sender on device buffers
 
-// Where statistics, clip or search and packing are one streaming launch for any width: above QP_ONE_LAUNCH_MIN_N elements with the
-// search, and above QP_ONE_LAUNCH_MIN_N_CLOSED with a closed-form clip.
+// Where statistics, clip or search and packing are one streaming launch: as far down as it goes (8 tiles of 1024 elements), and up to
+// any size but for a gap each.
 constexpr uint64_t QP_ONE_LAUNCH_MIN_N = 1ull << 21;
 constexpr uint64_t QP_ONE_LAUNCH_MIN_N_CLOSED = QP_ONE_LAUNCH_MIN_N + (1ull << 19);
 
-// Where the directed search with statistics and packing in front of and behind it is one launch of the streaming kernel: that
-// spends 15 to 25 us whatever the size (barriers, and one block's scoring, which grows with the levels), the
-// small-tensor launch scores every element against every candidate.  At 2^15, 2^16, 2^17, 2^18, 2^19 and 2^20 elements: 23.5,
-// 24.7, 26.8, 32.9, 43 and 64 us in the small-tensor launch; streaming 22.7, 23.5, 23, 24.7, 28.8, 28.8 at 2 bits, 26.7, 28.7,
-// 26.8, 28.8, 32, 33 at 3 and 31 to 33 up to 2^18, 35 to 37 from there on at 4.
+// The directed search.  Against the small-tensor launch, which scores every element against every candidate (fp32, 2^13, 2^15, 2^17,
+// 2^18, 2^19 and 2^20 elements: 22.6, 23.2, 26.7, 32.8, 43 and 63.5 us at any width): 12.3, 14.1, 14.4, 14.4, 16.4 and 16.4 us at 1 bit,
+// 16.4, 18.5, 19.1, 20.5, 22.6 and 22.6 at 2, 18.5, 20.5, 20.5, 22.3, 24.5 and 24.6 at 3, and at 4 bits, from 2^15 on, 22.6, 22.6, 22.6,
+// 24.8 and 25.7.
 // Above 15 * 2^17 up to QP_ONE_LAUNCH_MIN_N elements the separate calls' three launches run, although one is faster there too
-// (2.02 M elements at 2, 3 and 4 bits: 36.9, 39.2 and 43.1 us, in one launch 30.8, 34.8 and 37.0): the graph
+// (2.02 M elements at 2, 3 and 4 bits: 36.9, 39.2 and 43.1 us in three, 22.6, 24.6 and 26.7 in one): the graph
 // replay test sends 2 017 280 elements and asserts that the recorded calls hold several launches.
-static bool streaming_search(uint64_t n, int bits)
-{
-    const uint64_t from = bits <= 2 ? 1ull << 15 : bits == 3 ? 3ull << 16 : 3ull << 17;
-    return n > QP_ONE_LAUNCH_MIN_N || (n >= from && n <= 15ull << 17);
-}
+static bool streaming_search(uint64_t n) { return n > QP_ONE_LAUNCH_MIN_N || n <= 15ull << 17; }
 
-// And the closed-form clip: as one cluster up to 2^18 elements (12.4 us, against 14.4 in the small-tensor launch), then again
-// above what the small-tensor launch holds.  Between the two: the small-tensor launch up to 2^21 (14.4 to 18.1 us; streaming 14.4
-// to 16.4), and above it up to QP_ONE_LAUNCH_MIN_N_CLOSED the separate calls' launches, 22.6 us where one streaming launch
-// takes 16.4 to 17: the sender's range test asserts that the call falls back to the chain behind the small-tensor launch.
-static bool streaming_closed_form(uint64_t n)
-{
-    return n > QP_ONE_LAUNCH_MIN_N_CLOSED || n <= 1u << 18;
-}
+// And the closed-form clip: 10.3 us as one cluster, up to 2^18 elements, and 12.3 from there to 2^21, where the small-tensor launch
+// takes 14.4 up to 2^20 and 16.4 to 18.5 up to 2^21.  Above that, up to QP_ONE_LAUNCH_MIN_N_CLOSED, the separate calls' launches,
+// 22.6 us where one would take 13: the sender's range test asserts that the call falls back to the chain behind the small-tensor launch.
+static bool streaming_closed_form(uint64_t n) { return n > QP_ONE_LAUNCH_MIN_N_CLOSED || n <= QP_ONE_LAUNCH_MIN_N; }
 
 // statistics -> clip -> quantize+pack on device buffers: one cooperative launch where that
 // applies (small tensors), the kernel chain of the separate calls otherwise
@@ -796,7 +787,7 @@ static int32_t sender_on_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_
     const int use_ds = (method & 0xF) == QP_CLIP_DSACIQ;
     const int search_mode = bmode | ((method & QP_CLIP_MIDRISE) ? QP_B_MIDRISE : 0);
     if (use_ds && ctx->sender_path == QP_SENDER_AUTO && ctx->stats_path == QP_STATS_AUTO && ctx->search_path == QP_SEARCH_AUTO &&
-        streaming_search(n, bits) && check_x(ctx, d_x, dtype, n) == QP_OK && steps >= 1 && d_packed && !((uintptr_t)d_packed & 15u) &&
+        streaming_search(n) && check_x(ctx, d_x, dtype, n) == QP_OK && steps >= 1 && d_packed && !((uintptr_t)d_packed & 15u) &&
         !((uintptr_t)st & 7u) && !((uintptr_t)d_qp_out & 3u) && (bmode == QP_B_MAD || bmode == QP_B_MEAN_ABS) &&
         qp_stats_search_applies(ctx, d_x, dtype, n, hist_bins, bits, steps)) {
         qp_device_guard guard(ctx->device);

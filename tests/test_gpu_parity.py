@@ -1112,6 +1112,39 @@ def test_sender_search_streaming(ctx, bits, n, bf16, data):
     ctx.qp_get_status()
 
 
+# the sender's streaming launch against the small-tensor launch where either can run: the smallest, a cluster's last and a grid's
+# first tensor, the ends of both rules.  Each is within 2e-6 of a candidate's error, so they are within 4e-6 of one another.
+@pytest.mark.parametrize("bits,use_ds,n,bf16", [(1, True, 8192, False), (3, True, 8192, True), (2, True, 8191, False), (4, True, 32768, False),
+                                                (4, True, 65536, True), (3, True, (1 << 18) + 1, True), (4, True, (1 << 18) - 1, False),
+                                                (4, True, (1 << 19) + 5, False), (8, False, 8192, True), (5, False, (1 << 18) + 1, False),
+                                                (3, False, 700001, True), (8, False, 1 << 21, False)])
+def test_sender_streaming_against_the_small_tensor_launch(ctx, bits, use_ds, n, bf16):
+    x = dev(si.vit_activation((1, n, 1), 90 + bits, outlier_frac=0.001).reshape(-1))
+    x = x.to(torch.bfloat16) if bf16 else x
+    out = []
+    for path in (qp.QP_SENDER_AUTO, qp.QP_SENDER_FUSED):
+        ctx.qp_set_sender_path(path)
+        try:
+            before = ctx.qp_launch_count()
+            packed, q = ctx.qp_sender_device(x, bits, use_ds)
+            assert ctx.qp_launch_count() - before == 1
+        finally:
+            ctx.qp_set_sender_path(qp.QP_SENDER_AUTO)
+        assert torch.equal(packed, ctx.qp_quantize_pack(x, bits, q))
+        got = ctx.read_qparams(q)
+        curve = np.array(ctx.qp_dsaciq_curve(100)) if use_ds else np.zeros(1)
+        ends = [(c.lo, c.hi) for c in ctx.qp_dsaciq_candidates(100)] if use_ds else [(got.lo, got.hi)]
+        out.append((got, curve, ends.index((got.lo, got.hi))))
+    (a, ca, ka), (b, cb, kb) = out
+    assert np.array_equal(np.isinf(ca), np.isinf(cb))
+    ok = np.isfinite(ca)
+    assert np.all(np.abs(ca[ok] - cb[ok]) <= 4e-6 * cb[ok])
+    assert ka == kb or abs(cb[ka] - cb[kb]) <= 4e-6 * cb[kb]
+    if not use_ds:                                       # two roundings of the same fp64 ends
+        assert abs(a.lo - b.lo) <= 2.0 ** -22 * abs(b.lo) and abs(a.hi - b.hi) <= 2.0 ** -22 * abs(b.hi)
+    ctx.qp_get_status()
+
+
 # the separate search in that launch, from its smallest tensor (8 tiles) to the last cluster and the first grid
 @pytest.mark.parametrize("bits", [1, 2, 3, 4])
 @pytest.mark.parametrize("n", [8 * 1024, 16 * 1024 + 1, (1 << 18) - 3, 1 << 18, (1 << 18) + 1])
