@@ -28,6 +28,9 @@ __device__ __forceinline__ bool ss_range_fits(const qp_stats_t& st, float inv_w)
     return st.max - st.min <= 3.4028234663852886e38 && inv_w < __int_as_float(0x7F800000);
 }
 
+// 2^k as fp64, k from -1022 to 1023
+__device__ __forceinline__ double ss_two_to(int k) { return __hiloint2double((k + 1023) << 20, 0); }
+
 template <int HH>
 struct SsPlan {
     float m;                                                  // fp32 mean; y = x - m
@@ -48,15 +51,14 @@ __device__ inline void ss_make_plan(SsPlan<HH>& p, int i, double mean, double a0
     const bool any = R > 1e-30 && R < 1e30;
     if (i < 0) {
         const int e = any ? (int)((unsigned)__double2hiint(R) >> 20) - 1022 : 0;            // R < 2^e, a normal number
-        auto two_to = [](int k) { return __hiloint2double((k + 1023) << 20, 0); };
         p.m = (float)mean;
         p.ncand = ncand;
         p.kf = (float)ncand;
         p.down = a1 < a0;
-        p.inv_e = any ? (float)two_to(-e) : 0.f;
-        p.w = any ? two_to(e - 6) : 0.0;
+        p.inv_e = any ? (float)ss_two_to(-e) : 0.f;
+        p.w = any ? ss_two_to(e - 6) : 0.0;
         p.cell = (float)p.w;
-        p.u = any ? two_to(e - 6 - ub) : 1.0;
+        p.u = any ? ss_two_to(e - 6 - ub) : 1.0;
         // clip ends that are coarse against the smallest step (an ulp of the mean beyond 2^-15 of it, where a candidate's
         // error would move by 1e-8), or clips beyond what the formula's fp32 constants hold: the exact thresholds
         p.hard = HH > 0 && R > 0.0 && (!any || fabs(mean) * 1.1920928955078125e-7 > 3.0517578125e-5 * (2.0 * a_min / L1));

@@ -775,6 +775,7 @@ static bool streaming_search(uint64_t n) { return n > QP_ONE_LAUNCH_MIN_N || n <
 // And the closed-form clip: 10.3 us as one cluster, up to 2^18 elements, and 12.3 from there to 2^21, where the small-tensor launch
 // takes 14.4 up to 2^20 and 16.4 to 18.5 up to 2^21.  Above that, up to QP_ONE_LAUNCH_MIN_N_CLOSED, the separate calls' launches,
 // 22.6 us where one would take 13: the sender's range test asserts that the call falls back to the chain behind the small-tensor launch.
+// 16 bits go the same way: 8.4, 16.8 and 100 M fp32 elements 22.6, 37.0 and 167 us in one launch, 32.8, 49.0 and 176 in three.
 static bool streaming_closed_form(uint64_t n) { return n > QP_ONE_LAUNCH_MIN_N_CLOSED || n <= QP_ONE_LAUNCH_MIN_N; }
 
 // statistics -> clip -> quantize+pack on device buffers: one cooperative launch where that
@@ -805,7 +806,7 @@ static int32_t sender_on_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_
     // the closed-form clip in one launch, except that the packer's own launch reads a large bf16 tensor faster: 2^26, 2^27 and
     // 2^28 elements at 8 bits take 89, 158 and 292 us in one launch, 94, 155 and 279 in three
     if (!use_ds && (dtype == QP_F32 || n <= (1ull << 26)) && ctx->sender_path == QP_SENDER_AUTO &&
-        ctx->stats_path == QP_STATS_AUTO && streaming_closed_form(n) && bits <= 8 &&
+        ctx->stats_path == QP_STATS_AUTO && streaming_closed_form(n) && (bits <= 8 || bits == 16) &&
         check_x(ctx, d_x, dtype, n) == QP_OK && d_packed && !((uintptr_t)d_packed & 15u) && !((uintptr_t)st & 7u) &&
         !((uintptr_t)d_qp_out & 3u) && (bmode == QP_B_MAD || bmode == QP_B_MEAN_ABS) && qp_stats_onepass_applies(ctx, d_x, n)) {
         qp_device_guard guard(ctx->device);

@@ -30,6 +30,23 @@ __device__ __forceinline__ void qp_quads_to_words(const uint32_t* sw, int g, uin
     }
 }
 
+// A partial tile's elements: whole vectors as such (VEC), the others one by one, NaN for those that are missing.
+template <typename T, bool VEC>
+__device__ __forceinline__ void qp_load_part(const T* __restrict__ xt, int have, int lane, float (&e)[QP_TILE / (32 * qp_span<T>::EPV)][qp_span<T>::EPV])
+{
+    constexpr int EPV = qp_span<T>::EPV;
+#pragma unroll
+    for (int j = 0; j < QP_TILE / (32 * EPV); ++j) {
+        const int k = (j * 32 + lane) * EPV;
+        if (VEC && k + EPV <= have) {
+            qp_load_vec(xt + k, e[j]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < EPV; ++i) e[j][i] = k + i < have ? qp_load_one(xt + k + i) : __int_as_float(0x7FC00000);
+        }
+    }
+}
+
 // Packs tile `tile` of x (n elements; the last tile may be partial: its missing elements are NaN, code 0) into `out`,
 // of which nwords exist (pad words included).  VEC: x is 16-byte aligned; otherwise every lane loads the
 // elements of its vectors one by one (the loads of a vector touch the same lines, so they hit L1).
@@ -55,14 +72,7 @@ __device__ __forceinline__ void qp_pack_tile(const T* __restrict__ x, uint64_t n
             }
         }
     } else {
-        const int have = (int)(n - tile * QP_TILE);
-#pragma unroll
-        for (int j = 0; j < NLOAD; ++j)
-#pragma unroll
-            for (int i = 0; i < EPV; ++i) {
-                const int k = (j * 32 + lane) * EPV + i;
-                e[j][i] = k < have ? qp_load_one(xt + k) : __int_as_float(0x7FC00000);
-            }
+        qp_load_part<T, VEC>(xt, (int)(n - tile * QP_TILE), lane, e);
     }
     uint32_t* ot = out + tile * (32 * BITS);
     if constexpr (BITS == 8 || (BITS == 4 && EPV == 8)) {         // a vector's quads are whole words: straight to the output
@@ -111,4 +121,41 @@ __device__ __forceinline__ void qp_pack_tile(const T* __restrict__ x, uint64_t n
             if (m * 32 + lane < room) ot[m * 32 + lane] = sw[m * 32 + lane];
     }
     __syncwarp();
+}
+// The same at 16 bits, where a vector's codes are whole words.  x is 16-byte aligned.
+template <typename T>
+__device__ __forceinline__ void qp_pack_tile16(const T* __restrict__ x, uint64_t n, uint64_t tile, int lane, float lo, float hi,
+                                               float inv, uint32_t* __restrict__ out, uint64_t nwords)
+{
+    constexpr int EPV = qp_span<T>::EPV, NLOAD = QP_TILE / (32 * EPV);
+    const T* xt = x + tile * QP_TILE;
+    const bool full = (tile + 1) * QP_TILE <= n;                 // warp-uniform
+    const int have = full ? QP_TILE : (int)(n - tile * QP_TILE);
+    float e[NLOAD][EPV];
+    if (full) {
+#pragma unroll
+        for (int j = 0; j < NLOAD; ++j) qp_load_vec(xt + (j * 32 + lane) * EPV, e[j]);
+    } else {
+        qp_load_part<T, true>(xt, have, lane, e);
+    }
+    uint32_t* ot = out + tile * (QP_TILE / 2);
+    const uint64_t room = nwords - tile * (QP_TILE / 2);          // whole vectors: the stream is padded to 16 bytes
+#pragma unroll
+    for (int j = 0; j < NLOAD; ++j) {
+        const int v = j * 32 + lane;
+        unsigned w[EPV / 2];
+#pragma unroll
+        for (int i = 0; i < EPV; i += 2) {
+            unsigned a = qp_code(e[j][i], lo, hi, inv, 0xFFFFu), b = qp_code(e[j][i + 1], lo, hi, inv, 0xFFFFu);
+            if (!full) {
+                a = v * EPV + i < have ? a : 0u;
+                b = v * EPV + i + 1 < have ? b : 0u;
+            }
+            w[i / 2] = a | (b << 16);
+        }
+        if ((uint64_t)v * (EPV / 2) < room) {
+            if constexpr (EPV == 4) reinterpret_cast<uint2*>(ot)[v] = make_uint2(w[0], w[1]);
+            else reinterpret_cast<uint4*>(ot)[v] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
 }

@@ -216,7 +216,9 @@ struct OpDeviations {
     }
 };
 
-// BITS = 0: statistics only; 1..8: the sender.
+template <int N> struct Rows { static constexpr int value = N; };
+
+// BITS = 0: statistics only; 1..8 and 16: the sender.
 template <typename T, int BITS>
 __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpArgs a)
 {
@@ -224,6 +226,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
     using Tiles = SsTiles<T, SS_TILE>;
     constexpr int EPV = Tiles::EPV;
     __shared__ SsBlock s_block[3];
+    __shared__ SsRows s_rows[OP_ROWS];
     __shared__ int s_ok, s_full, s_again;
     __shared__ float s_c, s_delta;
     __shared__ double s_D, s_abs, s_below;
@@ -250,6 +253,20 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             qp_grid::barrier_warp0(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
         }
     };
+    // this block's partial into row r, by warp 0, and every block's rows
+    auto put = [&](int r, const uint4& v) {
+        if (a.cluster) ss_push(s_rows[r], G, v);
+        else if (lane == 0) part[r * G] = v;
+    };
+    auto merge = [&](auto rows, int r, auto&& take) {
+        if (a.cluster) ss_merge_pushed<decltype(rows)::value>(s_rows + r, G, take);
+        else ss_merge<decltype(rows)::value>(a.part + r * G, G, take);
+    };
+    // (a block's shared memory may be written from outside once the block runs: the wait is in front of the first push, and a
+    // cluster's tensors never have a pilot)
+    if (a.cluster) qp_grid::cluster_arrive();
+    SsTail tail;
+    tail.load(x, tail0, a.n, blockIdx.x == G - 1);
     auto leave = [&](unsigned gave_up) {
         if (threadIdx.x == 0 && qp_grid::last_out(qp_grid::count_out(a.bar, gave_up), G)) qp_grid::reset(a.bar);
     };
@@ -287,14 +304,14 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             if (m * m < __int_as_float(0x7F800000)) { p1 += m; p2 = fmaf(m, m, p2); ++pn; }
         }
         const SsParts v = ss_block_parts<false>({(double)p1, (double)p2, 0.f, 0.f, pn}, s_block[0]);
-        if (threadIdx.x == 0) {
-            part[OP_PILOT * G] = ss_row(v.a, v.b);
-            part[(OP_PILOT + 1) * G] = make_uint4(v.count, 0u, 0u, 0u);
+        if (threadIdx.x < 32) {
+            put(OP_PILOT, ss_row(v.a, v.b));
+            put(OP_PILOT + 1, make_uint4(v.count, 0u, 0u, 0u));
         }
         meet_warp0();
         if (threadIdx.x < 32) {
             double t1 = 0.0, t2 = 0.0, tn = 0.0;
-            ss_merge<2>(a.part + OP_PILOT * G, G, [&](const uint4 (&p)[2]) {
+            merge(Rows<2>{}, OP_PILOT, [&](const uint4 (&p)[2]) {
                 t1 += ss_row_first(p[0]);
                 t2 += ss_row_second(p[0]);
                 tn += (double)p[1].x;
@@ -347,12 +364,10 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             o.sy = f.sy; o.sa = f.sa; o.sv = f.sv; o.sx = f.sx;
             o.below = f.below;
         }
-        if (blockIdx.x == G - 1)
-            for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) {
-                const float v = qp_load_one(x + i);
-                o.one(v, c);
-                if (a.one && qp_is_finite(v)) f.window(__fsub_rn(v, c));
-            }
+        tail.each([&](float v) {
+            o.one(v, c);
+            if (a.one && qp_is_finite(v)) f.window(__fsub_rn(v, c));
+        });
     };
     if (a.one) {
         OpPass<true> f;
@@ -362,13 +377,14 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
         pass(f);
     }
     {
+        if (a.cluster) qp_grid::cluster_wait();
         const SsParts v = ss_block_parts<true>({o.sy, o.sx, o.mn, o.mx, o.bad}, s_block[1]);       // (its barrier also orders the window's counters)
         SsParts u = {0.0, 0.0, 0.f, 0.f, 0u};
         if (a.one) u = ss_block_parts<false>({o.sa, o.sv, 0.f, 0.f, o.below}, s_block[2]);
-        if (threadIdx.x == 0) {
-            part[OP_PASS * G] = ss_row(v.a, v.b);
-            part[(OP_PASS + 1) * G] = make_uint4(__float_as_uint(v.lo), __float_as_uint(v.hi), v.count, u.count);
-            if (a.one) part[(OP_PASS + 2) * G] = ss_row(u.a, u.b);
+        if (threadIdx.x < 32) {
+            put(OP_PASS, ss_row(v.a, v.b));
+            put(OP_PASS + 1, make_uint4(__float_as_uint(v.lo), __float_as_uint(v.hi), v.count, u.count));
+            if (a.one) put(OP_PASS + 2, ss_row(u.a, u.b));
         }
     }
     meet_warp0();
@@ -383,14 +399,14 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             bad += (double)q.z;                               // exact: counts are far below 2^53
         };
         if (a.one) {
-            ss_merge<3>(a.part + OP_PASS * G, G, [&](const uint4 (&p)[3]) {
+            merge(Rows<3>{}, OP_PASS, [&](const uint4 (&p)[3]) {
                 first_two(p[0], p[1]);
                 below += (double)p[1].w;
                 sa += ss_row_first(p[2]);
                 sv += ss_row_second(p[2]);
             });
         } else {
-            ss_merge<2>(a.part + OP_PASS * G, G, [&](const uint4 (&p)[2]) { first_two(p[0], p[1]); });
+            merge(Rows<2>{}, OP_PASS, [&](const uint4 (&p)[2]) { first_two(p[0], p[1]); });
         }
         __syncwarp();
         sy = ss_pair_sum(sy, sx);
@@ -449,14 +465,14 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             if (i == own) in_own += (unsigned)cn;
         }
         const SsParts v = ss_block_parts<false>({vn, vs, 0.f, 0.f, in_own}, s_block[0]);
-        if (threadIdx.x == 0) {
-            part[OP_WINDOW * G] = ss_row(v.a, v.b);
-            part[(OP_WINDOW + 1) * G] = make_uint4(v.count, (unsigned)s_full, 0u, 0u);
+        if (threadIdx.x < 32) {
+            put(OP_WINDOW, ss_row(v.a, v.b));
+            put(OP_WINDOW + 1, make_uint4(v.count, (unsigned)s_full, 0u, 0u));
         }
         meet_warp0();
         if (threadIdx.x < 32) {
             double tn = 0.0, ts = 0.0, to = 0.0, full = 0.0;
-            ss_merge<2>(a.part + OP_WINDOW * G, G, [&](const uint4 (&p)[2]) {
+            merge(Rows<2>{}, OP_WINDOW, [&](const uint4 (&p)[2]) {
                 tn += ss_row_first(p[0]);
                 ts += ss_row_second(p[0]);
                 to += (double)p[1].x;
@@ -497,20 +513,18 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             Tiles::template run<true>(x, a.ntiles, first, step, lane, f);
             sd = f.sd; sv = f.sv;
         }
-        if (blockIdx.x == G - 1)
-            for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) {
-                const float v = qp_load_one(x + i);
-                if (!qp_is_finite(v)) continue;
-                const float dd = __fsub_rn(__fsub_rn(v, m_hi), m_lo);
-                sd += (double)fabsf(dd);
-                sv += (double)(dd * dd);
-            }
+        tail.each([&](float v) {
+            if (!qp_is_finite(v)) return;
+            const float dd = __fsub_rn(__fsub_rn(v, m_hi), m_lo);
+            sd += (double)fabsf(dd);
+            sv += (double)(dd * dd);
+        });
         const SsParts v = ss_block_parts<false>({sd, sv, 0.f, 0.f, 0u}, s_block[2]);
-        if (threadIdx.x == 0) part[OP_SECOND * G] = ss_row(v.a, v.b);
+        if (threadIdx.x < 32) put(OP_SECOND, ss_row(v.a, v.b));
         meet_warp0();
         if (threadIdx.x < 32) {
             double td = 0.0, tv = 0.0;
-            ss_merge<1>(a.part + OP_SECOND * G, G, [&](const uint4 (&p)[1]) {
+            merge(Rows<1>{}, OP_SECOND, [&](const uint4 (&p)[1]) {
                 td += ss_row_first(p[0]);
                 tv += ss_row_second(p[0]);
             });
@@ -546,8 +560,10 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
         uint32_t* sw = reinterpret_cast<uint32_t*>(raw) + (threadIdx.x >> 5) * 256;
         const float lo = s_qp.lo, hi = s_qp.hi, inv = s_qp.inv_scale;
         const uint64_t tiles = (a.n + QP_TILE - 1) / QP_TILE;
-        for (uint64_t it = first; it < tiles; it += step)
-            qp_pack_tile<BITS, T, true>(x, a.n, tiles - 1 - it, lane, lo, hi, inv, a.packed, a.nwords, sw);
+        for (uint64_t it = first; it < tiles; it += step) {
+            if constexpr (BITS == 16) qp_pack_tile16<T>(x, a.n, tiles - 1 - it, lane, lo, hi, inv, a.packed, a.nwords);
+            else qp_pack_tile<BITS, T, true>(x, a.n, tiles - 1 - it, lane, lo, hi, inv, a.packed, a.nwords, sw);
+        }
     }
     if (a.cluster) return;
     __syncthreads();
@@ -566,7 +582,8 @@ void* op_kernel(int bits)
         case 5: return (void*)stats_onepass_kernel<T, 5>;
         case 6: return (void*)stats_onepass_kernel<T, 6>;
         case 7: return (void*)stats_onepass_kernel<T, 7>;
-        default: return (void*)stats_onepass_kernel<T, 8>;
+        case 8: return (void*)stats_onepass_kernel<T, 8>;
+        default: return (void*)stats_onepass_kernel<T, 16>;
     }
 }
 
@@ -577,7 +594,7 @@ bool op_usable(qp_ctx* ctx)
         int coop = 0;
         bool ok = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device) == cudaSuccess && coop &&
                   (size_t)ctx->sm_count * OP_ROWS * sizeof(uint4) <= sizeof(qp_stats_partial) * QP_MAX_BLOCKS;
-        for (int bits = 0; ok && bits <= 8; ++bits)
+        for (int bits = 0; ok && bits <= 9; ++bits)           // (9: 16 bits)
             for (int v = 0; ok && v < 2; ++v) {
                 void* k = v ? op_kernel<unsigned short>(bits) : op_kernel<float>(bits);
                 int per_sm = 0;
@@ -585,7 +602,7 @@ bool op_usable(qp_ctx* ctx)
                      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, SS_THREADS, OP_DYN_BYTES) == cudaSuccess && per_sm >= 1;
             }
         ctx->op_cluster = ok;
-        for (int bits = 0; ok && bits <= 8; ++bits)
+        for (int bits = 0; ok && bits <= 9; ++bits)
             for (int v = 0; v < 2; ++v)
                 ctx->op_cluster &= qp_cluster_fits(v ? op_kernel<unsigned short>(bits) : op_kernel<float>(bits), SS_THREADS, OP_DYN_BYTES);
         if (!ok) cudaGetLastError();
@@ -601,7 +618,7 @@ bool qp_stats_onepass_applies(qp_ctx* ctx, const void* d_x, uint64_t n)
     return !((uintptr_t)d_x & 15u) && n >= 8 * SS_TILE && op_usable(ctx);
 }
 
-// Statistics (bits = 0), or with bits 1..8 the sender with a closed-form clip.
+// Statistics (bits = 0), or with bits 1..8 or 16 the sender with a closed-form clip.
 int32_t qp_launch_stats_onepass(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, qp_stats_t* st_out, int bits, int method,
                                 int bmode, double F, qp_qparams_t* d_qp_out, void* d_packed, cudaStream_t s)
 {

@@ -19,14 +19,16 @@
 // step take the "hard" form below, with the exact thresholds.
 //
 // What bounds it, by time stamps that the blocks took (each figure from the last block before it to its own last block; the
-// stamps lengthen the launch by 2 to 3 us): on 129 MB (fp32, 2 bits) phase A 24 us, the read from DRAM; barrier and merge 3; B 18 and C
-// 21, the read, most of which L2 still holds, and the instructions (A and B 19 per element together, C 19, at 4 bits 35; one shared
-// atomic in B, two in C); between them histogram, barrier, merge and candidates 6; a block's prefix sums and errors 2, barrier and pick
-// 3; packing 20.  On 39 MB at 4 bits, which L2 holds: A 8, then 3, B 5, 6, C 12, 4, 3 and the packing 4: 45 and 3 for the launch.  Both
-// calls took 15 us longer (47 and 99 against 63 and 114) with the blocks' intervals added up by all of them in slices, behind a barrier of their own, the scoring
-// by block 0 alone with the others waiting, and block partials 64 bytes apart.
-// Shuffles by a warp that has not reconverged cost 250 cycles each instead of 30 (the finish 3.6 us instead of 1.3): hence the
-// __syncwarp before them and the grid barrier whose whole warp polls.
+// stamps lengthen the launch by 2 to 3 us): on 129 MB (fp32, 2 bits) phase A 23 us, the read from DRAM; barrier and merge 3.5; B 17.5 and C
+// 20, the read, most of which L2 still holds, and the instructions (A and B 19 per element together, C 19, at 4 bits 35; one shared
+// atomic in B, two in C); between them histogram, barrier, merge and candidates 5; a block's prefix sums and errors 2, barrier and pick
+// 3; packing 19.  On 39 MB at 4 bits, which L2 holds: A 8, then 3.5, B 5.5, 5, C 11, 4, 2.5 and the packing 4: 44 and 3 between launches.
+// Both calls took 15 us longer with the blocks' intervals added up by all of them in slices, behind a barrier of their own, the scoring
+// by block 0 alone with the others waiting, and block partials 64 bytes apart.  One image (151 K, a cluster of 10 blocks) at 2 bits, 17 us:
+// A 1.2, 1.9, B 1.9, 4.4 up to the candidates, C 2.3, 2 and 2.5 for scoring and pick, packing 0.9.
+// Shuffles by lanes that have parted cost 250 cycles each instead of 30 (the finish 3.6 us instead of 1.3; the whole launch on one
+// image 3.3 us longer without the __syncwarp behind the tail's elements): hence the __syncwarp before them and the grid barrier whose
+// whole warp polls.
 #include <type_traits>
 
 #include "qp_affine.cuh"
@@ -250,6 +252,7 @@ __device__ __forceinline__ void ss_flush(unsigned char* raw, int ni, int rs, ulo
             cd = (unsigned long long)d.x + d.y + ((unsigned long long)d.z + d.w);
             cnt[u] = sum[u] = make_uint4(0u, 0u, 0u, 0u);
         }
+        __syncwarp();
         for (int o = 1; o < (1 << ts); o <<= 1) {
             cn += __shfl_xor_sync(0xFFFFFFFFu, cn, o);
             cd += __shfl_xor_sync(0xFFFFFFFFu, cd, o);
@@ -277,6 +280,7 @@ __device__ __forceinline__ void ss_hist_out(const unsigned* bins, int nb, int sh
                 for (int r = 0; r < (1 << shift); ++r) c += bins[(u << shift) + r];
             }
         }
+        __syncwarp();
         for (int o = 1; o < (1 << ts); o <<= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
         if (u < units && (u & ((1 << ts) - 1)) == 0 && c) atomicAdd(&hist[min(u >> ts, nb - 1)], (unsigned long long)c);
     }
@@ -304,8 +308,10 @@ __device__ __forceinline__ uint2 ss_prefix(unsigned char* raw, int ni, int rs, c
     for (int g = 8; g <= 64; g += 8) cell += s_edge[g] <= i0 ? 8 : 0;
     int more = 0;
 #pragma unroll
-    for (int g = 1; g < 8; ++g) more += s_edge[min(cell + g, SS_GRID)] <= i0 ? 1 : 0;
-    cell = min(cell + more, SS_GRID);
+    for (int g = 1; g < 8; ++g) more += s_edge[min(cell + g, SS_GRID + 1)] <= i0 ? 1 : 0;
+    cell += more;
+    // (every cell starts an interval, so that an interval is in the cell of the one before it or in the next: no loop that parts lanes)
+    int next = s_edge[cell + 1];
     unsigned n = 0u;
     unsigned long long s = 0ull;
     for (int i = i0; i < i1; ++i) {
@@ -320,7 +326,8 @@ __device__ __forceinline__ uint2 ss_prefix(unsigned char* raw, int ni, int rs, c
             cn += c.x + c.y + (c.z + c.w);
             cd += (unsigned long long)d.x + d.y + ((unsigned long long)d.z + d.w);
         }
-        while (cell < SS_GRID && s_edge[cell + 1] <= i) ++cell;
+        cell += next <= i ? 1 : 0;
+        next = s_edge[cell + 1];
         if (row) { cn += (unsigned)row[e].x; cd += row[e].y; }
         *ss_slot(raw, e, rs) = make_ulonglong2(n, s);
         n += cn;
@@ -356,7 +363,7 @@ __device__ __forceinline__ uint2 ss_prefix(unsigned char* raw, int ni, int rs, c
 }
 
 // Where the boundaries of every candidate lie among the intervals: pos[k][b - 1], the first interval of code b = 1..HH of a
-// side.  s_edge: the interval that a grid cell starts with.
+// side.  s_edge: the interval that a grid cell starts with; behind the last, none.
 template <int HH>
 __device__ __forceinline__ void ss_places(const SsPlan<HH>& p, int ncand, int ni, int* s_edge, int* pos)
 {
@@ -364,7 +371,7 @@ __device__ __forceinline__ void ss_places(const SsPlan<HH>& p, int ncand, int ni
         const int k = w / HH, b = w - k * HH + 1;
         pos[w] = QP_CK(ss_place(p, k, b), ni);
     }
-    for (int g = threadIdx.x; g <= SS_GRID; g += SS_THREADS) s_edge[g] = ss_cell_start(p, g);
+    for (int g = threadIdx.x; g <= SS_GRID + 1; g += SS_THREADS) s_edge[g] = g <= SS_GRID ? ss_cell_start(p, g) : 1 << 30;
 }
 
 // The error of candidate k is, over the elements,
@@ -380,7 +387,7 @@ __device__ __forceinline__ void ss_errors(const SsPlan<HH>& p, int ncand, int ni
                                           const float4* s_cand, const int* s_valid, unsigned long long* acc)
 {
     constexpr int TPC = HH == 1 ? 2 : 4, RUN = (2 * HH + TPC - 1) / TPC;     // threads per candidate: one or two per side
-    const double unit = ldexp(1.0, fix);
+    const double unit = ss_two_to(fix);
     for (int w0 = threadIdx.x & ~31; w0 < ncand * TPC; w0 += SS_THREADS) {
         const int w = w0 + (threadIdx.x & 31), k = w / TPC, part = w % TPC;
         const int side = part / (TPC / 2), b0 = 1 + (part % (TPC / 2)) * RUN;
@@ -399,6 +406,7 @@ __device__ __forceinline__ void ss_errors(const SsPlan<HH>& p, int ncand, int ni
                 below = lv;
             }
         }
+        __syncwarp();
 #pragma unroll
         for (int o = TPC / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
         if (k < ncand && part == 0) atomicAdd(acc + k, (unsigned long long)__double2ll_rn(v * unit));
@@ -424,7 +432,7 @@ __device__ __forceinline__ int ss_finish(const SsArgs& a, float m, bool flat, co
         const double s_up = 0.5 * (s_abs + nf * dm), s_down = 0.5 * (s_abs - nf * dm);
         double best = inf;
         if (k < ncand) {
-            double v = HH || hard ? ldexp((double)(long long)__ldcg(a.acc + k), -fix) : 0.0;
+            double v = HH || hard ? (double)(long long)__ldcg(a.acc + k) * ss_two_to(-fix) : 0.0;
             if (hard) {
                 v -= 2.0 * (hard->lv_lo[k] * hard->e_lo + hard->lv_hi[k] * hard->e_hi);
             } else {
@@ -630,6 +638,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
     constexpr int H = SEARCH ? HH : 0;
     extern __shared__ __align__(16) unsigned char raw[];
     __shared__ SsBlock s_block[2];
+    __shared__ SsRows s_rows[STATS ? 4 : 1];
     __shared__ __align__(16) double s_red[SS_WARPS * 2];
     __shared__ int s_ok;
     __shared__ bool s_last;
@@ -644,8 +653,23 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
     const uint64_t tail0 = a.ntiles * SS_TILE;
     unsigned* bins = reinterpret_cast<unsigned*>(raw + SS_TABLE_BYTES);
     uint4* part = a.part + blockIdx.x;                        // this block's: row r at part[r * G]
-    unsigned waits = 0;
     const bool cluster = a.cluster;
+    // this block's partial into row r, by warp 0, and every block's rows r and r + 1 (behind a barrier; the statistics alone have none
+    // behind phase B)
+    auto pushed = [&](int r) { return cluster && (SEARCH || r < 2); };
+    auto put = [&](int r, const uint4& v) {
+        if (pushed(r)) ss_push(s_rows[r], G, v);
+        else if (lane == 0) part[r * G] = v;
+    };
+    auto merge2 = [&](int r, auto&& take) {
+        if (pushed(r)) ss_merge_pushed<2>(s_rows + r, G, take);
+        else ss_merge<2>(a.part + r * G, G, take);
+    };
+    // (a block's shared memory may be written from outside once the block runs: the wait is in front of the first push)
+    if (STATS && cluster) qp_grid::cluster_arrive();
+    SsTail tail;
+    tail.load(x, tail0, a.n, blockIdx.x == G - 1);
+    unsigned waits = 0;
     auto meet = [&]() {
         if (cluster) {
             qp_grid::cluster_arrive();
@@ -662,6 +686,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
             qp_grid::cluster_arrive();
             qp_grid::cluster_wait();
             if (threadIdx.x == 0) s_ok = 1;
+            __syncwarp();
         } else if (threadIdx.x < 32) {
             qp_grid::barrier_warp0(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
         }
@@ -689,19 +714,19 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
                 for (int j = 0; j < SS_TILE / 32 / Tiles::EPV; ++j)
                     for (int i = 0; i < Tiles::EPV; ++i) acc.one(qp_load_one(x + t * SS_TILE + (j * 32 + lane) * Tiles::EPV + i));
         }
-        if (blockIdx.x == G - 1)
-            for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) acc.one(qp_load_one(x + i));
+        tail.each([&](float v) { acc.one(v); });
+        if (cluster) qp_grid::cluster_wait();
         const SsParts v = ss_block_parts<true>({acc.s, acc.sa, acc.mn, acc.mx, acc.bad}, s_block[0]);
-        if (threadIdx.x == 0) {
-            part[0] = ss_row(v.a, v.b);
-            part[G] = make_uint4(__float_as_uint(v.lo), __float_as_uint(v.hi), v.count, 0u);
+        if (threadIdx.x < 32) {
+            put(0, ss_row(v.a, v.b));
+            put(1, make_uint4(__float_as_uint(v.lo), __float_as_uint(v.hi), v.count, 0u));
         }
         if (threadIdx.x >= 32) empty(threadIdx.x - 32, SS_THREADS - 32);          // while warp 0 waits and merges
         meet_warp0();
         if (threadIdx.x < 32) {
             double s = 0.0, sa = 0.0, bad = 0.0;
             float mn = __int_as_float(0x7F800000), mx = -mn;
-            ss_merge<2>(a.part, G, [&](const uint4 (&p)[2]) {
+            merge2(0, [&](const uint4 (&p)[2]) {
                 s += ss_row_first(p[0]);
                 sa += ss_row_second(p[0]);
                 mn = fminf(mn, __uint_as_float(p[1].x));
@@ -762,12 +787,11 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
                 SsDeviationsOf<STATS ? 0 : 1> f = {d};
                 SsTiles<T, SS_TILE>::template run<true>(x, a.ntiles, first, step, lane, f);
             }
-            if (blockIdx.x == G - 1)
-                for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) d.one(qp_load_one(x + i));
+            tail.each([&](float x) { d.one(x); });
             v = ss_block_parts<false>({d.sd[0] + d.sd[1], d.sv[0] + d.sv[1], 0.f, 0.f, d.below}, s_block[1]);   // (its barrier orders the counters)
-            if (STATS && threadIdx.x == 0) {
-                part[2 * G] = ss_row(v.a, v.b);
-                part[3 * G] = make_uint4(v.count, 0u, 0u, 0u);
+            if (STATS && threadIdx.x < 32) {
+                put(2, ss_row(v.a, v.b));
+                put(3, make_uint4(v.count, 0u, 0u, 0u));
             }
         }
         if (hist_on) ss_hist_out(bins, a.nb, a.hist_shift, a.hist);
@@ -792,7 +816,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
 #pragma unroll
             for (int u = 0; u < 4; ++u) c[u] = hist_on && lane + 32 * u < a.nb ? __ldcg(&a.hist[lane + 32 * u]) : 0ull;
             if (STATS)
-                ss_merge<2>(a.part + 2 * G, G, [&](const uint4 (&p)[2]) {
+                merge2(2, [&](const uint4 (&p)[2]) {
                     sd += ss_row_first(p[0]);
                     sv += ss_row_second(p[0]);
                     below += (double)p[1].x;
@@ -840,7 +864,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
         __shared__ float4 s_cand[QP_SS_MAX_CAND];
         __shared__ int s_valid[QP_SS_MAX_CAND];
         __shared__ double s_curve[QP_SS_MAX_CAND];
-        __shared__ int s_edge[SS_GRID + 1];                   // interval that a grid cell starts with
+        __shared__ int s_edge[SS_GRID + 2];                   // interval that a grid cell starts with, and one that there is not
         {                                                     // every thread the same set-up, then its part of the plan and its candidates
             const bool have = s_st.hist_bins == a.nb;
             if (!have && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, QP_DEV_HIST_MISSING);
@@ -874,8 +898,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
                 const SsPlan<H> p = s_plan;
                 SsSides f = {p.m, guard, 0u, 0u};
                 SsTiles<T, SS_TILE>::template run<false>(x, a.ntiles, first, step, lane, f);
-                if (blockIdx.x == G - 1)
-                    for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) f.one(qp_load_one(x + i));
+                tail.each([&](float x) { f.one(x); });
                 const SsParts v = ss_block_parts<false>({(double)f.all, 0.0, 0.f, 0.f, f.down}, s_block[0]);
                 if (threadIdx.x == 0) {
                     atomicAdd(a.acc + ncand, (unsigned long long)v.count);
@@ -910,11 +933,9 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
                     SsTiles<T, CT>::template run<false>(x, t1, t0 + first, step, lane, f);
                 }
             }
-            if (blockIdx.x == G - 1)
-                for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) {
-                    const float v = qp_load_one(x + i);
-                    if (qp_is_finite(v)) ss_count<H>(p, tb, v);
-                }
+            tail.each([&](float v) {
+                if (qp_is_finite(v)) ss_count<H>(p, tb, v);
+            });
             ss_places<H>(s_plan, ncand, ni, s_edge, pos);
             __syncthreads();
             const uint2 sides = ss_prefix(raw, ni, a.rep_shift, ntiles > per ? row : nullptr, s_edge, reinterpret_cast<ulonglong2*>(s_red));
@@ -943,8 +964,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
                     fresh = false;
                 }
             }
-            if (blockIdx.x == G - 1)
-                for (uint64_t i = tail0 + threadIdx.x; i < a.n; i += SS_THREADS) ss_hard_one(h, qp_load_one(x + i), e2[0], e2[1]);
+            tail.each([&](float x) { ss_hard_one(h, x, e2[0], e2[1]); });
             const SsParts e = ss_block_parts<false>({e2[0], e2[1], 0.f, 0.f, 0u}, s_block[0]);
             if (threadIdx.x == 0) part[0] = ss_row(e.a, e.b);         // (every block is done with the first rows)
             ss_hard_flush(h, row, fresh);
@@ -964,8 +984,6 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
                 return SS_DONE;
             }
             if (!meet()) return SS_GAVE_UP;
-            // (block 0 of a separate search: a warp that the rest does not wait for asks meanwhile who is out)
-            if (!a.packed && !cluster && threadIdx.x == SS_THREADS - 1) ss_out(a, qp_grid::count_out(a.bar));
         }
         SsBeyond beyond = {lv, lv + ncand, 0.0, 0.0};
         if (hard && H > 0) {
@@ -987,7 +1005,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
         const int best = ss_finish<H>(a, s_plan.m, flat, s_st, up, down, ncand, fix, s_cand, s_valid, s_curve, hard && H > 0 ? &beyond : nullptr,
                                       s_block[0].sum, reinterpret_cast<int*>(s_block[0].count));
         if (blockIdx.x == 0) {
-            if (threadIdx.x == 0) {
+            if (threadIdx.x == SS_THREADS - 32) {             // (a warp that has a tile less to pack than the first, or none)
                 qp_ds_write_result(best, s_curve, s_setup, a.steps, a.nb, BITS, s_cand[best], a.ds_out, a.qp_out, a.status);
                 *a.setup = s_setup;
             }
@@ -1000,6 +1018,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
             if (!STATS)
                 for (int k = threadIdx.x; k < ncand + 2; k += SS_THREADS) a.acc[k] = 0ull;
         }
+        if (!a.packed && !cluster && threadIdx.x == SS_THREADS - 1) ss_out(a, qp_grid::count_out(a.bar));
         if constexpr (!STATS) return SS_OUT;
         if constexpr (STATS) {                                // the sender: everybody packs, from the tensor's end
             const float4 q = s_cand[best];

@@ -118,6 +118,30 @@ __device__ __forceinline__ uint4 ss_row(double a, double b)
 }
 __device__ __forceinline__ double ss_row_first(const uint4& r) { return __hiloint2double((int)r.y, (int)r.x); }
 __device__ __forceinline__ double ss_row_second(const uint4& r) { return __hiloint2double((int)r.w, (int)r.z); }
+// In a cluster the rows go into every block's shared memory instead, rows[r][block]: by warp 0, a lane per block, before the
+// cluster's barrier; behind it lane b < G has block b's.
+typedef uint4 SsRows[16];                                     // of as many blocks as a cluster has at most
+__device__ __forceinline__ void ss_push(SsRows& row, unsigned G, const uint4& v)
+{
+    const unsigned lane = threadIdx.x & 31;
+    if (lane < G) {
+        unsigned at;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((unsigned)__cvta_generic_to_shared(&row[blockIdx.x])), "r"(lane));
+        asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+    }
+    __syncwarp();
+}
+template <int ROWS, typename F>
+__device__ __forceinline__ void ss_merge_pushed(const SsRows* rows, unsigned G, F&& take)
+{
+    const unsigned b = threadIdx.x & 31;
+    if (b < G) {
+        uint4 p[ROWS];
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) p[r] = rows[r][b];
+        take(p);
+    }
+}
 template <int ROWS, typename F>
 __device__ __forceinline__ void ss_merge(const uint4* part, unsigned G, F&& take)
 {
@@ -176,6 +200,33 @@ struct SsStream {
 };
 template <typename T, int ELEMS> using SsTiles = SsStream<T, ELEMS / 32 / qp_span<T>::EPV>;
 
+
+// The elements behind the last whole tile, for the last block: loaded once, up to two per thread, and kept for all passes.  (As loads in
+// every pass, after its own, they were the longest chain of a small tensor's.)
+struct SsTail {
+    float v[2];
+    int m;
+    template <typename T>
+    __device__ __forceinline__ void load(const T* x, uint64_t tail0, uint64_t n, bool mine)
+    {
+        static_assert(SS_TILE <= 2 * SS_THREADS, "two per thread");
+        m = 0;
+        v[0] = v[1] = 0.f;
+        const uint64_t i = tail0 + threadIdx.x;
+        if (mine && i < n) {
+            v[0] = qp_load_one(x + i);
+            m = 1;
+            if (i + SS_THREADS < n) { v[1] = qp_load_one(x + i + SS_THREADS); m = 2; }
+        }
+    }
+    template <typename F>
+    __device__ __forceinline__ void each(F&& f) const
+    {
+        if (m > 0) f(v[0]);
+        if (m > 1) f(v[1]);
+        __syncwarp();
+    }
+};
 
 // ---- launches whose blocks wait for one another: a cooperative grid, or one thread-block cluster
 constexpr unsigned QP_CLUSTER_BLOCKS = 16;        // the largest cluster (above 8: by attribute, where the device has the SMs)

@@ -1117,7 +1117,9 @@ def test_sender_search_streaming(ctx, bits, n, bf16, data):
 @pytest.mark.parametrize("bits,use_ds,n,bf16", [(1, True, 8192, False), (3, True, 8192, True), (2, True, 8191, False), (4, True, 32768, False),
                                                 (4, True, 65536, True), (3, True, (1 << 18) + 1, True), (4, True, (1 << 18) - 1, False),
                                                 (4, True, (1 << 19) + 5, False), (8, False, 8192, True), (5, False, (1 << 18) + 1, False),
-                                                (3, False, 700001, True), (8, False, 1 << 21, False)])
+                                                (3, False, 700001, True), (8, False, 1 << 21, False),
+                                                (16, False, 8192 + 5, False), (16, False, 9216 + 9, True), (16, False, (1 << 18) + 7, True),
+                                                (16, False, (5 << 19) + 1023, False)])
 def test_sender_streaming_against_the_small_tensor_launch(ctx, bits, use_ds, n, bf16):
     x = dev(si.vit_activation((1, n, 1), 90 + bits, outlier_frac=0.001).reshape(-1))
     x = x.to(torch.bfloat16) if bf16 else x
