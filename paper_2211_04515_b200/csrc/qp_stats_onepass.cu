@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
     const T* x = static_cast<const T*>(a.x);
     const int lane = threadIdx.x & 31;
     const unsigned G = gridDim.x;
-    const uint64_t first = (uint64_t)(threadIdx.x >> 5) * G + blockIdx.x, step = (uint64_t)G * SS_WARPS;
+    const uint64_t step = (uint64_t)G * SS_WARPS, first = ss_first_tile(a.ntiles, step);
     const uint64_t tail0 = a.ntiles * SS_TILE;
     const double inf = __longlong_as_double(0x7FF0000000000000ll);
     unsigned* table = reinterpret_cast<unsigned*>(raw);

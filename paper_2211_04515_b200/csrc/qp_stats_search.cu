@@ -649,7 +649,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
     const T* x = static_cast<const T*>(a.x);
     const int lane = threadIdx.x & 31;
     const unsigned G = gridDim.x;
-    const uint64_t first = (uint64_t)(threadIdx.x >> 5) * G + blockIdx.x, step = (uint64_t)G * SS_WARPS;
+    const uint64_t step = (uint64_t)G * SS_WARPS, first = ss_first_tile(a.ntiles, step);
     const uint64_t tail0 = a.ntiles * SS_TILE;
     unsigned* bins = reinterpret_cast<unsigned*>(raw + SS_TABLE_BYTES);
     uint4* part = a.part + blockIdx.x;                        // this block's: row r at part[r * G]

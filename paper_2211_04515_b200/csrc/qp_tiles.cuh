@@ -158,6 +158,16 @@ __device__ __forceinline__ void ss_merge(const uint4* part, unsigned G, F&& take
     }
 }
 
+// A warp's first tile; the others follow `step` tiles apart.  Up to 32 tiles a warp, warp w of block b starts with tile w G + b, so that
+// the last tiles are spread over the blocks (closed-form sender, 27 M bf16 elements at 6 bits: 38.6 us, 39.8 with a block's warps side
+// by side; 51 M fp32 at 3 bits 84.2 and 85.5); beyond that the last tiles count for less than the 64 KB that a block's warps
+// read side by side (90 M fp32 at 8 bits: 146 us spread, 141.8 side by side; 268 M: 392 and 386).
+__device__ __forceinline__ uint64_t ss_first_tile(uint64_t ntiles, uint64_t step)
+{
+    const unsigned w = threadIdx.x >> 5;
+    return ntiles <= 32 * step ? w * gridDim.x + blockIdx.x : blockIdx.x * SS_WARPS + w;
+}
+
 // ---- streaming.  A warp works on tiles of N 16-byte vectors per lane, held in registers; a vector's registers are
 // reloaded from the warp's next tile as soon as its elements have been taken out, so the loads of a whole tile are
 // in flight all the time without a second set of registers or moves between the two.
@@ -269,8 +279,7 @@ inline int qp_cluster_wanted(const qp_ctx* ctx, int fits, uint64_t n)
 }
 
 // Blocks of such a launch: a tile per warp.  (In a cluster a block per tile, up to 16, gains on the passes what it loses on the
-// barriers: one image at 8 bits the same, with the search at 2 bits 20.1 us against 19.0.)  Warp w of block b starts with tile
-// w G + b, so that the last tiles are spread over the blocks: 32 M elements at 8 bits 61.5 us, 62.1 with a block's warps side by side.
+// barriers: one image at 8 bits the same, with the search at 2 bits 20.1 us against 19.0.)
 inline unsigned qp_together_blocks(const qp_ctx* ctx, int cluster, uint64_t ntiles)
 {
     const uint64_t most = cluster ? QP_CLUSTER_BLOCKS : (uint64_t)ctx->sm_count, want = (ntiles + SS_WARPS - 1) / SS_WARPS;
