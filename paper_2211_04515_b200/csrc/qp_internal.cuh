@@ -293,6 +293,17 @@ template <int BITS>
 __device__ __forceinline__ unsigned qp_quad(const float* e, float lo, float hi, float inv)
 {
     const qp_f2 nlo = qp_pack2(-lo, -lo), inv2 = qp_pack2(inv, inv), magic = qp_pack2(QP_MAGIC, QP_MAGIC);
+    if constexpr (BITS == 8) {                                // a code is the low byte of its sum: three permutations
+        unsigned two[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float a = fminf(fmaxf(e[2 * h], lo), hi), b = fminf(fmaxf(e[2 * h + 1], lo), hi);
+            float pa, pb;
+            qp_unpack2(qp_add2(qp_mul2(qp_add2(qp_pack2(a, b), nlo), inv2), magic), pa, pb);
+            two[h] = __byte_perm(__float_as_uint(pa), __float_as_uint(pb), 0x0040);
+        }
+        return __byte_perm(two[0], two[1], 0x5410);
+    }
     constexpr unsigned MB = QP_MAGIC_BITS;
     constexpr unsigned offs = MB + (MB << BITS) + (BITS < 16 ? MB << ((2 * BITS) & 31) : 0u) + (3 * BITS < 32 ? MB << ((3 * BITS) & 31) : 0u);
     unsigned r = 0u - offs;

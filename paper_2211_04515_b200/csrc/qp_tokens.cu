@@ -555,17 +555,19 @@ __device__ __forceinline__ bool tok_row_stats(const T* row, int nvec, uint32_t C
 }
 
 constexpr int TR_WARPS = 8;                                   // warps per block
+// Blocks per SM, 48 registers a thread: a row is a chain of waits, and 72 % of the issue slots were taken with four.  fp32 of 25216 x 1280
+// at 4 and 8 bits 41.3 -> 39.0 and 37.2 -> 36.3 us, 16000 x 2048 at 8 bits 41.1 -> 35.3, 40000 x 192 bf16 at 4 bits 28.4 -> 26.7; six
+// (40 registers) are slower again (39.2, 37.1, 37.0).
+constexpr int TR_BLOCKS = 5;
 
-// bytes of shared memory a warp needs for a row (a multiple of 16): the row, and in the sender its quads
-__host__ __device__ constexpr size_t tok_row_bytes(uint32_t C, size_t esz, bool sender)
-{
-    return (size_t)C * esz + (sender ? (size_t)C : 0);
-}
+// bytes of shared memory a warp needs for a row (a multiple of 16).  The sender's quads, a byte per element, take the
+// place of the elements that they were made of, its words that of the elements behind.
+__host__ __device__ constexpr size_t tok_row_bytes(uint32_t C, size_t esz) { return (size_t)C * esz; }
 
 // BITS = 0: statistics only (any row of whole vectors).  BITS = 1..8: the whole sender, rows of whole
 // 32-element groups (a row is then whole words).
 template <int BITS, typename T>
-__global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __restrict__ x, uint64_t tokens, uint32_t C, int method,
+__global__ void __launch_bounds__(TR_WARPS * 32, TR_BLOCKS) tok_rows_kernel(const T* __restrict__ x, uint64_t tokens, uint32_t C, int method,
                                                                  int bmode, double F, uint32_t* __restrict__ out,
                                                                  uint64_t nwords, qp_qparams_t* __restrict__ qp_out,
                                                                  qp_stats_t* __restrict__ st_out, unsigned* __restrict__ status)
@@ -573,7 +575,7 @@ __global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __rest
     extern __shared__ __align__(16) unsigned char raw[];
     constexpr int EPV = qp_span<T>::EPV;
     const int lane = threadIdx.x & 31;
-    T* row = reinterpret_cast<T*>(raw + (threadIdx.x >> 5) * tok_row_bytes(C, sizeof(T), BITS > 0));
+    T* row = reinterpret_cast<T*>(raw + (threadIdx.x >> 5) * tok_row_bytes(C, sizeof(T)));
     const int nvec = (int)(C / EPV);
     unsigned raise = 0u;
     const uint64_t wstride = (uint64_t)gridDim.x * TR_WARPS;
@@ -596,7 +598,7 @@ __global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __rest
         if (lane == 0) st_out[t] = st;
         if constexpr (BITS > 0) {
             constexpr unsigned mask = (1u << BITS) - 1u;
-            uint32_t* sw = reinterpret_cast<uint32_t*>(row + C);
+            uint32_t* sw = reinterpret_cast<uint32_t*>(row);
             const int groups = (int)(C / 32);
             double lo_d, hi_d;
             qp_clip_ends(st, method, QP_DIST_LAPLACE, bmode, BITS, F, lo_d, hi_d);
@@ -617,9 +619,12 @@ __global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __rest
             }
             if (lane == 0) qp_out[t] = q;
             uint32_t* orow = out + t * (uint64_t)(groups * BITS);
+            constexpr bool STAGED = BITS != 8 && !(BITS == 4 && EPV == 8);
+            const unsigned lanes = nvec >= 32 ? 0xFFFFFFFFu : (1u << nvec) - 1u;       // those with a vector among the first 32
             auto quantize = [&](int v) {                     // vector v: its quads to the output (8 bits: a quad is a word) or to `sw`
                 float e[EPV];
                 tok_lds<T>(row + QP_CK(v, nvec) * EPV, e);
+                if (STAGED && v < 32) __syncwarp(lanes);     // the first 32 vectors' quads lie where those vectors were, the others' behind
                 if constexpr (EPV == 4) {
                     const unsigned qd = qp_quad<BITS>(e, q.lo, q.hi, q.inv_scale);
                     if constexpr (BITS == 8) orow[v] = qd;
@@ -636,10 +641,10 @@ __global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __rest
 #pragma unroll 4
             for (int v0 = 0; v0 < whole; v0 += 32) quantize(v0 + lane);
             if (whole + lane < nvec) quantize(whole + lane);
-            if constexpr (BITS != 8 && !(BITS == 4 && EPV == 8)) {
+            if constexpr (STAGED) {
                 // quads across the warp: 32 elements = BITS words per lane
                 __syncwarp();
-                uint32_t* words = reinterpret_cast<uint32_t*>(row);   // the row is no longer needed: room for its words
+                uint32_t* words = sw + C / 4;                 // behind the quads
                 for (int g = lane; g < groups; g += 32) {
                     uint32_t w[BITS];
                     qp_quads_to_words<BITS>(sw, QP_CK(g, groups), w);
@@ -651,12 +656,12 @@ __global__ void __launch_bounds__(TR_WARPS * 32) tok_rows_kernel(const T* __rest
                         orow[g] = w[0];
                     } else {
 #pragma unroll
-                        for (int m = 0; m < BITS; ++m) words[QP_CK(g * BITS + m, (int)(C * sizeof(T) / 4))] = w[m];
+                        for (int m = 0; m < BITS; ++m) words[QP_CK(g * BITS + m, (int)(C / 4))] = w[m];
                     }
                 }
                 if constexpr (BITS != 4 && BITS != 2 && BITS != 1) {
                     __syncwarp();
-                    for (int i = lane; i < groups * BITS; i += 32) orow[i] = words[QP_CK(i, (int)(C * sizeof(T) / 4))];
+                    for (int i = lane; i < groups * BITS; i += 32) orow[i] = words[QP_CK(i, (int)(C / 4))];
                 }
             }
             if (t == tokens - 1) {                           // pad words
@@ -751,14 +756,14 @@ bool tok_rows_apply(const void* x, int dtype, uint32_t C, bool sender)
     if (!x || (dtype != QP_F32 && dtype != QP_BF16)) return false;
     const size_t esz = dtype == QP_F32 ? 4 : 2;
     return C >= 32 && C % (sender ? 32 : 16 / esz) == 0 && ((uintptr_t)x & 15u) == 0 &&
-           tok_row_bytes(C, esz, sender) * TR_WARPS <= TR_SMEM_MAX;
+           (tok_row_bytes(C, esz) + (sender ? C : 0)) * TR_WARPS <= TR_SMEM_MAX;
 }
 
 template <int BITS, typename T>
 int32_t launch_rows(qp_ctx* ctx, const T* x, uint64_t tokens, uint32_t C, int method, int bmode, uint32_t* out,
                     qp_qparams_t* d_qp, qp_stats_t* d_stats, cudaStream_t s)
 {
-    const size_t smem = tok_row_bytes(C, sizeof(T), BITS > 0) * TR_WARPS;
+    const size_t smem = tok_row_bytes(C, sizeof(T)) * TR_WARPS;
     if (smem > 48 * 1024 && cudaFuncSetAttribute(tok_rows_kernel<BITS, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)TR_SMEM_MAX) != cudaSuccess)
         return qp_check_launch(ctx, "token rows (shared memory)");
