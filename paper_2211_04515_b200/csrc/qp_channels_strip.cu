@@ -14,8 +14,8 @@
 // What bounds it: the 32-byte sectors that a strip's rows touch (ct_choose), the instructions (A 4, B 11, C 14 + 2 per code
 // boundary and element) with their shared atomics, and the chain of small steps around the passes.  12608 x 1024 fp32 at 4 bits (52 MB), by
 // time stamps: A 14 us, its sums across the cluster 3, B 10 and 4, peaks and plans 5, C 20, interval sums across the cluster 6 (16
-// bytes a load; 8 with 4 bytes), prefix sums 3 (13 with a `while` over the cells per interval and a warp per side), errors 7, pick 1:
-// 74, and the whole stage (receiver, this, packing) 106; with strips of 14 channels, whose rows start anywhere in a sector, and
+// bytes a load; 8 with 4 bytes), prefix sums 3 (13 with a `while` over the cells per interval and a warp per side), errors 5 (7 by
+// codes instead of by boundaries), pick 1: 72, and the whole stage (receiver, this, packing) 104; with strips of 14 channels, whose rows start anywhere in a sector, and
 // those two forms 101 and 134.  Unrolling the errors' loop or three vectors of the interval sums at a time costs 2 us each (straight
 // code that runs once).  The ten kernels before (four for the statistics, histogram, set-up, thresholds sorted per
 // channel, a pass with binary searches, error curves, pick) took 255 us.
@@ -547,25 +547,25 @@ __global__ void __launch_bounds__(CT_THREADS, 1) ch_strip_kernel(const CtArgs a)
                 qp_ds_candidate(su, k, a.steps, BITS, a.bmode & QP_B_MIDRISE, cd, ok);
                 a.cand[(size_t)c * a.ncp + k] = cd;
                 a.valid[(size_t)c * a.ncp + k] = ok;
-                double v = 0.0, n_up = 0.0, n_down = 0.0, x_up = 0.0, x_down = 0.0;
                 // integers below 2^52 to fp64 by the exponent of 2^52 (the conversion unit is a quarter of the fp64 one's rate)
                 auto whole = [](unsigned hi, unsigned lo) { return __hiloint2double((int)(0x43300000u | hi), (int)lo) - 4503599627370496.0; };
+                // sum over the codes i of a side of N_i l_i^2 - 2 l_i S_i, by the boundaries between them: with P below a boundary,
+                // N l_top^2 - 2 S l_top - sum of (l_i - l_(i-1)) ((l_i + l_(i-1)) P_N - 2 P_S)
+                double v = 0.0;
                 if (ok) {
+                    const int top = flat ? 0 : H;             // (flat: everything has the first code of its side)
+                    double a1 = ss_level(cd, H + 1, p.m), a2 = -ss_level(cd, H, p.m);            // distances from the centre
 #pragma unroll 1
-                    for (int i = 0; i <= H; ++i) {            // code i of both sides, outwards
-                        const int p1 = i == H || flat ? ni : QP_CK(ss_place(p, k, i + 1), ni);
-                        double n1 = up, n2 = down, x1 = s_up, x2 = s_down;
-                        if (p1 < ni) {
-                            const unsigned w1 = c_up[p1], w2 = c_up[ni + p1];
-                            n1 = whole(0u, w1 & 0x1FFFFu);
-                            n2 = whole(0u, w2 & 0x1FFFFu);
-                            x1 = p.u * whole(w1 >> 17, t_up[p1]);
-                            x2 = p.u * whole(w2 >> 17, t_up[ni + p1]);
-                        }
-                        const double l1 = ss_level(cd, H + 1 + i, p.m), l2 = -ss_level(cd, H - i, p.m);   // distances from the centre
-                        v += ((n1 - n_up) * l1 * l1 - 2.0 * l1 * (x1 - x_up)) + ((n2 - n_down) * l2 * l2 - 2.0 * l2 * (x2 - x_down));
-                        n_up = n1; n_down = n2; x_up = x1; x_down = x2;
+                    for (int i = 1; i <= top; ++i) {          // boundary i of both sides, outwards
+                        const int at = QP_CK(ss_place(p, k, i), ni);
+                        const unsigned w1 = c_up[at], w2 = c_up[ni + at];
+                        const double l1 = ss_level(cd, H + 1 + i, p.m), l2 = -ss_level(cd, H - i, p.m);
+                        v += (l1 - a1) * (2.0 * p.u * whole(w1 >> 17, t_up[at]) - (l1 + a1) * whole(0u, w1 & 0x1FFFFu));
+                        v += (l2 - a2) * (2.0 * p.u * whole(w2 >> 17, t_up[ni + at]) - (l2 + a2) * whole(0u, w2 & 0x1FFFFu));
+                        a1 = l1;
+                        a2 = l2;
                     }
+                    v += (up * a1 * a1 - 2.0 * a1 * s_up) + (down * a2 * a2 - 2.0 * a2 * s_down);
                 }
                 mse = !ok ? inf : nf > 0.0 ? (nf * (q.var + dm * dm) + v) / nf : 0.0;
                 a.curve[(size_t)c * a.ncp + k] = mse;
