@@ -168,7 +168,7 @@ int32_t qp_make_qparams(double lo, double hi, int bits, qp_qparams_t* h_out);
  * d_x.  Two passes over x (sums/min/max, then deviations about the mean), fp64 merges in a
  * fixed order: results are bit-reproducible run to run.  n = 0 gives all-zero statistics.
  * 16-byte aligned tensors (8192 elements and more, 128 KB with the histogram) take one launch for
- * both, and without the histogram a single pass from 96 MB on: deviations about a pilot centre, the
+ * both, and without the histogram a single pass from 96 MB (fp32; bf16 224 MB) on: deviations about a pilot centre, the
  * split point moved to the mean afterwards (a second pass follows in the same launch where that
  * cannot be done to 1e-8), see qp_set_stats_path.
  * hist_bins > 0 asks the second pass to carry the directed search's histogram along

@@ -43,7 +43,7 @@ constexpr int OP_OCTAVES = 8;                      // octaves of |y| below delta
 constexpr int OP_CELLS = 64 * OP_OCTAVES + 1;      // per side; cell 0: what is below them
 constexpr int OP_REPS = 3;                         // log2 of the lane replicas of a cell
 constexpr unsigned OP_FULL = 65000u;               // most elements of a cell's replica: offsets of 16 bits add up to a word
-constexpr uint64_t OP_ONE_MIN_BYTES = 96ull << 20; // tensors from which one pass is the faster form
+constexpr uint64_t OP_ONE_MIN_BYTES_F32 = 96ull << 20, OP_ONE_MIN_BYTES_BF16 = 224ull << 20;   // tensors from which one pass is the faster form
 constexpr float OP_MAGIC = 8388608.0f;
 constexpr unsigned OP_ONE = 0x4B000000u;
 constexpr size_t OP_DYN_BYTES = (size_t)(2 * OP_CELLS * 2 << OP_REPS) * sizeof(unsigned);   // >= 16 KB: the packer's staging
@@ -642,10 +642,11 @@ int32_t qp_launch_stats_onepass(qp_ctx* ctx, const void* d_x, int dtype, uint64_
     a.cluster = qp_cluster_wanted(ctx, ctx->op_cluster, n);
     const unsigned G = qp_together_blocks(ctx, a.cluster, a.ntiles);
     const uint64_t share = n / (dtype == QP_F32 ? 4 : 8) / ((uint64_t)G * SS_THREADS * 16);   // a sixteenth of the tensor
-    // Two passes while the second one finds the tensor in L2, where it costs less than the pilot and the window; fp32 of 67, 134
-    // and 268 MB: 30.6, 41 and 62 us in one pass, 28.6, 45 and 82 us in two; bf16 of 34, 67 and 134 MB: 28.8, 38.9 and 57,
-    // and 26.7, 39.0 and 63.
-    a.one = n * (dtype == QP_F32 ? 4 : 2) >= OP_ONE_MIN_BYTES;
+    // Two passes while the second one finds enough of the tensor in L2 to cost less than the pilot and the window; fp32 of 67, 100 and
+    // 134 MB: 24.5, 31.6 and 40.9 us in two passes, 28.6, 34.1 and 39.1 in one (the sender at 8 bits 32.9, 51.1 and 66.5, and 36.9, 51.5
+    // and 61.5).  The pass with the window takes twice the elements a byte in bf16: 100, 134, 220 and 268 MB in 37.0, 47.3, 73.2 and 87.5 us in
+    // two passes, 45.1, 52.9, 75.6 and 87.8 in one (the sender, up to 134 MB, 65.4 and 86, and 68.7 and 86).
+    a.one = n * (dtype == QP_F32 ? 4 : 2) >= (dtype == QP_F32 ? OP_ONE_MIN_BYTES_F32 : OP_ONE_MIN_BYTES_BF16);
     a.sample = share < 1 ? 1 : share < OP_SAMPLE ? (int)share : OP_SAMPLE;
     void* k = dtype == QP_F32 ? op_kernel<float>(bits) : op_kernel<unsigned short>(bits);
     void* params[] = {&a};

@@ -1217,6 +1217,22 @@ def test_stats_streaming(ctx, n, data, bf16):
     ctx.qp_get_status()
 
 
+# bf16 on both sides of the line between two passes and one (224 MB): every block of rows against sums in 64 bits (fp32 chains of
+# at most 16 terms: 16 * 2^-24; the one pass accepts 1e-8 beside them), and the sender's quantizer from those statistics
+@pytest.mark.parametrize("n", [(112 << 20) - 1, 112 << 20])
+def test_stats_bf16_on_both_sides_of_the_one_pass_line(ctx, n):
+    g = torch.Generator(device="cuda").manual_seed(n % 97)
+    x = (torch.randn(n, device="cuda", generator=g) * 0.7 + 0.1).to(torch.bfloat16)
+    st = ctx.read_stats(ctx.qp_stats(x))
+    parts = [c.double() for c in x.split(1 << 24)]
+    mean = sum(float(c.sum()) for c in parts) / n
+    mad, var, ab = (sum(float(f(c).sum()) for c in parts) / n for f in (lambda c: (c - mean).abs(), lambda c: (c - mean) ** 2, lambda c: c.abs()))
+    assert (st.n, st.nonfinite, st.min, st.max) == (n, 0, float(x.min()), float(x.max()))
+    assert abs(st.mean - mean) <= 1e-6 * ab and abs(st.mad - mad) <= 1e-6 * mad and abs(st.var - var) <= 1e-6 * var
+    assert abs(st.mean_abs - ab) <= 1e-6 * ab
+    assert ctx.qp_get_status() == 0
+
+
 # statistics and search in one launch (the default from 8192 elements on, 32768 at 4 bits, the sender by width): every width it takes, tile
 # remainders, the largest and smallest number of steps, tables with few replicas, and the exact-threshold form
 SS_CASES = [(1, 0, 100, 100, (1 << 21) + 1, "vit"), (2, 0, 100, 100, (1 << 21) + 1023, "outliers"), (3, 0, 100, 100, (1 << 21) + 1024, "vit"),
