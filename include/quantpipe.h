@@ -139,7 +139,7 @@ const char* qp_status_string(int32_t status);
 /* 1 if the library was built with index checks (-DQP_CHECK_BOUNDS; `python -m paper_2211_04515_b200.build
  * --check` writes libquantpipe_check.so): every index into the kernels' shared-memory tables and scratch
  * rows is then range-checked, an index out of range is redirected to entry 0 (nothing traps or faults) and
- * qp_get_status reports QP_DEV_INDEX_RANGE.  The stand-in, on this library's own tables, for a memory
+ * qp_get_status reports QP_DEV_INDEX_RANGE; some blocks also come late where others could overtake them.  The stand-in, on this library's own tables, for a memory
  * checker where none can be run.  0 for the ordinary build. */
 int32_t qp_built_with_index_checks(void);
 /* Number of kernels this context has launched since qp_create (host-side count). */

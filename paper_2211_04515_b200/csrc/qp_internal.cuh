@@ -116,12 +116,14 @@ struct qp_ctx {
 };
 
 // Scratch of the cooperative kernels (d_fused): 256 bytes of barrier counters and the histogram (4096 x 8 bytes), both
-// zero between launches, and the search's sums per candidate, one set of the sender's, one of the separate search's (the latter
-// zero between launches).
+// zero between launches; the search's sums per candidate, one set of the sender's, one of the separate search's (the latter
+// zero between launches); and the search sender's histogram.  What is the sender's is emptied by the launch that uses it, in front of
+// its first barrier: a histogram emptied behind the last one would be empty too early for a block that still has to read it.
 constexpr int QP_SS_MAX_CAND = 256;              // candidates of the search in one launch with the statistics
 constexpr int QP_SS_TOTALS = 4096;               // most intervals of a block's row
 constexpr size_t QP_FUSED_TOTALS_AT = 256 + sizeof(unsigned long long) * 4096;
-constexpr size_t QP_FUSED_BYTES = QP_FUSED_TOTALS_AT + 2 * sizeof(unsigned long long) * (QP_SS_MAX_CAND + 2);
+constexpr size_t QP_FUSED_SENDER_HIST_AT = QP_FUSED_TOTALS_AT + 2 * sizeof(unsigned long long) * (QP_SS_MAX_CAND + 2);
+constexpr size_t QP_FUSED_BYTES = QP_FUSED_SENDER_HIST_AT + sizeof(unsigned long long) * 4096;
 
 constexpr long long QP_WAIT_CYCLES_DEFAULT = 4000000000ll;   // about two seconds
 constexpr unsigned QP_SPIN_LIMIT_DEFAULT = 1u << 22;          // x 64 ns sleeps: a quarter of a second at least
@@ -181,6 +183,13 @@ __device__ __forceinline__ I qp_ck(I i, N n)
     return i;
 }
 #define QP_CK(i, n) qp_ck((i), (n))
+// QP_LATE(c): in the debug build the threads that c names come here about half a millisecond late, so that what they
+// read must not depend on their being on time.
+#define QP_LATE(c)                                                                                          \
+    do {                                                                                                    \
+        if (c)                                                                                              \
+            for (int late = 0; late < 8; ++late) __nanosleep(100000);                                       \
+    } while (0)
 struct qp_ck_unit { qp_ck_unit* next; unsigned (*read_and_clear)(); };
 void qp_ck_register(qp_ck_unit* u);
 #define QP_CK_UNIT                                                                                          \
@@ -195,6 +204,7 @@ void qp_ck_register(qp_ck_unit* u);
     static const int qp_ck_registered = (qp_ck_register(&qp_ck_this_unit), 0);
 #else
 #define QP_CK(i, n) (i)
+#define QP_LATE(c)
 #define QP_CK_UNIT
 #endif
 

@@ -60,10 +60,10 @@ struct SsArgs {
     int* valid;
     qp_ds_setup* setup;
     uint4* part;                                  // [4][grid] block partials, 16 bytes each
-    unsigned long long* hist;                     // [nb], zero at entry and at exit
+    unsigned long long* hist;                     // [nb]; the sender's own, otherwise zero at entry and at exit
     ulonglong2* rows;                             // [grid][intervals] count, sum: what a block emptied its tables of on the way
-    unsigned long long* acc;                      // [ncand + 2]: errors of the candidates in fixed point; search only: the elements below the
-                                                  // centre and the others, all zero at entry and at exit
+    unsigned long long* acc;                      // [ncand + 2]: errors of the candidates in fixed point (the sender's own); search only: the
+                                                  // elements below the centre and the others, all zero at entry and at exit
     unsigned* bar;                                // [0] arrivals, [1] blocks that have left; zero at entry and at exit
     unsigned* status;
     unsigned spin_limit, bar_extra;
@@ -619,7 +619,7 @@ __host__ __device__ constexpr int ss_ctile(int hh) { return hh >= 3 ? 512 : 1024
 __device__ __forceinline__ void ss_out(const SsArgs& a, unsigned before)
 {
     if (!qp_grid::last_out(before, gridDim.x)) return;
-    if (before >= qp_grid::GAVE_UP) {                         // (block 0 of an undisturbed launch has cleaned)
+    if (before >= qp_grid::GAVE_UP && !(a.bits && !a.st_in)) {        // (block 0 of an undisturbed launch has cleaned)
         for (int b = 0; b < a.nb; ++b) a.hist[b] = 0ull;
         if (a.bits)
             for (int k = 0; k < a.steps + 3; ++k) a.acc[k] = 0ull;
@@ -702,8 +702,10 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
 
     // ---- phase A
     if constexpr (STATS) {
-        if (SEARCH && blockIdx.x == 0)                        // (their first use is behind the barrier)
+        if (SEARCH && blockIdx.x == 0) {                      // (their first use is behind the barrier)
             for (int k = threadIdx.x; k <= a.steps; k += SS_THREADS) a.acc[k] = 0ull;
+            for (int b = threadIdx.x; b < a.nb; b += SS_THREADS) a.hist[b] = 0ull;
+        }
         using Tiles = SsTiles<T, SS_TILE>;
         SsMoments acc;
         acc.clear();
@@ -813,6 +815,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
         if (threadIdx.x < 32) {
             double sd = 0.0, sv = 0.0, below = 0.0, peak = 0.0;
             unsigned long long c[4];
+            QP_LATE(SEARCH && G > 1 && blockIdx.x == G - 1);
 #pragma unroll
             for (int u = 0; u < 4; ++u) c[u] = hist_on && lane + 32 * u < a.nb ? __ldcg(&a.hist[lane + 32 * u]) : 0ull;
             if (STATS)
@@ -1014,9 +1017,10 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
                 a.cand[k] = s_cand[k];
                 a.valid[k] = s_valid[k];
             }
-            for (int b = threadIdx.x; b < a.nb; b += SS_THREADS) a.hist[b] = 0ull;       // (nobody needs it any more)
-            if (!STATS)
+            if constexpr (!STATS) {                           // (nobody needs them any more: every block has arrived since)
+                for (int b = threadIdx.x; b < a.nb; b += SS_THREADS) a.hist[b] = 0ull;
                 for (int k = threadIdx.x; k < ncand + 2; k += SS_THREADS) a.acc[k] = 0ull;
+            }
         }
         if (!a.packed && !cluster && threadIdx.x == SS_THREADS - 1) ss_out(a, qp_grid::count_out(a.bar));
         if constexpr (!STATS) return SS_OUT;
@@ -1127,7 +1131,7 @@ int32_t qp_launch_stats_search(qp_ctx* ctx, const void* d_x, int dtype, uint64_t
     a.part = reinterpret_cast<uint4*>(ctx->d_part);
     unsigned char* f = static_cast<unsigned char*>(ctx->d_fused);
     a.bar = reinterpret_cast<unsigned*>(f) + 16;              // words 16, 17 (the sender uses 0, 1, the statistics 8..10 and 24, 25)
-    a.hist = reinterpret_cast<unsigned long long*>(f + 256);
+    a.hist = reinterpret_cast<unsigned long long*>(f + (bits && !st_in ? QP_FUSED_SENDER_HIST_AT : 256));
     a.acc = reinterpret_cast<unsigned long long*>(f + QP_FUSED_TOTALS_AT) + (st_in ? QP_SS_MAX_CAND + 2 : 0);
     a.rows = reinterpret_cast<ulonglong2*>(ctx->d_iv_part);
     a.status = ctx->d_status;

@@ -4,7 +4,8 @@ No memory checker can be run on the kernels, so the library has a debug build
 (`python -m paper_2211_04515_b200.build --check`, -DQP_CHECK_BOUNDS) in which every index into the
 kernels' shared-memory tables and scratch rows is range-checked: an index out of range is redirected
 to entry 0 (nothing traps, nothing faults) and raises QP_DEV_INDEX_RANGE in what qp_get_status
-returns.  This test builds that variant, runs the small cases (c1, ragged sizes, degenerate and
+returns.  The build also makes some blocks come late where others could overtake them (QP_LATE), so that a missing wait
+shows in the results.  This test builds that variant, runs the small cases (c1, ragged sizes, degenerate and
 non-finite inputs, searches at 1 to 8 bits, channel-wise and token-wise shapes, the streaming launches as
 clusters and as grids, the channel strips and the token rows) in a child process
 that loads it through QUANTPIPE_LIB, and expects them to pass with the bit clear (the child's
@@ -25,7 +26,7 @@ SUBSET = ("test_stats_configs or test_stats_ragged or test_stats_special or stat
           "test_search_ragged or test_search_degenerate or test_fused_sender_c1 or fused_sender_special or "
           "test_channels_shapes or test_search_channels_vit or test_tokens_shapes or "
           "test_stats_streaming or test_sender_search_streaming or test_search_streaming_small or test_search_channels_strips or "
-          "test_tokens_rows_edges or beyond_fp32")
+          "test_tokens_rows_edges or beyond_fp32 or one_bit_blocks")
 
 
 def test_small_cases_run_clean_under_the_index_checked_build():

@@ -1112,6 +1112,24 @@ def test_sender_search_streaming(ctx, bits, n, bf16, data):
     ctx.qp_get_status()
 
 
+# one bit, where nothing but phase B's barrier lies between the histogram and the launch's end: all blocks quantize with the same
+# quantizer, and it is the one that the separate calls find (in the index-checked build the last block reads the histogram late)
+@pytest.mark.parametrize("n,bf16", [(1 << 15, False), ((1 << 18) - 1, True), ((1 << 18) + 1, False), ((5 << 18) + 1023, True)])
+def test_sender_one_bit_blocks_agree(ctx, n, bf16):
+    x = dev(si.vit_activation((1, n, 1), 640, outlier_frac=0.001).reshape(-1))
+    x = x.to(torch.bfloat16) if bf16 else x
+    st = ctx.qp_stats(x, hist_bins=100)
+    res = ctx.read_ds_result(ctx.qp_dsaciq_search(x, st, 1)[0])
+    for _ in range(3):                                   # (what a launch leaves behind is the next one's start)
+        got = torch.zeros(80, dtype=torch.uint8, device="cuda")
+        packed, q = ctx.qp_sender_device(x, 1, True, out_stats=got)
+        assert ctx.read_stats(got).hist_peak == ctx.read_stats(st).hist_peak
+        assert torch.equal(packed, ctx.qp_quantize_pack(x, 1, q))
+        # (ends are fp32 roundings of fp64 sums in another order; neighbouring steps that tie are b_R / 1000 apart)
+        assert abs(ctx.read_qparams(q).hi - ctx.read_qparams(q).lo - 2 * res.alpha_star) <= 2e-2 * res.alpha_star
+    assert ctx.qp_get_status() == 0
+
+
 # the sender's streaming launch against the small-tensor launch where either can run: the smallest, a cluster's last and a grid's
 # first tensor, the ends of both rules.  Each is within 2e-6 of a candidate's error, so they are within 4e-6 of one another.
 @pytest.mark.parametrize("bits,use_ds,n,bf16", [(1, True, 8192, False), (3, True, 8192, True), (2, True, 8191, False), (4, True, 32768, False),
