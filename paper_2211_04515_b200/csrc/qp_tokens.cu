@@ -378,9 +378,8 @@ __device__ __forceinline__ void tok_lds8(const T* row, int v, qp_f2 (&p)[4])
 
 // a 16-byte vector of the row as floats
 template <typename T>
-__device__ __forceinline__ void tok_lds(const T* p, float (&e)[qp_span<T>::EPV])
+__device__ __forceinline__ void tok_widen(const uint4& r, float (&e)[qp_span<T>::EPV])
 {
-    const uint4 r = *reinterpret_cast<const uint4*>(p);
     const unsigned w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -391,6 +390,11 @@ __device__ __forceinline__ void tok_lds(const T* p, float (&e)[qp_span<T>::EPV])
             e[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
         }
     }
+}
+template <typename T>
+__device__ __forceinline__ void tok_lds(const T* p, float (&e)[qp_span<T>::EPV])
+{
+    tok_widen<T>(*reinterpret_cast<const uint4*>(p), e);
 }
 
 // sum of 8 magnitudes as a tree, and of 8 values: no longer chain of roundings than a run of four
@@ -559,6 +563,10 @@ constexpr int TR_WARPS = 8;                                   // warps per block
 // at 4 and 8 bits 41.3 -> 39.0 and 37.2 -> 36.3 us, 16000 x 2048 at 8 bits 41.1 -> 35.3, 40000 x 192 bf16 at 4 bits 28.4 -> 26.7; six
 // (40 registers) are slower again (39.2, 37.1, 37.0).
 constexpr int TR_BLOCKS = 5;
+// Rounds of 32 vectors that the staged widths load before they store.  One, two and four of them, 12608 rows of 1280 fp32 at 5 bits:
+// 21.9, 20.6 and 20.8 us, 2560 bf16 at 6: 32.9, 31.8 and 31.5, 2560 fp32 at 4: 43.1, 41.1 and 41.1 (quads in a room of their own, four
+// blocks an SM: 22.2, 32.9 and 41.1).
+constexpr int TR_ROUNDS = 4;
 
 // bytes of shared memory a warp needs for a row (a multiple of 16).  The sender's quads, a byte per element, take the
 // place of the elements that they were made of, its words that of the elements behind.
@@ -620,11 +628,10 @@ __global__ void __launch_bounds__(TR_WARPS * 32, TR_BLOCKS) tok_rows_kernel(cons
             if (lane == 0) qp_out[t] = q;
             uint32_t* orow = out + t * (uint64_t)(groups * BITS);
             constexpr bool STAGED = BITS != 8 && !(BITS == 4 && EPV == 8);
-            const unsigned lanes = nvec >= 32 ? 0xFFFFFFFFu : (1u << nvec) - 1u;       // those with a vector among the first 32
-            auto quantize = [&](int v) {                     // vector v: its quads to the output (8 bits: a quad is a word) or to `sw`
+            auto load = [&](int v) { return *reinterpret_cast<const uint4*>(row + QP_CK(v, nvec) * EPV); };
+            auto quantize = [&](int v, const uint4& r) {     // vector v: its quads to the output (8 bits: a quad is a word) or to `sw`
                 float e[EPV];
-                tok_lds<T>(row + QP_CK(v, nvec) * EPV, e);
-                if (STAGED && v < 32) __syncwarp(lanes);     // the first 32 vectors' quads lie where those vectors were, the others' behind
+                tok_widen<T>(r, e);
                 if constexpr (EPV == 4) {
                     const unsigned qd = qp_quad<BITS>(e, q.lo, q.hi, q.inv_scale);
                     if constexpr (BITS == 8) orow[v] = qd;
@@ -638,9 +645,30 @@ __global__ void __launch_bounds__(TR_WARPS * 32, TR_BLOCKS) tok_rows_kernel(cons
                 }
             };
             const int whole = nvec & ~31;
+            if constexpr (STAGED) {
+                // A round of 32 vectors leaves its quads where vectors of that round and of earlier ones were, which other lanes have
+                // read: all lanes load, then all store.
+                int v0 = 0;
+                for (; v0 + 32 * TR_ROUNDS <= whole; v0 += 32 * TR_ROUNDS) {
+                    uint4 r[TR_ROUNDS];
+#pragma unroll
+                    for (int u = 0; u < TR_ROUNDS; ++u) r[u] = load(v0 + 32 * u + lane);
+                    __syncwarp();
+#pragma unroll
+                    for (int u = 0; u < TR_ROUNDS; ++u) quantize(v0 + 32 * u + lane, r[u]);
+                }
+                for (; v0 < nvec; v0 += 32) {
+                    const bool mine = v0 + lane < nvec;
+                    uint4 r = make_uint4(0u, 0u, 0u, 0u);
+                    if (mine) r = load(v0 + lane);
+                    __syncwarp();
+                    if (mine) quantize(v0 + lane, r);
+                }
+            } else {
 #pragma unroll 4
-            for (int v0 = 0; v0 < whole; v0 += 32) quantize(v0 + lane);
-            if (whole + lane < nvec) quantize(whole + lane);
+                for (int v0 = 0; v0 < whole; v0 += 32) quantize(v0 + lane, load(v0 + lane));
+                if (whole + lane < nvec) quantize(whole + lane, load(whole + lane));
+            }
             if constexpr (STAGED) {
                 // quads across the warp: 32 elements = BITS words per lane
                 __syncwarp();

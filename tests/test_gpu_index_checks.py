@@ -26,7 +26,7 @@ SUBSET = ("test_stats_configs or test_stats_ragged or test_stats_special or stat
           "test_search_ragged or test_search_degenerate or test_fused_sender_c1 or fused_sender_special or "
           "test_channels_shapes or test_search_channels_vit or test_tokens_shapes or "
           "test_stats_streaming or test_sender_search_streaming or test_search_streaming_small or test_search_channels_strips or "
-          "test_tokens_rows_edges or beyond_fp32 or one_bit_blocks")
+          "test_tokens_rows or beyond_fp32 or one_bit_blocks")
 
 
 def test_small_cases_run_clean_under_the_index_checked_build():

@@ -1881,6 +1881,19 @@ def test_tokens_rows_edges(ctx, channels, bits):
     assert ctx.qp_get_status() == qp.QP_DEV_NONFINITE | qp.QP_DEV_DEGENERATE
 
 
+# the quads of 1 to 7 bits take the place of elements that other lanes read: rows of more than 512 channels, where a round's quads
+# lie over vectors of an earlier round, with whole groups of four rounds (fp32 512, bf16 1024 channels), single rounds and a partial one
+@pytest.mark.parametrize("bits", range(1, 8))
+@pytest.mark.parametrize("channels", [544, 800, 1280, 2080, 2816])
+def test_tokens_rows_in_place(ctx, channels, bits):
+    x = si.vit_activation((1, 21, channels), 530 + channels).reshape(-1)
+    check_tokens(ctx, x, dev(x), channels, bits)
+    h = si.to_bf16_bits(x)
+    d = torch.from_numpy(h.view(np.int16)).cuda().view(torch.bfloat16)
+    check_tokens(ctx, oracle.widen_bf16(h), d, channels, bits)
+    assert ctx.qp_get_status() == 0
+
+
 def test_tokens_misaligned_nonfinite_bf16_and_errors(ctx):
     x = si.vit_activation((1, 301, 96), 167, outlier_frac=0.03).reshape(-1).astype(np.float32)
     big = dev(np.concatenate([np.zeros(1, np.float32), x]))
