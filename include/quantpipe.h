@@ -128,7 +128,8 @@ int32_t qp_get_status(qp_ctx* ctx, void* stream);
  * wait give up at the first attempt that finds the copy still in flight.  (The second wait that
  * a block which gave up grants its own copies in flight before it leaves always keeps the
  * default.)  barrier_extra_arrivals = 1 makes every grid barrier wait for one arrival more
- * than there are blocks, so that it can only end by running out.  A wait that runs out
+ * than there are blocks, so that it can only end by running out; -k (k = 1..8) only the k-th one of
+ * a launch and those behind it.  A wait that runs out
  * raises QP_DEV_STREAM_TIMEOUT, the kernel leaves without output, and nothing faults.
  * Drops the stored graphs (they carry the old limits).  Errors: QP_ERR_INVALID_ARG. */
 int32_t qp_set_wait_limit_for_testing(qp_ctx* ctx, long long tile_wait_cycles, uint32_t barrier_polls,

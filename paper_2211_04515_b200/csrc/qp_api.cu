@@ -208,10 +208,10 @@ extern "C" int32_t qp_set_wait_limit_for_testing(qp_ctx* ctx, long long tile_wai
                                                  int barrier_extra_arrivals)
 {
     if (!ctx) return QP_ERR_INVALID_ARG;
-    if (barrier_extra_arrivals < 0 || barrier_extra_arrivals > 1) return qp_fail(ctx, QP_ERR_INVALID_ARG, "barrier_extra_arrivals");
+    if (barrier_extra_arrivals < -8 || barrier_extra_arrivals > 1) return qp_fail(ctx, QP_ERR_INVALID_ARG, "barrier_extra_arrivals");
     ctx->wait_cycles = tile_wait_cycles < 0 ? QP_WAIT_CYCLES_DEFAULT : tile_wait_cycles;
     ctx->spin_limit = barrier_polls == 0 ? QP_SPIN_LIMIT_DEFAULT : barrier_polls;
-    ctx->bar_extra = barrier_extra_arrivals;
+    ctx->bar_extra = barrier_extra_arrivals < 0 ? -barrier_extra_arrivals : barrier_extra_arrivals;
     qp_device_guard guard(ctx->device);
     qp_drop_graphs(ctx);                      // recorded launches carry the old limits
     return QP_OK;

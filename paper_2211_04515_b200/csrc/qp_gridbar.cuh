@@ -24,6 +24,10 @@ __device__ __forceinline__ void arrive_release(unsigned* p)
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
 }
 
+// Arrivals that a launch's barrier number `nr` (from 1 on) waits for.  extra: 0, or the number of the first barrier that a test makes
+// wait for one arrival more than there are blocks.
+__device__ __forceinline__ unsigned target(unsigned nr, unsigned blocks, unsigned extra) { return nr * blocks + (extra - 1u < nr ? 1u : 0u); }
+
 // One thread polls until `target` arrivals; false when the wait ran out.
 __device__ __forceinline__ bool poll(const unsigned* bar, unsigned target, unsigned spin_limit, unsigned* status)
 {

@@ -86,7 +86,7 @@ struct qp_ctx {
     int ct_clusters[9];                  // how many clusters of 1..8 blocks run at a time
     long long wait_cycles;               // limit of a wait for a tile copy (clock cycles)
     unsigned spin_limit;                 // limit of a grid-barrier wait (polls)
-    int bar_extra;                       // test only: arrivals a grid barrier waits for beyond the grid size
+    int bar_extra;                       // test only: number of a launch's first grid barrier that waits for one arrival too many (0: none)
     size_t fused_dyn_max;                // largest slice (bytes of dynamic shared memory) per block
     void* d_fused;                       // scratch of the cooperative kernels (QP_FUSED_BYTES, see below)
     void* d_ch_part;                     // channel-wise statistics: block partials, allocated on first use

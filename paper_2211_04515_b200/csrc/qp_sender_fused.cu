@@ -59,7 +59,7 @@ struct FsArgs {
     unsigned* bar;                                // arrival counter, zero at entry
     unsigned* status;
     unsigned spin_limit;                          // polls a grid-barrier wait may take
-    unsigned bar_extra;                           // 0; a test makes the barriers wait for more arrivals than blocks
+    unsigned bar_extra;                           // 0; a test makes the barriers from this one on wait for more arrivals than blocks
 };
 
 // Block reduction of N values at once; every thread gets the results, merged in warp order (the
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(FS_THREADS, 1) sender_fused_kernel(const FsArg
             p[0] = v5[0]; p[1] = v5[1]; p[2] = v5[2]; p[3] = v5[3]; p[4] = v5[4];
         }
     }
-    if (!qp_grid::barrier(a.bar, G + a.bar_extra, a.spin_limit, a.status, &s_ok)) return;
+    if (!qp_grid::barrier(a.bar, qp_grid::target(1, G, a.bar_extra), a.spin_limit, a.status, &s_ok)) return;
 
     // ---- phase 1: tensor-wide first moments (same in every block), then deviations and histogram
     double mean, mean_abs, mn_all, mx_all;
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(FS_THREADS, 1) sender_fused_kernel(const FsArg
                 if (c) atomicAdd(&a.hist[b], (unsigned long long)c);
             }
     }
-    if (!qp_grid::barrier(a.bar, 2 * G + a.bar_extra, a.spin_limit, a.status, &s_ok)) return;
+    if (!qp_grid::barrier(a.bar, qp_grid::target(2, G, a.bar_extra), a.spin_limit, a.status, &s_ok)) return;
 
     // ---- phase 2: statistics, then the clip range
     {
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(FS_THREADS, 1) sender_fused_kernel(const FsArg
             s_st.hist_bins = a.use_ds ? a.nb : 0;
             s_st.reserved = 0;
             if (blockIdx.x == 0) {
-                *a.st_out = s_st;
+                if (!a.use_ds) *a.st_out = s_st;               // (the search has a barrier yet: no output if that runs out)
                 if (nbad) atomicOr(a.status, QP_DEV_NONFINITE);
             }
             if (a.use_ds) {
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(FS_THREADS, 1) sender_fused_kernel(const FsArg
             for (int j = 0; j < per_group; ++j) t += s_acc[j * groups + cg][ck];
             a.sums[(size_t)blockIdx.x * (FS_MAX_STEPS + 1) + c] = t;
         }
-        if (!qp_grid::barrier(a.bar, 3 * G + a.bar_extra, a.spin_limit, a.status, &s_ok)) return;
+        if (!qp_grid::barrier(a.bar, qp_grid::target(3, G, a.bar_extra), a.spin_limit, a.status, &s_ok)) return;
 
         // ---- phase 3: error curve, first minimum wins.  The G block sums of a candidate are merged
         // by four threads, each over a quarter of the blocks in index order (loads issued in
@@ -414,6 +414,7 @@ __global__ void __launch_bounds__(FS_THREADS, 1) sender_fused_kernel(const FsArg
                 a.cand[k] = s_cand[k];
             }
             if (tid == 0) {
+                *a.st_out = s_st;
                 *a.setup = s_setup;
                 qp_ds_write_result(s_best, s_curve, s_setup, a.steps, a.nb, a.bits, s_cand[s_best], a.ds_out, a.qp_out,
                                    a.status);

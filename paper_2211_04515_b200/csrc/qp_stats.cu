@@ -655,7 +655,7 @@ __global__ void __launch_bounds__(SF_THREADS, 1) stats_fused_kernel(const SfArgs
         __syncthreads();
     };
     if (!ok) give_up();
-    const bool met = qp_grid::barrier(a.bar, (unsigned)G + a.bar_extra, a.spin_limit, a.status, &s_ok);
+    const bool met = qp_grid::barrier(a.bar, qp_grid::target(1, (unsigned)G, a.bar_extra), a.spin_limit, a.status, &s_ok);
     if (!met && threadIdx.x == 0) atomicExch(a.bar + 2, 1u);
     ok = ok && met && qp_grid::ld_acquire(a.bar + 2) == 0u;  // (the flag is read by all threads after the barrier's block barrier)
 

@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             if (threadIdx.x == 0) s_ok = 1;
             __syncwarp();
         } else if (threadIdx.x < 32) {
-            qp_grid::barrier_warp0(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
+            qp_grid::barrier_warp0(a.bar, qp_grid::target(waits, G, a.bar_extra), a.spin_limit, a.status, &s_ok);
         }
     };
     // this block's partial into row r, by warp 0, and every block's rows

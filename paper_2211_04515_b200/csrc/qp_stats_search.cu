@@ -677,7 +677,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
             return true;
         }
         ++waits;
-        return qp_grid::barrier(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
+        return qp_grid::barrier(a.bar, qp_grid::target(waits, G, a.bar_extra), a.spin_limit, a.status, &s_ok);
     };
     // for what warp 0 wrote and reads next; the others learn from s_ok behind the next block barrier
     auto meet_warp0 = [&]() {
@@ -688,7 +688,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
             if (threadIdx.x == 0) s_ok = 1;
             __syncwarp();
         } else if (threadIdx.x < 32) {
-            qp_grid::barrier_warp0(a.bar, waits * G + a.bar_extra, a.spin_limit, a.status, &s_ok);
+            qp_grid::barrier_warp0(a.bar, qp_grid::target(waits, G, a.bar_extra), a.spin_limit, a.status, &s_ok);
         }
     };
     auto empty = [&](int t, int threads) {                    // the tables, by threads t = 0 .. threads - 1
@@ -844,7 +844,7 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
                 }
                 s_st.hist_peak = (unsigned long long)peak;
                 s_st.hist_bins = a.nb;
-                if (STATS && (!SEARCH || blockIdx.x == 0)) {
+                if (!SEARCH) {                                // (the sender's go out with its result, behind its last barrier)
                     *a.st_out = s_st;
                     if (s_st.nonfinite) atomicOr(a.status, QP_DEV_NONFINITE);
                 }
@@ -1011,6 +1011,10 @@ __device__ __forceinline__ int ss_run(const SsArgs& a)
             if (threadIdx.x == SS_THREADS - 32) {             // (a warp that has a tile less to pack than the first, or none)
                 qp_ds_write_result(best, s_curve, s_setup, a.steps, a.nb, BITS, s_cand[best], a.ds_out, a.qp_out, a.status);
                 *a.setup = s_setup;
+            }
+            if (STATS && threadIdx.x == SS_THREADS - 64) {
+                *a.st_out = s_st;
+                if (s_st.nonfinite) atomicOr(a.status, QP_DEV_NONFINITE);
             }
             for (int k = threadIdx.x; k < ncand; k += SS_THREADS) {
                 a.curve[k] = s_curve[k];

@@ -136,6 +136,52 @@ def test_default_launch_whose_barrier_runs_out_leaves_no_trace(call, n):
     c.close()
 
 
+# the same with the later barriers of a launch: what the ones before them have told is not written either
+@pytest.mark.parametrize("call,n,barriers", [("stats", 300 * 1024 + 5, 2), ("stats", 96 << 18, 3), ("search_counts", 300 * 1024 + 5, 2),
+                                             ("sender_search", 300 * 1024 + 5, 3), ("sender_one_bit", 300 * 1024 + 5, 2),
+                                             ("sender", 300 * 1024 + 5, 2), ("sender_fused", 300 * 1024 + 5, 2),
+                                             ("sender_fused_search", 300 * 1024 + 5, 3)])
+def test_a_later_barrier_that_runs_out_leaves_no_output(call, n, barriers):
+    c = qp.Context(0)
+    d = dev(np.resize(si.vit_activation((1, 1024, 1024), 306).reshape(-1), n))
+    d_stats = c.qp_stats(d)
+    fused = "fused" in call
+    c.qp_set_sender_path(qp.QP_SENDER_FUSED if fused else qp.QP_SENDER_AUTO)
+    bits = 1 if call == "sender_one_bit" else 2
+    sizes = {"stats": [ctypes.sizeof(qp.Stats)],
+             "search": [ctypes.sizeof(qp.DSResult), ctypes.sizeof(qp.QParams)],
+             "sender": [qp.qp_packed_bytes(n, bits), ctypes.sizeof(qp.QParams), ctypes.sizeof(qp.Stats)]}[call.split("_")[0]]
+
+    def run():
+        out = [torch.full((b,), 0xEE, dtype=torch.uint8, device="cuda") for b in sizes]
+        before = c.qp_launch_count()
+        if call == "stats":
+            c.qp_stats(d, out=out[0])
+        elif call == "search_counts":
+            c.qp_dsaciq_search(d, d_stats, 2, out_result=out[0], out_qp=out[1])
+        else:
+            c.qp_sender_device(d, bits, call not in ("sender", "sender_fused"), out_packed=out[0], out_qp=out[1], out_stats=out[2])
+        assert c.qp_launch_count() - before == 1
+        torch.cuda.synchronize()
+        return out
+
+    want = run()
+    for nr in range(2, barriers + 1):
+        c.qp_set_wait_limit_for_testing(barrier_polls=500, barrier_extra_arrivals=-nr)
+        assert all(bool((o == 0xEE).all()) for o in run()), nr
+        c.qp_set_wait_limit_for_testing()
+        if not fused:                                    # (the small-tensor sender's scratch is put back by qp_get_status)
+            assert all(torch.equal(a, b) for a, b in zip(run(), want))
+        with pytest.raises(qp.QuantPipeError) as e:
+            c.qp_get_status()
+        assert e.value.status == qp.QP_ERR_TIMEOUT
+        assert all(torch.equal(a, b) for a, b in zip(run(), want))
+        assert c.qp_get_status() == 0
+    with pytest.raises(qp.QuantPipeError):
+        c.qp_set_wait_limit_for_testing(barrier_extra_arrivals=-9)
+    c.close()
+
+
 def test_graph_replay_keeps_calls_with_different_options_apart():
     """Stored graphs are keyed by every argument.  Pairs of calls that differ only in the clip method
     and the histogram's bin count (fields that once shared bits of one key word) must each replay
