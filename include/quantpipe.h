@@ -539,14 +539,14 @@ int32_t qp_sender_tokens_device(qp_ctx* ctx, const void* d_x, int dtype, uint64_
  *                    the sums are merged in another order: statistics agree with the chain to
  *                    ~1e-15 relative, the error curve to ~1e-6, so the clip range can differ in
  *                    its last fp32 bit or, where two steps of the search tie, by one step.
- *   QP_SENDER_AUTO   the default.  For 16-byte aligned tensors a streaming launch that reads x again for
- *                    every step (closed-form clips up to 2^18 elements and above
- *                    2.6e6, bf16 up to 2^26; the search at 1..4 bits from 2^15, 3 * 2^16 or 3 * 2^17
- *                    elements (up to 2, 3 and 4 bits) to 1.9e6 and above 2^21); else fused for n <= 2^20
- *                    with the search and n <= 2^21 otherwise; else the chain.  The fastest of the
- *                    three on a B200 but for what lies between those ranges: above 1.9e6 up to 2^21
- *                    elements with the search and above 2^21 up to 2.6e6 without, the chain takes 6 us
- *                    longer than one launch would
+ *   QP_SENDER_AUTO   the default.  For 16-byte aligned tensors and packed streams, from 8192 elements on, a
+ *                    streaming launch that reads x again for every step: closed-form clips at 1..8 and
+ *                    16 bits up to 2^21 elements and above 2^21 + 2^19 (bf16 up to 2^26), the search at
+ *                    1..4 bits (at 4 from 128 KB on; steps <= 255, hist_bins <= 4096) up to 15 * 2^17
+ *                    elements and above 2^21; else fused for n <= 2^20 with the search and
+ *                    n <= 2^21 otherwise; else the chain.  The fastest of the three on a B200 but for what
+ *                    lies between those ranges: with the search (2.02e6 fp32 elements) the chain takes 14 to
+ *                    17 us longer there than one launch would, with a closed-form clip 10
  * A grid barrier that does not complete within about a quarter of a second sets
  * QP_DEV_STREAM_TIMEOUT in the status word and the launch ends without output
  * (qp_get_status then returns QP_ERR_TIMEOUT). */
