@@ -237,6 +237,8 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
     const unsigned G = gridDim.x;
     const uint64_t step = (uint64_t)G * SS_WARPS, first = ss_first_tile(a.ntiles, step);
     const uint64_t tail0 = a.ntiles * SS_TILE;
+    // (16 bits an element take one pass from 224 MB on, which is beyond what the sender brings here: no pilot and no window in its code)
+    const bool one = (sizeof(T) == 4 || BITS == 0) && a.one;
     const double inf = __longlong_as_double(0x7FF0000000000000ll);
     unsigned* table = reinterpret_cast<unsigned*>(raw);
     uint4* part = a.part + blockIdx.x;             // this block's: row r at part[r * G]
@@ -270,14 +272,14 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
     auto leave = [&](unsigned gave_up) {
         if (threadIdx.x == 0 && qp_grid::last_out(qp_grid::count_out(a.bar, gave_up), G)) qp_grid::reset(a.bar);
     };
-    if (a.one)                                                // the window's table
+    if (one)                                                  // the window's table
         for (int i = threadIdx.x; i < (int)(OP_DYN_BYTES / 16); i += SS_THREADS) reinterpret_cast<uint4*>(raw)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x == 0) s_full = 0;
 
     // ---- pilot: sample i, four neighbouring vectors (the bytes of one DRAM burst) by four lanes, lies at a random place of
     // the i-th of equal parts of the tensor
     float c = 0.f, delta = 1.f;
-    if (a.one) {
+    if (one) {
         const uint64_t nv4 = a.n / (4 * EPV);
         const unsigned total = (unsigned)a.sample * G * (SS_THREADS / 4);
         const uint64_t each = nv4 / total;                    // >= 1
@@ -366,10 +368,10 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
         }
         tail.each([&](float v) {
             o.one(v, c);
-            if (a.one && qp_is_finite(v)) f.window(__fsub_rn(v, c));
+            if (one && qp_is_finite(v)) f.window(__fsub_rn(v, c));
         });
     };
-    if (a.one) {
+    if (one) {
         OpPass<true> f;
         pass(f);
     } else {
@@ -380,11 +382,11 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
         if (a.cluster) qp_grid::cluster_wait();
         const SsParts v = ss_block_parts<true>({o.sy, o.sx, o.mn, o.mx, o.bad}, s_block[1]);       // (its barrier also orders the window's counters)
         SsParts u = {0.0, 0.0, 0.f, 0.f, 0u};
-        if (a.one) u = ss_block_parts<false>({o.sa, o.sv, 0.f, 0.f, o.below}, s_block[2]);
+        if (one) u = ss_block_parts<false>({o.sa, o.sv, 0.f, 0.f, o.below}, s_block[2]);
         if (threadIdx.x < 32) {
             put(OP_PASS, ss_row(v.a, v.b));
             put(OP_PASS + 1, make_uint4(__float_as_uint(v.lo), __float_as_uint(v.hi), v.count, u.count));
-            if (a.one) put(OP_PASS + 2, ss_row(u.a, u.b));
+            if (one) put(OP_PASS + 2, ss_row(u.a, u.b));
         }
     }
     meet_warp0();
@@ -398,7 +400,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             mx = fmaxf(mx, __uint_as_float(q.y));
             bad += (double)q.z;                               // exact: counts are far below 2^53
         };
-        if (a.one) {
+        if (one) {
             merge(Rows<3>{}, OP_PASS, [&](const uint4 (&p)[3]) {
                 first_two(p[0], p[1]);
                 below += (double)p[1].w;
@@ -414,7 +416,7 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
         bad = ss_pair_sum(bad, below);
         sx = __shfl_sync(0xFFFFFFFFu, sy, 16);
         mx = -__shfl_sync(0xFFFFFFFFu, mn, 16);
-        if (a.one) {
+        if (one) {
             sa = ss_pair_sum(sa, sv);
             sv = __shfl_sync(0xFFFFFFFFu, sa, 16);
             below = __shfl_sync(0xFFFFFFFFu, bad, 16);
@@ -432,19 +434,19 @@ __global__ void __launch_bounds__(SS_THREADS, 1) stats_onepass_kernel(const OpAr
             s_st.hist_peak = 0;
             s_st.hist_bins = 0;
             s_st.reserved = 0;
-            if (a.one) {
+            if (one) {
                 s_st.var = nf > 0.0 ? fmax(0.0, sv / nf - D * D) : 0.0;
                 s_D = D;
                 s_abs = sa;
                 s_below = below;
             }
-            s_again = !a.one || !(fabs(D) < (double)delta) || !(sv < inf);
+            s_again = !one || !(fabs(D) < (double)delta) || !(sv < inf);
         }
     }
     __syncthreads();
     if (!s_ok) { leave(qp_grid::GAVE_UP); return; }
     // ---- this block's share of the elements between c and the mean
-    if (!s_again) {                                           // uniform over the grid
+    if (one && !s_again) {                                    // uniform over the grid
         const double D = s_D;
         const int side = D < 0.0;
         const float aD = (float)fabs(D);
