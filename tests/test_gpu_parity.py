@@ -1188,7 +1188,7 @@ def test_search_bf16_at_128_kb(ctx, n):
     assert ctx.qp_get_status() == 0
 
 
-# statistics about a pilot centre (96 MB and more: 25165824 fp32 elements) and in two streaming passes (below), tiles of 1024
+# statistics about a pilot centre (fp32 of 96 MB and more: 25165824 elements) and in two streaming passes (below, bf16), tiles of 1024
 # elements, 16 warps a block; with the closed-form sender from 2^21 + 2^19 elements.  Data that the one pass cannot
 # finish ("mass", "two_levels") or finishes at once, and elements that its sums must leave out.
 @pytest.mark.parametrize("n,data,bf16", [(8 * 1024, "plain", False), ((1 << 15) + 1, "plain", True), (1 << 18, "outliers", False),
@@ -1236,19 +1236,43 @@ def test_stats_streaming(ctx, n, data, bf16):
 
 
 # bf16 on both sides of the line between two passes and one (224 MB): every block of rows against sums in 64 bits (fp32 chains of
-# at most 16 terms: 16 * 2^-24; the one pass accepts 1e-8 beside them), and the sender's quantizer from those statistics
-@pytest.mark.parametrize("n", [(112 << 20) - 1, 112 << 20])
-def test_stats_bf16_on_both_sides_of_the_one_pass_line(ctx, n):
+# at most 16 terms: 16 * 2^-24; the one pass accepts 1e-8 beside them), and the sender's quantizer from those statistics.  Ragged
+# tensors with elements that the sums must leave out, and data that the one pass cannot finish, as for fp32 above.
+@pytest.mark.parametrize("n,data", [((112 << 20) - 1, "plain"), (112 << 20, "plain"), ((112 << 20) + 1025, "nonfinite"),
+                                    ((112 << 20) + 9, "mass"), ((112 << 20) + 1023, "two_levels"), (112 << 20, "constant"),
+                                    ((112 << 20) + 5, "offset")])
+def test_stats_bf16_on_both_sides_of_the_one_pass_line(ctx, n, data):
     g = torch.Generator(device="cuda").manual_seed(n % 97)
-    x = (torch.randn(n, device="cuda", generator=g) * 0.7 + 0.1).to(torch.bfloat16)
-    st = ctx.read_stats(ctx.qp_stats(x))
-    parts = [c.double() for c in x.split(1 << 24)]
-    mean = sum(float(c.sum()) for c in parts) / n
-    mad, var, ab = (sum(float(f(c).sum()) for c in parts) / n for f in (lambda c: (c - mean).abs(), lambda c: (c - mean) ** 2, lambda c: c.abs()))
-    assert (st.n, st.nonfinite, st.min, st.max) == (n, 0, float(x.min()), float(x.max()))
+    x = torch.randn(n, device="cuda", generator=g) * 0.7 + 0.1
+    if data == "nonfinite":
+        x[[0, 1023, n // 2, n - 1]] = torch.tensor([np.nan, np.inf, -np.inf, np.nan], device="cuda")
+    elif data == "mass":                                 # half of the elements at the mean
+        x -= 0.1
+        x[::2] = 0.0
+    elif data == "two_levels":
+        x[:] = 2.0
+        x[::3] = -1.0
+    elif data == "constant":
+        x[:] = -2.5
+    elif data == "offset":
+        x += 500.0
+    x = x.to(torch.bfloat16)
+    out = ctx.qp_stats(x)
+    st = ctx.read_stats(out)
+    parts = [c[torch.isfinite(c)].double() for c in x.split(1 << 24)]
+    nf = sum(c.numel() for c in parts)
+    mean = sum(float(c.sum()) for c in parts) / nf
+    mad, var, ab = (sum(float(f(c).sum()) for c in parts) / nf for f in (lambda c: (c - mean).abs(), lambda c: (c - mean) ** 2, lambda c: c.abs()))
+    assert (st.n, st.nonfinite) == (n, n - nf) and n - nf == (4 if data == "nonfinite" else 0)
+    assert (st.min, st.max) == (min(float(c.min()) for c in parts), max(float(c.max()) for c in parts))
     assert abs(st.mean - mean) <= 1e-6 * ab and abs(st.mad - mad) <= 1e-6 * mad and abs(st.var - var) <= 1e-6 * var
     assert abs(st.mean_abs - ab) <= 1e-6 * ab
-    assert ctx.qp_get_status() == 0
+    assert bytes(st) == bytes(ctx.read_stats(ctx.qp_stats(x)))
+    packed, q = ctx.qp_sender_device(x, 6, False)        # (bf16 of this size goes through the separate calls' launches)
+    want = ctx.qp_clip_qparams_device(out, 6, qp.QP_CLIP_ACIQ)
+    assert torch.equal(q.view(torch.uint8).reshape(-1), want.view(torch.uint8).reshape(-1))
+    assert torch.equal(packed, ctx.qp_quantize_pack(x, 6, want))
+    assert ctx.qp_get_status() == (qp.QP_DEV_NONFINITE if data == "nonfinite" else qp.QP_DEV_DEGENERATE if data == "constant" else 0)
 
 
 # statistics and search in one launch (the default from 8192 elements on, 32768 at 4 bits, the sender by width): every width it takes, tile
