@@ -563,6 +563,11 @@ constexpr int TR_WARPS = 8;                                   // warps per block
 // at 4 and 8 bits 41.3 -> 39.0 and 37.2 -> 36.3 us, 16000 x 2048 at 8 bits 41.1 -> 35.3, 40000 x 192 bf16 at 4 bits 28.4 -> 26.7; six
 // (40 registers) are slower again (39.2, 37.1, 37.0).
 constexpr int TR_BLOCKS = 5;
+// Statistics of rows so long that shared memory has no room for five blocks keep 64 registers: 12608 rows of 2048, 2560 and 3072 fp32
+// channels 22.4, 31.3 and 34.1 us with 48, 21.5, 30.1 and 33.5 with 64 (no bound: 21.3, 29.5 and 33.3, but 18.0 at 1600 against
+// 16.9).  The sender's gain or lose 1 to 3 % by width and type, on both sides of nothing.
+constexpr int TR_LONG_BLOCKS = 4;
+constexpr size_t TR_SM_BYTES = 228 * 1024;                    // shared memory of an SM, of which a block takes 1 KB more than it asks for
 // Rounds of 32 vectors that the staged widths load before they store.  One, two and four of them, 12608 rows of 1280 fp32 at 5 bits:
 // 21.9, 20.6 and 20.8 us, 2560 bf16 at 6: 32.9, 31.8 and 31.5, 2560 fp32 at 4: 43.1, 41.1 and 41.1 (quads in a room of their own, four
 // blocks an SM: 22.2, 32.9 and 41.1).
@@ -574,8 +579,8 @@ __host__ __device__ constexpr size_t tok_row_bytes(uint32_t C, size_t esz) { ret
 
 // BITS = 0: statistics only (any row of whole vectors).  BITS = 1..8: the whole sender, rows of whole
 // 32-element groups (a row is then whole words).
-template <int BITS, typename T>
-__global__ void __launch_bounds__(TR_WARPS * 32, TR_BLOCKS) tok_rows_kernel(const T* __restrict__ x, uint64_t tokens, uint32_t C, int method,
+template <int BITS, typename T, int BLOCKS>
+__global__ void __launch_bounds__(TR_WARPS * 32, BLOCKS) tok_rows_kernel(const T* __restrict__ x, uint64_t tokens, uint32_t C, int method,
                                                                  int bmode, double F, uint32_t* __restrict__ out,
                                                                  uint64_t nwords, qp_qparams_t* __restrict__ qp_out,
                                                                  qp_stats_t* __restrict__ st_out, unsigned* __restrict__ status)
@@ -777,7 +782,8 @@ int32_t unpack_tokens_typed(qp_ctx* ctx, const void* d_packed, uint64_t n, uint3
 }
 
 // Rows go through shared memory where a row fits: TR_WARPS of them in the 48 KB every block may have would
-// stop at 1536 fp32 channels; blocks ask for more, up to what leaves two blocks (16 warps) per SM.
+// stop at 1536 fp32 channels; blocks ask for more, up to what leaves two blocks (16 warps) per SM.  The sender's rows stop
+// a byte per element earlier, at 2848 fp32 and 4768 bf16 channels: quads had room of their own when that line was measured.
 constexpr size_t TR_SMEM_MAX = 112 * 1024;
 bool tok_rows_apply(const void* x, int dtype, uint32_t C, bool sender)
 {
@@ -792,11 +798,12 @@ int32_t launch_rows(qp_ctx* ctx, const T* x, uint64_t tokens, uint32_t C, int me
                     qp_qparams_t* d_qp, qp_stats_t* d_stats, cudaStream_t s)
 {
     const size_t smem = tok_row_bytes(C, sizeof(T)) * TR_WARPS;
-    if (smem > 48 * 1024 && cudaFuncSetAttribute(tok_rows_kernel<BITS, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)TR_SMEM_MAX) != cudaSuccess)
+    const bool five = TR_BLOCKS * (smem + 1024) <= TR_SM_BYTES;
+    const auto kernel = five ? tok_rows_kernel<BITS, T, TR_BLOCKS> : tok_rows_kernel<BITS, T, BITS == 0 ? TR_LONG_BLOCKS : TR_BLOCKS>;
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TR_SMEM_MAX) != cudaSuccess)
         return qp_check_launch(ctx, "token rows (shared memory)");
     const uint64_t want = (tokens + TR_WARPS - 1) / TR_WARPS, cap = (uint64_t)ctx->sm_count * 64;
-    tok_rows_kernel<BITS, T><<<(unsigned)(want < cap ? want : cap), TR_WARPS * 32, smem, s>>>(
+    kernel<<<(unsigned)(want < cap ? want : cap), TR_WARPS * 32, smem, s>>>(
         x, tokens, C, method, bmode, BITS > 0 ? qp_host_aciq_F(BITS, QP_DIST_LAPLACE) : 0.0, out,
         BITS > 0 ? qp_packed_bytes(tokens * C, BITS) / 4 : 0, d_qp, d_stats, ctx->d_status);
     ctx->launches += 1;

@@ -1918,6 +1918,23 @@ def test_tokens_rows_in_place(ctx, channels, bits):
     assert ctx.qp_get_status() == 0
 
 
+# statistics of rows on both sides of the line behind which shared memory holds fewer than five blocks (1427 fp32, 2854 bf16
+# channels), with rows of whole vectors that are no whole groups, up to the longest rows in shared memory
+@pytest.mark.parametrize("channels,bf16", [(1424, False), (1428, False), (3584, False), (2848, True), (2856, True), (7168, True)])
+def test_tokens_rows_statistics_of_long_rows(ctx, channels, bf16):
+    x = si.vit_activation((1, 37, channels), 560 + channels).reshape(-1)
+    d = dev(x)
+    if bf16:
+        h = si.to_bf16_bits(x)
+        d, x = torch.from_numpy(h.view(np.int16)).cuda().view(torch.bfloat16), oracle.widen_bf16(h)
+    before = ctx.qp_launch_count()
+    out = ctx.qp_stats_tokens(d, channels)
+    assert ctx.qp_launch_count() - before == 1
+    for st, st_o in zip(_read_array(out, qp.Stats, 37), oracle.stats_tokens(x, channels)):
+        check_stats(st, st_o)
+    assert ctx.qp_get_status() == 0
+
+
 def test_tokens_misaligned_nonfinite_bf16_and_errors(ctx):
     x = si.vit_activation((1, 301, 96), 167, outlier_frac=0.03).reshape(-1).astype(np.float32)
     big = dev(np.concatenate([np.zeros(1, np.float32), x]))
