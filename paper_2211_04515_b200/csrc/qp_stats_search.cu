@@ -198,7 +198,7 @@ struct SsDeviationsOf {                                       // the stream's vi
 };
 
 // The guarded pass, out of line: inlined, its code moves the compiler's schedule of the ordinary pass (128-image search sender
-// 117.8 us inlined, 113.1 as a call; 64 images at 4 bits 62.9 and 62.1).
+// 101.3 us inlined, 98.9 as a call; 64 images at 4 bits 47.7 and 45.9).
 template <typename T>
 __device__ __noinline__ void ss_guarded_deviations(const T* x, uint64_t ntiles, uint64_t first, uint64_t step, int lane, SsDeviations& d)
 {
@@ -1092,9 +1092,10 @@ bool ss_usable(qp_ctx* ctx)
 }  // namespace
 
 // 16-byte aligned tensors; statistics with the histogram from 128 KB on (where qp_stats_carries_histogram says so), the search
-// from 8 tiles on, at 4 bits from 128 KB: 12 to 23 us by width up to 2^20 elements, where the candidates scored one by one take 23 us at
-// 2^15, 33 at 2^18 and 60 at 2^20.  (Below 128 KB the statistics carry no histogram and the launch counts it as well: 17 to 28 us at 1..3
-// bits, 33 at 4, against 25 to 29.)  At 1..4 bits (each further code boundary costs two instructions per element: at 5 bits and up the
+// from 8 tiles on, at 4 bits from 128 KB: 8.4 to 17.2 us by width up to 2^20 elements, where the candidates scored one by one take 23 us at
+// 2^15, 36 at 2^18 and 62 at 2^20.  Below 128 KB the statistics carry no histogram and the launch counts it as well: fp32 of 8192 to
+// 32760 elements 13 to 15 us at 1 bit, 16 to 18 at 2, 17 to 19 at 3 and 19 to 21 at 4, against 25 to 27.  (The line at 4 bits was drawn
+// when the launch took 33 us there.)  At 1..4 bits (each further code boundary costs two instructions per element: at 5 bits and up the
 // interval pass with its table is the cheaper one) and up to 256 candidates (tables that leave a replica to every
 // eighth lane at least).
 bool qp_stats_search_applies(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int hist_bins, int bits, int steps)

@@ -241,8 +241,9 @@ struct SsTail {
 // ---- launches whose blocks wait for one another: a cooperative grid, or one thread-block cluster
 constexpr unsigned QP_CLUSTER_BLOCKS = 16;        // the largest cluster (above 8: by attribute, where the device has the SMs)
 
-// One cluster while every warp of it has at most one tile; the search with 2 bits at 2^17, 2^18 and 3 * 2^17 elements takes 23,
-// 24.7 and 28.8 us in a cluster, 26.7, 28.1 and 28.8 in a grid, at 2^20 35 and 28.8.
+// One cluster while every warp of it has at most one tile.  The search sender with 2 bits at 2^17, 2^18, 3 * 2^17 and 2^20 fp32 elements
+// takes 19.6, 20.9, 23.0 and 31.2 us in a cluster, 22.6, 22.9, 23.0 and 23.0 in a grid; the closed form at 8 bits 10.6, 10.6, 11.6 and
+// 16.1, and 12.7 in a grid.
 constexpr uint64_t QP_CLUSTER_MAX_N = (uint64_t)QP_CLUSTER_BLOCKS * SS_WARPS * SS_TILE;
 
 inline cudaLaunchConfig_t qp_cluster_config(cudaLaunchAttribute* at, unsigned G, unsigned threads, size_t bytes, cudaStream_t s)
