@@ -43,14 +43,14 @@ MIN_TIMED_S = 0.5              # the K-step region is repeated until this much d
 # digest of the kernel's source files at capture time: when those files have changed since, the entry
 # is stale and the benchmark reports traffic = null.
 NCU_TRAFFIC = {
-    "stats": {"bytes": 135.7e6, "kernel": "stats_onepass_kernel<float, 0>", "summary": "profiles/streaming_kernels.md",
-              "files": ("qp_stats_onepass.cu", "qp_tiles.cuh", "qp_gridbar.cuh", "qp_packtile.cuh", "qp_internal.cuh"), "digest": "7cb53f6d6fbec9d3"},
-    "clip": {"bytes": 132.4e6, "kernel": "stats_search_kernel<float, 0, 1>", "summary": "profiles/streaming_kernels.md",
-             "files": ("qp_stats_search.cu", "qp_affine.cuh", "qp_tiles.cuh", "qp_gridbar.cuh", "qp_packtile.cuh", "qp_internal.cuh"), "digest": "70dfab9c8e2d3d6e"},
-    "quantize_pack": {"bytes": 144.4e6, "kernel": "pack_kernel<8, float>", "summary": "profiles/streaming_kernels.md",
-                      "files": ("qp_pack.cu", "qp_packtile.cuh", "qp_internal.cuh"), "digest": "d5a2f9791cf70b2f"},
-    "unpack_dequantize": {"bytes": 103.2e6, "kernel": "unpack_kernel<8, float>", "summary": "profiles/streaming_kernels.md",
-                          "files": ("qp_unpack.cu", "qp_internal.cuh"), "digest": "e449d247ca7d5ff2"},
+    "stats": {"bytes": 136.3e6, "kernel": "stats_onepass_kernel<float, 0>", "summary": "profiles/streaming_kernels.md",
+              "files": ("qp_stats_onepass.cu", "qp_tiles.cuh", "qp_gridbar.cuh", "qp_packtile.cuh", "qp_internal.cuh"), "digest": "f86f79566c4d7e9f"},
+    "clip": {"bytes": 133.1e6, "kernel": "stats_search_kernel<float, 0, 1>", "summary": "profiles/streaming_kernels.md",
+             "files": ("qp_stats_search.cu", "qp_affine.cuh", "qp_tiles.cuh", "qp_gridbar.cuh", "qp_packtile.cuh", "qp_internal.cuh"), "digest": "d4939068129ced64"},
+    "quantize_pack": {"bytes": 144.3e6, "kernel": "pack_kernel<8, float>", "summary": "profiles/streaming_kernels.md",
+                      "files": ("qp_pack.cu", "qp_packtile.cuh", "qp_internal.cuh"), "digest": "97210ccaf7acdd41"},
+    "unpack_dequantize": {"bytes": 103.3e6, "kernel": "unpack_kernel<8, float>", "summary": "profiles/streaming_kernels.md",
+                          "files": ("qp_unpack.cu", "qp_internal.cuh"), "digest": "609e925b9ae2cbdd"},
 }
 
 

@@ -914,10 +914,10 @@ int32_t qp_launch_stats(qp_ctx* ctx, const void* d_x, int dtype, uint64_t n, int
     }
     const uint64_t ntiles = ((uintptr_t)d_x & 15u) ? 0 : n * (dtype == QP_F32 ? 4 : 2) / ST_TILE;
     // QP_STATS_AUTO takes the streaming launches wherever they apply: 11.5 us at 2^20 fp32 elements against 15.3 in one launch of
-    // bulk-copied tiles and 17.5 in two kernels, 101 against 152 and 159 at 2^27; with the histogram 23.5 us for 52 MB, 27.3 and 35.4.  But fp32 with the
-    // histogram above 2^25 elements: there the bulk-copied tiles, the last of which stay in shared memory for the second pass, read
-    // DRAM faster: 2^25, 2^26, 2^27 and 2^28 elements in 53, 90, 165 and 319 us, streaming 53, 97, 185 and 361, two kernels 59,
-    // 98, 177 and 331.  (bf16 is bound by its instructions: streaming 211 us at 2^28, 279 and 233 in the others.)
+    // bulk-copied tiles and 17.5 in two kernels, 101 against 152 and 159 at 2^27; with the histogram 23.5 us for 52 MB, against 27.3 and
+    // 35.4.  But fp32 with the histogram above 2^25 elements: there the bulk-copied tiles, the last of which stay in shared memory for the second pass, read
+    // DRAM faster: 2^25, 2^26, 2^27 and 2^28 elements in 53, 90, 165 and 313 us, streaming 52, 95, 179 and 348, two kernels 62,
+    // 99, 177 and 350.  (bf16 is bound by its instructions: streaming 205 us at 2^28, 271 and 229 in the others.)
     // QP_STATS_FUSED and QP_STATS_TWO_KERNELS force the other two.
     const bool with_hist = hist_bins >= 1 && hist_bins <= ST_FUSED_HIST_MAX;
     const bool tiles = with_hist && dtype == QP_F32 && n > (1ull << 25) && ntiles >= 8 && stats_fused_usable(ctx);
